@@ -54,7 +54,10 @@ enum { OSAM_LINEAR_ELASTIC = 0, OSAM_NEO_HOOKEAN = 1, OSAM_SAINT_VENANT_KIRCHHOF
  * Newmark (beta = 1/4, gamma = 1/2, average acceleration) */
 enum { OSAM_EXPLICIT = 0, OSAM_IMPLICIT = 1 };
 enum { OSAM_MULTIPLICATIVE = 0, OSAM_ADDITIVE = 1 };
-/* OSAM_FP64: native FP64 everywhere.  OSAM_FP32_FORCE: internal force in FP32 (checked to 1e-5).
+/* OSAM_FP64: FP64 state and arithmetic; the internal force of explicit Neo-Hookean subdomains whose scatter
+ * is OSAM_SCATTER_AUTO is evaluated in 64-bit fixed point with an error below native FP64's (elements
+ * outside its range -- displacement gradients of order one half, displacements beyond 12 element edges --
+ * in native FP64).  OSAM_FP32_FORCE: internal force in FP32 (checked to 1e-5).
  * OSAM_F32X2_FORCE: internal force in double-float arithmetic (pairs of FP32 values, ~48-bit
  * significands) on the FP32 pipes, state and time integration in FP64 (checked to 1e-9 like FP64);
  * uses the deterministic gather scatter.  OSAM_FP64_TANGENT32: OSAM_FP64, except that the Newton
@@ -70,7 +73,8 @@ enum { OSAM_FP64 = 0, OSAM_FP32_FORCE = 1, OSAM_F32X2_FORCE = 2, OSAM_FP64_TANGE
  * GATHER_TILED the gather scheme with the FP64 force evaluated by 8x4x4 element tiles that share
  * their edge interpolation (same results bit for bit), GATHER_TILED_LOWREG the tiled kernel capped at
  * 128 registers (4 instead of 3 resident tiles per SM); the FP32 variants ignore these.  AUTO times
- * the candidates at initialisation and keeps the fastest */
+ * the candidates at initialisation and keeps the fastest (explicit Neo-Hookean FP64 subdomains: element
+ * blocks of the fixed-point force, gather scheme) */
 enum {
     OSAM_SCATTER_AUTO = 0,
     OSAM_SCATTER_ATOMIC = 1,

@@ -44,7 +44,7 @@ int fom_substep(osam_ctx* ctx, int s, int j, const int* active, long long ne) {
         for (CplH& c : ctx->cpls)
             if (c.src == s) LK(launch_trace_b(c.d, active, g, g.u[j & 1], j, ctx->stream));
     const int pk = ctx->prof_begin();
-    LK(launch_force_b(g, active, ctx->scatter, ctx->stream, fuse ? &tr : nullptr));
+    LK(launch_force_b(g, active, ctx->scatter, ctx->stream, fuse ? &tr : nullptr, X));
     ctx->prof_end(pk, ne);
     LK(launch_node_b(g, active, ctx->scatter, j + 1, (j + 2 <= S.nsub) ? j + 2 : -1, 0, X, Y, S.dt, ctx->stream));
     return OSAM_OK;

@@ -1,0 +1,238 @@
+// Neo-Hookean internal force and explicit node update in 64-bit fixed point (fixed_math.cuh).
+//
+// The force of the FP64 explicit path when the launch is left to the library: one thread per element, the
+// predicted displacement read as fixed-point u / h (written by the node kernel), the element forces left
+// as 64-bit integers in the element buffer, so the node kernel's sums are exact and cost integer
+// additions.  An element outside the range of the formats is evaluated in FP64 (far_element) into a second
+// buffer and marked in the first.
+//
+// k_force_fx_b is bound by the integer multiply-add pipe: ncu counts 1969 instructions on it and 2994 on
+// the integer ALU per warp, against 717 FP64 instructions (67 to 80 cycles each) of the tiled FP64 kernel.
+// Measured on 40x40x80: 43 us per launch, 186 us for the FP64 kernel; on 96x96x192 480 us, 2360 us.
+// The Gauss points are fully unrolled (43.4 us; with the two planes as a loop 45.3), 255 registers and
+// two warps per scheduler: capping at 168 or 128 registers (480 to 680 bytes of spills read back per thread)
+// measured 45.3 and 47.5 us on 40x40x80, 510 and 523 us on 96x96x192.
+#include <cuda_runtime.h>
+
+#include <cstdint>
+
+#include "fixed_math.cuh"
+#include "hex8_math.cuh"
+#include "osam_internal.h"
+#include "trace_item.cuh"
+
+namespace osam {
+
+namespace {
+
+using namespace fx;
+
+// Fixed-point material factor of a positive FP64 value below 2^k (62 fraction bits of value / 2^k)
+__device__ __forceinline__ i64 fixed_factor(double m, int k) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(m);
+    const int s = (int)(b >> 52) - 1023 - k + 10;    // 62 - 52 bits, scaled by 2^(e - k)
+    const i64 v = (i64)((b & 0xfffffffffffffULL) | 0x10000000000000ULL);
+    if (s >= 0) return shl(v, s);
+    return s < -53 ? 0 : (v + ((i64)1 << (-s - 1))) >> -s;
+}
+
+// Element e in FP64: its 24 contributions go to fe2, the fixed-point buffer gets the mark.  Not inlined,
+// so that its registers and code stay out of the fixed-point path.
+__device__ __noinline__ void far_element(const FomB& g, const InstFom& I, const double* u, int e, int n0) {
+    using namespace hex8;
+    const int sy = I.nx + 1, sz = (I.nx + 1) * (I.ny + 1);
+    double m1, m2, m3;
+    if (I.lam_e || I.mu_e)
+        material_factors<OSAM_NEO_HOOKEAN, double>(I.lam_e ? I.lam_e[e] : I.lam, I.mu_e ? I.mu_e[e] : I.mu, I.wq, I.wq3,
+                                                   m1, m2, m3);
+    else { m1 = I.m1; m2 = I.m2; m3 = I.m3; }
+    double Dx[3][2][2], Dy[3][2][2], Dz[3][2][2], F[3][8];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        double U[8];
+#pragma unroll
+        for (int c8 = 0; c8 < 8; ++c8)
+            U[c8] = u[(long long)c * g.NN + I.node_off + n0 + (c8 & 1) + ((c8 >> 1) & 1) * sy + ((c8 >> 2) & 1) * sz];
+        edge_differences<double>(U, I.invh, Dx[c], Dy[c], Dz[c]);
+    }
+    element_force<OSAM_NEO_HOOKEAN, double>(Dx, Dy, Dz, m1, m2, m3, F);
+    i64* fe = static_cast<i64*>(g.fe) + I.elem_off + e;
+    double* fe2 = g.fe2 + I.elem_off + e;
+#pragma unroll
+    for (int c8 = 0; c8 < 8; ++c8)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            fe[(long long)(c8 * 3 + c) * g.NE] = kBadF;
+            fe2[(long long)(c8 * 3 + c) * g.NE] = F[c][c8];
+        }
+}
+
+__global__ void __launch_bounds__(128) k_force_fx_b(const __grid_constant__ FomB g, const int* __restrict__ active,
+                                                    const __grid_constant__ TraceFuse tr, const double* u) {
+    if ((int)blockIdx.x >= g.n_eblk) {
+        trace::fused_trace_block(tr, active, g, (int)blockIdx.x - g.n_eblk);
+        return;
+    }
+    const int2 b = g.eblk[blockIdx.x];
+    if (active && !active[b.x]) return;
+    const InstFom& I = g.inst[b.x];
+    const int e = b.y + threadIdx.x;
+    if (e >= I.ne) return;
+    const int nx = I.nx, ny = I.ny;
+    const int i = e % nx;
+    const int t = e / nx;
+    const int j = t % ny;
+    const int k = t / ny;
+    const int sy = nx + 1, sz = (nx + 1) * (ny + 1);
+    const int n0 = i + sy * j + sz * k;
+    WalshIn w[3];
+    bool bad = false;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        const i64* x = g.ux + (long long)c * g.NN + I.node_off + n0;
+        i64 V[8];
+#pragma unroll
+        for (int c8 = 0; c8 < 8; ++c8) V[c8] = x[(c8 & 1) + ((c8 >> 1) & 1) * sy + ((c8 >> 2) & 1) * sz];
+        bad |= spread_bad(V);
+        w[c] = walsh_in(V, c);
+    }
+    i64 kap2 = I.fk2, mu = I.fmu;
+    if (I.lam_e || I.mu_e) {
+        const double le = I.lam_e ? I.lam_e[e] : I.lam, me = I.mu_e ? I.mu_e[e] : I.mu;
+        double m1, m2, m3;
+        hex8::material_factors<OSAM_NEO_HOOKEAN, double>(le, me, I.wq, I.wq3, m1, m2, m3);
+        kap2 = fixed_factor(m1, kFracOut - I.fscale);
+        mu = fixed_factor(m2, kFracOut - I.fscale);
+    }
+    i64 F[3][8];
+    bad |= !element_force_nh(w, kap2, mu, mul_third(mu), F);
+    if (bad) {
+        far_element(g, I, u, e, n0);
+        return;
+    }
+    i64* fe = static_cast<i64*>(g.fe) + I.elem_off + e;
+#pragma unroll
+    for (int c8 = 0; c8 < 8; ++c8)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) fe[(long long)(c8 * 3 + c) * g.NE] = F[c][c8];
+}
+
+// Corrector of substep j and predictor of substep j + 1 (the arithmetic of k_node_b) on the fixed-point
+// element buffer: the 24 contributions of a node are summed exactly as integers and converted once per
+// component; the predictor is written in FP64 and as fixed-point u / h.
+__global__ void __launch_bounds__(kNodeBlock) k_node_fx_b(const __grid_constant__ FomB g,
+                                                          const int* __restrict__ active, int slot1, int slot2,
+                                                          int predict_only, const double* ucur, double* unext,
+                                                          double dt) {
+    const int2 b = g.nblk[blockIdx.x];
+    if (active && !active[b.x]) return;
+    const InstFom& I = g.inst[b.x];
+    const int n = b.y + threadIdx.x;
+    if (n >= I.nn) return;
+    const int nx = I.nx, ny = I.ny, nz = I.nz;
+    const int i = n % (nx + 1);
+    const int t = n / (nx + 1);
+    const int j = t % (ny + 1);
+    const int k = t / (ny + 1);
+    const long long gn = I.node_off + n;
+    const uint8_t cm = g.clamp[gn];
+    const int row = g.srow[gn];
+    const double hdt = 0.5 * dt, hdt2 = 0.5 * dt * dt;
+    const double minv = g.minv[gn];
+    const double* h1 = slot1 >= 0 ? g.hist + I.hist_off + (long long)slot1 * 9 * I.ns : nullptr;
+    const double* h2 = slot2 >= 0 ? g.hist + I.hist_off + (long long)slot2 * 9 * I.ns : nullptr;
+    double uc[3], vc[3], ac[3], f[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        const long long d = (long long)c * g.NN + gn;
+        uc[c] = ucur[d];
+        vc[c] = g.v[d];
+        ac[c] = g.a[d];
+    }
+    if (!predict_only && row < 0 && cm != 7) {
+        const i64* fe = static_cast<const i64*>(g.fe) + I.elem_off;
+        i64 s[3] = {0, 0, 0};
+        unsigned int far = 0;
+#pragma unroll
+        for (int az = 0; az < 2; ++az) {
+            const int ke = k - az;
+#pragma unroll
+            for (int ay = 0; ay < 2; ++ay) {
+                const int je = j - ay;
+#pragma unroll
+                for (int ax = 0; ax < 2; ++ax) {
+                    const int ie = i - ax;
+                    const int corner = ax + 2 * ay + 4 * az;
+                    if (ke < 0 || ke >= nz || je < 0 || je >= ny || ie < 0 || ie >= nx) continue;
+                    const long long e = ie + (long long)nx * (je + ny * ke);
+                    i64 x[3];
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) x[c] = __ldg(fe + (long long)(corner * 3 + c) * g.NE + e);
+                    if (x[0] == kBadF) { far |= 1u << corner; continue; }
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) s[c] += x[c];
+                }
+            }
+        }
+#pragma unroll
+        for (int c = 0; c < 3; ++c) f[c] = f64_scaled(s[c], I.fscale);
+        while (far) {   // elements held in FP64
+            const int corner = __ffs((int)far) - 1;
+            far &= far - 1;
+            const long long e = (i - (corner & 1)) +
+                                (long long)nx * ((j - ((corner >> 1) & 1)) + ny * (k - (corner >> 2)));
+#pragma unroll
+            for (int c = 0; c < 3; ++c) f[c] += g.fe2[(long long)(corner * 3 + c) * g.NE + I.elem_off + e];
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        const long long d = (long long)c * g.NN + gn;
+        double un;
+        if (cm & (1 << c)) {
+            g.v[d] = 0.0;
+            g.a[d] = 0.0;
+            un = 0.0;
+        } else if (row >= 0) {
+            if (!predict_only) {
+                g.v[d] = h1[(long long)(3 + c) * I.ns + row];
+                g.a[d] = h1[(long long)(6 + c) * I.ns + row];
+            }
+            un = h2 ? h2[(long long)c * I.ns + row] : 0.0;
+        } else {
+            double vn = vc[c], an = ac[c];
+            if (!predict_only) {
+                const double anew = -f[c] * minv;
+                vn = fma(hdt, an + anew, vn);
+                an = anew;
+                g.v[d] = vn;
+                g.a[d] = an;
+            }
+            un = fma(hdt2, an, fma(dt, vn, uc[c]));
+        }
+        if (h2) {
+            unext[d] = un;
+            g.ux[d] = fixed_u(un, I.ihm, I.ihe);
+        }
+    }
+}
+
+}  // namespace
+
+cudaError_t launch_force_fx_b(const FomB& g, const int* active, const TraceFuse& tr, const double* upred,
+                              cudaStream_t s) {
+    if (!upred || g.eblock > 128) return cudaErrorInvalidValue;
+    long long items = 0;
+    for (int k = 0; k < tr.n; ++k) items += 3LL * tr.c[k].R;
+    const int grid = g.n_eblk + (int)((items + g.eblock - 1) / g.eblock);
+    k_force_fx_b<<<grid, g.eblock, 0, s>>>(g, active, tr, upred);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_node_fx_b(const FomB& g, const int* active, int slot1, int slot2, int predict_only,
+                             const double* ucur, double* unext, double dt, cudaStream_t s) {
+    k_node_fx_b<<<g.n_nblk, kNodeBlock, 0, s>>>(g, active, slot1, slot2, predict_only, ucur, unext, dt);
+    return cudaGetLastError();
+}
+
+}  // namespace osam

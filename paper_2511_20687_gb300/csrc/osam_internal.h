@@ -62,6 +62,10 @@ struct InstFom {
     const double* lam_e;      // absolute device pointers or null (uniform lam / mu)
     const double* mu_e;
     long long node_off, elem_off, hist_off;
+    // fixed-point force (fixed_math.cuh): kappa/2 and mu factors with 62 fraction bits in units of
+    // 2^(54 - fscale) (fscale: fraction bits of the element forces), 1/h as ihm 2^(ihe - 62)
+    long long fk2, fmu, ihm;
+    int ihe, fscale;
 };
 
 // kernel view of a FOM slot across instances; nodal arrays are SoA over the concatenated nodes:
@@ -124,6 +128,9 @@ struct FomB {
     float* linf;              // the same in FP32 (OSAM_FP64_TANGENT32; lin is then null)
     float* fe32;              // FP32 element buffer [24][NE] of the FP32 tangent action
     int df32;                 // 1: internal force in double-float arithmetic (element buffer of float2)
+    int fixed;                // 1: internal force in 64-bit fixed point (element buffer of int64; force_fx.cu)
+    long long* ux;            // fixed-point predicted displacement / h [3][NN]
+    double* fe2;              // FP64 contributions of the elements outside the fixed-point range [24][NE]
 };
 
 // one instance of a ROM slot
@@ -214,8 +221,9 @@ cudaError_t launch_zero_clamped(int nn, const uint8_t* clamp, double* u, double*
 // batched per-step kernels (step_kernels.cu); `active` masks instances that have converged
 // ------------------------------------------------------------------------------------------------
 // internal force of the predicted displacement held (divided by h) in g.us / g.u2
+// (upred: that displacement itself, required by fixed-point groups)
 cudaError_t launch_force_b(const FomB& g, const int* active, int scatter, cudaStream_t s,
-                           const TraceFuse* tr = nullptr);
+                           const TraceFuse* tr = nullptr, const double* upred = nullptr);
 cudaError_t launch_force_init_b(const FomB& g, const int* active, cudaStream_t s);  // FP64 gather of f(u[0]) into fe
 cudaError_t launch_init_accel_b(const FomB& g, const int* active, cudaStream_t s);  // a = -M^-1 f from fe
 cudaError_t launch_node_b(const FomB& g, const int* active, int scatter, int slot1, int slot2, int predict_only,
@@ -223,6 +231,11 @@ cudaError_t launch_node_b(const FomB& g, const int* active, int scatter, int slo
 cudaError_t launch_saverest_fom_b(const FomB& g, const int* active, int restore, cudaStream_t s);
 cudaError_t launch_norms_fom_b(const FomB& g, const int* active, double dt, cudaStream_t s);
 cudaError_t launch_copy_u10_b(const FomB& g, const int* active, cudaStream_t s);
+// fixed-point groups (force_fx.cu)
+cudaError_t launch_force_fx_b(const FomB& g, const int* active, const TraceFuse& tr, const double* upred,
+                              cudaStream_t s);
+cudaError_t launch_node_fx_b(const FomB& g, const int* active, int slot1, int slot2, int predict_only,
+                             const double* ucur, double* unext, double dt, cudaStream_t s);
 // double-float mode (force_df.cu)
 cudaError_t launch_split_u2_b(const FomB& g, cudaStream_t s);
 cudaError_t launch_force_df_b(const FomB& g, const int* active, const TraceFuse& tr, cudaStream_t s);

@@ -107,7 +107,8 @@ int set_eblocks(osam_ctx* ctx, FomGroupH& G, int block) {
 // 2 mu_e)) (element eigenvalue bound of the lumped-mass system at the reference configuration; the
 // Neo-Hookean law linearises to the same lambda, mu).  A relative allowance of 1e-9 keeps a step that
 // sits exactly on the limit.
-int check_stability(osam_ctx* ctx, FomGroupH& G, int s, int n, const osam_problem_desc* descs) {
+int check_stability(osam_ctx* ctx, FomGroupH& G, int s, int n, const osam_problem_desc* descs,
+                    std::vector<double>& modulus) {
     unsigned long long* mod = ctx->alloc<unsigned long long>(n);
     int* bad = ctx->alloc<int>(1);
     CKA(mod); CKA(bad);
@@ -123,6 +124,7 @@ int check_stability(osam_ctx* ctx, FomGroupH& G, int s, int n, const osam_proble
     for (int i = 0; i < n; ++i) {
         double m;
         std::memcpy(&m, &mh[i], sizeof(double));
+        modulus.push_back(m);
         const double lim = G.grid[i].h * std::sqrt(descs[i].subdomains[s].rho / m);
         const double dt = ctx->slots[s].dt;
         if (!G.d.implicit && dt > lim * (1.0 + 1e-9))
@@ -147,6 +149,21 @@ int set_tiles(osam_ctx* ctx, FomGroupH& G) {
     G.d.tblk = d;
     G.d.n_tblk = (int)tb.size();
     return OSAM_OK;
+}
+
+// Scales of the fixed-point force of one Neo-Hookean instance.  The unit of its element forces is the
+// power of two at or above the largest material factor: of the uniform kappa/2 and mu, or, with
+// per-element parameters, of mu <= modulus / 2 (modulus = max(3 lambda + 2 mu, 2 mu) >= 6 kappa/2).
+void fixed_point_scales(InstFom& I, double modulus) {
+    const double top = I.lam_e || I.mu_e ? 0.5 * modulus * I.wq : std::max(I.m1, I.m2);
+    int k;
+    std::frexp(top, &k);
+    I.fscale = 54 - k;
+    I.fk2 = std::llrint(std::ldexp(I.m1, 62 - k));
+    I.fmu = std::llrint(std::ldexp(I.m2, 62 - k));
+    int e;
+    I.ihm = (long long)std::ldexp(std::frexp(I.invh, &e), 63);
+    I.ihe = e - 1;
 }
 
 int setup_fom_group(osam_ctx* ctx, FomGroupH& G, int s, int n, const osam_problem_desc* descs) {
@@ -198,6 +215,14 @@ int setup_fom_group(osam_ctx* ctx, FomGroupH& G, int s, int n, const osam_proble
     CKA(B.us = ctx->alloc<double>(3 * NN));
     if (B.df32 || B.fp32) CKA(B.u2 = ctx->alloc<float2>(3 * NN));   // the FP32 forces' split of u/h
     B.implicit = descs[0].subdomains[s].integrator == OSAM_IMPLICIT;
+    // Fixed-point force: explicit Neo-Hookean groups of the FP64 modes whose scatter is left to the
+    // library (a scatter mode asked for by name runs its own FP64 kernel).
+    B.fixed = B.material == OSAM_NEO_HOOKEAN && !B.implicit && descs[0].scatter == OSAM_SCATTER_AUTO &&
+              (ctx->precision == OSAM_FP64 || ctx->precision == OSAM_FP64_TANGENT32);
+    if (B.fixed) {
+        CKA(B.ux = ctx->alloc<long long>(3 * NN));
+        CKA(B.fe2 = ctx->alloc<double>(24 * NE));
+    }
     if (B.implicit) {
         ctx->any_implicit = true;
         CKA(B.ut = ctx->alloc<double>(3 * NN));
@@ -278,7 +303,12 @@ int setup_fom_group(osam_ctx* ctx, FomGroupH& G, int s, int n, const osam_proble
     if (B.implicit) CKA(B.ipart = ctx->alloc<double>(2LL * B.n_nblk));
     RET(set_eblocks(ctx, G, 128));
     RET(set_tiles(ctx, G));
-    RET(check_stability(ctx, G, s, n, descs));
+    std::vector<double> modulus;
+    RET(check_stability(ctx, G, s, n, descs, modulus));
+    if (B.fixed) {
+        for (int i = 0; i < n; ++i) fixed_point_scales(G.inst[i], modulus[i]);
+        RET(upload(ctx, G.inst_d, G.inst.data(), sizeof(InstFom) * n));
+    }
     if (B.df32 || B.fp32) CK(launch_split_u2_b(B, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
     return OSAM_OK;
@@ -620,15 +650,17 @@ int initial_accel(osam_ctx* ctx, const int* mask) {
     return OSAM_OK;
 }
 
-// time force + node kernels of the largest FOM group for (element block, scatter) candidates on
-// scratch copies of its state; keep the fastest (the deterministic gather scatter unless atomics are
-// more than 5% faster)
-int autotune(osam_ctx* ctx) {
+// time force + node kernels of the largest FOM group of one kind (fixed-point force or not) for (element
+// block, scatter) candidates on scratch copies of its state; keep the fastest for every group of that
+// kind (the deterministic gather scatter unless atomics are more than 5% faster)
+int autotune(osam_ctx* ctx, bool fixed) {
     FomGroupH* best_g = nullptr;
     const Slot* best_s = nullptr;
     long long ne = -1;
     for (Slot& S : ctx->slots)
-        if (S.kind == OSAM_FOM && S.fom.d.NE > ne) { ne = S.fom.d.NE; best_g = &S.fom; best_s = &S; }
+        if (S.kind == OSAM_FOM && (S.fom.d.fixed != 0) == fixed && S.fom.d.NE > ne) {
+            ne = S.fom.d.NE; best_g = &S.fom; best_s = &S;
+        }
     if (!best_g) return OSAM_OK;
     FomGroupH& G = *best_g;
     FomB g = G.d;
@@ -657,6 +689,7 @@ int autotune(osam_ctx* ctx) {
         const int mode = cd[0], block = cd[1], tiled = cd[2], occ = cd[3];
         if (g.df32 && (mode == kAtomic || block > 128 || tiled)) continue;  // double-float force: gather, <= 128 threads
         if (tiled && g.fp32) continue;                                    // the tiled kernel is FP64
+        if (fixed && (mode == kAtomic || tiled || block > 128)) continue; // the fixed-point force: gather, <= 128 threads
         RET(set_eblocks(ctx, G, block));
         g.eblk = G.d.eblk;
         g.n_eblk = G.d.n_eblk;
@@ -665,7 +698,7 @@ int autotune(osam_ctx* ctx) {
         g.tiled = tiled;
         for (int rep = 0; rep < 4; ++rep) {
             if (rep == 1) CK(cudaEventRecord(ctx->ev0, ctx->stream));
-            CK(launch_force_b(g, nullptr, mode, ctx->stream));
+            CK(launch_force_b(g, nullptr, mode, ctx->stream, nullptr, u));
             CK(launch_node_b(g, nullptr, mode, 1, slot2, 0, u, un, best_s->dt, ctx->stream));
         }
         CK(cudaEventRecord(ctx->ev1, ctx->stream));
@@ -682,9 +715,9 @@ int autotune(osam_ctx* ctx) {
     }
     CK(cudaMemsetAsync(G.d.f, 0, sizeof(double) * 3 * NN, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
-    ctx->scatter = best_scatter;
+    if (!fixed) ctx->scatter = best_scatter;
     for (Slot& S : ctx->slots)
-        if (S.kind == OSAM_FOM) {
+        if (S.kind == OSAM_FOM && (S.fom.d.fixed != 0) == fixed) {
             RET(set_eblocks(ctx, S.fom, best_block));
             S.fom.d.tiled = best_tiled;
             S.fom.d.occ = best_occ;
@@ -805,7 +838,10 @@ int init_impl(osam_ctx* ctx, int n, const osam_problem_desc* descs) {
     // initial boundary data: zero-order hold of the initial states (before the accelerations)
     for (CplH& c : ctx->cpls) RET(zoh_cpl(ctx, c, nullptr));
     RET(initial_accel(ctx, nullptr));
-    if (d0.scatter == OSAM_SCATTER_AUTO) RET(autotune(ctx));
+    if (d0.scatter == OSAM_SCATTER_AUTO) {
+        RET(autotune(ctx, false));
+        RET(autotune(ctx, true));
+    }
     const bool fp64_force = d0.precision == OSAM_FP64 || d0.precision == OSAM_FP64_TANGENT32;
     if (d0.scatter == OSAM_SCATTER_GATHER_LOWREG && fp64_force)
         for (Slot& S : ctx->slots)
