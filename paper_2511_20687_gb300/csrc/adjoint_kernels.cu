@@ -5,17 +5,12 @@
 // at element level is the force-like contraction of the directional derivative dP[Gbar] with
 // Gbar = grad(ybar):  ubar_b = sum_gp w detJ dP[Gbar] grad N_b.  Parameter cotangents are
 // lambda_bar_e = sum_gp w detJ P_lambda : Gbar and mu_bar_e = sum_gp w detJ P_mu : Gbar.
-// Neo-Hookean (cofactor form P = beta cof(F) + alpha F, alpha = mu J^-2/3,
-// beta = [kappa/2 (J^2-1) - mu/3 J^-2/3 tr C] / J):
-//   dJ = cof(F) : G,  d trC = 2 F : G,  d alpha = -2/3 alpha dJ / J,
-//   d beta = [kappa J dJ - 1/3 (d alpha trC + alpha d trC)] / J - beta dJ / J,
-//   dP = d beta cof + beta dcof[G] + d alpha F + alpha G,  dcof linear in G (cof is quadratic in F).
+// The Neo-Hookean contraction is in lane_kernels.cu.
 #include <cuda_runtime.h>
 
 #include <cstdint>
 
 #include "hex8_math.cuh"
-#include "nh_tangent.cuh"
 #include "osam_internal.h"
 
 namespace osam {
@@ -41,14 +36,12 @@ __device__ __forceinline__ void edge_diffs(const double* x, int sn, long long sc
     }
 }
 
-using tangent::nh_tangent;
-
-// One thread per element.  MODE kAtomic adds ubar into a.f ([3] x strided nodes); kGather writes the
+// Linear elastic, one thread per element.  MODE kAtomic adds ubar into a.f ([3] x strided nodes); kGather writes the
 // element's 24 contributions to the element buffer a.fe [24][ne] (corner-major, component), which a
 // fixed-order gather sums per node (deterministic).  The transposed interpolation is the force's
 // Walsh-basis stage (hex8::walsh_transpose), so the material factors carry its 1/4.
-template <int MAT, int MODE>
-__global__ void __launch_bounds__(128) k_hex8_vjp(const ElemArgs a, const double* ybar, int ysn, long long ysc,
+template <int MODE>
+__global__ void __launch_bounds__(128) k_hex8_vjp_le(const ElemArgs a, const double* ybar, int ysn, long long ysc,
                                                   double* lam_bar, double* mu_bar, int accumulate) {
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= a.ne) return;
@@ -74,7 +67,7 @@ __global__ void __launch_bounds__(128) k_hex8_vjp(const ElemArgs a, const double
         hex8::lerp2(Ex[c], Bx[c]); hex8::lerp2(Ey[c], By[c]); hex8::lerp2(Ez[c], Bz[c]);
     }
     double m1, m2, m3;
-    hex8::material_factors<MAT, double>(lam, mu, a.wq, a.wq3, m1, m2, m3);
+    hex8::material_factors<OSAM_LINEAR_ELASTIC, double>(lam, mu, a.wq, a.wq3, m1, m2, m3);
     double Sx[3][2][2], Sy[3][2][2], Sz[3][2][2];
     double lb = 0.0, mb = 0.0;
 #pragma unroll
@@ -89,25 +82,18 @@ __global__ void __launch_bounds__(128) k_hex8_vjp(const ElemArgs a, const double
                     Hm[c][0] = Gx[c][q][r]; Hm[c][1] = Gy[c][p][r]; Hm[c][2] = Gz[c][p][q];
                     Gm[c][0] = Bx[c][q][r]; Gm[c][1] = By[c][p][r]; Gm[c][2] = Bz[c][p][q];
                 }
-                if (MAT == OSAM_NEO_HOOKEAN) {
-                    double pk, pm;
-                    nh_tangent(Hm, Gm, m1, m2, m3, dP, pk, pm);
-                    lb += pk;
-                    mb = fma(2.0 / 3.0, pk, mb + pm);
-                } else {
-                    const double trG = Gm[0][0] + Gm[1][1] + Gm[2][2];
-                    const double trH = Hm[0][0] + Hm[1][1] + Hm[2][2];
-                    double symHG = 0.0;
+                const double trG = Gm[0][0] + Gm[1][1] + Gm[2][2];
+                const double trH = Hm[0][0] + Hm[1][1] + Hm[2][2];
+                double symHG = 0.0;
 #pragma unroll
-                    for (int x = 0; x < 3; ++x)
+                for (int x = 0; x < 3; ++x)
 #pragma unroll
-                        for (int y = 0; y < 3; ++y) {
-                            dP[x][y] = m2 * (Gm[x][y] + Gm[y][x]) + (x == y ? m1 * trG : 0.0);
-                            symHG = fma(Hm[x][y] + Hm[y][x], Gm[x][y], symHG);
-                        }
-                    lb = fma(trH, trG, lb);
-                    mb += symHG;
-                }
+                    for (int y = 0; y < 3; ++y) {
+                        dP[x][y] = m2 * (Gm[x][y] + Gm[y][x]) + (x == y ? m1 * trG : 0.0);
+                        symHG = fma(Hm[x][y] + Hm[y][x], Gm[x][y], symHG);
+                    }
+                lb = fma(trH, trG, lb);
+                mb += symHG;
 #pragma unroll
                 for (int c = 0; c < 3; ++c) {
                     if (p == 0) Sx[c][q][r] = dP[c][0]; else Sx[c][q][r] += dP[c][0];
@@ -141,15 +127,10 @@ __global__ void __launch_bounds__(128) k_hex8_vjp(const ElemArgs a, const double
 cudaError_t launch_hex8_vjp(int material, int scatter, const ElemArgs& a, const double* ybar, int ysn, long long ysc,
                             double* lam_bar, double* mu_bar, int acc, cudaStream_t s) {
     if (a.ne <= 0) return cudaSuccess;
+    if (material == OSAM_NEO_HOOKEAN) return launch_elem_vjp_nh(scatter, a, ybar, ysn, ysc, lam_bar, mu_bar, acc, s);
     const int g = grid_for(a.ne, 128);
-    const bool at = scatter == kAtomic;
-    if (material == OSAM_NEO_HOOKEAN) {
-        if (at) k_hex8_vjp<OSAM_NEO_HOOKEAN, kAtomic><<<g, 128, 0, s>>>(a, ybar, ysn, ysc, lam_bar, mu_bar, acc);
-        else k_hex8_vjp<OSAM_NEO_HOOKEAN, kGather><<<g, 128, 0, s>>>(a, ybar, ysn, ysc, lam_bar, mu_bar, acc);
-    } else {
-        if (at) k_hex8_vjp<OSAM_LINEAR_ELASTIC, kAtomic><<<g, 128, 0, s>>>(a, ybar, ysn, ysc, lam_bar, mu_bar, acc);
-        else k_hex8_vjp<OSAM_LINEAR_ELASTIC, kGather><<<g, 128, 0, s>>>(a, ybar, ysn, ysc, lam_bar, mu_bar, acc);
-    }
+    if (scatter == kAtomic) k_hex8_vjp_le<kAtomic><<<g, 128, 0, s>>>(a, ybar, ysn, ysc, lam_bar, mu_bar, acc);
+    else k_hex8_vjp_le<kGather><<<g, 128, 0, s>>>(a, ybar, ysn, ysc, lam_bar, mu_bar, acc);
     return cudaGetLastError();
 }
 

@@ -76,8 +76,19 @@ constexpr int kCgCheck = 8;            // CG iterations between host checks of t
 constexpr double kCgTol2 = 1e-26;      // floor of the CG test r.z <= eta^2 (r.z)_0 (eta: the Newton forcing term)
 constexpr double kCgTol2F32 = 1e-12;   // the floor with the FP32 tangent (eta >= 1e-6, above its rounding)
 
-// the stored-linearisation path (Neo-Hookean groups), and the CG floor that goes with its precision
-bool stored_lin(const FomB& g) { return g.lin || g.linf; }
+// Newton residual force and tangent action of an implicit group, and the CG floor that goes with the
+// tangent's precision
+cudaError_t newton_force(const FomB& g, cudaStream_t s) {
+    if (g.linf) return launch_force_lin_b(g, g.nact, s);
+    if (g.material == OSAM_NEO_HOOKEAN) return launch_imp_force_nh_b(g, g.nact, s);
+    return launch_force_b(g, g.nact, kGather, s, nullptr);
+}
+cudaError_t newton_tangent(const FomB& g, cudaStream_t s) {
+    if (g.linf) return launch_tangent_lin_b(g, g.cgact, s);
+    if (g.material == OSAM_NEO_HOOKEAN) return launch_imp_tangent_nh_b(g, g.cgact, s);
+    if (g.fixed == 2) return launch_tangent_le_b(g, g.cgact, s);
+    return launch_tangent_b(g, g.cgact, s);
+}
 double cg_floor(const FomB& g) { return g.linf ? kCgTol2F32 : kCgTol2; }
 
 // Implicit Newmark interval of FOM slot s (beta = 1/4, gamma = 1/2): per substep the predictor, a
@@ -97,8 +108,7 @@ int advance_implicit(osam_ctx* ctx, int s, const int* active) {
         LK(launch_mask_copy(n, active, g.nact, ctx->stream));
         LK(launch_mask_copy(n, active, g.cgact, ctx->stream));
         for (int it = 0; it < kNewtonMax; ++it) {
-            if (stored_lin(g)) LK(launch_force_lin_b(g, g.nact, ctx->stream));
-            else LK(launch_force_b(g, g.nact, kGather, ctx->stream, nullptr));
+            LK(newton_force(g, ctx->stream));
             LK(launch_imp_residual_b(g, g.nact, c0, ctx->stream));
             LK(launch_imp_reduce_b(g, g.nact, 0, it == 0, kNewtonTol2, ctx->stream));
             bool any = false;
@@ -107,8 +117,7 @@ int advance_implicit(osam_ctx* ctx, int s, const int* active) {
             for (int k = 0; k < kCgMax;) {
                 for (int q = 0; q < kCgCheck; ++q, ++k) {
                     const int pk = ctx->prof_begin(1);
-                    if (stored_lin(g)) LK(launch_tangent_lin_b(g, g.cgact, ctx->stream));
-                    else LK(launch_tangent_b(g, g.cgact, ctx->stream));
+                    LK(newton_tangent(g, ctx->stream));
                     ctx->prof_end(pk, 0);
                     LK(launch_cg_ap_b(g, g.cgact, c0, ctx->stream));
                     LK(launch_cg_step_b(g, g.cgact, c0, cg_floor(g), ctx->stream));
@@ -183,8 +192,7 @@ int enqueue_implicit_captured(osam_ctx* ctx, int s, const int* active) {
         {
             cudaStream_t a = ctx->cap[0];
             auto body = [&]() -> int {
-                if (stored_lin(g)) LK(launch_force_lin_b(g, g.nact, a));
-                else LK(launch_force_b(g, g.nact, kGather, a, nullptr));
+                LK(newton_force(g, a));
                 LK(launch_imp_residual_b(g, g.nact, c0, a));
                 LK(launch_imp_reduce_b(g, g.nact, 0, -1, kNewtonTol2, a));
                 RET(while_handle(ctx, a, &hc));
@@ -196,8 +204,7 @@ int enqueue_implicit_captured(osam_ctx* ctx, int s, const int* active) {
                 cudaStream_t b = ctx->cap[1];
                 int rc2 = OSAM_OK;
                 auto cg = [&]() -> int {
-                    if (stored_lin(g)) LK(launch_tangent_lin_b(g, g.cgact, b));
-                    else LK(launch_tangent_b(g, g.cgact, b));
+                    LK(newton_tangent(g, b));
                     LK(launch_cg_ap_b(g, g.cgact, c0, b));
                     LK(launch_cg_step_b(g, g.cgact, c0, cg_floor(g), b));
                     LK(launch_cg_dir_b(g, g.cgact, c0, b));

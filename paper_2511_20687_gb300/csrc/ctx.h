@@ -75,6 +75,7 @@ struct osam_ctx {
     int max_it = 1;
     int precision = OSAM_FP64;
     int scatter = kGather;
+    bool integer_force = false;   // integer force kernels with a scatter mode asked for by name (the adjoint)
     std::vector<Slot> slots;
     std::vector<CplH> cpls;
     std::vector<void*> allocs;

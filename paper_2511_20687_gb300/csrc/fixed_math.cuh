@@ -212,44 +212,56 @@ OSAM_HD WalshIn walsh_in(const i64 V[8], int axis) {
     return w;
 }
 
-// One Gauss point: alpha (60 fraction bits) and beta cof(F) added to the pair sums.
+// Constitutive quantities of one Gauss point: cof(F) (61), J (58), J^-2/3 (62), 1/J (62), alpha (60) and beta (57).
 //   F0, F1, F2: columns of F (61), nF1 = -F1, nF2 = -F2, n: |F|^2 (58); kap2, mu, mu3: material factors (62)
 // cof(F) has entries below |col||col| < 2.25 and is carried with 61 bits.
-OSAM_HD void gauss_point(const D F0[3], const D F1[3], const D F2[3], const D nF1[3], const D nF2[3], i64 n, D kap2,
-                         D mu, D mu3, Range& g, i64& alpha, i64 X[3], i64 Y[3], i64 Z[3]) {
-    D c0[3], c1[3], c2[3];
+struct NhPoint {
+    D c0[3], c1[3], c2[3], r3, inv;
+    i64 J, alpha, beta, invJ;   // invJ: 1/J with 60 fraction bits
+};
+OSAM_HD NhPoint nh_point(const D F0[3], const D F1[3], const D F2[3], const D nF1[3], const D nF2[3], i64 n, D kap2,
+                         D mu, D mu3, Range& g) {
+    NhPoint s;
 #ifdef __CUDACC__
 #pragma unroll
 #endif
     for (int a = 0; a < 3; ++a) {
         const int b = (a + 1) % 3, c = (a + 2) % 3;
-        c0[a] = split(shl(dot2(F1[b], F2[c], nF1[c], F2[b]), 3));
-        c1[a] = split(shl(dot2(F2[b], F0[c], nF2[c], F0[b]), 3));
-        c2[a] = split(shl(dot2(F0[b], F1[c], F0[c], nF1[b]), 3));
+        s.c0[a] = split(shl(dot2(F1[b], F2[c], nF1[c], F2[b]), 3));
+        s.c1[a] = split(shl(dot2(F2[b], F0[c], nF2[c], F0[b]), 3));
+        s.c2[a] = split(shl(dot2(F0[b], F1[c], F0[c], nF1[b]), 3));
     }
-    const i64 J = dot3(F0[0], c0[0], F1[0], c1[0], F2[0], c2[0]);    // 58
-    g.jmin = imin(g.jmin, hi(J));
-    g.jmax = imax(g.jmax, hi(J));
-    const i64 s1 = rcbrt58(J);                                        // 62
+    s.J = dot3(F0[0], s.c0[0], F1[0], s.c1[0], F2[0], s.c2[0]);      // 58
+    g.jmin = imin(g.jmin, hi(s.J));
+    g.jmax = imax(g.jmax, hi(s.J));
+    const i64 s1 = rcbrt58(s.J);                                      // 62
     const D s1d = split(s1);
-    const D r3 = split(shl(mul(s1d, s1d), 2));                        // J^-2/3, 62 (below 1.53)
-    const i64 inv = mul(r3, s1d);                                     // 1/J, 60
-    const D inv62 = split(shl(inv, 2));
-    alpha = mul(mu, r3);                                              // 60
-    const i64 q = mul(r3, inv62);                                     // J^-5/3, 60 (below 2.9)
+    s.r3 = split(shl(mul(s1d, s1d), 2));                              // J^-2/3, 62 (below 1.53)
+    s.invJ = mul(s.r3, s1d);                                          // 1/J, 60
+    s.inv = split(shl(s.invJ, 2));
+    s.alpha = mul(mu, s.r3);                                          // 60
+    const i64 q = mul(s.r3, s.inv);                                   // J^-5/3, 60 (below 2.9)
     const i64 mq = shl(mul(mu3, split(q)), 3);                        // 61 (mu3 <= 1/3)
-    const i64 b1 = mul(kap2, split(shl(J, 3) - shl(inv, 1)));         // 59
-    const i64 beta = (b1 >> 2) - mul(split(mq), split(shl(n, 2)));    // 57
-    g.bmax = imax(g.bmax, hi(beta));
-    g.bmin = imin(g.bmin, hi(beta));
-    const D B = split(shl(beta, 3));                                  // 60
+    const i64 b1 = mul(kap2, split(shl(s.J, 3) - shl(s.invJ, 1)));    // 59
+    s.beta = (b1 >> 2) - mul(split(mq), split(shl(n, 2)));            // 57
+    g.bmax = imax(g.bmax, hi(s.beta));
+    g.bmin = imin(g.bmin, hi(s.beta));
+    return s;
+}
+
+// One Gauss point: alpha (60 fraction bits) and beta cof(F) added to the pair sums
+OSAM_HD void gauss_point(const D F0[3], const D F1[3], const D F2[3], const D nF1[3], const D nF2[3], i64 n, D kap2,
+                         D mu, D mu3, Range& g, i64& alpha, i64 X[3], i64 Y[3], i64 Z[3]) {
+    const NhPoint s = nh_point(F0, F1, F2, nF1, nF2, n, kap2, mu, mu3, g);
+    alpha = s.alpha;
+    const D B = split(shl(s.beta, 3));                                // 60
 #ifdef __CUDACC__
 #pragma unroll
 #endif
     for (int a = 0; a < 3; ++a) {
-        X[a] = mul_add(B, c0[a], X[a]);                               // 57
-        Y[a] = mul_add(B, c1[a], Y[a]);
-        Z[a] = mul_add(B, c2[a], Z[a]);
+        X[a] = mul_add(B, s.c0[a], X[a]);                             // 57
+        Y[a] = mul_add(B, s.c1[a], Y[a]);
+        Z[a] = mul_add(B, s.c2[a], Z[a]);
     }
 }
 
@@ -401,6 +413,325 @@ OSAM_HD bool element_force_nh(const WalshIn w[3], i64 kap2i, i64 mui, i64 mu3i, 
                   (d1 - d0) + aby[c] + abz[c], Fo[c]);
     }
     return !out_of_range(g);
+}
+
+// ---- one Gauss point on its own (the kernels with one Gauss point per lane) ----------------------
+
+// a b + c d + e f + g h as one rounded high word
+OSAM_HD i64 dot4(D a, D b, D c, D d, D e, D f, D g, D h) {
+    i64 m = mad(a.h, b.l, (i64)1 << 31);
+    m = mad(a.l, b.h, m);
+    m = mad(c.h, d.l, m);
+    m = mad(c.l, d.h, m);
+    m = mad(e.h, f.l, m);
+    m = mad(e.l, f.h, m);
+    m = mad(g.h, h.l, m);
+    m = mad(g.l, h.h, m);
+    return mad(g.h, h.h, mad(e.h, f.h, mad(c.h, d.h, mad(a.h, b.h, m >> 32))));
+}
+
+// Columns of F (or of a direction's gradient G) at one Gauss point, 61 fraction bits
+struct Cols {
+    i64 x[3][3];   // [column][component]
+};
+
+constexpr int kOne25 = 1 << 25;
+
+// Piola stress P[column][component] (57 fraction bits, below 1) of one Gauss point; false out of range
+OSAM_HD bool stress_point(const Cols& C, D kap2, D mu, D mu3, i64 P[3][3]) {
+    D F[3][3], nF1[3], nF2[3];
+    i64 n = 0;
+    Range g;
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+    for (int k = 0; k < 3; ++k) {
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+        for (int c = 0; c < 3; ++c) F[k][c] = split(C.x[k][c]);
+        const i64 m = norm3(F[k][0], F[k][1], F[k][2]);
+        g.nmax = g.nmax > (unsigned int)hi(m) ? g.nmax : (unsigned int)hi(m);
+        n += m;
+    }
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+    for (int c = 0; c < 3; ++c) { nF1[c] = split(-C.x[1][c]); nF2[c] = split(-C.x[2][c]); }
+    const NhPoint s = nh_point(F[0], F[1], F[2], nF1, nF2, n, kap2, mu, mu3, g);
+    const D A = split(s.alpha), B = split(shl(s.beta, 3));            // 60, 60
+    int top = 0;
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+    for (int c = 0; c < 3; ++c) {
+        P[0][c] = dot2(B, s.c0[c], A, F[0][c]);                       // 57
+        P[1][c] = dot2(B, s.c1[c], A, F[1][c]);
+        P[2][c] = dot2(B, s.c2[c], A, F[2][c]);
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+        for (int k = 0; k < 3; ++k) top |= hi(P[k][c]) ^ (hi(P[k][c]) >> 31);
+    }
+    return !out_of_range(g) && top < kOne25;
+}
+
+// Directional derivative dP[G] (nh_tangent.cuh) of one Gauss point and the parameter contractions
+// pk = P_kappa : G (60 fraction bits) and pm = P_mu : G (56).  G is scaled so that every Walsh coefficient of
+// the direction is below 2^58 (|G_ij| < 0.32, 61 fraction bits); dP has 56 fraction bits and is below 2.
+// Checked besides the force's range: |dJ| < 1 and the bracket of dbeta below 4.  Against a 113-bit
+// reference the element action is closer than the same formula in double (tests/test_fixed_point.py).
+OSAM_HD bool tangent_point(const Cols& C, const Cols& E, D kap2, D mu, D mu3, i64 dP[3][3], i64& pk, i64& pm) {
+    D F[3][3], N[3][3], G[3][3];
+    i64 n = 0;
+    Range g;
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+    for (int k = 0; k < 3; ++k) {
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+        for (int c = 0; c < 3; ++c) {
+            F[k][c] = split(C.x[k][c]);
+            N[k][c] = split(-C.x[k][c]);
+            G[k][c] = split(E.x[k][c]);
+        }
+        const i64 m = norm3(F[k][0], F[k][1], F[k][2]);
+        g.nmax = g.nmax > (unsigned int)hi(m) ? g.nmax : (unsigned int)hi(m);
+        n += m;
+    }
+    const NhPoint s = nh_point(F[0], F[1], F[2], N[1], N[2], n, kap2, mu, mu3, g);
+    i64 dJ = dot3(s.c0[0], G[0][0], s.c0[1], G[0][1], s.c0[2], G[0][2]);
+    dJ += dot3(s.c1[0], G[1][0], s.c1[1], G[1][1], s.c1[2], G[1][2]);
+    dJ += dot3(s.c2[0], G[2][0], s.c2[1], G[2][1], s.c2[2], G[2][2]);   // 58, below 3.6
+    i64 FG = 0;
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+    for (int k = 0; k < 3; ++k) FG += dot3(F[k][0], G[k][0], F[k][1], G[k][1], F[k][2], G[k][2]);   // 58, below 2.4
+    bool ok = !out_of_range(g) && (hi(dJ) ^ (hi(dJ) >> 31)) < (1 << 26);
+    const D dJd = split(shl(dJ, 4));                                   // 62
+    const D al = split(shl(s.alpha, 2));                               // 62
+    const D nd = split(shl(n, 2));                                     // 60
+    const D FGd = split(shl(FG, 2));                                   // 60
+    // dalpha = -2/3 alpha dJ / J, below 2
+    const i64 a13 = mul_third(mul(al, s.inv));                         // alpha / (3 J), 60
+    const i64 da = -mul(split(shl(a13, 2)), dJd);                      // 59
+    // dbeta = [(2 kap2 J - beta) dJ - (dalpha trC + 2 alpha F:G) / 3] / J
+    const i64 cf = shl(mul(kap2, split(shl(s.J, 3))), 1) - shl(s.beta, 2);      // 59, below 8
+    const i64 T = mul(split(shl(da, 2)), nd) + mul(al, FGd);                    // 57
+    const i64 Q = mul(split(cf), dJd) - mul_third(T);                           // 57, below 14
+    ok = ok && (hi(Q) ^ (hi(Q) >> 31)) < (4 << 25);
+    const D db = split(mul(s.inv, split(shl(Q, 4))));                  // 59
+    const D be = split(shl(s.beta, 2)), dad = split(da), ah = split((s.alpha + 1) >> 1);   // 59
+    int top = 0;
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+    for (int a = 0; a < 3; ++a) {
+        const int b = (a + 1) % 3, c = (a + 2) % 3;
+        const i64 d0 = dot4(G[1][b], F[2][c], G[1][c], N[2][b], F[1][b], G[2][c], N[1][c], G[2][b]);   // 58, below 1.7
+        const i64 d1 = dot4(G[2][b], F[0][c], G[2][c], N[0][b], F[2][b], G[0][c], N[2][c], G[0][b]);
+        const i64 d2 = dot4(G[0][b], F[1][c], G[0][c], N[1][b], F[0][b], G[1][c], N[0][c], G[1][b]);
+        dP[0][a] = dot4(db, s.c0[a], be, split(shl(d0, 3)), dad, F[0][a], ah, G[0][a]);                // 56
+        dP[1][a] = dot4(db, s.c1[a], be, split(shl(d1, 3)), dad, F[1][a], ah, G[1][a]);
+        dP[2][a] = dot4(db, s.c2[a], be, split(shl(d2, 3)), dad, F[2][a], ah, G[2][a]);
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+        for (int k = 0; k < 3; ++k) top |= hi(dP[k][a]) ^ (hi(dP[k][a]) >> 31);
+    }
+    const D jd = split(shl(shl(s.J, 2) - s.invJ, 2));                  // J - 1/J, 62
+    pk = (mul(jd, dJd) + 1) >> 1;                                      // (J - 1/J) dJ / 2, 60
+    const i64 qn = mul_third(mul(split(mul(s.r3, s.inv)), nd));        // J^-5/3 trC / 3, 56
+    pm = (mul(s.r3, FGd) - mul(split(shl(qn, 4)), dJd) + 2) >> 2;      // 56
+    return ok && top < kOne25;
+}
+
+// ---- operands with a block exponent --------------------------------------------------------------
+// The 8 nodal values of one component of an element's direction (or linear displacement) share one
+// exponent e: value = V 2^(e - 1081), |V| < 2^59, exact for values within 2^-6 of the largest, else rounded at
+// 2^-60 of it.  So differences of nearly equal values stay exact in each component; the Walsh coefficients of
+// the three components are then brought to one exponent, the largest coefficient in [2^57, 2^58).
+OSAM_HD unsigned int hi_word(double x) {
+    unsigned long long b;
+#ifdef __CUDA_ARCH__
+    b = (unsigned long long)__double_as_longlong(x);
+#else
+    __builtin_memcpy(&b, &x, 8);
+#endif
+    return (unsigned int)(b >> 32);
+}
+// biased exponent with the sign bit off (the maximum of hi_word() & 0x7fffffff, shifted)
+OSAM_HD i64 block_value(double x, int emax) {
+    unsigned long long b;
+#ifdef __CUDA_ARCH__
+    b = (unsigned long long)__double_as_longlong(x);
+#else
+    __builtin_memcpy(&b, &x, 8);
+#endif
+    const int e = (int)((b >> 52) & 0x7ff), s = emax - e;
+    if (e == 0 || s > 60) return 0;
+    const unsigned long long m = ((b & 0xfffffffffffffULL) | 0x10000000000000ULL) << 6;
+    const i64 v = (i64)((m + ((1ULL << s) >> 1)) >> s);
+    return (i64)b < 0 ? -v : v;
+}
+OSAM_HD int lead_zeros(i64 x) {   // of a non-negative value
+    if (x == 0) return 64;
+#ifdef __CUDA_ARCH__
+    return __clzll(x);
+#else
+    return __builtin_clzll((unsigned long long)x);
+#endif
+}
+OSAM_HD i64 mag(i64 x) { return x ^ (x >> 63); }
+// x 2^n, rounded if n < 0 (|x| < 2^62)
+OSAM_HD i64 shift(i64 x, int n) {
+    if (n >= 0) return shl(x, n);
+    return n < -62 ? 0 : (x + ((i64)1 << (-n - 1))) >> -n;
+}
+// exponent of a component's largest coefficient (of magnitudes or-ed into any); kNoExponent for zero
+constexpr int kNoExponent = -100000;
+OSAM_HD int top_exponent(i64 any, int e) { return any == 0 ? kNoExponent : e - lead_zeros(any); }
+
+// Two factors a, b (any finite values) as integers with a common exponent: value = A 2^(e - 1084), |A| < 2^62
+OSAM_HD int factor_exponent(double a, double b) {
+    const unsigned int x = hi_word(a) & 0x7fffffffu, y = hi_word(b) & 0x7fffffffu;
+    return (int)((x > y ? x : y) >> 20);
+}
+OSAM_HD i64 factor_value(double x, int e) { return shl(block_value(x, e), 3); }
+
+// ---- linear elasticity ---------------------------------------------------------------------------
+// Element force of isotropic linear elasticity in the Walsh basis of the 8 corners.  With raw Walsh
+// coefficients w_S of the nodal values (S a set of axes: signs of those axes), the 2x2x2 Gauss sums of
+// sigma(grad u) grad N are diagonal in the sign patterns (they are orthogonal on the Gauss points), so
+//   F(s) = h/16 sum_S f_S s^S,
+//   f_i   of component i: lam tr + 2 mu w_i^i (tr = w_x^x + w_y^y + w_z^z), of component c: mu (w_i^c + w_c^i),
+//   f_ij  of component i: [lam (w_ij^i + w_jk^k) + 3 mu w_ij^i] / 3,
+//         of component k: mu (2 w_ij^k + w_jk^i + w_ik^j) / 3   (k: the third axis),
+//   f_xyz of component c: (lam + 4 mu) w_xyz^c / 9:
+// the 1/sqrt3 of the Gauss points enters squared only, and no stress at a point is formed.  About 60
+// products per element against 300 with the tensor-product interpolation.
+// w: [component][pattern] with pattern bits x = 1, y = 2, z = 4, |w| < 2^59; lam, mu < 2^62; f: [component][pattern],
+// w lam / 2^64, below 2^62.
+OSAM_HD void le_coefficients(const i64 w[3][8], i64 lam, i64 mu, i64 f[3][8]) {
+    const D L = split(lam), M = split(mu);
+    const i64 lt = mul(L, split(w[0][1] + w[1][2] + w[2][4]));
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+    for (int i = 0; i < 3; ++i) {
+        const int j = (i + 1) % 3, k = (i + 2) % 3;
+        const int I = 1 << i, J = 1 << j, K = 1 << k;
+        f[i][0] = 0;
+        f[i][I] = mul_add(M, split(2 * w[i][I]), lt);
+        const i64 sh = mul(M, split(w[i][J] + w[j][I]));
+        f[i][J] = sh;
+        f[j][I] = sh;
+        // patterns {i, j} and {i, k} of component i, {j, k} of component i
+        f[i][I | J] = mul_third(mul_add(L, split(w[i][I | J] + w[k][J | K]), mul(M, split(3 * w[i][I | J]))));
+        f[i][I | K] = mul_third(mul_add(L, split(w[i][I | K] + w[j][J | K]), mul(M, split(3 * w[i][I | K]))));
+        f[i][J | K] = mul_third(mul(M, split(2 * w[i][J | K] + w[j][I | K] + w[k][I | J])));
+        const i64 x = mul_add(L, split(w[i][7]), mul(M, split(4 * w[i][7])));
+        f[i][7] = mul_third(mul_third(x));
+    }
+}
+
+// The 24 nodal forces of an element from its 24 nodal displacements: exact Walsh sums of the block values,
+// the coefficients above, the inverse sums.  lam, mu: Lame parameters times the factor h / 16 (divided by
+// the factor that the displacements carry).  Returns false for operands outside the formats (not finite,
+// or so small or large that the result's exponent leaves the normal range): the caller then uses FP64.
+OSAM_HD double f64_scaled(i64 x, int scale);
+OSAM_HD bool element_force_le(const double U[3][8], double lam, double mu, double F[3][8]) {
+    const int ek = factor_exponent(lam, mu);
+    if (ek == 2047) return false;
+    i64 w[3][8], f[3][8];
+    int e[3], T = kNoExponent;
+    bool bad = false;
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+    for (int c = 0; c < 3; ++c) {
+        unsigned int top = 0;
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+        for (int a = 0; a < 8; ++a) {
+            const unsigned int h = hi_word(U[c][a]) & 0x7fffffffu;
+            top = top > h ? top : h;
+        }
+        e[c] = (int)(top >> 20);
+        bad |= e[c] == 2047;
+        if (e[c] == 0) {                       // all zero, or subnormal displacements
+            unsigned long long bits = 0;
+            for (int a = 0; a < 8; ++a) {
+                unsigned long long b;
+                __builtin_memcpy(&b, &U[c][a], 8);
+                bits |= b << 1;
+            }
+            bad |= bits != 0;
+        }
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+        for (int a = 0; a < 8; ++a) w[c][a] = block_value(U[c][a], e[c]);
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+        for (int b = 1; b < 8; b <<= 1)
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+            for (int a = 0; a < 8; ++a)
+                if (!(a & b)) {
+                    const i64 lo = w[c][a], up = w[c][a | b];
+                    w[c][a] = lo + up;
+                    w[c][a | b] = up - lo;
+                }
+        i64 any = 0;
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+        for (int a = 1; a < 8; ++a) any |= mag(w[c][a]);
+        T = imax(T, top_exponent(any, e[c]));
+    }
+    // |w| < 2^58 after the shift: 4 w fits beside it, and the 7 terms of a corner below 2^61 each
+    const bool zero = T == kNoExponent;
+    const int scale = 2095 - T - ek;           // 1081 + 1084 - 64 - 6
+    if (bad || (!zero && (scale > 1000 || scale < -900))) return false;
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+    for (int c = 0; c < 3; ++c)
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+        for (int a = 1; a < 8; ++a) w[c][a] = zero ? 0 : shift(w[c][a], e[c] - T - 6);
+    le_coefficients(w, factor_value(lam, ek), factor_value(mu, ek), f);
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+    for (int c = 0; c < 3; ++c) {
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+        for (int b = 1; b < 8; b <<= 1)
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+            for (int a = 0; a < 8; ++a)
+                if (!(a & b)) {
+                    const i64 lo = f[c][a], up = f[c][a | b];
+                    f[c][a] = lo - up;
+                    f[c][a | b] = lo + up;
+                }
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+        for (int a = 0; a < 8; ++a) F[c][a] = f64_scaled(f[c][a], scale);
+    }
+    return true;
 }
 
 // x / 2^scale as an FP64 value, rounded to nearest (integer operations; |x| < 2^63)

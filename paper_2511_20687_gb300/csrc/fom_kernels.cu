@@ -15,7 +15,7 @@ namespace {
 using namespace hex8;
 
 // one thread per element of a single mesh, strided input / output (see ElemArgs)
-template <int MAT, typename T, int MODE>
+template <int MAT, int MODE>
 __global__ void __launch_bounds__(128) k_hex8_force(const ElemArgs a) {
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= a.ne) return;
@@ -30,27 +30,27 @@ __global__ void __launch_bounds__(128) k_hex8_force(const ElemArgs a) {
     for (int c8 = 0; c8 < 8; ++c8) node[c8] = n0 + (c8 & 1) + ((c8 >> 1) & 1) * sy + ((c8 >> 2) & 1) * sz;
     const double lam = a.lam_e ? a.lam_e[e] : a.lam;
     const double mu = a.mu_e ? a.mu_e[e] : a.mu;
-    T m1, m2, m3;
-    material_factors<MAT, T>(lam, mu, a.wq, a.wq3, m1, m2, m3);
-    T Dx[3][2][2], Dy[3][2][2], Dz[3][2][2];
+    double m1, m2, m3;
+    material_factors<MAT, double>(lam, mu, a.wq, a.wq3, m1, m2, m3);
+    double Dx[3][2][2], Dy[3][2][2], Dz[3][2][2];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
         double U[8];
         const double* uc = a.u + (long long)c * a.usc;
 #pragma unroll
         for (int c8 = 0; c8 < 8; ++c8) U[c8] = uc[(long long)node[c8] * a.usn];
-        edge_differences<T>(U, a.invh, Dx[c], Dy[c], Dz[c]);
+        edge_differences<double>(U, a.invh, Dx[c], Dy[c], Dz[c]);
     }
-    T F[3][8];
-    element_force<MAT, T>(Dx, Dy, Dz, m1, m2, m3, F);
+    double F[3][8];
+    element_force<MAT, double>(Dx, Dy, Dz, m1, m2, m3, F);
     if (MODE == kAtomic) {
-        T* f = static_cast<T*>(a.f);
+        double* f = static_cast<double*>(a.f);
 #pragma unroll
         for (int c = 0; c < 3; ++c)
 #pragma unroll
             for (int c8 = 0; c8 < 8; ++c8) atomic_add(f + (long long)c * a.fsc + (long long)node[c8] * a.fsn, F[c][c8]);
     } else {
-        T* fe = static_cast<T*>(a.fe);
+        double* fe = static_cast<double*>(a.fe);
 #pragma unroll
         for (int c8 = 0; c8 < 8; ++c8)
 #pragma unroll
@@ -164,21 +164,14 @@ __global__ void k_cfl_modulus(const FomB g, unsigned long long* out, int* bad) {
 
 int grid_for(long long n, int block) { return (int)((n + block - 1) / block); }
 
-cudaError_t launch_hex8_force(int material, bool fp32, int scatter, const ElemArgs& a, cudaStream_t s) {
+cudaError_t launch_hex8_force(int material, int scatter, const ElemArgs& a, cudaStream_t s) {
     if (a.ne <= 0) return cudaSuccess;
+    // Neo-Hookean and linear elastic: in 64-bit integers, no FP64 pipe (lane_kernels.cu, force_le.cu)
+    if (material == OSAM_NEO_HOOKEAN) return launch_elem_force_nh(scatter, a, s);
+    if (material == OSAM_LINEAR_ELASTIC) return launch_elem_force_le(scatter, a, s);
     const int g = grid_for(a.ne, 128);
-#define OSAM_LAUNCH(MAT, T, MODE) k_hex8_force<MAT, T, MODE><<<g, 128, 0, s>>>(a)
-    if (material == OSAM_NEO_HOOKEAN) {
-        if (fp32) { if (scatter == kAtomic) OSAM_LAUNCH(OSAM_NEO_HOOKEAN, float, kAtomic); else OSAM_LAUNCH(OSAM_NEO_HOOKEAN, float, kGather); }
-        else { if (scatter == kAtomic) OSAM_LAUNCH(OSAM_NEO_HOOKEAN, double, kAtomic); else OSAM_LAUNCH(OSAM_NEO_HOOKEAN, double, kGather); }
-    } else if (material == OSAM_SAINT_VENANT_KIRCHHOFF) {
-        if (fp32) { if (scatter == kAtomic) OSAM_LAUNCH(OSAM_SAINT_VENANT_KIRCHHOFF, float, kAtomic); else OSAM_LAUNCH(OSAM_SAINT_VENANT_KIRCHHOFF, float, kGather); }
-        else { if (scatter == kAtomic) OSAM_LAUNCH(OSAM_SAINT_VENANT_KIRCHHOFF, double, kAtomic); else OSAM_LAUNCH(OSAM_SAINT_VENANT_KIRCHHOFF, double, kGather); }
-    } else {
-        if (fp32) { if (scatter == kAtomic) OSAM_LAUNCH(OSAM_LINEAR_ELASTIC, float, kAtomic); else OSAM_LAUNCH(OSAM_LINEAR_ELASTIC, float, kGather); }
-        else { if (scatter == kAtomic) OSAM_LAUNCH(OSAM_LINEAR_ELASTIC, double, kAtomic); else OSAM_LAUNCH(OSAM_LINEAR_ELASTIC, double, kGather); }
-    }
-#undef OSAM_LAUNCH
+    if (scatter == kAtomic) k_hex8_force<OSAM_SAINT_VENANT_KIRCHHOFF, kAtomic><<<g, 128, 0, s>>>(a);
+    else k_hex8_force<OSAM_SAINT_VENANT_KIRCHHOFF, kGather><<<g, 128, 0, s>>>(a);
     return cudaGetLastError();
 }
 

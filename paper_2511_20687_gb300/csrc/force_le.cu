@@ -1,0 +1,144 @@
+// Linear elastic element force in the Walsh basis with block exponents (element_force_le, fixed_math.cuh):
+// element level, explicit step, and (the force being linear) the tangent action of implicit groups.
+//
+// The FP64 tensor-product form issues about 500 FP64 instructions of 67 to 80 cycles per element; here an
+// element takes about 60 integer products and 400 additions of 2 to 4 cycles, and no FP64 instruction
+// (uniform material).  Its rounding is 2^-58 of the element's largest displacement gradient against 2^-53 at
+// every FP64 operation.  One thread per element.
+#include <cuda_runtime.h>
+
+#include <cstdint>
+
+#include "fixed_math.cuh"
+#include "hex8_math.cuh"
+#include "osam_internal.h"
+#include "trace_item.cuh"
+
+namespace osam {
+
+namespace {
+
+using namespace fx;
+
+constexpr int kElemBlock = 64;   // element level: two warps, so that a small mesh spreads over the SMs
+
+// The same element in FP64, for operands outside the formats; lam and mu carry h / 16 (material_factors: h^2 / 32).
+// Reads the nodal values again, so that the integer path's operands stay in registers.
+__device__ __noinline__ void far_force_le(const double* u, int usn, long long usc, int sy, int sz, double lam, double mu,
+                                          double F[3][8]) {
+    using namespace hex8;
+    double Dx[3][2][2], Dy[3][2][2], Dz[3][2][2];
+    for (int c = 0; c < 3; ++c) {
+        double U[8];
+        for (int c8 = 0; c8 < 8; ++c8)
+            U[c8] = u[c * usc + (long long)((c8 & 1) + ((c8 >> 1) & 1) * sy + (c8 >> 2) * sz) * usn];
+        edge_differences_prescaled<double>(U, Dx[c], Dy[c], Dz[c]);
+    }
+    element_force<OSAM_LINEAR_ELASTIC, double>(Dx, Dy, Dz, 0.5 * lam, 0.5 * mu, 0.0, F);
+}
+
+template <int MODE>
+__device__ __forceinline__ void put(const ElemArgs& a, int e, int n0, int sy, int sz, int c8, int c, double v) {
+    if (MODE == kAtomic) {
+        const long long n = n0 + (c8 & 1) + ((c8 >> 1) & 1) * sy + (c8 >> 2) * sz;
+        atomicAdd(static_cast<double*>(a.f) + (long long)c * a.fsc + n * a.fsn, v);
+    } else {
+        static_cast<double*>(a.fe)[(long long)(c8 * 3 + c) * a.ne + e] = v;
+    }
+}
+
+template <int MODE>
+__global__ void __launch_bounds__(kElemBlock) k_elem_force_le(const __grid_constant__ ElemArgs a, double w) {
+    const int e = blockIdx.x * kElemBlock + threadIdx.x;
+    if (e >= a.ne) return;
+    const int i = e % a.nx, t = e / a.nx, j = t % a.ny, k = t / a.ny;
+    const int sy = a.nx + 1, sz = (a.nx + 1) * (a.ny + 1);
+    const int n0 = i + sy * j + sz * k;
+    double U[3][8], F[3][8];
+#pragma unroll
+    for (int c8 = 0; c8 < 8; ++c8) {
+        const long long n = n0 + (c8 & 1) + ((c8 >> 1) & 1) * sy + (c8 >> 2) * sz;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) U[c][c8] = a.u[(long long)c * a.usc + n * a.usn];
+    }
+    const double lam = (a.lam_e ? a.lam_e[e] : a.lam) * w, mu = (a.mu_e ? a.mu_e[e] : a.mu) * w;
+    if (!element_force_le(U, lam, mu, F)) {
+        double Ff[3][8];
+        far_force_le(a.u + (long long)n0 * a.usn, a.usn, a.usc, sy, sz, lam, mu, Ff);
+        for (int c8 = 0; c8 < 8; ++c8)
+            for (int c = 0; c < 3; ++c) put<MODE>(a, e, n0, sy, sz, c8, c, Ff[c][c8]);
+        return;
+    }
+#pragma unroll
+    for (int c8 = 0; c8 < 8; ++c8)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) put<MODE>(a, e, n0, sy, sz, c8, c, F[c][c8]);
+}
+
+// FomB groups: x = u / h (g.us) or the CG direction; element buffer [24][NE], trace blocks at the end of the grid
+template <bool TANGENT>
+__global__ void __launch_bounds__(128) k_fom_force_le(const __grid_constant__ FomB g, const int* __restrict__ active,
+                                                      const __grid_constant__ TraceFuse tr) {
+    if ((int)blockIdx.x >= g.n_eblk) {
+        trace::fused_trace_block(tr, active, g, (int)blockIdx.x - g.n_eblk);
+        return;
+    }
+    const int2 b = g.eblk[blockIdx.x];
+    if (active && !active[b.x]) return;
+    const InstFom& I = g.inst[b.x];
+    const int e = b.y + threadIdx.x;
+    if (e >= I.ne) return;
+    const int nx = I.nx, ny = I.ny, i = e % nx, t = e / nx, j = t % ny, k = t / ny;
+    const int sy = nx + 1, sz = (nx + 1) * (ny + 1);
+    const double* x = (TANGENT ? g.cg_p : g.us) + I.node_off + (i + sy * j + sz * k);
+    double U[3][8], F[3][8];
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+#pragma unroll
+        for (int c8 = 0; c8 < 8; ++c8)
+            U[c][c8] = x[(long long)c * g.NN + (c8 & 1) + ((c8 >> 1) & 1) * sy + (c8 >> 2) * sz];
+    double lam = TANGENT ? I.t1 : I.s1, mu = TANGENT ? I.t2 : I.s2;
+    if (I.lam_e || I.mu_e) {
+        const double w = 2.0 * (TANGENT ? I.wqi : I.wq);
+        lam = (I.lam_e ? I.lam_e[e] : I.lam) * w;
+        mu = (I.mu_e ? I.mu_e[e] : I.mu) * w;
+    }
+    double* fe = static_cast<double*>(g.fe) + I.elem_off + e;
+    if (!element_force_le(U, lam, mu, F)) {
+        double Ff[3][8];
+        far_force_le(x, 1, g.NN, sy, sz, lam, mu, Ff);
+        for (int c8 = 0; c8 < 8; ++c8)
+            for (int c = 0; c < 3; ++c) fe[(long long)(c8 * 3 + c) * g.NE] = Ff[c][c8];
+        return;
+    }
+#pragma unroll
+    for (int c8 = 0; c8 < 8; ++c8)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) fe[(long long)(c8 * 3 + c) * g.NE] = F[c][c8];
+}
+
+}  // namespace
+
+cudaError_t launch_elem_force_le(int scatter, const ElemArgs& a, cudaStream_t s) {
+    const int grid = grid_for(a.ne, kElemBlock);
+    const double w = 2.0 * a.wq * a.invh;   // h / 16
+    if (scatter == kAtomic) k_elem_force_le<kAtomic><<<grid, kElemBlock, 0, s>>>(a, w);
+    else k_elem_force_le<kGather><<<grid, kElemBlock, 0, s>>>(a, w);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_force_le_b(const FomB& g, const int* active, const TraceFuse& tr, cudaStream_t s) {
+    if (g.eblock > 128) return cudaErrorInvalidValue;
+    long long items = 0;
+    for (int k = 0; k < tr.n; ++k) items += 3LL * tr.c[k].R;
+    k_fom_force_le<false><<<g.n_eblk + (int)((items + g.eblock - 1) / g.eblock), g.eblock, 0, s>>>(g, active, tr);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_tangent_le_b(const FomB& g, const int* mask, cudaStream_t s) {
+    if (g.eblock > 128) return cudaErrorInvalidValue;
+    k_fom_force_le<true><<<g.n_eblk, g.eblock, 0, s>>>(g, mask, TraceFuse{});
+    return cudaGetLastError();
+}
+
+}  // namespace osam

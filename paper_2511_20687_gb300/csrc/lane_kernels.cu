@@ -1,0 +1,264 @@
+// Neo-Hookean element kernels with one element on 8 lanes (lanes.cuh), in 64-bit integers: the element-level
+// force and its vector-Jacobian product, the force of the implicit Newton residual and the tangent action of
+// its CG iterations.
+//
+// The FP64 forms were bound by the FP64 pipe at every size: a warp that carries 32 elements issues 720
+// (force) to 1500 (vector-Jacobian product) FP64 instructions of 67 to 80 cycles, 25 to 55 us however few elements
+// there are.  Here a Gauss point takes about 250 (force) or 550 (tangent) integer multiply-adds of 4 cycles, and
+// 8 lanes per element put 8 times as many warps in flight on a small mesh.  An element outside the formats'
+// range is evaluated in FP64 by one of its lanes.
+#include <cuda_runtime.h>
+
+#include <cmath>
+#include <cstdint>
+
+#include "hex8_math.cuh"
+#include "lanes.cuh"
+#include "nh_tangent.cuh"
+#include "osam_internal.h"
+
+namespace osam {
+
+namespace {
+
+using namespace fx;
+
+constexpr int kLaneBlock = 128;                   // 16 elements
+
+// FP64 evaluation of one element (all 24 values, parameter contractions) for operands outside the formats.
+// x(c, corner) and p(c, corner) read the displacement and the direction.  Not inlined into the lane path's registers.
+struct FarIn {
+    const double *u, *p;
+    int usn, psn;
+    long long usc, psc;
+    int n0, sy, sz;
+    double invh, lam, mu, wq, wq3;
+    __device__ long long node(int c8) const { return n0 + (c8 & 1) + ((c8 >> 1) & 1) * sy + ((c8 >> 2) & 1) * (long long)sz; }
+};
+
+__device__ __noinline__ void far_force(const FarIn& x, double F[3][8]) {
+    using namespace hex8;
+    double Dx[3][2][2], Dy[3][2][2], Dz[3][2][2], m1, m2, m3;
+    material_factors<OSAM_NEO_HOOKEAN, double>(x.lam, x.mu, x.wq, x.wq3, m1, m2, m3);
+    for (int c = 0; c < 3; ++c) {
+        double U[8];
+        for (int c8 = 0; c8 < 8; ++c8) U[c8] = x.u[c * x.usc + x.node(c8) * x.usn];
+        edge_differences<double>(U, x.invh, Dx[c], Dy[c], Dz[c]);
+    }
+    element_force<OSAM_NEO_HOOKEAN, double>(Dx, Dy, Dz, m1, m2, m3, F);
+}
+
+__device__ __noinline__ void far_tangent(const FarIn& x, double F[3][8], double& lb, double& mb) {
+    using namespace hex8;
+    double Gx[3][2][2], Gy[3][2][2], Gz[3][2][2], Bx[3][2][2], By[3][2][2], Bz[3][2][2], m1, m2, m3;
+    material_factors<OSAM_NEO_HOOKEAN, double>(x.lam, x.mu, x.wq, x.wq3, m1, m2, m3);
+    for (int c = 0; c < 3; ++c) {
+        double U[8], Dx[2][2], Dy[2][2], Dz[2][2];
+        for (int c8 = 0; c8 < 8; ++c8) U[c8] = x.u[c * x.usc + x.node(c8) * x.usn];
+        edge_differences<double>(U, x.invh, Dx, Dy, Dz);
+        lerp2(Dx, Gx[c]); lerp2(Dy, Gy[c]); lerp2(Dz, Gz[c]);
+        for (int c8 = 0; c8 < 8; ++c8) U[c8] = x.p[c * x.psc + x.node(c8) * x.psn];
+        edge_differences<double>(U, x.invh, Dx, Dy, Dz);
+        lerp2(Dx, Bx[c]); lerp2(Dy, By[c]); lerp2(Dz, Bz[c]);
+    }
+    double Sx[3][2][2] = {}, Sy[3][2][2] = {}, Sz[3][2][2] = {};
+    lb = mb = 0.0;
+    for (int g = 0; g < 8; ++g) {
+        const int p = g >> 2, q = (g >> 1) & 1, r = g & 1;
+        double H[3][3], G[3][3], dP[3][3], pk, pm;
+        for (int c = 0; c < 3; ++c) {
+            H[c][0] = Gx[c][q][r]; H[c][1] = Gy[c][p][r]; H[c][2] = Gz[c][p][q];
+            G[c][0] = Bx[c][q][r]; G[c][1] = By[c][p][r]; G[c][2] = Bz[c][p][q];
+        }
+        tangent::nh_tangent(H, G, m1, m2, m3, dP, pk, pm);
+        lb += pk;
+        mb = fma(2.0 / 3.0, pk, mb + pm);
+        for (int c = 0; c < 3; ++c) { Sx[c][q][r] += dP[c][0]; Sy[c][p][r] += dP[c][1]; Sz[c][p][q] += dP[c][2]; }
+    }
+    walsh_transpose<double>(Sx, Sy, Sz, F);
+}
+
+// The element of a lane group in one mesh; lanes beyond the last element repeat it (all lanes take part in
+// the shuffles) and write nothing
+struct Elem {
+    int e, n0, sy, sz;
+    bool live;
+};
+__device__ __forceinline__ Elem element(int e, int nx, int ny, int ne) {
+    Elem x;
+    x.live = e < ne;
+    x.e = x.live ? e : ne - 1;
+    const int i = x.e % nx, t = x.e / nx, j = t % ny, k = t / ny;
+    x.sy = nx + 1;
+    x.sz = (nx + 1) * (ny + 1);
+    x.n0 = i + x.sy * j + x.sz * k;
+    return x;
+}
+__device__ __forceinline__ int corner_node(const Elem& x, int a) {
+    return x.n0 + (a & 1) + ((a >> 1) & 1) * x.sy + (a >> 2) * x.sz;
+}
+
+// ---- element level: one mesh, strided operands (ElemArgs) ----------------------------------------
+template <int MODE>
+__device__ __forceinline__ void put(const ElemArgs& a, const Elem& x, int corner, int c, double v) {
+    if (MODE == kAtomic)
+        atomicAdd(static_cast<double*>(a.f) + (long long)c * a.fsc + (long long)corner_node(x, corner) * a.fsn, v);
+    else
+        static_cast<double*>(a.fe)[(long long)(corner * 3 + c) * a.ne + x.e] = v;
+}
+
+__device__ __forceinline__ FarIn far_in(const ElemArgs& a, const Elem& x, const double* p, int psn, long long psc,
+                                        double lam, double mu) {
+    return FarIn{a.u, p, a.usn, psn, a.usc, psc, x.n0, x.sy, x.sz, a.invh, lam, mu, a.wq, a.wq3};
+}
+
+template <int MODE>
+__global__ void __launch_bounds__(kLaneBlock) k_elem_force(const __grid_constant__ ElemArgs a, i64 ihm, int ihe) {
+    const Elem x = element((int)(blockIdx.x * (kLaneBlock / 8) + (threadIdx.x >> 3)), a.nx, a.ny, a.ne);
+    const Lane L = make_lane();
+    const int node = corner_node(x, L.a);
+    i64 U[3], F[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) U[c] = fixed_u(a.u[(long long)c * a.usc + (long long)node * a.usn], ihm, ihe);
+    const double lam = a.lam_e ? a.lam_e[x.e] : a.lam, mu = a.mu_e ? a.mu_e[x.e] : a.mu;
+    Material M;
+    bool bad = !material(lam, mu, a.wq, M);
+    const bool ok = force_lanes(L, U, M.kap2, M.mu, M.mu3, bad || M.k < -900 || M.k > 900, F);
+    if (!x.live) return;
+    if (ok) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) put<MODE>(a, x, L.a, c, f64_scaled(F[c], 57 - M.k));
+    } else if (L.a == 0) {
+        double Ff[3][8];
+        far_force(far_in(a, x, nullptr, 0, 0, lam, mu), Ff);
+        for (int c8 = 0; c8 < 8; ++c8)
+            for (int c = 0; c < 3; ++c) put<MODE>(a, x, c8, c, Ff[c][c8]);
+    }
+}
+
+template <int MODE>
+__global__ void __launch_bounds__(kLaneBlock) k_elem_vjp(const __grid_constant__ ElemArgs a, const double* ybar, int ysn,
+                                                         long long ysc, double* lam_bar, double* mu_bar, int accumulate,
+                                                         i64 ihm, int ihe, double wqi, double vol) {
+    const Elem x = element((int)(blockIdx.x * (kLaneBlock / 8) + (threadIdx.x >> 3)), a.nx, a.ny, a.ne);
+    const Lane L = make_lane();
+    const int node = corner_node(x, L.a);
+    i64 U[3], F[3], pk = 0, pm = 0;
+    double p[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        U[c] = fixed_u(a.u[(long long)c * a.usc + (long long)node * a.usn], ihm, ihe);
+        p[c] = ybar[(long long)c * ysc + (long long)node * ysn];
+    }
+    const double lam = a.lam_e ? a.lam_e[x.e] : a.lam, mu = a.mu_e ? a.mu_e[x.e] : a.mu;
+    Material M;
+    const bool bad = !material(lam, mu, wqi, M);
+    int scale, base;
+    const bool ok = tangent_lanes(L, U, p, M, bad, lam_bar || mu_bar, F, scale, pk, pm, base);
+    if (!x.live) return;
+    double lb = 0.0, mb = 0.0;
+    if (ok) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) put<MODE>(a, x, L.a, c, f64_scaled(F[c], scale));
+        lb = vol * f64_scaled(pk, 60 + base);
+        mb = vol * f64_scaled(pm, 56 + base);
+    } else if (L.a == 0) {
+        double Ff[3][8];
+        far_tangent(far_in(a, x, ybar, ysn, ysc, lam, mu), Ff, lb, mb);
+        for (int c8 = 0; c8 < 8; ++c8)
+            for (int c = 0; c < 3; ++c) put<MODE>(a, x, c8, c, Ff[c][c8]);
+        lb *= a.w8 / a.invh;
+        mb *= a.w8 / a.invh;
+    }
+    if (L.a != 0) return;
+    if (lam_bar) lam_bar[x.e] = (accumulate ? lam_bar[x.e] : 0.0) + lb;
+    if (mu_bar) mu_bar[x.e] = (accumulate ? mu_bar[x.e] : 0.0) + mb;
+}
+
+// ---- implicit groups (FomB): element buffer [24][NE] ----------------------------------------------
+// TANGENT: K(u) p of the CG direction; else the internal force of u
+template <bool TANGENT>
+__global__ void __launch_bounds__(kLaneBlock) k_fom_lanes(const __grid_constant__ FomB g, const int* __restrict__ mask) {
+    const int per = g.eblock * 8 / kLaneBlock;   // thread blocks per element block
+    const int2 b = g.eblk[blockIdx.x / per];
+    if (mask && !mask[b.x]) return;
+    const InstFom& I = g.inst[b.x];
+    const int first = b.y + (int)(blockIdx.x % per) * (kLaneBlock / 8);
+    if (first >= I.ne) return;
+    const Elem x = element(first + (int)(threadIdx.x >> 3), I.nx, I.ny, I.ne);
+    const Lane L = make_lane();
+    const long long gn = I.node_off + corner_node(x, L.a);
+    i64 U[3], F[3], pk, pm;
+    double p[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        U[c] = fixed_u(g.u[0][c * g.NN + gn], I.ihm, I.ihe);
+        if (TANGENT) p[c] = g.cg_p[c * g.NN + gn];
+    }
+    const double lam = I.lam_e ? I.lam_e[x.e] : I.lam, mu = I.mu_e ? I.mu_e[x.e] : I.mu;
+    Material M;
+    const bool bad = !material(lam, mu, TANGENT ? I.wqi : I.wq, M);
+    int scale = 57 - M.k, base;
+    const bool ok = TANGENT ? tangent_lanes(L, U, p, M, bad, false, F, scale, pk, pm, base)
+                            : force_lanes(L, U, M.kap2, M.mu, M.mu3, bad || M.k < -900 || M.k > 900, F);
+    if (!x.live) return;
+    double* fe = static_cast<double*>(g.fe) + I.elem_off + x.e;
+    if (ok) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) fe[(long long)(L.a * 3 + c) * g.NE] = f64_scaled(F[c], scale);
+    } else if (L.a == 0) {
+        const FarIn in{g.u[0] + I.node_off, TANGENT ? g.cg_p + I.node_off : nullptr, 1, 1, g.NN, g.NN, x.n0, x.sy, x.sz,
+                       I.invh, lam, mu, I.wq, I.wq3};
+        double Ff[3][8], lb, mb;
+        if (TANGENT) far_tangent(in, Ff, lb, mb);
+        else far_force(in, Ff);
+        for (int c8 = 0; c8 < 8; ++c8)
+            for (int c = 0; c < 3; ++c) fe[(long long)(c8 * 3 + c) * g.NE] = Ff[c][c8];
+    }
+}
+
+int elem_grid(int ne) { return grid_for(8LL * ne, kLaneBlock); }
+
+}  // namespace
+
+void fixed_point_inverse(double x, long long& m, int& e) {
+    int k;
+    m = (long long)std::ldexp(std::frexp(x, &k), 63);
+    e = k - 1;
+}
+
+cudaError_t launch_elem_force_nh(int scatter, const ElemArgs& a, cudaStream_t s) {
+    long long m;
+    int e;
+    fixed_point_inverse(a.invh, m, e);
+    if (scatter == kAtomic) k_elem_force<kAtomic><<<elem_grid(a.ne), kLaneBlock, 0, s>>>(a, m, e);
+    else k_elem_force<kGather><<<elem_grid(a.ne), kLaneBlock, 0, s>>>(a, m, e);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_elem_vjp_nh(int scatter, const ElemArgs& a, const double* ybar, int ysn, long long ysc,
+                               double* lam_bar, double* mu_bar, int acc, cudaStream_t s) {
+    long long m;
+    int e;
+    fixed_point_inverse(a.invh, m, e);
+    const double wqi = a.wq * a.invh, vol = a.w8;   // h^3 / 8 per Gauss point; the gradients carry 1 / h
+    if (scatter == kAtomic)
+        k_elem_vjp<kAtomic><<<elem_grid(a.ne), kLaneBlock, 0, s>>>(a, ybar, ysn, ysc, lam_bar, mu_bar, acc, m, e, wqi, vol);
+    else
+        k_elem_vjp<kGather><<<elem_grid(a.ne), kLaneBlock, 0, s>>>(a, ybar, ysn, ysc, lam_bar, mu_bar, acc, m, e, wqi, vol);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_imp_force_nh_b(const FomB& g, const int* mask, cudaStream_t s) {
+    if (g.eblock % 32) return cudaErrorInvalidValue;
+    k_fom_lanes<false><<<g.n_eblk * (g.eblock * 8 / kLaneBlock), kLaneBlock, 0, s>>>(g, mask);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_imp_tangent_nh_b(const FomB& g, const int* mask, cudaStream_t s) {
+    if (g.eblock % 32) return cudaErrorInvalidValue;
+    k_fom_lanes<true><<<g.n_eblk * (g.eblock * 8 / kLaneBlock), kLaneBlock, 0, s>>>(g, mask);
+    return cudaGetLastError();
+}
+
+}  // namespace osam

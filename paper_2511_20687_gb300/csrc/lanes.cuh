@@ -1,0 +1,175 @@
+// One hex8 element on 8 lanes: lane a (bits x, y, z) holds corner a, then Walsh pattern a, then Gauss point
+// a, then corner a again.  In the sign basis (s = 2 bit - 1 per axis) interpolation to the Gauss points and its
+// transpose are butterflies over lane bits, so the 8 lanes share all of an element's work and nothing is
+// computed twice; every value is a 64-bit integer (fixed_math.cuh), so the sums are exact.
+#pragma once
+
+#include <cuda_runtime.h>
+
+#include "fixed_math.cuh"
+
+namespace osam {
+namespace fx {
+
+struct Lane {
+    int a;             // corner / pattern / Gauss point
+    i64 n[3];          // -1 where the lane's bit of an axis is set, else 0
+    D k;               // factor of the lane's pattern: t^(order - 1) - keep
+    bool keep;
+};
+
+__device__ __forceinline__ Lane make_lane() {
+    Lane L;
+    L.a = (int)(threadIdx.x & 7u);
+#pragma unroll
+    for (int d = 0; d < 3; ++d) L.n[d] = -(i64)((L.a >> d) & 1);
+    const int order = __popc((unsigned int)L.a);
+    L.k = order == 2 ? split(kTm1) : (order == 3 ? split(kThird) : split(0));
+    L.keep = order != 3;
+    return L;
+}
+
+__device__ __forceinline__ i64 other(i64 v, int axis) { return __shfl_xor_sync(0xffffffffu, v, 1 << axis); }
+__device__ __forceinline__ i64 flip(i64 x, i64 n) { return (x ^ n) - n; }   // -x where n is -1
+
+// sums over an axis: pattern bit 0 lower + upper, bit 1 upper - lower
+__device__ __forceinline__ i64 sum_stage(const Lane& L, i64 v, int axis) { return v + flip(other(v, axis), L.n[axis]); }
+// values at the signs of an axis: lower f0 - f1, upper f0 + f1
+__device__ __forceinline__ i64 eval_stage(const Lane& L, i64 v, int axis) { return v + flip(other(v, axis), ~L.n[axis]); }
+// plain sum over an axis on the lanes whose bit is set, zero on the others
+__device__ __forceinline__ i64 set_sum(const Lane& L, i64 v, int axis) { return (v + other(v, axis)) & L.n[axis]; }
+
+__device__ __forceinline__ i64 walsh_sums(const Lane& L, i64 v) {
+    return sum_stage(L, sum_stage(L, sum_stage(L, v, 0), 1), 2);
+}
+__device__ __forceinline__ i64 corner_values(const Lane& L, i64 v) {
+    return eval_stage(L, eval_stage(L, eval_stage(L, v, 0), 1), 2);
+}
+// the 1/sqrt3 powers of the lane's pattern
+__device__ __forceinline__ i64 pattern_scale(const Lane& L, i64 v) { return mul_add(split(v), L.k, L.keep ? v : 0); }
+
+// derivatives along the three axes at the lane's Gauss point from the scaled coefficients of one component
+__device__ __forceinline__ void gauss_columns(const Lane& L, i64 w, int c, Cols& C) {
+    const i64 z = eval_stage(L, w, 2), y = eval_stage(L, w, 1);
+    const i64 gx = eval_stage(L, z, 1), gy = eval_stage(L, z, 0), gz = eval_stage(L, y, 0);
+    const int lane = (int)(threadIdx.x & 31u);
+    C.x[0][c] = __shfl_sync(0xffffffffu, gx, lane | 1);
+    C.x[1][c] = __shfl_sync(0xffffffffu, gy, lane | 2);
+    C.x[2][c] = __shfl_sync(0xffffffffu, gz, lane | 4);
+}
+// its transpose: the coefficients of the corner forces from the stress columns (p0, p1, p2) of one component
+__device__ __forceinline__ i64 gauss_transpose(const Lane& L, i64 p0, i64 p1, i64 p2) {
+    i64 A = set_sum(L, p0, 0), B = sum_stage(L, p1, 0), C = sum_stage(L, p2, 0);
+    A = sum_stage(L, A, 1);
+    B = set_sum(L, B, 1);
+    C = sum_stage(L, C, 1);
+    return sum_stage(L, A + B, 2) + set_sum(L, C, 2);
+}
+
+// true in all 8 lanes of an element if it is in any of them
+__device__ __forceinline__ bool any_lane(bool x) {
+    return ((__ballot_sync(0xffffffffu, x) >> (threadIdx.x & 24u)) & 0xffu) != 0;
+}
+template <typename T, typename Op>
+__device__ __forceinline__ T reduce8(T x, Op op) {
+#pragma unroll
+    for (int b = 1; b < 8; b <<= 1) x = op(x, __shfl_xor_sync(0xffffffffu, x, b));
+    return x;
+}
+
+// Columns of F from this lane's fixed-point u / h (59 fraction bits); bad: a node outside the format, or a Walsh
+// coefficient at or above 11 (found from the values cut to 23 fraction bits, which cannot wrap)
+__device__ __forceinline__ void deformation(const Lane& L, const i64 U[3], Cols& C, bool& bad) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        bad |= hi(U[c]) < -((kMaxU + 1) << 27);
+        int v = hi(U[c]) >> 4;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            const int o = __shfl_xor_sync(0xffffffffu, v, 1 << d), n = (int)L.n[d];
+            v += (o ^ n) - n;
+        }
+        bad |= L.a != 0 && (v >= (11 << 23) || v <= -(11 << 23));
+        i64 w = walsh_sums(L, U[c]);
+        if (L.a == 1 << c) w += (i64)1 << kFracF;
+        gauss_columns(L, pattern_scale(L, L.a ? w : 0), c, C);
+    }
+}
+
+// A direction in block format: its scaled gradient columns, gradient = G 2^-base / h; returns the base
+__device__ __forceinline__ int direction(const Lane& L, const double p[3], Cols& G, bool& bad) {
+    i64 w[3];
+    int e[3], T = kNoExponent;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        e[c] = (int)(reduce8(hi_word(p[c]) & 0x7fffffffu, [](unsigned int a, unsigned int b) { return max(a, b); }) >> 20);
+        w[c] = walsh_sums(L, block_value(p[c], e[c]));
+        if (L.a == 0) w[c] = 0;
+        T = max(T, top_exponent(mag(w[c]), e[c]));
+        bad |= e[c] == 2047 || (e[c] == 0 && shl(__double_as_longlong(p[c]), 1) != 0);   // not finite, subnormal
+    }
+    T = reduce8(T, [](int a, int b) { return max(a, b); });
+    const bool zero = T == kNoExponent;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) gauss_columns(L, pattern_scale(L, zero ? 0 : shift(w[c], e[c] - T - 6)), c, G);
+    return zero ? 0 : 1016 - T;                // 1081 - 59 - 6
+}
+
+// Material factors kappa/2 and mu times w as integers: value = X 2^(k - 62), the larger in [2^61, 2^62);
+// false unless both are positive and finite
+struct Material {
+    D kap2, mu, mu3;
+    int k;
+};
+__device__ __forceinline__ bool material(double lam, double mu, double w, Material& M) {
+    const int e = factor_exponent(lam, mu), ew = factor_exponent(w, 0.0);
+    const i64 l = factor_value(lam, e), m = factor_value(mu, e);
+    const D wd = split(factor_value(w, ew));
+    const i64 K = mul(split((l >> 1) + mul_third(m)), wd), U = mul(split(m), wd);
+    if (e == 2047 || ew == 2047 || ew == 0 || K <= 0 || U <= 0) return false;
+    const int n = lead_zeros(K | U) - 2;
+    const i64 us = shl(U, n);
+    M.kap2 = split(shl(K, n));
+    M.mu = split(us);
+    M.mu3 = split(mul_third(us));
+    M.k = e + ew - 2042 - n;     // 2 x 1084 - 64 - 62
+    return true;
+}
+
+// corner forces of the lane's corner (57 fraction bits, units 2^k); false if the element is out of range
+__device__ __forceinline__ bool force_lanes(const Lane& L, const i64 U[3], D kap2, D mu, D mu3, bool bad, i64 F[3]) {
+    Cols C;
+    deformation(L, U, C, bad);
+    i64 P[3][3];
+    bad |= !stress_point(C, kap2, mu, mu3, P);
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+        F[c] = corner_values(L, pattern_scale(L, gauss_transpose(L, P[0][c], P[1][c], P[2][c])));
+    return !any_lane(bad);
+}
+
+// tangent action on a direction p (FP64): value of the lane's corner = F 2^-scale; the sums over the Gauss points
+// of pk (60 fraction bits) and pm + 2/3 pk (56) with `base` more from the direction's own exponent
+__device__ __forceinline__ bool tangent_lanes(const Lane& L, const i64 U[3], const double p[3], const Material& M,
+                                              bool bad, bool contract, i64 F[3], int& scale, i64& pk, i64& pm, int& base) {
+    Cols C, G;
+    deformation(L, U, C, bad);
+    base = direction(L, p, G, bad);
+    i64 dP[3][3];
+    bad |= !tangent_point(C, G, M.kap2, M.mu, M.mu3, dP, pk, pm);
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+        F[c] = corner_values(L, pattern_scale(L, gauss_transpose(L, dP[0][c], dP[1][c], dP[2][c])));
+    scale = 56 + base - M.k;
+    if (contract) {
+        pm += mul_third(pk) >> 3;
+        pk = reduce8(pk, [](i64 a, i64 b) { return a + b; });
+        pm = reduce8(pm, [](i64 a, i64 b) { return a + b; });
+    }
+    // the results' exponents stay inside the normal range
+    bad |= scale > 1000 || base > 950 || scale < -900 || base < -960;
+    return !any_lane(bad);
+}
+
+}  // namespace fx
+}  // namespace osam

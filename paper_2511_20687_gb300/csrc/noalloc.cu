@@ -83,7 +83,7 @@ int device_setup(cudaStream_t s, double** out) {
         a.u = base + 24; a.usn = 3; a.usc = 1;
         a.fe = base;
         for (int m : {OSAM_LINEAR_ELASTIC, OSAM_NEO_HOOKEAN, OSAM_SAINT_VENANT_KIRCHHOFF})
-            if (e == cudaSuccess) e = osam::launch_hex8_force(m, false, osam::kGather, a, s);
+            if (e == cudaSuccess) e = osam::launch_hex8_force(m, osam::kGather, a, s);
         if (e == cudaSuccess) {
             k_gather_aos<<<1, 32, 0, s>>>(1, 1, 1, base, base + 48);
             e = cudaGetLastError();
@@ -137,7 +137,7 @@ extern "C" OSAM_API int osam_hex8_force_noalloc(int nx, int ny, int nz, double h
     a.u = u; a.usn = 3; a.usc = 1;
     a.fe = fe;
     // every element writes all 24 of its entries, so the buffer needs no clearing between calls
-    cudaError_t e = osam::launch_hex8_force(material, false, osam::kGather, a, s);
+    cudaError_t e = osam::launch_hex8_force(material, osam::kGather, a, s);
     if (e == cudaSuccess) {
         const long long nn = (long long)(nx + 1) * (ny + 1) * (nz + 1);
         k_gather_aos<<<(int)((3 * nn + 255) / 256), 256, 0, s>>>(nx, ny, nz, fe, f);

@@ -440,7 +440,7 @@ int osam_hex8_force(int nx, int ny, int nz, double h, int material, double lambd
     if (cudaMemsetAsync(f, 0, sizeof(double) * 3 * nn, s) != cudaSuccess) return OSAM_ECUDA;
     ElemArgs a = standalone_args(nx, ny, nz, h, lambda, mu, lambda_e, mu_e, u);
     a.f = f;
-    return launch_hex8_force(material, false, kAtomic, a, s) == cudaSuccess ? OSAM_OK : OSAM_ECUDA;
+    return launch_hex8_force(material, kAtomic, a, s) == cudaSuccess ? OSAM_OK : OSAM_ECUDA;
 }
 
 int osam_hex8_force_vjp(int nx, int ny, int nz, double h, int material, double lambda, double mu,
@@ -491,10 +491,14 @@ int osam_adjoint(const osam_adjoint_desc* d, osam_adjoint_out* out) {
     pd.scatter = OSAM_SCATTER_GATHER;   // element buffer + fixed-order gather: bitwise repeatable gradients
     pd.stream = d->stream;
     pd.device = d->device;
-    osam_ctx* raw = nullptr;
-    if (int rc = osam_batch_init(1, &pd, &raw)) return rc;
-    std::unique_ptr<osam_ctx> holder(raw);
-    osam_ctx* ctx = raw;
+    g_init_error.clear();
+    std::unique_ptr<osam_ctx> holder(new osam_ctx());
+    osam_ctx* ctx = holder.get();
+    ctx->integer_force = true;          // exact integer sums: as repeatable as the fixed-order gather
+    if (int rc = init_impl(ctx, 1, &pd)) {
+        g_init_error = ctx->err;
+        return rc;
+    }
     FomB& F = ctx->slots[0].fom.d;
     const InstFom& I = ctx->slots[0].fom.inst[0];
     const int nn = I.nn, ne = I.ne;
@@ -525,7 +529,7 @@ int osam_adjoint(const osam_adjoint_desc* d, osam_adjoint_out* out) {
     // one explicit step in place on (u[0], v, a), deterministic element-buffer scatter
     auto step = [&](double* u_store, cudaStream_t st) -> int {
         CK(launch_node_b(F, nullptr, kGather, -1, 1, 1, F.u[0], F.u[1], dt, st));
-        CK(launch_force_b(F, nullptr, kGather, st));
+        CK(launch_force_b(F, nullptr, kGather, st, nullptr, F.u[1]));
         CK(launch_node_b(F, nullptr, kGather, 1, -1, 0, F.u[1], F.u[0], dt, st));
         CK(cudaMemcpyAsync(F.u[0], F.u[1], sizeof(double) * n3, cudaMemcpyDeviceToDevice, st));
         if (u_store) CK(cudaMemcpyAsync(u_store, F.u[0], sizeof(double) * n3, cudaMemcpyDeviceToDevice, st));

@@ -23,7 +23,7 @@ namespace osam {
 enum Scatter { kAtomic = 1, kGather = 2 };
 
 constexpr int kMaxSlots = 8;    // subdomains per instance
-constexpr int kLinPerGp = 22;   // doubles per Gauss point of the stored Neo-Hookean Newton linearisation
+constexpr int kLinPerGp = 22;   // floats per Gauss point of the stored Neo-Hookean Newton linearisation
 constexpr int kNodeBlock = 128; // nodes per block of the node kernels
 
 struct Grid {
@@ -66,6 +66,8 @@ struct InstFom {
     // 2^(54 - fscale) (fscale: fraction bits of the element forces), 1/h as ihm 2^(ihe - 62)
     long long fk2, fmu, ihm;
     int ihe, fscale;
+    double wqi;               // wq / h (weight of the tangent action on a direction that is not divided by h)
+    double s1, s2, t1, t2;    // linear elastic: lam and mu times 2 wq and 2 wqi (element_force_le)
 };
 
 // kernel view of a FOM slot across instances; nodal arrays are SoA over the concatenated nodes:
@@ -124,11 +126,11 @@ struct FomB {
     int* nact;                // per instance Newton state: 1 iterating, 0 converged, 2 failed
     int* cgact;               // per instance: CG still iterating
     long long* istat;         // per instance: Newton linear solves, CG iterations (since the last reset)
-    double* lin;              // Neo-Hookean implicit groups: stored Newton linearisation [kLinPerGp][8][NE]
-    float* linf;              // the same in FP32 (OSAM_FP64_TANGENT32; lin is then null)
+    float* linf;              // OSAM_FP64_TANGENT32, Neo-Hookean implicit groups: Newton linearisation [kLinPerGp][8][NE]
     float* fe32;              // FP32 element buffer [24][NE] of the FP32 tangent action
     int df32;                 // 1: internal force in double-float arithmetic (element buffer of float2)
-    int fixed;                // 1: internal force in 64-bit fixed point (element buffer of int64; force_fx.cu)
+    int fixed;                // internal force in 64-bit integers: 1 Neo-Hookean (element buffer of int64; force_fx.cu),
+                              // 2 linear elastic (element buffer of double; force_le.cu)
     long long* ux;            // fixed-point predicted displacement / h [3][NN]
     double* fe2;              // FP64 contributions of the elements outside the fixed-point range [24][NE]
 };
@@ -208,7 +210,7 @@ struct CtlB {
 // element level, set-up and I/O (fom_kernels.cu)
 // ------------------------------------------------------------------------------------------------
 int grid_for(long long n, int block);
-cudaError_t launch_hex8_force(int material, bool fp32, int scatter, const ElemArgs& a, cudaStream_t s);
+cudaError_t launch_hex8_force(int material, int scatter, const ElemArgs& a, cudaStream_t s);
 cudaError_t launch_lumped_minv(const Grid& g, double rho, double* minv, cudaStream_t s, double* mass = nullptr);
 cudaError_t launch_donor(const Grid& src, const Grid& dst, const int* dst_nodes, int nrow, int* dnode, double* dw,
                          int* err, cudaStream_t s);
@@ -236,6 +238,18 @@ cudaError_t launch_force_fx_b(const FomB& g, const int* active, const TraceFuse&
                               cudaStream_t s);
 cudaError_t launch_node_fx_b(const FomB& g, const int* active, int slot1, int slot2, int predict_only,
                              const double* ucur, double* unext, double dt, cudaStream_t s);
+// Neo-Hookean element level and implicit groups in 64-bit integers, 8 lanes per element (lane_kernels.cu);
+// fixed_point_inverse: x as m 2^(e - 62), m in [2^62, 2^63)
+void fixed_point_inverse(double x, long long& m, int& e);
+cudaError_t launch_elem_force_nh(int scatter, const ElemArgs& a, cudaStream_t s);
+cudaError_t launch_elem_vjp_nh(int scatter, const ElemArgs& a, const double* ybar, int ysn, long long ysc,
+                               double* lam_bar, double* mu_bar, int acc, cudaStream_t s);
+cudaError_t launch_imp_force_nh_b(const FomB& g, const int* mask, cudaStream_t s);
+cudaError_t launch_imp_tangent_nh_b(const FomB& g, const int* mask, cudaStream_t s);
+// linear elastic in 64-bit integers (force_le.cu)
+cudaError_t launch_elem_force_le(int scatter, const ElemArgs& a, cudaStream_t s);
+cudaError_t launch_force_le_b(const FomB& g, const int* active, const TraceFuse& tr, cudaStream_t s);
+cudaError_t launch_tangent_le_b(const FomB& g, const int* mask, cudaStream_t s);
 // double-float mode (force_df.cu)
 cudaError_t launch_split_u2_b(const FomB& g, cudaStream_t s);
 cudaError_t launch_force_df_b(const FomB& g, const int* active, const TraceFuse& tr, cudaStream_t s);
@@ -268,8 +282,8 @@ cudaError_t launch_imp_residual_b(const FomB& g, const int* mask, double c0, cud
 // products are reduced inside k_cg_ap_b / k_cg_step_b by each instance's last block.
 cudaError_t launch_imp_reduce_b(const FomB& g, const int* mask, int mode, int first, double tol2, cudaStream_t s);
 cudaError_t launch_tangent_b(const FomB& g, const int* mask, cudaStream_t s);
-// Neo-Hookean implicit groups: Newton force that also stores the Gauss-point linearisation, and the
-// tangent action that reads it
+// Neo-Hookean implicit groups with the FP32 tangent: Newton force that also stores the Gauss-point
+// linearisation, and the tangent action that reads it
 cudaError_t launch_force_lin_b(const FomB& g, const int* mask, cudaStream_t s);
 cudaError_t launch_tangent_lin_b(const FomB& g, const int* mask, cudaStream_t s);
 cudaError_t launch_cg_ap_b(const FomB& g, const int* mask, double c0, cudaStream_t s);
@@ -300,6 +314,11 @@ cudaError_t launch_gemm_nn(int m, int n, int k, const double* A, int lda, const 
                            int ldc, double alpha, double beta, cudaStream_t s);
 cudaError_t launch_gemm_nt(int m, int n, int k, const double* A, int lda, const double* B, int ldb, double* C,
                            int ldc, double alpha, double beta, cudaStream_t s);
+// the same on the bf16 tensor cores by exact splitting (split_gemm.cu); element strides (ai, ak), (bk, bj)
+constexpr int kSplitChunk = 1024;
+cudaError_t launch_split_gemm(int m, int n, int k, const double* A, long long ai, long long ak, const double* B,
+                              long long bk, long long bj, double* C, long long ldc, double alpha, double beta,
+                              cudaStream_t s);
 cudaError_t launch_kron_features(const double* Ubar, int r, int nsnap, double* D, int ldd, int col0,
                                  cudaStream_t s);
 // compressed Kronecker cube (q_i q_j q_k)_{i<=j<=k} of every snapshot into columns col0.. of D

@@ -161,9 +161,6 @@ void fixed_point_scales(InstFom& I, double modulus) {
     I.fscale = 54 - k;
     I.fk2 = std::llrint(std::ldexp(I.m1, 62 - k));
     I.fmu = std::llrint(std::ldexp(I.m2, 62 - k));
-    int e;
-    I.ihm = (long long)std::ldexp(std::frexp(I.invh, &e), 63);
-    I.ihe = e - 1;
 }
 
 int setup_fom_group(osam_ctx* ctx, FomGroupH& G, int s, int n, const osam_problem_desc* descs) {
@@ -181,6 +178,10 @@ int setup_fom_group(osam_ctx* ctx, FomGroupH& G, int s, int n, const osam_proble
         I.wq = g.h * g.h / 32.0;
         I.wq3 = g.h * g.h / 96.0;
         I.lam = d.lambda; I.mu = d.mu;
+        I.wqi = I.wq * I.invh;
+        I.s1 = 2.0 * I.wq * I.lam; I.s2 = 2.0 * I.wq * I.mu;
+        I.t1 = 2.0 * I.wqi * I.lam; I.t2 = 2.0 * I.wqi * I.mu;
+        fixed_point_inverse(I.invh, I.ihm, I.ihe);
         if (d.material == OSAM_NEO_HOOKEAN) {
             const double kappa = d.lambda + (2.0 / 3.0) * d.mu;
             I.m1 = 0.5 * kappa * I.wq; I.m2 = d.mu * I.wq; I.m3 = d.mu * I.wq3;
@@ -215,11 +216,12 @@ int setup_fom_group(osam_ctx* ctx, FomGroupH& G, int s, int n, const osam_proble
     CKA(B.us = ctx->alloc<double>(3 * NN));
     if (B.df32 || B.fp32) CKA(B.u2 = ctx->alloc<float2>(3 * NN));   // the FP32 forces' split of u/h
     B.implicit = descs[0].subdomains[s].integrator == OSAM_IMPLICIT;
-    // Fixed-point force: explicit Neo-Hookean groups of the FP64 modes whose scatter is left to the
-    // library (a scatter mode asked for by name runs its own FP64 kernel).
-    B.fixed = B.material == OSAM_NEO_HOOKEAN && !B.implicit && descs[0].scatter == OSAM_SCATTER_AUTO &&
-              (ctx->precision == OSAM_FP64 || ctx->precision == OSAM_FP64_TANGENT32);
-    if (B.fixed) {
+    // Force in 64-bit integers: explicit Neo-Hookean groups and linear elastic groups of the FP64 modes
+    // whose scatter is left to the library (a scatter mode asked for by name runs its own FP64 kernel).
+    const bool integers = (descs[0].scatter == OSAM_SCATTER_AUTO || ctx->integer_force) &&
+                          (ctx->precision == OSAM_FP64 || ctx->precision == OSAM_FP64_TANGENT32);
+    B.fixed = !integers ? 0 : B.material == OSAM_NEO_HOOKEAN && !B.implicit ? 1 : B.material == OSAM_LINEAR_ELASTIC ? 2 : 0;
+    if (B.fixed == 1) {
         CKA(B.ux = ctx->alloc<long long>(3 * NN));
         CKA(B.fe2 = ctx->alloc<double>(24 * NE));
     }
@@ -242,8 +244,6 @@ int setup_fom_group(osam_ctx* ctx, FomGroupH& G, int s, int n, const osam_proble
         if (B.material == OSAM_NEO_HOOKEAN && ctx->precision == OSAM_FP64_TANGENT32) {
             CKA(B.linf = ctx->alloc<float>((long long)kLinPerGp * 8 * NE));
             CKA(B.fe32 = ctx->alloc<float>(24 * NE));
-        } else if (B.material == OSAM_NEO_HOOKEAN) {
-            CKA(B.lin = ctx->alloc<double>((long long)kLinPerGp * 8 * NE));
         }
         CK(cudaMemsetAsync(B.istat, 0, sizeof(long long) * 2 * n, ctx->stream));
         CKA(B.nact = ctx->alloc<int>(n));
@@ -305,7 +305,7 @@ int setup_fom_group(osam_ctx* ctx, FomGroupH& G, int s, int n, const osam_proble
     RET(set_tiles(ctx, G));
     std::vector<double> modulus;
     RET(check_stability(ctx, G, s, n, descs, modulus));
-    if (B.fixed) {
+    if (B.fixed == 1) {
         for (int i = 0; i < n; ++i) fixed_point_scales(G.inst[i], modulus[i]);
         RET(upload(ctx, G.inst_d, G.inst.data(), sizeof(InstFom) * n));
     }
@@ -683,13 +683,14 @@ int autotune(osam_ctx* ctx, bool fixed) {
     // measured level with their natural builds on the bench meshes (tiled: 192.8 vs 193.1 us per launch
     // on 40x40x80, the fourth resident tile per SM paid for by its spills), so AUTO does not try them
     // (OSAM_SCATTER_GATHER_LOWREG / _TILED_LOWREG select them).
-    const int cands[8][4] = {{kGather, 64, 0, 0}, {kGather, 128, 0, 0}, {kGather, 256, 0, 0}, {kGather, 128, 1, 0},
+    const int cands[9][4] = {{kGather, 32, 0, 0}, {kGather, 64, 0, 0}, {kGather, 128, 0, 0}, {kGather, 256, 0, 0}, {kGather, 128, 1, 0},
                              {kAtomic, 64, 0, 0}, {kAtomic, 128, 0, 0}, {kAtomic, 256, 0, 0}, {kAtomic, 128, 1, 0}};
     for (const auto& cd : cands) {
         const int mode = cd[0], block = cd[1], tiled = cd[2], occ = cd[3];
         if (g.df32 && (mode == kAtomic || block > 128 || tiled)) continue;  // double-float force: gather, <= 128 threads
         if (tiled && g.fp32) continue;                                    // the tiled kernel is FP64
-        if (fixed && (mode == kAtomic || tiled || block > 128)) continue; // the fixed-point force: gather, <= 128 threads
+        if (fixed && (mode == kAtomic || tiled || block > 128)) continue; // the integer forces: gather, <= 128 threads
+        if (!fixed && block < 64) continue;
         RET(set_eblocks(ctx, G, block));
         g.eblk = G.d.eblk;
         g.n_eblk = G.d.n_eblk;

@@ -819,7 +819,8 @@ cudaError_t launch_force_b(const FomB& g, const int* active, int scatter, cudaSt
     for (int k = 0; k < tr.n; ++k) items += 3LL * tr.c[k].R;
     const int grid = g.n_eblk + (int)((items + b - 1) / b);
     if (g.df32) return launch_force_df_b(g, active, tr, s);
-    if (g.fixed) return launch_force_fx_b(g, active, tr, upred, s);
+    if (g.fixed == 1) return launch_force_fx_b(g, active, tr, upred, s);
+    if (g.fixed == 2) return launch_force_le_b(g, active, tr, s);
 #define OSAM_LAUNCH(MAT, T, MODE) k_force_b<MAT, T, MODE><<<grid, b, 0, s>>>(g, active, tr)
     const bool fp32 = g.fp32 != 0;
     if (g.tiled && !fp32) {
@@ -886,7 +887,8 @@ cudaError_t launch_node_b(const FomB& g, const int* active, int scatter, int slo
                           const double* ucur, double* unext, double dt, cudaStream_t s) {
     const bool fp32 = g.fp32 != 0;
     if (g.df32) return launch_node_df_b(g, active, slot1, slot2, predict_only, ucur, unext, dt, s);
-    if (g.fixed) return launch_node_fx_b(g, active, slot1, slot2, predict_only, ucur, unext, dt, s);
+    if (g.fixed == 1) return launch_node_fx_b(g, active, slot1, slot2, predict_only, ucur, unext, dt, s);
+    if (g.fixed == 2) scatter = kGather;
     if (fp32) {
         if (scatter == kAtomic) k_node_b<float, kAtomic><<<g.n_nblk, kNodeBlock, 0, s>>>(g, active, slot1, slot2, predict_only, ucur, unext, dt);
         else k_node_b<float, kGather><<<g.n_nblk, kNodeBlock, 0, s>>>(g, active, slot1, slot2, predict_only, ucur, unext, dt);

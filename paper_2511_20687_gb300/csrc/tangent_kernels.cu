@@ -8,7 +8,6 @@
 #include <cuda_runtime.h>
 
 #include "hex8_math.cuh"
-#include "nh_tangent.cuh"
 #include "osam_internal.h"
 
 namespace osam {
@@ -96,13 +95,7 @@ __global__ void __launch_bounds__(256) k_tangent_b(const FomB g, const int* __re
     }
     const double lam = I.lam_e ? I.lam_e[e] : I.lam;
     const double mu = I.mu_e ? I.mu_e[e] : I.mu;
-    double m1, m2, m3;
-    if (MAT == OSAM_NEO_HOOKEAN) {
-        const double kappa = lam + (2.0 / 3.0) * mu;
-        m1 = 0.5 * kappa * I.w8; m2 = mu * I.w8; m3 = mu * I.w8 / 3.0;
-    } else {
-        m1 = lam * I.w8; m2 = mu * I.w8; m3 = 0.0;
-    }
+    const double m1 = lam * I.w8, m2 = mu * I.w8;
     double Sx[3][2][2], Sy[3][2][2], Sz[3][2][2];
 #pragma unroll
     for (int p = 0; p < 2; ++p)
@@ -116,10 +109,7 @@ __global__ void __launch_bounds__(256) k_tangent_b(const FomB g, const int* __re
                     Hm[c][0] = Gx[c][q][r]; Hm[c][1] = Gy[c][p][r]; Hm[c][2] = Gz[c][p][q];
                     Gm[c][0] = Bx[c][q][r]; Gm[c][1] = By[c][p][r]; Gm[c][2] = Bz[c][p][q];
                 }
-                if (MAT == OSAM_NEO_HOOKEAN) {
-                    double pk, pm;
-                    tangent::nh_tangent(Hm, Gm, m1, m2, m3, dP, pk, pm);
-                } else if (MAT == OSAM_SAINT_VENANT_KIRCHHOFF) {
+                if (MAT == OSAM_SAINT_VENANT_KIRCHHOFF) {
                     svk_tangent(Hm, Gm, m1, m2, dP);
                 } else {
                     stress_le<double>(Gm, m1, m2, dP);  // linear: the tangent applied to G is sigma(G)
@@ -166,19 +156,6 @@ __global__ void __launch_bounds__(256) k_tangent_b(const FomB g, const int* __re
 // beta, a1, b1.
 static_assert(kLinPerGp == 22, "stored linearisation: F, cof F, alpha, beta, a1, b1");
 
-__device__ __forceinline__ void nodal_grads(const FomB& g, const InstFom& I, const double* x, double scale,
-                                            const int node[8], double Gx[3][2][2], double Gy[3][2][2],
-                                            double Gz[3][2][2]) {
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        double V[8], Dx[2][2], Dy[2][2], Dz[2][2];
-#pragma unroll
-        for (int c8 = 0; c8 < 8; ++c8) V[c8] = x[(long long)c * g.NN + I.node_off + node[c8]] * scale;
-        edge_differences_prescaled<double>(V, Dx, Dy, Dz);
-        lerp2<double>(Dx, Gx[c]); lerp2<double>(Dy, Gy[c]); lerp2<double>(Dz, Gz[c]);
-    }
-}
-
 // transposed interpolation of the Gauss-point sums (scaled like the force's: Walsh basis, factor 4 in
 // the material factors) and the element-buffer write
 template <typename T>
@@ -222,16 +199,14 @@ __device__ __forceinline__ ElemIdx elem_idx(const FomB& g, const int* mask) {
 // instruction would take a slot of the FP64 pipe, the bound of the Newton force, 176 times per
 // element; the entries -- F, cof F and the material-scaled factors -- lie far inside the FP32 range,
 // and the rounding toward zero is at the CG operator's own FP32 level).
-__device__ __forceinline__ double lin_value(double x, double*) { return x; }
-__device__ __forceinline__ float lin_value(double x, float*) { return f32_rz(x); }
+__device__ __forceinline__ float lin_value(double x) { return f32_rz(x); }
 
 // The per-Gauss-point quantities of the Newton linearisation, stored by the Neo-Hookean Gauss sums'
 // hook (TL: the storage type); a1 and b1 from the force's own 1/J (the cube of its reciprocal cube
 // root, no division).  Material factors scaled by h^2/32 like the force's (the Walsh-basis transposed
 // interpolation carries the remaining factor 4), so the tangent's dP is scaled alike.
-template <typename TL>
 struct LinStore {
-    TL* lin;             // this element's first entry
+    float* lin;             // this element's first entry
     long long st;        // stride between quantities (8 NE)
     long long ne;        // stride between Gauss points (NE)
     double kap2;         // m1 of the material factors
@@ -240,22 +215,21 @@ struct LinStore {
         (void)J;
         const double a1 = -(2.0 / 3.0) * alpha * invJ;
         const double b1 = 2.0 * kap2 - invJ * fma(a1, trC * (1.0 / 3.0), beta);
-        TL* lg = lin + (long long)(4 * p + 2 * q + r) * ne;
+        float* lg = lin + (long long)(4 * p + 2 * q + r) * ne;
 #pragma unroll
         for (int a = 0; a < 9; ++a) {
-            lg[a * st] = lin_value(Fm[a / 3][a % 3], lg);
-            lg[(9 + a) * st] = lin_value(Cm[a / 3][a % 3], lg);
+            lg[a * st] = lin_value(Fm[a / 3][a % 3]);
+            lg[(9 + a) * st] = lin_value(Cm[a / 3][a % 3]);
         }
-        lg[18 * st] = lin_value(alpha, lg); lg[19 * st] = lin_value(beta, lg);
-        lg[20 * st] = lin_value(a1, lg); lg[21 * st] = lin_value(b1, lg);
+        lg[18 * st] = lin_value(alpha); lg[19 * st] = lin_value(beta);
+        lg[20 * st] = lin_value(a1); lg[21 * st] = lin_value(b1);
     }
 };
 
 // Newton residual force of a Neo-Hookean group at u (from u / h) plus the stored linearisation: the
 // explicit force's arithmetic (1 of F's diagonal in the first interpolation stage, paired Gauss-point
 // sums, Walsh-basis transposed interpolation) with the linearisation written at each Gauss point
-template <typename TL>
-__global__ void __launch_bounds__(256) k_force_lin_b(const FomB g, TL* __restrict__ lin_base,
+__global__ void __launch_bounds__(256) k_force_lin_b(const FomB g, float* __restrict__ lin_base,
                                                      const int* __restrict__ mask) {
     const ElemIdx x = elem_idx(g, mask);
     if (!x.ok) return;
@@ -277,7 +251,7 @@ __global__ void __launch_bounds__(256) k_force_lin_b(const FomB g, TL* __restric
         material_factors<OSAM_NEO_HOOKEAN, double>(I.lam_e ? I.lam_e[e] : I.lam, I.mu_e ? I.mu_e[e] : I.mu, I.wq,
                                                    I.wq3, m1, m2, m3);
     else { m1 = I.m1; m2 = I.m2; m3 = I.m3; }
-    const LinStore<TL> store{lin_base + I.elem_off + e, 8LL * g.NE, g.NE, m1};
+    const LinStore store{lin_base + I.elem_off + e, 8LL * g.NE, g.NE, m1};
     double Sx[3][2][2], Sy[3][2][2], Sz[3][2][2], F[3][8];
     nh_gauss_sums<double>(Gx, Gy, Gz, m1, m2, m3, Sx, Sy, Sz, store);
     walsh_transpose<double>(Sx, Sy, Sz, F);
@@ -288,71 +262,7 @@ __global__ void __launch_bounds__(256) k_force_lin_b(const FomB g, TL* __restric
         for (int c = 0; c < 3; ++c) fe[(long long)(c8 * 3 + c) * g.NE + e] = F[c][c8];
 }
 
-// tangent action from the stored linearisation: per Gauss point 166 FP64 flops instead of 243, and
-// no interpolation of u
-__global__ void __launch_bounds__(256) k_tangent_lin_b(const FomB g, const int* __restrict__ mask) {
-    const ElemIdx x = elem_idx(g, mask);
-    if (!x.ok) return;
-    const InstFom& I = x.I;
-    const int e = x.e;
-    double Bx[3][2][2], By[3][2][2], Bz[3][2][2];
-    nodal_grads(g, I, g.cg_p, I.invh, x.node, Bx, By, Bz);
-    const double* lin = g.lin + I.elem_off + e;
-    const long long st = 8LL * g.NE;
-    double Sx[3][2][2], Sy[3][2][2], Sz[3][2][2];
-#pragma unroll
-    for (int p = 0; p < 2; ++p)
-#pragma unroll
-        for (int q = 0; q < 2; ++q)
-#pragma unroll
-            for (int r = 0; r < 2; ++r) {
-                const int gp = 4 * p + 2 * q + r;
-                const double* lg = lin + (long long)gp * g.NE;
-                double F[3][3], cf[3][3], G[3][3], dc[3][3];
-#pragma unroll
-                for (int a = 0; a < 9; ++a) {
-                    F[a / 3][a % 3] = __ldg(lg + a * st);
-                    cf[a / 3][a % 3] = __ldg(lg + (9 + a) * st);
-                }
-                const double alpha = __ldg(lg + 18 * st), beta = __ldg(lg + 19 * st);
-                const double a1 = __ldg(lg + 20 * st), b1 = __ldg(lg + 21 * st);
-#pragma unroll
-                for (int c = 0; c < 3; ++c) { G[c][0] = Bx[c][q][r]; G[c][1] = By[c][p][r]; G[c][2] = Bz[c][p][q]; }
-                double dJ = 0.0, FG = 0.0;
-#pragma unroll
-                for (int a = 0; a < 9; ++a) {
-                    dJ = fma(cf[a / 3][a % 3], G[a / 3][a % 3], dJ);
-                    FG = fma(F[a / 3][a % 3], G[a / 3][a % 3], FG);
-                }
-                dc[0][0] = G[1][1] * F[2][2] + F[1][1] * G[2][2] - G[1][2] * F[2][1] - F[1][2] * G[2][1];
-                dc[0][1] = G[1][2] * F[2][0] + F[1][2] * G[2][0] - G[1][0] * F[2][2] - F[1][0] * G[2][2];
-                dc[0][2] = G[1][0] * F[2][1] + F[1][0] * G[2][1] - G[1][1] * F[2][0] - F[1][1] * G[2][0];
-                dc[1][0] = G[0][2] * F[2][1] + F[0][2] * G[2][1] - G[0][1] * F[2][2] - F[0][1] * G[2][2];
-                dc[1][1] = G[0][0] * F[2][2] + F[0][0] * G[2][2] - G[0][2] * F[2][0] - F[0][2] * G[2][0];
-                dc[1][2] = G[0][1] * F[2][0] + F[0][1] * G[2][0] - G[0][0] * F[2][1] - F[0][0] * G[2][1];
-                dc[2][0] = G[0][1] * F[1][2] + F[0][1] * G[1][2] - G[0][2] * F[1][1] - F[0][2] * G[1][1];
-                dc[2][1] = G[0][2] * F[1][0] + F[0][2] * G[1][0] - G[0][0] * F[1][2] - F[0][0] * G[1][2];
-                dc[2][2] = G[0][0] * F[1][1] + F[0][0] * G[1][1] - G[0][1] * F[1][0] - F[0][1] * G[1][0];
-                const double dalpha = a1 * dJ;
-                const double dbeta = fma(b1, dJ, a1 * FG);
-                double dP[3][3];
-#pragma unroll
-                for (int a = 0; a < 3; ++a)
-#pragma unroll
-                    for (int b2 = 0; b2 < 3; ++b2)
-                        dP[a][b2] = fma(dbeta, cf[a][b2], fma(beta, dc[a][b2], fma(dalpha, F[a][b2], alpha * G[a][b2])));
-#pragma unroll
-                for (int c = 0; c < 3; ++c) {
-                    if (p == 0) Sx[c][q][r] = dP[c][0]; else Sx[c][q][r] += dP[c][0];
-                    if (q == 0) Sy[c][p][r] = dP[c][1]; else Sy[c][p][r] += dP[c][1];
-                    if (r == 0) Sz[c][p][q] = dP[c][2]; else Sz[c][p][q] += dP[c][2];
-                }
-            }
-    write_element<double>(static_cast<double*>(g.fe) + I.elem_off, g.NE, e, Sx, Sy, Sz);
-}
-
-// The tangent action of k_tangent_lin_b in FP32 (OSAM_FP64_TANGENT32): the linearisation read as
-// stored in FP32 (half the bytes), the direction p converted once per nodal value, every Gauss-point
+// Tangent action from the stored linearisation in FP32 (OSAM_FP64_TANGENT32): the direction p converted once per nodal value, every Gauss-point
 // operation on the FP32 pipes, and the element contributions written in FP32 to the FP32 element
 // buffer (the CG's Ap kernel sums them in FP32 and adds them to its FP64 mass term).  p is converted
 // with the integer-only f32_rz, so no FP64-pipe instruction is left.
@@ -437,26 +347,22 @@ __global__ void __launch_bounds__(256) k_tangent_lin32_b(const FomB g, const int
 
 cudaError_t launch_force_lin_b(const FomB& g, const int* mask, cudaStream_t s) {
     if (g.n_eblk == 0) return cudaSuccess;
-    if (g.eblock > 256 || (!g.lin && !g.linf) || g.material != OSAM_NEO_HOOKEAN) return cudaErrorInvalidValue;
-    if (g.linf) k_force_lin_b<float><<<g.n_eblk, g.eblock, 0, s>>>(g, g.linf, mask);
-    else k_force_lin_b<double><<<g.n_eblk, g.eblock, 0, s>>>(g, g.lin, mask);
+    if (g.eblock > 256 || !g.linf || g.material != OSAM_NEO_HOOKEAN) return cudaErrorInvalidValue;
+    k_force_lin_b<<<g.n_eblk, g.eblock, 0, s>>>(g, g.linf, mask);
     return cudaGetLastError();
 }
 
 cudaError_t launch_tangent_lin_b(const FomB& g, const int* mask, cudaStream_t s) {
     if (g.n_eblk == 0) return cudaSuccess;
-    if (g.eblock > 256 || g.material != OSAM_NEO_HOOKEAN) return cudaErrorInvalidValue;
-    if (g.linf && g.fe32) k_tangent_lin32_b<<<g.n_eblk, g.eblock, 0, s>>>(g, mask);
-    else if (g.lin) k_tangent_lin_b<<<g.n_eblk, g.eblock, 0, s>>>(g, mask);
-    else return cudaErrorInvalidValue;
+    if (g.eblock > 256 || !g.linf || !g.fe32 || g.material != OSAM_NEO_HOOKEAN) return cudaErrorInvalidValue;
+    k_tangent_lin32_b<<<g.n_eblk, g.eblock, 0, s>>>(g, mask);
     return cudaGetLastError();
 }
 
 cudaError_t launch_tangent_b(const FomB& g, const int* mask, cudaStream_t s) {
     if (g.n_eblk == 0) return cudaSuccess;
     if (g.eblock > 256) return cudaErrorInvalidConfiguration;
-    if (g.material == OSAM_NEO_HOOKEAN) k_tangent_b<OSAM_NEO_HOOKEAN><<<g.n_eblk, g.eblock, 0, s>>>(g, mask);
-    else if (g.material == OSAM_SAINT_VENANT_KIRCHHOFF)
+    if (g.material == OSAM_SAINT_VENANT_KIRCHHOFF)
         k_tangent_b<OSAM_SAINT_VENANT_KIRCHHOFF><<<g.n_eblk, g.eblock, 0, s>>>(g, mask);
     else k_tangent_b<OSAM_LINEAR_ELASTIC><<<g.n_eblk, g.eblock, 0, s>>>(g, mask);
     return cudaGetLastError();
