@@ -85,6 +85,7 @@ __global__ void k_build_Rt(int nrow, int r, const int* dnode, const double* dw, 
 // alpha and beta.  The output tiles are numbered along grid.x, column tile fastest (blocks that
 // share a row tile of A run together and find it in L2), so m is bounded only by 32-bit indices.
 constexpr int TM = 64, TN = 64, TK = 16;
+constexpr double kSplitMin = 4.2e6;
 
 // The GEMM runs on the FP64 tensor cores: 128 threads per 64x64 output tile, each warp a 32x32 quarter
 // as 4 x 4 accumulators of mma.sync m8n8k4 (FP64 in and out, each MMA 8x8x4 fused multiply-adds).
@@ -213,6 +214,10 @@ cudaError_t launch_gemm_impl(int m, int n, int k, const double* A, long long ai,
                              long long bk, long long bj, double* C, long long ldc, double alpha, double beta,
                              cudaStream_t s) {
     if (m <= 0 || n <= 0) return cudaSuccess;
+    // From a few million products on, on the bf16 tensor cores (split_gemm.cu); below, the splitting's extra
+    // launches cost more than the FP64 tensor pipe takes.
+    if (k >= 16 && (double)m * n * k >= kSplitMin)
+        return launch_split_gemm(m, n, k, A, ai, ak, B, bk, bj, C, ldc, alpha, beta, s);
     const long long tiles = (long long)grid_for(n, TN) * grid_for(m, TM);
     int dev = 0, sms = 152;
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);

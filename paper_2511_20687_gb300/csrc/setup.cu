@@ -683,14 +683,13 @@ int autotune(osam_ctx* ctx, bool fixed) {
     // measured level with their natural builds on the bench meshes (tiled: 192.8 vs 193.1 us per launch
     // on 40x40x80, the fourth resident tile per SM paid for by its spills), so AUTO does not try them
     // (OSAM_SCATTER_GATHER_LOWREG / _TILED_LOWREG select them).
-    const int cands[9][4] = {{kGather, 32, 0, 0}, {kGather, 64, 0, 0}, {kGather, 128, 0, 0}, {kGather, 256, 0, 0}, {kGather, 128, 1, 0},
+    const int cands[8][4] = {{kGather, 64, 0, 0}, {kGather, 128, 0, 0}, {kGather, 256, 0, 0}, {kGather, 128, 1, 0},
                              {kAtomic, 64, 0, 0}, {kAtomic, 128, 0, 0}, {kAtomic, 256, 0, 0}, {kAtomic, 128, 1, 0}};
     for (const auto& cd : cands) {
         const int mode = cd[0], block = cd[1], tiled = cd[2], occ = cd[3];
         if (g.df32 && (mode == kAtomic || block > 128 || tiled)) continue;  // double-float force: gather, <= 128 threads
         if (tiled && g.fp32) continue;                                    // the tiled kernel is FP64
         if (fixed && (mode == kAtomic || tiled || block > 128)) continue; // the integer forces: gather, <= 128 threads
-        if (!fixed && block < 64) continue;
         RET(set_eblocks(ctx, G, block));
         g.eblk = G.d.eblk;
         g.n_eblk = G.d.n_eblk;
