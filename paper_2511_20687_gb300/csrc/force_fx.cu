@@ -120,6 +120,7 @@ __global__ void __launch_bounds__(128) k_force_fx_b(const __grid_constant__ FomB
 // Corrector of substep j and predictor of substep j + 1 (the arithmetic of k_node_b) on the fixed-point
 // element buffer: the 24 contributions of a node are summed exactly as integers and converted once per
 // component; the predictor is written in FP64 and as fixed-point u / h.
+template <int NC>
 __global__ void __launch_bounds__(kNodeBlock) k_node_fx_b(const __grid_constant__ FomB g,
                                                           const int* __restrict__ active, int slot1, int slot2,
                                                           int predict_only, const double* ucur, double* unext,
@@ -135,23 +136,24 @@ __global__ void __launch_bounds__(kNodeBlock) k_node_fx_b(const __grid_constant_
     const int j = t % (ny + 1);
     const int k = t / (ny + 1);
     const long long gn = I.node_off + n;
+    const int c0 = NC == 3 ? 0 : (int)blockIdx.y;   // the thread's components c0 .. c0 + NC - 1
     const uint8_t cm = g.clamp[gn];
     const int row = g.srow[gn];
     const double hdt = 0.5 * dt, hdt2 = 0.5 * dt * dt;
     const double minv = g.minv[gn];
     const double* h1 = slot1 >= 0 ? g.hist + I.hist_off + (long long)slot1 * 9 * I.ns : nullptr;
     const double* h2 = slot2 >= 0 ? g.hist + I.hist_off + (long long)slot2 * 9 * I.ns : nullptr;
-    double uc[3], vc[3], ac[3], f[3] = {0.0, 0.0, 0.0};
+    double uc[NC], vc[NC], ac[NC], f[NC] = {};
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        const long long d = (long long)c * g.NN + gn;
-        uc[c] = ucur[d];
-        vc[c] = g.v[d];
-        ac[c] = g.a[d];
+    for (int q = 0; q < NC; ++q) {
+        const long long d = (long long)(c0 + q) * g.NN + gn;
+        uc[q] = ucur[d];
+        vc[q] = g.v[d];
+        ac[q] = g.a[d];
     }
     if (!predict_only && row < 0 && cm != 7) {
         const i64* fe = static_cast<const i64*>(g.fe) + I.elem_off;
-        i64 s[3] = {0, 0, 0};
+        i64 s[NC] = {};
         unsigned int far = 0;
 #pragma unroll
         for (int az = 0; az < 2; ++az) {
@@ -165,28 +167,29 @@ __global__ void __launch_bounds__(kNodeBlock) k_node_fx_b(const __grid_constant_
                     const int corner = ax + 2 * ay + 4 * az;
                     if (ke < 0 || ke >= nz || je < 0 || je >= ny || ie < 0 || ie >= nx) continue;
                     const long long e = ie + (long long)nx * (je + ny * ke);
-                    i64 x[3];
+                    i64 x[NC];
 #pragma unroll
-                    for (int c = 0; c < 3; ++c) x[c] = __ldg(fe + (long long)(corner * 3 + c) * g.NE + e);
+                    for (int q = 0; q < NC; ++q) x[q] = __ldg(fe + (long long)(corner * 3 + c0 + q) * g.NE + e);
                     if (x[0] == kBadF) { far |= 1u << corner; continue; }
 #pragma unroll
-                    for (int c = 0; c < 3; ++c) s[c] += x[c];
+                    for (int q = 0; q < NC; ++q) s[q] += x[q];
                 }
             }
         }
 #pragma unroll
-        for (int c = 0; c < 3; ++c) f[c] = f64_scaled(s[c], I.fscale);
+        for (int q = 0; q < NC; ++q) f[q] = f64_scaled(s[q], I.fscale);
         while (far) {   // elements held in FP64
             const int corner = __ffs((int)far) - 1;
             far &= far - 1;
             const long long e = (i - (corner & 1)) +
                                 (long long)nx * ((j - ((corner >> 1) & 1)) + ny * (k - (corner >> 2)));
 #pragma unroll
-            for (int c = 0; c < 3; ++c) f[c] += g.fe2[(long long)(corner * 3 + c) * g.NE + I.elem_off + e];
+            for (int q = 0; q < NC; ++q) f[q] += g.fe2[(long long)(corner * 3 + c0 + q) * g.NE + I.elem_off + e];
         }
     }
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
+    for (int q = 0; q < NC; ++q) {
+        const int c = c0 + q;
         const long long d = (long long)c * g.NN + gn;
         double un;
         if (cm & (1 << c)) {
@@ -200,15 +203,15 @@ __global__ void __launch_bounds__(kNodeBlock) k_node_fx_b(const __grid_constant_
             }
             un = h2 ? h2[(long long)c * I.ns + row] : 0.0;
         } else {
-            double vn = vc[c], an = ac[c];
+            double vn = vc[q], an = ac[q];
             if (!predict_only) {
-                const double anew = -f[c] * minv;
+                const double anew = -f[q] * minv;
                 vn = fma(hdt, an + anew, vn);
                 an = anew;
                 g.v[d] = vn;
                 g.a[d] = an;
             }
-            un = fma(hdt2, an, fma(dt, vn, uc[c]));
+            un = fma(hdt2, an, fma(dt, vn, uc[q]));
         }
         if (h2) {
             unext[d] = un;
@@ -231,7 +234,9 @@ cudaError_t launch_force_fx_b(const FomB& g, const int* active, const TraceFuse&
 
 cudaError_t launch_node_fx_b(const FomB& g, const int* active, int slot1, int slot2, int predict_only,
                              const double* ucur, double* unext, double dt, cudaStream_t s) {
-    k_node_fx_b<<<g.n_nblk, kNodeBlock, 0, s>>>(g, active, slot1, slot2, predict_only, ucur, unext, dt);
+    if (node_split(g))
+        k_node_fx_b<1><<<dim3(g.n_nblk, 3), kNodeBlock, 0, s>>>(g, active, slot1, slot2, predict_only, ucur, unext, dt);
+    else k_node_fx_b<3><<<g.n_nblk, kNodeBlock, 0, s>>>(g, active, slot1, slot2, predict_only, ucur, unext, dt);
     return cudaGetLastError();
 }
 

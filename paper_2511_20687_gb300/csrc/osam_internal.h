@@ -135,6 +135,12 @@ struct FomB {
     double* fe2;              // FP64 contributions of the elements outside the fixed-point range [24][NE]
 };
 
+// A node kernel takes one thread per node and component instead of one per node while that leaves it
+// below eight warps per scheduler: its time is then the length of one thread's chain of FP64 instructions
+// and loads, a third with one component.
+constexpr int kNodeSplitBlocks = 152 * 8 / 3;
+inline bool node_split(const FomB& g) { return g.n_nblk <= kNodeSplitBlocks; }
+
 // one instance of a ROM slot
 struct InstRom {
     int r, rs, nsdof, d, nq, nc, gx, gy;   // nc: cubic columns r(r+1)(r+2)/6 (0: quadratic ROM)

@@ -294,7 +294,7 @@ __global__ void __launch_bounds__(kNodeBlock) k_init_accel_b(const FomB g, const
 //   clamped:    u = v = a = 0
 //   Schwarz:    v, a from history slot j+1 (slot1); u^{j+2} from history slot j+2 (slot2)
 // predict_only: write the predictor of ucur with the current (v, a) (start of an interval).
-template <typename TF, int MODE>
+template <typename TF, int MODE, int NC>
 __global__ void __launch_bounds__(kNodeBlock) k_node_b(const FomB g, const int* __restrict__ active, int slot1,
                                                       int slot2, int predict_only, const double* ucur, double* unext,
                                                       double dt) {
@@ -308,6 +308,7 @@ __global__ void __launch_bounds__(kNodeBlock) k_node_b(const FomB g, const int* 
     const int j = t % (I.ny + 1);
     const int k = t / (I.ny + 1);
     const long long gn = I.node_off + n;
+    const int c0 = NC == 3 ? 0 : (int)blockIdx.y;   // the thread's components c0 .. c0 + NC - 1
     const uint8_t cm = g.clamp[gn];
     const int row = g.srow[gn];
     const double hdt = 0.5 * dt, hdt2 = 0.5 * dt * dt;
@@ -318,14 +319,14 @@ __global__ void __launch_bounds__(kNodeBlock) k_node_b(const FomB g, const int* 
     TF* fa = static_cast<TF*>(g.f);
     // all loads of a free node first (state and the element contributions of the three components,
     // summed per component in the fixed corner order), so that they are in flight together
-    double uc[3], vc[3], ac[3], f[3] = {0.0, 0.0, 0.0};
-    TF fs[3] = {TF(0), TF(0), TF(0)};   // the gather sums in the element buffer's precision
+    double uc[NC], vc[NC], ac[NC], f[NC] = {};
+    TF fs[NC] = {};   // the gather sums in the element buffer's precision
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        const long long d = (long long)c * g.NN + gn;
-        uc[c] = ucur[d];
-        vc[c] = g.v[d];
-        ac[c] = g.a[d];
+    for (int q = 0; q < NC; ++q) {
+        const long long d = (long long)(c0 + q) * g.NN + gn;
+        uc[q] = ucur[d];
+        vc[q] = g.v[d];
+        ac[q] = g.a[d];
     }
     if (!predict_only && row < 0 && cm != 7) {
         if (MODE == kGather) {
@@ -344,27 +345,28 @@ __global__ void __launch_bounds__(kNodeBlock) k_node_b(const FomB g, const int* 
                         const long long e = ie + (long long)I.nx * (je + I.ny * ke);
                         const int corner = ax + 2 * ay + 4 * az;
 #pragma unroll
-                        for (int c = 0; c < 3; ++c) fs[c] += __ldg(fe + (long long)(corner * 3 + c) * g.NE + e);
+                        for (int q = 0; q < NC; ++q) fs[q] += __ldg(fe + (long long)(corner * 3 + c0 + q) * g.NE + e);
                     }
                 }
             }
             // FP64: the same sums; FP32 force: summed in FP32 (its own precision) and widened once, by
             // integer operations (f64_of: exact)
 #pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                if constexpr (sizeof(TF) == 4) f[c] = f64_of(fs[c]);
-                else f[c] = fs[c];
+            for (int q = 0; q < NC; ++q) {
+                if constexpr (sizeof(TF) == 4) f[q] = f64_of(fs[q]);
+                else f[q] = fs[q];
             }
         } else {
 #pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                if constexpr (sizeof(TF) == 4) f[c] = f64_of(fa[(long long)c * g.NN + gn]);
-                else f[c] = fa[(long long)c * g.NN + gn];
+            for (int q = 0; q < NC; ++q) {
+                if constexpr (sizeof(TF) == 4) f[q] = f64_of(fa[(long long)(c0 + q) * g.NN + gn]);
+                else f[q] = fa[(long long)(c0 + q) * g.NN + gn];
             }
         }
     }
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
+    for (int q = 0; q < NC; ++q) {
+        const int c = c0 + q;
         const long long d = (long long)c * g.NN + gn;
         double un;
         if (cm & (1 << c)) {
@@ -380,16 +382,16 @@ __global__ void __launch_bounds__(kNodeBlock) k_node_b(const FomB g, const int* 
             }
             un = h2 ? h2[(long long)c * I.ns + row] : 0.0;
         } else {
-            double vn = vc[c], an = ac[c];
+            double vn = vc[q], an = ac[q];
             if (!predict_only) {
                 if (MODE == kAtomic) fa[d] = TF(0);
-                const double anew = -f[c] * minv;
+                const double anew = -f[q] * minv;
                 vn = fma(hdt, an + anew, vn);
                 an = anew;
                 g.v[d] = vn;
                 g.a[d] = an;
             }
-            un = fma(hdt2, an, fma(dt, vn, uc[c]));
+            un = fma(hdt2, an, fma(dt, vn, uc[q]));
         }
         if (h2) {
             unext[d] = un;
@@ -889,13 +891,21 @@ cudaError_t launch_node_b(const FomB& g, const int* active, int scatter, int slo
     if (g.df32) return launch_node_df_b(g, active, slot1, slot2, predict_only, ucur, unext, dt, s);
     if (g.fixed == 1) return launch_node_fx_b(g, active, slot1, slot2, predict_only, ucur, unext, dt, s);
     if (g.fixed == 2) scatter = kGather;
+    const bool split = node_split(g);
+    const dim3 grid(g.n_nblk, split ? 3 : 1);
+#define OSAM_NODE(T, M)                                                                                                   \
+    do {                                                                                                                  \
+        if (split) k_node_b<T, M, 1><<<grid, kNodeBlock, 0, s>>>(g, active, slot1, slot2, predict_only, ucur, unext, dt); \
+        else k_node_b<T, M, 3><<<grid, kNodeBlock, 0, s>>>(g, active, slot1, slot2, predict_only, ucur, unext, dt);       \
+    } while (0)
     if (fp32) {
-        if (scatter == kAtomic) k_node_b<float, kAtomic><<<g.n_nblk, kNodeBlock, 0, s>>>(g, active, slot1, slot2, predict_only, ucur, unext, dt);
-        else k_node_b<float, kGather><<<g.n_nblk, kNodeBlock, 0, s>>>(g, active, slot1, slot2, predict_only, ucur, unext, dt);
+        if (scatter == kAtomic) OSAM_NODE(float, kAtomic);
+        else OSAM_NODE(float, kGather);
     } else {
-        if (scatter == kAtomic) k_node_b<double, kAtomic><<<g.n_nblk, kNodeBlock, 0, s>>>(g, active, slot1, slot2, predict_only, ucur, unext, dt);
-        else k_node_b<double, kGather><<<g.n_nblk, kNodeBlock, 0, s>>>(g, active, slot1, slot2, predict_only, ucur, unext, dt);
+        if (scatter == kAtomic) OSAM_NODE(double, kAtomic);
+        else OSAM_NODE(double, kGather);
     }
+#undef OSAM_NODE
     return cudaGetLastError();
 }
 
