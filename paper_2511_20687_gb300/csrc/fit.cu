@@ -16,8 +16,13 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
+#include <condition_variable>
+#include <functional>
+#include <mutex>
 #include <string>
+#include <thread>
 #include <vector>
 
 #include "osam.h"
@@ -29,152 +34,256 @@ namespace {
 
 thread_local std::string g_fit_error;
 
+// a . b with eight partial sums (vector instructions without a reassociating compiler flag)
+double dot(const double* a, const double* b, int n) {
+    double s[8] = {};
+    int i = 0;
+    for (; i + 8 <= n; i += 8)
+        for (int q = 0; q < 8; ++q) s[q] += a[i + q] * b[i + q];
+    double t = ((s[0] + s[4]) + (s[1] + s[5])) + ((s[2] + s[6]) + (s[3] + s[7]));
+    for (; i < n; ++i) t += a[i] * b[i];
+    return t;
+}
+
+// The host threads of one call.  run(f) calls f(t) for every thread number t, 0 on the calling thread;
+// sync() is a barrier among them.  With fewer threads than asked for (or none beside the caller) the work is
+// split over those there are; the results do not depend on their number.
+class Team {
+public:
+    explicit Team(int want) {
+        try {
+            threads_.reserve(std::max(want, 1));
+            for (int t = 1; t < want; ++t) threads_.emplace_back([this, t] { loop(t); });
+        } catch (...) {
+        }
+        n_ = (int)threads_.size() + 1;
+    }
+    ~Team() {
+        {
+            std::lock_guard<std::mutex> g(m_);
+            stop_ = true;
+        }
+        go_.notify_all();
+        for (auto& t : threads_) t.join();
+    }
+    int size() const { return n_; }
+    void run(const std::function<void(int)>& f) {
+        {
+            std::lock_guard<std::mutex> g(m_);
+            f_ = &f;
+            left_ = n_ - 1;
+            ++epoch_;
+        }
+        go_.notify_all();
+        f(0);
+        std::unique_lock<std::mutex> g(m_);
+        done_.wait(g, [this] { return left_ == 0; });
+        f_ = nullptr;
+    }
+    void sync() {
+        if (n_ == 1) return;
+        const unsigned int e = turn_.load(std::memory_order_acquire);
+        if (arrived_.fetch_add(1, std::memory_order_acq_rel) + 1 == n_) {
+            arrived_.store(0, std::memory_order_relaxed);
+            turn_.store(e + 1, std::memory_order_release);
+        } else {
+            for (int spin = 0; turn_.load(std::memory_order_acquire) == e; ++spin)
+                if (spin > 2000) std::this_thread::yield();
+        }
+    }
+
+private:
+    void loop(int t) {
+        unsigned int seen = 0;
+        for (;;) {
+            const std::function<void(int)>* f;
+            {
+                std::unique_lock<std::mutex> g(m_);
+                go_.wait(g, [&] { return stop_ || epoch_ != seen; });
+                if (stop_) return;
+                seen = epoch_;
+                f = f_;
+            }
+            (*f)(t);
+            std::lock_guard<std::mutex> g(m_);
+            if (--left_ == 0) done_.notify_one();
+        }
+    }
+    std::vector<std::thread> threads_;
+    int n_ = 1, left_ = 0;
+    unsigned int epoch_ = 0;
+    bool stop_ = false;
+    const std::function<void(int)>* f_ = nullptr;
+    std::mutex m_;
+    std::condition_variable go_, done_;
+    std::atomic<int> arrived_{0};
+    std::atomic<unsigned int> turn_{0};
+};
+
+// threads for an n x n problem: none beside the caller for small ones, whose barriers would cost more than the work
+int team_size(int n) {
+    const int hw = (int)std::thread::hardware_concurrency();
+    return n < 96 ? 1 : std::max(1, std::min({hw, 8, n / 32}));
+}
+
 // Symmetric eigen-decomposition by Householder reduction to tridiagonal form followed by the
 // implicit QL iteration with Wilkinson-type shifts (Householder 1958; Bowdler, Martin, Reinsch and
 // Wilkinson 1968).  A is n x n, row-major, symmetric; on return A's diagonal holds the eigenvalues
-// and V (row-major) the eigenvectors as columns.  About 9 n^3 flops with contiguous row access.
+// and V (row-major) the eigenvectors as columns.  The reduction's rows are shared out cyclically among the
+// threads; the rows of the accumulated transformation are independent through both the accumulation and the
+// QL rotations, so each thread takes a block of them and repeats the (cheap) scalar QL recurrence.
 void sym_eig(std::vector<double>& A, int n, std::vector<double>& V) {
-    std::vector<double> d(n), e(n, 0.0), tau(n, 0.0), p(n), w(n);
-    // (1) A <- H_k A H_k, H_k = I - tau_k v_k v_k^T acting on rows / columns k+1..n-1; v_k is kept in
-    //     row k to the right of the diagonal (the part of A that the reduction no longer needs)
-    for (int k = 0; k + 2 < n; ++k) {
-        double* ak = &A[(size_t)k * n];
-        const int m0 = k + 1;
-        double scale = 0.0;
-        for (int i = m0; i < n; ++i) scale = std::max(scale, std::fabs(ak[i]));
-        if (scale == 0.0) { e[k] = 0.0; tau[k] = 0.0; continue; }
-        double ss = 0.0;
-        for (int i = m0; i < n; ++i) { ak[i] /= scale; ss += ak[i] * ak[i]; }
-        const double nrm = std::sqrt(ss);
-        const double alpha = ak[m0] > 0.0 ? -nrm : nrm;      // reflect x onto alpha e_1
-        e[k] = alpha * scale;
-        ak[m0] -= alpha;                                     // v = x - alpha e_1
-        const double vv = ss - 2.0 * alpha * (ak[m0] + alpha) + alpha * alpha;  // |v|^2
-        const double t = vv > 0.0 ? 2.0 / vv : 0.0;
-        tau[k] = t;
-        // p = t B v with B = A[m0.., m0..] (symmetric: use rows), then w = p - (t/2)(p.v) v
-        for (int i = m0; i < n; ++i) {
-            const double* ai = &A[(size_t)i * n];
-            double s = 0.0;
-            for (int j = m0; j < n; ++j) s += ai[j] * ak[j];
-            p[i] = t * s;
-        }
-        double pv = 0.0;
-        for (int i = m0; i < n; ++i) pv += p[i] * ak[i];
-        const double kk = 0.5 * t * pv;
-        for (int i = m0; i < n; ++i) w[i] = p[i] - kk * ak[i];
-        // B <- B - v w^T - w v^T
-        for (int i = m0; i < n; ++i) {
-            double* ai = &A[(size_t)i * n];
-            const double vi = ak[i], wi = w[i];
-            for (int j = m0; j < n; ++j) ai[j] -= vi * w[j] + wi * ak[j];
-        }
-    }
-    for (int k = 0; k < n; ++k) d[k] = A[(size_t)k * n + k];
-    if (n >= 2) e[n - 2] = A[(size_t)(n - 2) * n + (n - 1)];
-    // (2) Q = H_0 H_1 ... H_{n-3}, accumulated from the last reflector; Z = Q^T (rows = vectors)
-    std::vector<double> Q((size_t)n * n, 0.0);
-    for (int i = 0; i < n; ++i) Q[(size_t)i * n + i] = 1.0;
-    for (int k = n - 3; k >= 0; --k) {
-        const double t = tau[k];
-        if (t == 0.0) continue;
-        const double* v = &A[(size_t)k * n];
-        const int m0 = k + 1;
-        // Q[m0.., m0..] <- (I - t v v^T) Q[m0.., m0..]: s_j = t sum_i v_i Q_ij, Q_ij -= v_i s_j
-        std::fill(p.begin(), p.end(), 0.0);
-        for (int i = m0; i < n; ++i) {
-            const double vi = v[i];
-            const double* qi = &Q[(size_t)i * n];
-            for (int j = m0; j < n; ++j) p[j] += vi * qi[j];
-        }
-        for (int i = m0; i < n; ++i) {
-            const double vi = t * v[i];
-            double* qi = &Q[(size_t)i * n];
-            for (int j = m0; j < n; ++j) qi[j] -= vi * p[j];
-        }
-    }
-    std::vector<double> Z((size_t)n * n);
-    for (int i = 0; i < n; ++i)
-        for (int j = 0; j < n; ++j) Z[(size_t)j * n + i] = Q[(size_t)i * n + j];
-    // (3) implicit QL on (d, e), e[i] coupling d[i] and d[i+1]; each plane rotation of rows i, i+1 of
-    //     the tridiagonal matrix is applied to rows i, i+1 of Z
-    for (int l = 0; l < n; ++l) {
-        for (int iter = 0; iter < 60; ++iter) {
-            int m = l;
-            for (; m + 1 < n; ++m) {
-                const double dd = std::fabs(d[m]) + std::fabs(d[m + 1]);
-                if (std::fabs(e[m]) <= 1e-16 * dd) break;
-            }
-            if (m == l) break;
-            double g = (d[l + 1] - d[l]) / (2.0 * e[l]);
-            double r = std::hypot(g, 1.0);
-            g = d[m] - d[l] + e[l] / (g + (g >= 0.0 ? r : -r));   // shifted so that the shift is the
-            double s = 1.0, c = 1.0, pp = 0.0;                     // eigenvalue of the leading 2x2 closer to d[l]
-            int i = m - 1;
-            bool deflated = false;
-            for (; i >= l; --i) {
-                const double f = s * e[i], b = c * e[i];
-                r = std::hypot(f, g);
-                e[i + 1] = r;
-                if (r == 0.0) { d[i + 1] -= pp; e[m] = 0.0; deflated = true; break; }
-                s = f / r;
-                c = g / r;
-                g = d[i + 1] - pp;
-                r = (d[i] - g) * s + 2.0 * c * b;
-                pp = s * r;
-                d[i + 1] = g + pp;
-                g = c * r - b;
-                double* zi = &Z[(size_t)i * n];
-                double* zj = &Z[(size_t)(i + 1) * n];
-                for (int k = 0; k < n; ++k) {
-                    const double a0 = zi[k], a1 = zj[k];
-                    zj[k] = s * a0 + c * a1;
-                    zi[k] = c * a0 - s * a1;
+    std::vector<double> d(n), e(n, 0.0), tau(n, 0.0), p(n), eig(n);
+    V.assign((size_t)n * n, 0.0);
+    Team team(team_size(n));
+    const int T = team.size();
+    // every thread's work space, allocated here: w, q, d, e and its block of Z
+    std::vector<double> work((size_t)T * 4 * n), Zall((size_t)n * n);
+    team.run([&](int me) {
+        double* w = &work[(size_t)me * 4 * n];
+        double *q = w + n, *dl = q + n, *el = dl + n;
+        // (1) A <- H_k A H_k, H_k = I - tau_k v_k v_k^T acting on rows / columns k+1..n-1; v_k is kept in
+        //     row k to the right of the diagonal (the part of A that the reduction no longer needs)
+        for (int k = 0; k + 2 < n; ++k) {
+            double* ak = &A[(size_t)k * n];
+            const int m0 = k + 1;
+            if (me == 0) {
+                double scale = 0.0;
+                for (int i = m0; i < n; ++i) scale = std::max(scale, std::fabs(ak[i]));
+                e[k] = 0.0;
+                tau[k] = 0.0;
+                if (scale != 0.0) {
+                    for (int i = m0; i < n; ++i) ak[i] /= scale;
+                    const double ss = dot(ak + m0, ak + m0, n - m0);
+                    const double nrm = std::sqrt(ss);
+                    const double alpha = ak[m0] > 0.0 ? -nrm : nrm;      // reflect x onto alpha e_1
+                    e[k] = alpha * scale;
+                    ak[m0] -= alpha;                                     // v = x - alpha e_1
+                    const double vv = ss - 2.0 * alpha * (ak[m0] + alpha) + alpha * alpha;  // |v|^2
+                    tau[k] = vv > 0.0 ? 2.0 / vv : 0.0;
                 }
             }
-            if (deflated) continue;
-            d[l] -= pp;
-            e[l] = g;
-            e[m] = 0.0;
+            team.sync();
+            const double t = tau[k];
+            if (t == 0.0) continue;   // nothing to reflect; the next v waits for every thread at its own barrier
+            // p = t B v with B = A[m0.., m0..] (symmetric: use rows), then w = p - (t/2)(p.v) v
+            const int first = m0 + (me - m0 % T + T) % T;
+            for (int i = first; i < n; i += T) p[i] = t * dot(&A[(size_t)i * n + m0], ak + m0, n - m0);
+            team.sync();
+            const double kk = 0.5 * t * dot(&p[m0], ak + m0, n - m0);
+            for (int i = m0; i < n; ++i) w[i] = p[i] - kk * ak[i];
+            // B <- B - v w^T - w v^T
+            for (int i = first; i < n; i += T) {
+                double* ai = &A[(size_t)i * n];
+                const double vi = ak[i], wi = w[i];
+                for (int j = m0; j < n; ++j) ai[j] -= vi * w[j] + wi * ak[j];
+            }
+            team.sync();
         }
-    }
-    V.assign((size_t)n * n, 0.0);
+        if (me == 0) {
+            for (int k = 0; k < n; ++k) d[k] = A[(size_t)k * n + k];
+            if (n >= 2) e[n - 2] = A[(size_t)(n - 2) * n + (n - 1)];
+        }
+        team.sync();
+        // (2) rows r0 .. r1 of Q = H_0 H_1 ... H_{n-3}, transposed into Z (a column per row of Q)
+        const int r0 = (int)((long long)n * me / T), r1 = (int)((long long)n * (me + 1) / T), nr = r1 - r0;
+        double* Z = Zall.data() + (size_t)n * r0;
+        for (int r = r0; r < r1; ++r) {
+            std::fill(q, q + n, 0.0);
+            q[r] = 1.0;
+            for (int k = 0; k + 2 < n; ++k) {
+                if (tau[k] == 0.0) continue;
+                const double* v = &A[(size_t)k * n];
+                const double s = tau[k] * dot(v + k + 1, q + k + 1, n - k - 1);
+                for (int j = k + 1; j < n; ++j) q[j] -= s * v[j];
+            }
+            for (int j = 0; j < n; ++j) Z[(size_t)j * nr + (r - r0)] = q[j];
+        }
+        // (3) implicit QL on (d, e), e[i] coupling d[i] and d[i+1]; each plane rotation of rows i, i+1 of
+        //     the tridiagonal matrix is applied to rows i, i+1 of Z
+        std::copy(d.begin(), d.end(), dl);
+        std::copy(e.begin(), e.end(), el);
+        for (int l = 0; l < n; ++l) {
+            for (int iter = 0; iter < 60; ++iter) {
+                int m = l;
+                for (; m + 1 < n; ++m) {
+                    const double dd = std::fabs(dl[m]) + std::fabs(dl[m + 1]);
+                    if (std::fabs(el[m]) <= 1e-16 * dd) break;
+                }
+                if (m == l) break;
+                double g = (dl[l + 1] - dl[l]) / (2.0 * el[l]);
+                double r = std::hypot(g, 1.0);
+                g = dl[m] - dl[l] + el[l] / (g + (g >= 0.0 ? r : -r));   // shifted so that the shift is the
+                double s = 1.0, c = 1.0, pp = 0.0;                       // eigenvalue of the leading 2x2 closer to d[l]
+                int i = m - 1;
+                bool deflated = false;
+                for (; i >= l; --i) {
+                    const double f = s * el[i], b = c * el[i];
+                    r = std::hypot(f, g);
+                    el[i + 1] = r;
+                    if (r == 0.0) { dl[i + 1] -= pp; el[m] = 0.0; deflated = true; break; }
+                    s = f / r;
+                    c = g / r;
+                    g = dl[i + 1] - pp;
+                    r = (dl[i] - g) * s + 2.0 * c * b;
+                    pp = s * r;
+                    dl[i + 1] = g + pp;
+                    g = c * r - b;
+                    double* zi = Z + (size_t)i * nr;
+                    double* zj = zi + nr;
+                    for (int k = 0; k < nr; ++k) {
+                        const double a0 = zi[k], a1 = zj[k];
+                        zj[k] = s * a0 + c * a1;
+                        zi[k] = c * a0 - s * a1;
+                    }
+                }
+                if (deflated) continue;
+                dl[l] -= pp;
+                el[l] = g;
+                el[m] = 0.0;
+            }
+        }
+        for (int i = 0; i < n; ++i)
+            for (int k = r0; k < r1; ++k) V[(size_t)k * n + i] = Z[(size_t)i * nr + (k - r0)];
+        if (me == 0) std::copy(dl, dl + n, eig.begin());
+    });
     for (int i = 0; i < n; ++i)
-        for (int k = 0; k < n; ++k) V[(size_t)k * n + i] = Z[(size_t)i * n + k];
-    for (int i = 0; i < n; ++i)
-        for (int j = 0; j < n; ++j) A[(size_t)i * n + j] = i == j ? d[i] : 0.0;
+        for (int j = 0; j < n; ++j) A[(size_t)i * n + j] = i == j ? eig[i] : 0.0;
 }
 
 // Cholesky L L^T = A (row-major, lower triangle written into A); false if not positive definite
 bool cholesky(std::vector<double>& A, int n) {
     for (int j = 0; j < n; ++j) {
-        double s = A[(size_t)j * n + j];
-        for (int k = 0; k < j; ++k) s -= A[(size_t)j * n + k] * A[(size_t)j * n + k];
+        const double* aj = &A[(size_t)j * n];
+        const double s = aj[j] - dot(aj, aj, j);
         if (!(s > 0.0)) return false;
         const double d = std::sqrt(s);
         A[(size_t)j * n + j] = d;
         for (int i = j + 1; i < n; ++i) {
-            double t = A[(size_t)i * n + j];
-            for (int k = 0; k < j; ++k) t -= A[(size_t)i * n + k] * A[(size_t)j * n + k];
-            A[(size_t)i * n + j] = t / d;
+            double* ai = &A[(size_t)i * n];
+            ai[j] = (ai[j] - dot(ai, aj, j)) / d;
         }
     }
     return true;
 }
 
-// solve L L^T X = B in place (B row-major n x m)
+// solve L L^T X = B in place (B row-major n x m), all columns at once
 void chol_solve(const std::vector<double>& L, int n, std::vector<double>& B, int m) {
-    for (int c = 0; c < m; ++c) {
-        for (int i = 0; i < n; ++i) {
-            double t = B[(size_t)i * m + c];
-            for (int k = 0; k < i; ++k) t -= L[(size_t)i * n + k] * B[(size_t)k * m + c];
-            B[(size_t)i * m + c] = t / L[(size_t)i * n + i];
-        }
-        for (int i = n - 1; i >= 0; --i) {
-            double t = B[(size_t)i * m + c];
-            for (int k = i + 1; k < n; ++k) t -= L[(size_t)k * n + i] * B[(size_t)k * m + c];
-            B[(size_t)i * m + c] = t / L[(size_t)i * n + i];
-        }
+    const auto take = [&](int i, int k, double l) {
+        double* bi = &B[(size_t)i * m];
+        const double* bk = &B[(size_t)k * m];
+        for (int c = 0; c < m; ++c) bi[c] -= l * bk[c];
+    };
+    const auto divide = [&](int i) {
+        for (int c = 0; c < m; ++c) B[(size_t)i * m + c] /= L[(size_t)i * n + i];
+    };
+    for (int i = 0; i < n; ++i) {
+        for (int k = 0; k < i; ++k) take(i, k, L[(size_t)i * n + k]);
+        divide(i);
+    }
+    for (int i = n - 1; i >= 0; --i) {
+        for (int k = i + 1; k < n; ++k) take(i, k, L[(size_t)k * n + i]);
+        divide(i);
     }
 }
 
