@@ -207,8 +207,7 @@ int enqueue_implicit_captured(osam_ctx* ctx, int s, const int* active) {
                     LK(newton_tangent(g, b));
                     LK(launch_cg_ap_b(g, g.cgact, c0, b));
                     LK(launch_cg_step_b(g, g.cgact, c0, cg_floor(g), b));
-                    LK(launch_cg_dir_b(g, g.cgact, c0, b));
-                    LK(launch_imp_loop_cond(g, hc, 1, kCgMax, b));
+                    LK(launch_cg_dir_b(g, g.cgact, c0, b, hc, kCgMax));
                     return OSAM_OK;
                 };
                 rc2 = cg();

@@ -273,8 +273,22 @@ __global__ void __launch_bounds__(kNodeBlock) k_cg_step_b(const FomB g, const in
     }
 }
 
-// p = z + beta p
-__global__ void __launch_bounds__(kNodeBlock) k_cg_dir_b(const FomB g, const int* __restrict__ mask, double ic0) {
+// Device-side loop control at the end of a pass (conditional WHILE nodes of a CUDA graph): which = 0 the
+// Newton loop, 1 the CG loop.  Counts the pass and continues while some instance is still iterating and the
+// cap is not reached (the loops end after at most max_it passes).
+__device__ __forceinline__ void loop_cond(const FomB& g, cudaGraphConditionalHandle h, int which, int max_it) {
+    const int it = ++g.iloop[which];
+    const int* m = which == 0 ? g.nact : g.cgact;
+    unsigned int go = 0;
+    for (int i = 0; i < g.n_inst; ++i) go |= m[i] == 1 ? 1u : 0u;
+    cudaGraphSetConditional(h, (go && it < max_it) ? 1u : 0u);
+}
+
+// p = z + beta p; in a graph (max_it > 0) one thread also closes the pass of the CG loop (the activity masks are
+// final since the step kernel), which saves a launch per iteration
+__global__ void __launch_bounds__(kNodeBlock) k_cg_dir_b(const FomB g, const int* __restrict__ mask, double ic0,
+                                                         cudaGraphConditionalHandle h, int max_it) {
+    if (max_it > 0 && blockIdx.x == 0 && threadIdx.x == 0) loop_cond(g, h, 1, max_it);
     const NodeCtx x = node_ctx(g, mask);
     if (!x.ok) return;
     const double beta = g.beta[x.inst];
@@ -344,10 +358,7 @@ __global__ void __launch_bounds__(kNodeBlock) k_imp_finish_b(const FomB g, const
     }
 }
 
-// Device-side loop control (conditional WHILE nodes of a CUDA graph): which = 0 the Newton loop,
-// 1 the CG loop.  Entry: reset the loop's counter, enter (Newton) or enter if an instance still has
-// a CG solve to do.  Condition at the end of a pass: count the pass, continue while some instance is
-// still iterating and the cap is not reached (the loops end after at most max_it passes).
+// Entry of a loop: reset its counter, enter (Newton) or enter if an instance still has a CG solve to do
 __global__ void k_imp_loop_entry(const FomB g, cudaGraphConditionalHandle h, int which) {
     if (threadIdx.x != 0 || blockIdx.x != 0) return;
     g.iloop[which] = 0;
@@ -361,11 +372,7 @@ __global__ void k_imp_loop_entry(const FomB g, cudaGraphConditionalHandle h, int
 
 __global__ void k_imp_loop_cond(const FomB g, cudaGraphConditionalHandle h, int which, int max_it) {
     if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    const int it = ++g.iloop[which];
-    const int* m = which == 0 ? g.nact : g.cgact;
-    unsigned int go = 0;
-    for (int i = 0; i < g.n_inst; ++i) go |= m[i] == 1 ? 1u : 0u;
-    cudaGraphSetConditional(h, (go && it < max_it) ? 1u : 0u);
+    loop_cond(g, h, which, max_it);
 }
 
 __global__ void k_mask_copy(int n, const int* __restrict__ src, int* dst) {
@@ -395,8 +402,9 @@ cudaError_t launch_cg_step_b(const FomB& g, const int* mask, double c0, double t
     k_cg_step_b<<<g.n_nblk, kNodeBlock, 0, s>>>(g, mask, 1.0 / c0, tol2);
     return cudaGetLastError();
 }
-cudaError_t launch_cg_dir_b(const FomB& g, const int* mask, double c0, cudaStream_t s) {
-    k_cg_dir_b<<<g.n_nblk, kNodeBlock, 0, s>>>(g, mask, 1.0 / c0);
+cudaError_t launch_cg_dir_b(const FomB& g, const int* mask, double c0, cudaStream_t s, cudaGraphConditionalHandle h,
+                            int max_it) {
+    k_cg_dir_b<<<g.n_nblk, kNodeBlock, 0, s>>>(g, mask, 1.0 / c0, h, max_it);
     return cudaGetLastError();
 }
 cudaError_t launch_imp_update_b(const FomB& g, const int* mask, cudaStream_t s) {

@@ -294,7 +294,9 @@ cudaError_t launch_force_lin_b(const FomB& g, const int* mask, cudaStream_t s);
 cudaError_t launch_tangent_lin_b(const FomB& g, const int* mask, cudaStream_t s);
 cudaError_t launch_cg_ap_b(const FomB& g, const int* mask, double c0, cudaStream_t s);
 cudaError_t launch_cg_step_b(const FomB& g, const int* mask, double c0, double tol2, cudaStream_t s);
-cudaError_t launch_cg_dir_b(const FomB& g, const int* mask, double c0, cudaStream_t s);
+// max_it > 0: also closes the pass of the CG loop whose handle is h
+cudaError_t launch_cg_dir_b(const FomB& g, const int* mask, double c0, cudaStream_t s, cudaGraphConditionalHandle h = 0,
+                            int max_it = 0);
 cudaError_t launch_imp_update_b(const FomB& g, const int* mask, cudaStream_t s);
 cudaError_t launch_imp_finish_b(const FomB& g, const int* active, int slot1, double dt, double c0, cudaStream_t s);
 cudaError_t launch_mask_copy(int n, const int* src, int* dst, cudaStream_t s);
