@@ -153,21 +153,33 @@ __global__ void k_adjoint_pre(int nn, double dt, const uint8_t* clamp, const dou
 }
 
 // ubar' += VJP (gathered from the element buffer in a fixed order); then the adjoints at the previous
-// step:  abar = dt/2 vbar' + dt^2/2 ubar',  vbar = vbar' + dt ubar',  ubar = ubar'
+// step:  abar = dt/2 vbar' + dt^2/2 ubar',  vbar = vbar' + dt ubar',  ubar = ubar'; with minv also that step's
+// k_adjoint_pre, which takes the same dof's values
 __global__ void k_adjoint_post(int nx, int ny, int nz, double dt, const uint8_t* clamp, const double* fe, double* ub,
-                               double* vb, double* ab) {
+                               double* vb, double* ab, const double* minv, double* y) {
     const int nn = (nx + 1) * (ny + 1) * (nz + 1);
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= 3 * nn) return;
-    const int c = t / nn, n = t % nn;
-    if (clamp[n] & (1 << c)) { ub[t] = 0.0; vb[t] = 0.0; ab[t] = 0.0; return; }
+    const int n = blockIdx.x * blockDim.x + threadIdx.x;
+    if (n >= nn) return;
+    const int c = blockIdx.y;
+    const long long t = (long long)c * nn + n;
+    if (clamp[n] & (1 << c)) {
+        ub[t] = 0.0; vb[t] = 0.0; ab[t] = 0.0;
+        if (minv) y[t] = 0.0;
+        return;
+    }
     const int i = n % (nx + 1), q = n / (nx + 1);
     const double g = hex8::gather_force(fe, nx, ny, nz, nx * ny * nz, i, q % (ny + 1), q / (ny + 1), c);
     const double u = ub[t] + g;
-    const double v = vb[t];
+    double v = vb[t];
     ub[t] = u;
-    ab[t] = fma(0.5 * dt * dt, u, 0.5 * dt * v);
-    vb[t] = fma(dt, u, v);
+    double a = fma(0.5 * dt * dt, u, 0.5 * dt * v);
+    v = fma(dt, u, v);
+    vb[t] = v;
+    if (minv) {
+        a = fma(0.5 * dt, v, a);
+        y[t] = -a * minv[n];
+    }
+    ab[t] = a;
 }
 
 }  // namespace
@@ -179,9 +191,9 @@ cudaError_t launch_adjoint_pre(int nn, double dt, const uint8_t* clamp, const do
 }
 
 cudaError_t launch_adjoint_post(int nx, int ny, int nz, double dt, const uint8_t* clamp, const double* fe, double* ub,
-                                double* vb, double* ab, cudaStream_t s) {
+                                double* vb, double* ab, const double* minv, double* y, cudaStream_t s) {
     const long long nn = (long long)(nx + 1) * (ny + 1) * (nz + 1);
-    k_adjoint_post<<<grid_for(3 * nn, 256), 256, 0, s>>>(nx, ny, nz, dt, clamp, fe, ub, vb, ab);
+    k_adjoint_post<<<dim3(grid_for(nn, 128), 3), 128, 0, s>>>(nx, ny, nz, dt, clamp, fe, ub, vb, ab, minv, y);
     return cudaGetLastError();
 }
 

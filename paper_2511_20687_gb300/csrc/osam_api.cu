@@ -526,14 +526,27 @@ int osam_adjoint(const osam_adjoint_desc* d, osam_adjoint_out* out) {
     for (auto& x : ev.e) CK(cudaEventCreateWithFlags(&x, cudaEventDisableTiming));
     cudaEvent_t ev_rec[2] = {ev.e[0], ev.e[1]}, ev_rev[2] = {ev.e[2], ev.e[3]}, ev_start = ev.e[4];
     CK(cudaEventRecord(ctx->ev0, R));
-    // one explicit step in place on (u[0], v, a), deterministic element-buffer scatter
-    auto step = [&](double* u_store, cudaStream_t st) -> int {
-        CK(launch_node_b(F, nullptr, kGather, -1, 1, 1, F.u[0], F.u[1], dt, st));
-        CK(launch_force_b(F, nullptr, kGather, st, nullptr, F.u[1]));
-        CK(launch_node_b(F, nullptr, kGather, 1, -1, 0, F.u[1], F.u[0], dt, st));
-        CK(cudaMemcpyAsync(F.u[0], F.u[1], sizeof(double) * n3, cudaMemcpyDeviceToDevice, st));
-        if (u_store) CK(cudaMemcpyAsync(u_store, F.u[0], sizeof(double) * n3, cudaMemcpyDeviceToDevice, st));
+    // n explicit steps from (u at x(0), v, a): the displacement of step j is written to x(j).  The node
+    // kernel of step j corrects v and a and predicts step j + 1, so a step is a force and a node launch.
+    auto steps = [&](int n, const std::function<double*(int)>& x, cudaStream_t st) -> int {
+        if (n < 1) return OSAM_OK;
+        CK(launch_node_b(F, nullptr, kGather, -1, 1, 1, x(0), x(1), dt, st));
+        for (int j = 1; j <= n; ++j) {
+            CK(launch_force_b(F, nullptr, kGather, st, nullptr, x(j)));
+            CK(launch_node_b(F, nullptr, kGather, 1, j < n ? 1 : -1, 0, x(j), j < n ? x(j + 1) : x(j - 1), dt, st));
+        }
         return OSAM_OK;
+    };
+    // forward sweep: u in alternating buffers, back in u[0] at the end
+    auto forward = [&](int n, cudaStream_t st) -> int {
+        RET(steps(n, [&](int j) { return F.u[j & 1]; }, st));
+        if (n & 1) CK(cudaMemcpyAsync(F.u[0], F.u[1], sizeof(double) * n3, cudaMemcpyDeviceToDevice, st));
+        return OSAM_OK;
+    };
+    // a segment again, every displacement kept in buf
+    auto recompute = [&](int n, double* buf, cudaStream_t st) -> int {
+        CK(cudaMemcpyAsync(buf, F.u[0], sizeof(double) * n3, cudaMemcpyDeviceToDevice, st));
+        return steps(n, [&](int j) { return buf + (size_t)j * n3; }, st);
     };
     auto save_ck = [&](int idx) -> int {
         double* base = ck + (size_t)idx * 3 * n3;
@@ -555,12 +568,15 @@ int osam_adjoint(const osam_adjoint_desc* d, osam_adjoint_out* out) {
     va.lam_e = I.lam_e; va.mu_e = I.mu_e;
     va.usn = 1; va.usc = nn;
     va.fe = vfe;
-    // reverse of step t + 1 of a segment starting at t0 (state u_{t+1} stored at buf[t + 1 - t0])
-    auto reverse = [&](int t, int t0, const double* buf, cudaStream_t st) -> int {
+    // reverse of the n steps of a segment whose displacements are in buf; the adjoint update of a step also
+    // forms the cotangent of the step before it
+    auto reverse = [&](int n, const double* buf, cudaStream_t st) -> int {
         CK(launch_adjoint_pre(nn, dt, F.clamp, F.minv, vb, ab, y, st));
-        va.u = buf + (size_t)(t + 1 - t0) * n3;
-        CK(launch_hex8_vjp(F.material, kGather, va, y, 1, nn, glam, gmu, 1, st));
-        CK(launch_adjoint_post(I.nx, I.ny, I.nz, dt, F.clamp, vfe, ub, vb, ab, st));
+        for (int t = n; t >= 1; --t) {
+            va.u = buf + (size_t)t * n3;
+            CK(launch_hex8_vjp(F.material, kGather, va, y, 1, nn, glam, gmu, 1, st));
+            CK(launch_adjoint_post(I.nx, I.ny, I.nz, dt, F.clamp, vfe, ub, vb, ab, t > 1 ? F.minv : nullptr, y, st));
+        }
         return OSAM_OK;
     };
     // A full segment of Cp steps is the same sequence of launches every time (the checkpoint is loaded
@@ -584,17 +600,10 @@ int osam_adjoint(const osam_adjoint_desc* d, osam_adjoint_out* out) {
         return OSAM_OK;
     };
     if (T >= Cp) {
-        RET(capture(0, [&]() -> int { for (int t = 0; t < Cp; ++t) RET(step(nullptr, R)); return OSAM_OK; }));
+        RET(capture(0, [&]() -> int { return forward(Cp, R); }));
         for (int b = 0; b < 2; ++b) {
-            RET(capture(1 + b, [&]() -> int {
-                CK(cudaMemcpyAsync(useg[b], F.u[0], sizeof(double) * n3, cudaMemcpyDeviceToDevice, R));
-                for (int t = 1; t <= Cp; ++t) RET(step(useg[b] + (size_t)t * n3, R));
-                return OSAM_OK;
-            }));
-            RET(capture(3 + b, [&]() -> int {
-                for (int t = Cp - 1; t >= 0; --t) RET(reverse(t, 0, useg[b], R));
-                return OSAM_OK;
-            }));
+            RET(capture(1 + b, [&]() -> int { return recompute(Cp, useg[b], R); }));
+            RET(capture(3 + b, [&]() -> int { return reverse(Cp, useg[b], R); }));
         }
     }
     RET(save_ck(0));
@@ -603,7 +612,7 @@ int osam_adjoint(const osam_adjoint_desc* d, osam_adjoint_out* out) {
             CK(cudaGraphLaunch(graphs.g[0], R));
             RET(save_ck((t0 + Cp) / Cp));
         } else {
-            for (int t = t0 + 1; t <= T; ++t) RET(step(nullptr, R));
+            RET(forward(T - t0, R));
         }
     }
     // J = w . u_T
@@ -624,9 +633,8 @@ int osam_adjoint(const osam_adjoint_desc* d, osam_adjoint_out* out) {
     if (seg >= 0 && T - seg * Cp < Cp) {
         const int t0 = seg * Cp;
         RET(load_ck(seg, R));
-        CK(cudaMemcpyAsync(useg[0], F.u[0], sizeof(double) * n3, cudaMemcpyDeviceToDevice, R));
-        for (int t = t0 + 1; t <= T; ++t) RET(step(useg[0] + (size_t)(t - t0) * n3, R));
-        for (int t = T - 1; t >= t0; --t) RET(reverse(t, t0, useg[0], R));
+        RET(recompute(T - t0, useg[0], R));
+        RET(reverse(T - t0, useg[0], R));
         --seg;
     }
     if (seg >= 0) {
@@ -652,7 +660,7 @@ int osam_adjoint(const osam_adjoint_desc* d, osam_adjoint_out* out) {
     RET(load_ck(0, R));
     va.u = F.u[0];
     CK(launch_hex8_vjp(F.material, kGather, va, y, 1, nn, glam, gmu, 1, R));
-    CK(launch_adjoint_post(I.nx, I.ny, I.nz, 0.0, F.clamp, vfe, ub, vb, ab, R));
+    CK(launch_adjoint_post(I.nx, I.ny, I.nz, 0.0, F.clamp, vfe, ub, vb, ab, nullptr, y, R));
     CK(cudaEventRecord(ctx->ev1, ctx->stream));
     CK(cudaEventSynchronize(ctx->ev1));
     float ms = 0.f;

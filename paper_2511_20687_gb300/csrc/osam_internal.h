@@ -344,7 +344,7 @@ cudaError_t launch_hex8_vjp(int material, int scatter, const ElemArgs& a, const 
 cudaError_t launch_adjoint_pre(int nn, double dt, const uint8_t* clamp, const double* minv, const double* vb, double* ab,
                                double* y, cudaStream_t s);
 cudaError_t launch_adjoint_post(int nx, int ny, int nz, double dt, const uint8_t* clamp, const double* fe, double* ub,
-                                double* vb, double* ab, cudaStream_t s);
+                                double* vb, double* ab, const double* minv, double* y, cudaStream_t s);
 
 // message returned by osam_last_error(NULL) on the calling thread
 void set_thread_error(const std::string& msg);
