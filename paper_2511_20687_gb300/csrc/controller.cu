@@ -79,7 +79,6 @@ constexpr double kCgTol2F32 = 1e-12;   // the floor with the FP32 tangent (eta >
 // Newton residual force and tangent action of an implicit group, and the CG floor that goes with the
 // tangent's precision
 cudaError_t newton_force(const FomB& g, cudaStream_t s) {
-    if (g.linf) return launch_force_lin_b(g, g.nact, s);
     if (g.material == OSAM_NEO_HOOKEAN) return launch_imp_force_nh_b(g, g.nact, s);
     return launch_force_b(g, g.nact, kGather, s, nullptr);
 }

@@ -437,8 +437,15 @@ struct Cols {
 
 constexpr int kOne25 = 1 << 25;
 
+// Linearisation of one Gauss point: F and cof F [column][component] (61 fraction bits), alpha (60), beta (57),
+// a1 = -2/3 alpha / J (60), b1 = kappa - (a1 trC / 3 + beta) / J (57)
+struct Linear {
+    i64 F[3][3], cof[3][3], alpha, beta, a1, b1;
+};
+OSAM_HD i64 whole(D x) { return shl((i64)x.h, 32) + x.l; }
+
 // Piola stress P[column][component] (57 fraction bits, below 1) of one Gauss point; false out of range
-OSAM_HD bool stress_point(const Cols& C, D kap2, D mu, D mu3, i64 P[3][3]) {
+OSAM_HD bool stress_point(const Cols& C, D kap2, D mu, D mu3, i64 P[3][3], Linear* lin = nullptr) {
     D F[3][3], nF1[3], nF2[3];
     i64 n = 0;
     Range g;
@@ -472,6 +479,18 @@ OSAM_HD bool stress_point(const Cols& C, D kap2, D mu, D mu3, i64 P[3][3]) {
 #pragma unroll
 #endif
         for (int k = 0; k < 3; ++k) top |= hi(P[k][c]) ^ (hi(P[k][c]) >> 31);
+    }
+    if (lin) {
+        for (int c = 0; c < 3; ++c) {
+            lin->cof[0][c] = whole(s.c0[c]); lin->cof[1][c] = whole(s.c1[c]); lin->cof[2][c] = whole(s.c2[c]);
+            for (int k = 0; k < 3; ++k) lin->F[k][c] = C.x[k][c];
+        }
+        lin->alpha = s.alpha;
+        lin->beta = s.beta;
+        const i64 a13 = mul_third(mul(split(shl(s.alpha, 2)), s.inv));             // alpha / (3 J), 60
+        lin->a1 = -shl(a13, 1);
+        const i64 e = s.beta - mul_third(mul(split(shl(a13, 2)), split(shl(n, 2))));   // 57, below 9
+        lin->b1 = (whole(kap2) >> 4) - mul(s.inv, split(shl(e, 2)));               // 57
     }
     return !out_of_range(g) && top < kOne25;
 }
@@ -754,6 +773,46 @@ OSAM_HD double f64_scaled(i64 x, int scale) {
     __builtin_memcpy(&r, &b, 8);
 #endif
     return r;
+}
+
+// x / 2^scale as an FP32 value, rounded toward zero (integer operations; zero below the normal range, largest
+// exponent above it)
+OSAM_HD float f32_scaled(i64 x, int scale) {
+    if (x == 0) return 0.0f;
+    const unsigned long long m = x < 0 ? 0ULL - (unsigned long long)x : (unsigned long long)x;
+    const int lz = lead_zeros((i64)(m >> 1)) - 1;       // m < 2^63
+    const int e = 127 + 63 - lz - scale;
+    const unsigned int f = (unsigned int)((m << lz) >> 40);   // 24 bits, leading bit set
+    const unsigned int b = (x < 0 ? 0x80000000u : 0u) |
+                           (e < 1 ? 0u : e > 254 ? 0x7f800000u : ((unsigned int)(e - 1) << 23) + f);
+    float r;
+#ifdef __CUDA_ARCH__
+    r = __uint_as_float(b);
+#else
+    __builtin_memcpy(&r, &b, 4);
+#endif
+    return r;
+}
+
+// (hi, lo) FP32 split of u / h by integer operations: hi the product cut to 24 bits, lo the remainder cut to 24 bits
+// (|u / h - (hi + lo)| < 2^-47 |u / h|).  ihm, ihe: 1/h as in fixed_u.
+OSAM_HD void split_scaled(double u, i64 ihm, int ihe, float& hif, float& lof) {
+    unsigned long long b;
+#ifdef __CUDA_ARCH__
+    b = (unsigned long long)__double_as_longlong(u);
+#else
+    __builtin_memcpy(&b, &u, 8);
+#endif
+    const int e = (int)((b >> 52) & 0x7ff);
+    const i64 m = e == 0 ? 0 : (i64)(((b & 0xfffffffffffffULL) | 0x10000000000000ULL) << 10);   // u = m 2^(e - 1085)
+    const i64 p = mul(m, ihm);                                       // below 2^62: u / h = p 2^(e - 1085 + ihe + 2)
+    const int lz = lead_zeros(p);
+    const i64 q = shl(p, lz == 64 ? 0 : lz - 1), top = q & ~(((i64)1 << 39) - 1);   // 24 leading bits of [2^62, 2^63)
+    const int scale = 1083 - e - ihe + (lz == 64 ? 0 : lz - 1);
+    const bool neg = (b >> 63) != 0, odd = e == 2047;
+    const i64 h = odd ? (i64)1 << 62 : top, l = q - top;
+    hif = f32_scaled(neg ? -h : h, odd ? -200 : scale);              // infinite for operands that are not finite
+    lof = odd ? 0.0f : f32_scaled(neg ? -l : l, scale);
 }
 
 // fixed-point u / h of a nodal displacement: mantissa (53 bits) times the 63-bit mantissa of 1/h, shifted

@@ -24,6 +24,10 @@ namespace {
 using namespace fx;
 
 constexpr int kLaneBlock = 128;                   // 16 elements
+// Blocks per SM asked of the compiler: the lane kernels wait on their own results, so warps in flight count.
+// 64x64x64, force 149.9 us at the natural 157 registers, 143.7 at 128, 139.5 at 5 blocks; vector-Jacobian product
+// 361.8 at 248 registers, 306 at 168, 301 at 128 (20x20x40: 31.1, 26.8, 24.9).
+constexpr int kForceBlocks = 5, kTangentBlocks = 4;
 
 // FP64 evaluation of one element (all 24 values, parameter contractions) for operands outside the formats.
 // x(c, corner) and p(c, corner) read the displacement and the direction.  Not inlined into the lane path's registers.
@@ -78,6 +82,46 @@ __device__ __noinline__ void far_tangent(const FarIn& x, double F[3][8], double&
     walsh_transpose<double>(Sx, Sy, Sz, F);
 }
 
+// The Newton linearisation of the FP32 tangent (k_tangent_lin32_b): F, cof F, alpha, beta and the coefficients of
+// dalpha = a1 dJ and dbeta = b1 dJ + a1 (F : G), dJ = cof : G, per Gauss point; layout [kLinPerGp][8 Gauss points][NE],
+// Gauss point 4 x + 2 y + z:
+//   a1 = -2/3 alpha / J,  b1 = 2 kappa/2 - (a1 trC / 3 + beta) / J   (from P = alpha F + beta cof,
+//   alpha = mu J^-2/3, beta = (kappa/2 (J^2 - 1) - mu/3 J^-2/3 trC) / J).
+static_assert(kLinPerGp == 22, "stored linearisation: F, cof F, alpha, beta, a1, b1");
+__device__ __forceinline__ int lin_point(int a) { return 4 * (a & 1) + (a & 2) + (a >> 2); }
+
+struct LinStore {
+    float* lin;          // this element's first entry
+    long long ne;        // stride between Gauss points
+    double kap2;         // m1 of the material factors
+    __device__ void operator()(int p, int q, int r, const double (&Fm)[3][3], const double (&Cm)[3][3], double, double trC,
+                               double invJ, double alpha, double beta) const {
+        const double a1 = -(2.0 / 3.0) * alpha * invJ;
+        const double b1 = 2.0 * kap2 - invJ * fma(a1, trC * (1.0 / 3.0), beta);
+        const long long st = 8 * ne;
+        float* lg = lin + (long long)(4 * p + 2 * q + r) * ne;
+        for (int a = 0; a < 9; ++a) {
+            lg[a * st] = (float)Fm[a / 3][a % 3];
+            lg[(9 + a) * st] = (float)Cm[a / 3][a % 3];
+        }
+        lg[18 * st] = (float)alpha; lg[19 * st] = (float)beta; lg[20 * st] = (float)a1; lg[21 * st] = (float)b1;
+    }
+};
+
+__device__ __noinline__ void far_linearise(const FarIn& x, float* lin, long long ne, double F[3][8]) {
+    using namespace hex8;
+    double Gx[3][2][2], Gy[3][2][2], Gz[3][2][2], Sx[3][2][2], Sy[3][2][2], Sz[3][2][2], m1, m2, m3;
+    material_factors<OSAM_NEO_HOOKEAN, double>(x.lam, x.mu, x.wq, x.wq3, m1, m2, m3);
+    for (int c = 0; c < 3; ++c) {
+        double U[8], Dx[2][2], Dy[2][2], Dz[2][2];
+        for (int c8 = 0; c8 < 8; ++c8) U[c8] = x.u[c * x.usc + x.node(c8) * x.usn];
+        edge_differences<double>(U, x.invh, Dx, Dy, Dz);
+        lerp2<double>(Dx, Gx[c], c == 0); lerp2<double>(Dy, Gy[c], c == 1); lerp2<double>(Dz, Gz[c], c == 2);
+    }
+    nh_gauss_sums<double>(Gx, Gy, Gz, m1, m2, m3, Sx, Sy, Sz, LinStore{lin, ne, m1});
+    walsh_transpose<double>(Sx, Sy, Sz, F);
+}
+
 // The element of a lane group in one mesh; lanes beyond the last element repeat it (all lanes take part in
 // the shuffles) and write nothing
 struct Elem {
@@ -113,7 +157,7 @@ __device__ __forceinline__ FarIn far_in(const ElemArgs& a, const Elem& x, const 
 }
 
 template <int MODE>
-__global__ void __launch_bounds__(kLaneBlock) k_elem_force(const __grid_constant__ ElemArgs a, i64 ihm, int ihe) {
+__global__ void __launch_bounds__(kLaneBlock, kForceBlocks) k_elem_force(const __grid_constant__ ElemArgs a, i64 ihm, int ihe) {
     const Elem x = element((int)(blockIdx.x * (kLaneBlock / 8) + (threadIdx.x >> 3)), a.nx, a.ny, a.ne);
     const Lane L = make_lane();
     const int node = corner_node(x, L.a);
@@ -137,7 +181,7 @@ __global__ void __launch_bounds__(kLaneBlock) k_elem_force(const __grid_constant
 }
 
 template <int MODE>
-__global__ void __launch_bounds__(kLaneBlock) k_elem_vjp(const __grid_constant__ ElemArgs a, const double* ybar, int ysn,
+__global__ void __launch_bounds__(kLaneBlock, kTangentBlocks) k_elem_vjp(const __grid_constant__ ElemArgs a, const double* ybar, int ysn,
                                                          long long ysc, double* lam_bar, double* mu_bar, int accumulate,
                                                          i64 ihm, int ihe, double wqi, double vol) {
     const Elem x = element((int)(blockIdx.x * (kLaneBlock / 8) + (threadIdx.x >> 3)), a.nx, a.ny, a.ne);
@@ -176,9 +220,12 @@ __global__ void __launch_bounds__(kLaneBlock) k_elem_vjp(const __grid_constant__
 }
 
 // ---- implicit groups (FomB): element buffer [24][NE] ----------------------------------------------
-// TANGENT: K(u) p of the CG direction; else the internal force of u
-template <bool TANGENT>
-__global__ void __launch_bounds__(kLaneBlock) k_fom_lanes(const __grid_constant__ FomB g, const int* __restrict__ mask) {
+// OP kOpTangent: K(u) p of the CG direction; else the internal force of u, with kOpLinearise also the Newton
+// linearisation of the FP32 tangent
+enum { kOpForce, kOpLinearise, kOpTangent };
+template <int OP>
+__global__ void __launch_bounds__(kLaneBlock, OP == kOpTangent ? kTangentBlocks : kForceBlocks) k_fom_lanes(const __grid_constant__ FomB g, const int* __restrict__ mask) {
+    constexpr bool TANGENT = OP == kOpTangent;
     const int per = g.eblock * 8 / kLaneBlock;   // thread blocks per element block
     const int2 b = g.eblk[blockIdx.x / per];
     if (mask && !mask[b.x]) return;
@@ -199,9 +246,26 @@ __global__ void __launch_bounds__(kLaneBlock) k_fom_lanes(const __grid_constant_
     Material M;
     const bool bad = !material(lam, mu, TANGENT ? I.wqi : I.wq, M);
     int scale = 57 - M.k, base;
+    Linear q;
+    Linear* lin = OP == kOpLinearise ? &q : nullptr;
     const bool ok = TANGENT ? tangent_lanes(L, U, p, M, bad, false, F, scale, pk, pm, base)
-                            : force_lanes(L, U, M.kap2, M.mu, M.mu3, bad || M.k < -900 || M.k > 900, F);
+                            : force_lanes(L, U, M.kap2, M.mu, M.mu3, bad || M.k < -900 || M.k > 900, F, lin);
     if (!x.live) return;
+    if (OP == kOpLinearise && ok) {
+        float* lg = g.linf + I.elem_off + x.e + (long long)lin_point(L.a) * g.NE;
+        const long long st = 8LL * g.NE;
+#pragma unroll
+        for (int d = 0; d < 3; ++d)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                lg[(3 * c + d) * st] = f32_scaled(q.F[d][c], 61);
+                lg[(9 + 3 * c + d) * st] = f32_scaled(q.cof[d][c], 61);
+            }
+        lg[18 * st] = f32_scaled(q.alpha, 60 - M.k);
+        lg[19 * st] = f32_scaled(q.beta, 57 - M.k);
+        lg[20 * st] = f32_scaled(q.a1, 60 - M.k);
+        lg[21 * st] = f32_scaled(q.b1, 57 - M.k);
+    }
     double* fe = static_cast<double*>(g.fe) + I.elem_off + x.e;
     if (ok) {
 #pragma unroll
@@ -211,6 +275,7 @@ __global__ void __launch_bounds__(kLaneBlock) k_fom_lanes(const __grid_constant_
                        I.invh, lam, mu, I.wq, I.wq3};
         double Ff[3][8], lb, mb;
         if (TANGENT) far_tangent(in, Ff, lb, mb);
+        else if (OP == kOpLinearise) far_linearise(in, g.linf + I.elem_off + x.e, g.NE, Ff);
         else far_force(in, Ff);
         for (int c8 = 0; c8 < 8; ++c8)
             for (int c = 0; c < 3; ++c) fe[(long long)(c8 * 3 + c) * g.NE] = Ff[c][c8];
@@ -251,13 +316,15 @@ cudaError_t launch_elem_vjp_nh(int scatter, const ElemArgs& a, const double* yba
 
 cudaError_t launch_imp_force_nh_b(const FomB& g, const int* mask, cudaStream_t s) {
     if (g.eblock % 32) return cudaErrorInvalidValue;
-    k_fom_lanes<false><<<g.n_eblk * (g.eblock * 8 / kLaneBlock), kLaneBlock, 0, s>>>(g, mask);
+    const int grid = g.n_eblk * (g.eblock * 8 / kLaneBlock);
+    if (g.linf) k_fom_lanes<kOpLinearise><<<grid, kLaneBlock, 0, s>>>(g, mask);
+    else k_fom_lanes<kOpForce><<<grid, kLaneBlock, 0, s>>>(g, mask);
     return cudaGetLastError();
 }
 
 cudaError_t launch_imp_tangent_nh_b(const FomB& g, const int* mask, cudaStream_t s) {
     if (g.eblock % 32) return cudaErrorInvalidValue;
-    k_fom_lanes<true><<<g.n_eblk * (g.eblock * 8 / kLaneBlock), kLaneBlock, 0, s>>>(g, mask);
+    k_fom_lanes<kOpTangent><<<g.n_eblk * (g.eblock * 8 / kLaneBlock), kLaneBlock, 0, s>>>(g, mask);
     return cudaGetLastError();
 }
 

@@ -137,11 +137,13 @@ __device__ __forceinline__ bool material(double lam, double mu, double w, Materi
 }
 
 // corner forces of the lane's corner (57 fraction bits, units 2^k); false if the element is out of range
-__device__ __forceinline__ bool force_lanes(const Lane& L, const i64 U[3], D kap2, D mu, D mu3, bool bad, i64 F[3]) {
+// (lin: also the linearisation of the lane's Gauss point)
+__device__ __forceinline__ bool force_lanes(const Lane& L, const i64 U[3], D kap2, D mu, D mu3, bool bad, i64 F[3],
+                                            Linear* lin = nullptr) {
     Cols C;
     deformation(L, U, C, bad);
     i64 P[3][3];
-    bad |= !stress_point(C, kap2, mu, mu3, P);
+    bad |= !stress_point(C, kap2, mu, mu3, P, lin);
 #pragma unroll
     for (int c = 0; c < 3; ++c)
         F[c] = corner_values(L, pattern_scale(L, gauss_transpose(L, P[0][c], P[1][c], P[2][c])));

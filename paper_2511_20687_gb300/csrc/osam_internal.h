@@ -288,9 +288,7 @@ cudaError_t launch_imp_residual_b(const FomB& g, const int* mask, double c0, cud
 // products are reduced inside k_cg_ap_b / k_cg_step_b by each instance's last block.
 cudaError_t launch_imp_reduce_b(const FomB& g, const int* mask, int mode, int first, double tol2, cudaStream_t s);
 cudaError_t launch_tangent_b(const FomB& g, const int* mask, cudaStream_t s);
-// Neo-Hookean implicit groups with the FP32 tangent: Newton force that also stores the Gauss-point
-// linearisation, and the tangent action that reads it
-cudaError_t launch_force_lin_b(const FomB& g, const int* mask, cudaStream_t s);
+// Neo-Hookean implicit groups with the FP32 tangent: the tangent action from the stored linearisation
 cudaError_t launch_tangent_lin_b(const FomB& g, const int* mask, cudaStream_t s);
 cudaError_t launch_cg_ap_b(const FomB& g, const int* mask, double c0, cudaStream_t s);
 cudaError_t launch_cg_step_b(const FomB& g, const int* mask, double c0, double tol2, cudaStream_t s);

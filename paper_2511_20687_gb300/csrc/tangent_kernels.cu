@@ -145,17 +145,10 @@ __global__ void __launch_bounds__(256) k_tangent_b(const FomB g, const int* __re
     }
 }
 
-// ---- Neo-Hookean Newton linearisation stored once per Newton step --------------------------------
+// ---- FP32 tangent from the stored Neo-Hookean linearisation ---------------------------------------
 // The tangent at u is applied ~6 times per Newton step (CG iterations) while u stays fixed, so the
 // u-dependent part of dP = dbeta cof + beta dcof[G] + dalpha F + alpha G is computed once, with the
-// force of the Newton residual, and stored per Gauss point: F, cof F, alpha, beta and the two
-// coefficients of the scalar derivatives, dalpha = a1 dJ and dbeta = b1 dJ + a1 (F : G), dJ = cof : G,
-//   a1 = -2/3 alpha / J,  b1 = 2 kappa/2 - (a1 trC / 3 + beta) / J   (from P = alpha F + beta cof,
-//   alpha = mu J^-2/3, beta = (kappa/2 (J^2 - 1) - mu/3 J^-2/3 trC) / J).
-// Layout [kLinPerGp][8 Gauss points][NE], element index fastest (coalesced): F (9), cof F (9), alpha,
-// beta, a1, b1.
-static_assert(kLinPerGp == 22, "stored linearisation: F, cof F, alpha, beta, a1, b1");
-
+// force of the Newton residual (lane_kernels.cu), and stored per Gauss point in FP32.
 // transposed interpolation of the Gauss-point sums (scaled like the force's: Walsh basis, factor 4 in
 // the material factors) and the element-buffer write
 template <typename T>
@@ -193,73 +186,6 @@ __device__ __forceinline__ ElemIdx elem_idx(const FomB& g, const int* mask) {
 #pragma unroll
     for (int c8 = 0; c8 < 8; ++c8) x.node[c8] = n0 + (c8 & 1) + ((c8 >> 1) & 1) * sy + ((c8 >> 2) & 1) * sz;
     return x;
-}
-
-// FP64 -> FP32 for the stored FP32 linearisation by integer operations (f32_rz: a conversion
-// instruction would take a slot of the FP64 pipe, the bound of the Newton force, 176 times per
-// element; the entries -- F, cof F and the material-scaled factors -- lie far inside the FP32 range,
-// and the rounding toward zero is at the CG operator's own FP32 level).
-__device__ __forceinline__ float lin_value(double x) { return f32_rz(x); }
-
-// The per-Gauss-point quantities of the Newton linearisation, stored by the Neo-Hookean Gauss sums'
-// hook (TL: the storage type); a1 and b1 from the force's own 1/J (the cube of its reciprocal cube
-// root, no division).  Material factors scaled by h^2/32 like the force's (the Walsh-basis transposed
-// interpolation carries the remaining factor 4), so the tangent's dP is scaled alike.
-struct LinStore {
-    float* lin;             // this element's first entry
-    long long st;        // stride between quantities (8 NE)
-    long long ne;        // stride between Gauss points (NE)
-    double kap2;         // m1 of the material factors
-    __device__ __forceinline__ void operator()(int p, int q, int r, const double (&Fm)[3][3], const double (&Cm)[3][3],
-                                               double J, double trC, double invJ, double alpha, double beta) const {
-        (void)J;
-        const double a1 = -(2.0 / 3.0) * alpha * invJ;
-        const double b1 = 2.0 * kap2 - invJ * fma(a1, trC * (1.0 / 3.0), beta);
-        float* lg = lin + (long long)(4 * p + 2 * q + r) * ne;
-#pragma unroll
-        for (int a = 0; a < 9; ++a) {
-            lg[a * st] = lin_value(Fm[a / 3][a % 3]);
-            lg[(9 + a) * st] = lin_value(Cm[a / 3][a % 3]);
-        }
-        lg[18 * st] = lin_value(alpha); lg[19 * st] = lin_value(beta);
-        lg[20 * st] = lin_value(a1); lg[21 * st] = lin_value(b1);
-    }
-};
-
-// Newton residual force of a Neo-Hookean group at u (from u / h) plus the stored linearisation: the
-// explicit force's arithmetic (1 of F's diagonal in the first interpolation stage, paired Gauss-point
-// sums, Walsh-basis transposed interpolation) with the linearisation written at each Gauss point
-__global__ void __launch_bounds__(256) k_force_lin_b(const FomB g, float* __restrict__ lin_base,
-                                                     const int* __restrict__ mask) {
-    const ElemIdx x = elem_idx(g, mask);
-    if (!x.ok) return;
-    const InstFom& I = x.I;
-    const int e = x.e;
-    double Gx[3][2][2], Gy[3][2][2], Gz[3][2][2];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        double V[8], Dx[2][2], Dy[2][2], Dz[2][2];
-#pragma unroll
-        for (int c8 = 0; c8 < 8; ++c8) V[c8] = g.us[(long long)c * g.NN + I.node_off + x.node[c8]];
-        edge_differences_prescaled<double>(V, Dx, Dy, Dz);
-        lerp2<double>(Dx, Gx[c], c == 0);
-        lerp2<double>(Dy, Gy[c], c == 1);
-        lerp2<double>(Dz, Gz[c], c == 2);
-    }
-    double m1, m2, m3;
-    if (I.lam_e || I.mu_e)
-        material_factors<OSAM_NEO_HOOKEAN, double>(I.lam_e ? I.lam_e[e] : I.lam, I.mu_e ? I.mu_e[e] : I.mu, I.wq,
-                                                   I.wq3, m1, m2, m3);
-    else { m1 = I.m1; m2 = I.m2; m3 = I.m3; }
-    const LinStore store{lin_base + I.elem_off + e, 8LL * g.NE, g.NE, m1};
-    double Sx[3][2][2], Sy[3][2][2], Sz[3][2][2], F[3][8];
-    nh_gauss_sums<double>(Gx, Gy, Gz, m1, m2, m3, Sx, Sy, Sz, store);
-    walsh_transpose<double>(Sx, Sy, Sz, F);
-    double* fe = static_cast<double*>(g.fe) + I.elem_off;
-#pragma unroll
-    for (int c8 = 0; c8 < 8; ++c8)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) fe[(long long)(c8 * 3 + c) * g.NE + e] = F[c][c8];
 }
 
 // Tangent action from the stored linearisation in FP32 (OSAM_FP64_TANGENT32): the direction p converted once per nodal value, every Gauss-point
@@ -344,13 +270,6 @@ __global__ void __launch_bounds__(256) k_tangent_lin32_b(const FomB g, const int
 }
 
 }  // namespace
-
-cudaError_t launch_force_lin_b(const FomB& g, const int* mask, cudaStream_t s) {
-    if (g.n_eblk == 0) return cudaSuccess;
-    if (g.eblock > 256 || !g.linf || g.material != OSAM_NEO_HOOKEAN) return cudaErrorInvalidValue;
-    k_force_lin_b<<<g.n_eblk, g.eblock, 0, s>>>(g, g.linf, mask);
-    return cudaGetLastError();
-}
 
 cudaError_t launch_tangent_lin_b(const FomB& g, const int* mask, cudaStream_t s) {
     if (g.n_eblk == 0) return cudaSuccess;
