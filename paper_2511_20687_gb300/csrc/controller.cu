@@ -73,6 +73,7 @@ constexpr double kNewtonTol2 = 1e-24;  // |R|^2 <= kNewtonTol2 |R(u~)|^2
 constexpr double kNewtonInc2 = 1e-28;  // or an increment |du|^2 <= kNewtonInc2 |u|^2 (rounding level of u)
 constexpr int kCgMax = 1000;           // CG iterations per Newton step
 constexpr int kCgCheck = 8;            // CG iterations between host checks of the activity mask
+constexpr int kCgUnroll = 2;           // CG iterations per pass of the device-side loop (kCgMax is a multiple)
 constexpr double kCgTol2 = 1e-26;      // floor of the CG test r.z <= eta^2 (r.z)_0 (eta: the Newton forcing term)
 constexpr double kCgTol2F32 = 1e-12;   // the floor with the FP32 tangent (eta >= 1e-6, above its rounding)
 
@@ -203,10 +204,12 @@ int enqueue_implicit_captured(osam_ctx* ctx, int s, const int* active) {
                 cudaStream_t b = ctx->cap[1];
                 int rc2 = OSAM_OK;
                 auto cg = [&]() -> int {
-                    LK(newton_tangent(g, b));
-                    LK(launch_cg_ap_b(g, g.cgact, c0, b));
-                    LK(launch_cg_step_b(g, g.cgact, c0, cg_floor(g), b));
-                    LK(launch_cg_dir_b(g, g.cgact, c0, b, hc, kCgMax));
+                    for (int u = 1; u <= kCgUnroll; ++u) {
+                        LK(newton_tangent(g, b));
+                        LK(launch_cg_ap_b(g, g.cgact, c0, b));
+                        LK(launch_cg_step_b(g, g.cgact, c0, cg_floor(g), b));
+                        LK(launch_cg_dir_b(g, g.cgact, c0, b, hc, u == kCgUnroll ? kCgMax / kCgUnroll : 0));
+                    }
                     return OSAM_OK;
                 };
                 rc2 = cg();

@@ -38,6 +38,12 @@ __device__ __forceinline__ double block_sum1(double x) {
     return a;
 }
 
+// Partial sums of a node kernel: one per block, in the plane of its component (blockIdx.y, with one component
+// per thread) of [2 quantities][3][n_nblk]; every plane of a launch is summed in a fixed order.
+__device__ __forceinline__ double* ipart(const FomB& g, int quantity, int plane) {
+    return g.ipart + (long long)(3 * quantity + plane) * g.n_nblk;
+}
+
 struct NodeCtx {
     int inst, n;
     long long gn;
@@ -84,6 +90,7 @@ __global__ void __launch_bounds__(kNodeBlock) k_imp_predict_b(const FomB g, cons
 // R = M (u - ut) c0 + f (free dofs; the element forces of u are in the element buffer).  CG start
 // x = 0, r = -R, z = p = M^-1 r / c0 (the mass part of the tangent as preconditioner); partials
 // |R|^2 and r . z
+template <int NC>
 __global__ void __launch_bounds__(kNodeBlock) k_imp_residual_b(const FomB g, const int* __restrict__ mask, double c0,
                                                                double ic0) {
     const NodeCtx x = node_ctx(g, mask);
@@ -97,7 +104,8 @@ __global__ void __launch_bounds__(kNodeBlock) k_imp_residual_b(const FomB g, con
         const double m = g.mass[x.gn];
         const double pz = g.minv[x.gn] * ic0;
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
+        for (int q = 0; q < NC; ++q) {
+            const int c = NC == 3 ? q : (int)blockIdx.y;
             const long long d = (long long)c * g.NN + x.gn;
             double R = 0.0;
             if (is_free(g, x.gn, c)) {
@@ -114,22 +122,23 @@ __global__ void __launch_bounds__(kNodeBlock) k_imp_residual_b(const FomB g, con
     s = block_sum1(s);
     sz = block_sum1(sz);
     if (threadIdx.x == 0) {
-        g.ipart[blockIdx.x] = s;
-        g.ipart[g.n_nblk + blockIdx.x] = sz;
+        ipart(g, 0, blockIdx.y)[blockIdx.x] = s;
+        ipart(g, 1, blockIdx.y)[blockIdx.x] = sz;
     }
 }
 
 // per-instance fixed-order sums of the node-block partials, and the decisions that depend on them
-__global__ void k_imp_reduce_b(const FomB g, const int* __restrict__ mask, int mode, int first, double tol2) {
+__global__ void k_imp_reduce_b(const FomB g, const int* __restrict__ mask, int mode, int first, double tol2, int planes) {
     const int inst = blockIdx.x;
     if (!run(mask, inst)) return;
     if (first < 0) first = g.iloop[0] == 0;  // device-side Newton loop: its counter says which step this is
     const int b0 = g.nblk_off[inst], b1 = g.nblk_off[inst + 1];
     double s = 0.0, sz = 0.0;
-    for (int b = b0 + (int)threadIdx.x; b < b1; b += blockDim.x) {
-        s += g.ipart[b];
-        sz += g.ipart[g.n_nblk + b];
-    }
+    for (int y = 0; y < planes; ++y)
+        for (int b = b0 + (int)threadIdx.x; b < b1; b += blockDim.x) {
+            s += ipart(g, 0, y)[b];
+            sz += ipart(g, 1, y)[b];
+        }
     s = block_sum1(s);
     sz = block_sum1(sz);
     if (threadIdx.x != 0) return;
@@ -166,14 +175,15 @@ __device__ __forceinline__ bool last_block_sum(const FomB& g, int inst, double& 
     if (threadIdx.x == 0) {
         __threadfence();
         const unsigned int t = atomicAdd(g.iticket + inst, 1u);
-        last = t == (unsigned int)(g.nblk_off[inst + 1] - g.nblk_off[inst] - 1);
+        last = t == gridDim.y * (unsigned int)(g.nblk_off[inst + 1] - g.nblk_off[inst]) - 1u;
     }
     __syncthreads();
     if (!last) return false;
     __threadfence();
     const int b0 = g.nblk_off[inst], b1 = g.nblk_off[inst + 1];
     double s = 0.0;
-    for (int b = b0 + (int)threadIdx.x; b < b1; b += blockDim.x) s += __ldcg(g.ipart + b);
+    for (int y = 0; y < (int)gridDim.y; ++y)
+        for (int b = b0 + (int)threadIdx.x; b < b1; b += blockDim.x) s += __ldcg(ipart(g, 0, y) + b);
     s = block_sum1(s);
     if (threadIdx.x != 0) return false;
     g.iticket[inst] = 0u;
@@ -207,6 +217,7 @@ __device__ __forceinline__ double gather_tangent32(const float* fe, int nx, int 
 
 // Ap = M p c0 + K p (free dofs; K p from the FP64 element buffer, or the FP32 one of the FP32 tangent);
 // p . Ap summed per instance by its last block, which sets alpha = (r . z) / (p . Ap) for the step kernel
+template <int NC>
 __global__ void __launch_bounds__(kNodeBlock) k_cg_ap_b(const FomB g, const int* __restrict__ mask, double c0) {
     const NodeCtx x = node_ctx(g, mask);
     double s = 0.0;
@@ -219,7 +230,8 @@ __global__ void __launch_bounds__(kNodeBlock) k_cg_ap_b(const FomB g, const int*
         const float* fe32 = g.fe32 ? g.fe32 + x.I.elem_off : nullptr;
         const double m = g.mass[x.gn];
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
+        for (int q = 0; q < NC; ++q) {
+            const int c = NC == 3 ? q : (int)blockIdx.y;
             const long long d = (long long)c * g.NN + x.gn;
             double ap = 0.0;
             if (is_free(g, x.gn, c)) {
@@ -232,7 +244,7 @@ __global__ void __launch_bounds__(kNodeBlock) k_cg_ap_b(const FomB g, const int*
         }
     }
     s = block_sum1(s);
-    if (threadIdx.x == 0) g.ipart[blockIdx.x] = s;
+    if (threadIdx.x == 0) ipart(g, 0, blockIdx.y)[blockIdx.x] = s;
     double pap;
     if (last_block_sum(g, x.inst, pap) && run(mask, x.inst)) {
         g.pap[x.inst] = pap;
@@ -243,6 +255,7 @@ __global__ void __launch_bounds__(kNodeBlock) k_cg_ap_b(const FomB g, const int*
 // x += alpha p, r -= alpha Ap; r . z of the new residual summed per instance by its last block, which
 // counts the iteration, ends the instance's CG solve at the forcing tolerance (floor tol2) and sets
 // beta = (r . z)_new / (r . z) and r . z <- (r . z)_new for the direction kernel
+template <int NC>
 __global__ void __launch_bounds__(kNodeBlock) k_cg_step_b(const FomB g, const int* __restrict__ mask, double ic0,
                                                           double tol2) {
     const NodeCtx x = node_ctx(g, mask);
@@ -251,7 +264,8 @@ __global__ void __launch_bounds__(kNodeBlock) k_cg_step_b(const FomB g, const in
         const double alpha = g.alpha[x.inst];
         const double pz = g.minv[x.gn] * ic0;
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
+        for (int q = 0; q < NC; ++q) {
+            const int c = NC == 3 ? q : (int)blockIdx.y;
             const long long d = (long long)c * g.NN + x.gn;
             g.cg_x[d] = fma(alpha, g.cg_p[d], g.cg_x[d]);
             const double r = fma(-alpha, g.cg_ap[d], g.cg_r[d]);
@@ -260,7 +274,7 @@ __global__ void __launch_bounds__(kNodeBlock) k_cg_step_b(const FomB g, const in
         }
     }
     s = block_sum1(s);
-    if (threadIdx.x == 0) g.ipart[blockIdx.x] = s;
+    if (threadIdx.x == 0) ipart(g, 0, blockIdx.y)[blockIdx.x] = s;
     double rrn;
     if (last_block_sum(g, x.inst, rrn) && run(mask, x.inst)) {
         const int inst = x.inst;
@@ -286,27 +300,31 @@ __device__ __forceinline__ void loop_cond(const FomB& g, cudaGraphConditionalHan
 
 // p = z + beta p; in a graph (max_it > 0) one thread also closes the pass of the CG loop (the activity masks are
 // final since the step kernel), which saves a launch per iteration
+template <int NC>
 __global__ void __launch_bounds__(kNodeBlock) k_cg_dir_b(const FomB g, const int* __restrict__ mask, double ic0,
                                                          cudaGraphConditionalHandle h, int max_it) {
-    if (max_it > 0 && blockIdx.x == 0 && threadIdx.x == 0) loop_cond(g, h, 1, max_it);
+    if (max_it > 0 && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) loop_cond(g, h, 1, max_it);
     const NodeCtx x = node_ctx(g, mask);
     if (!x.ok) return;
     const double beta = g.beta[x.inst];
     const double pz = g.minv[x.gn] * ic0;
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
+    for (int q = 0; q < NC; ++q) {
+        const int c = NC == 3 ? q : (int)blockIdx.y;
         const long long d = (long long)c * g.NN + x.gn;
         g.cg_p[d] = fma(beta, g.cg_p[d], g.cg_r[d] * pz);
     }
 }
 
 // u += x on free dofs, refreshed u / h for the force kernel; partials |x|^2 and |u|^2 (free dofs)
+template <int NC>
 __global__ void __launch_bounds__(kNodeBlock) k_imp_update_b(const FomB g, const int* __restrict__ mask) {
     const NodeCtx x = node_ctx(g, mask);
     double sx = 0.0, su = 0.0;
     if (x.ok) {
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
+        for (int q = 0; q < NC; ++q) {
+            const int c = NC == 3 ? q : (int)blockIdx.y;
             const long long d = (long long)c * g.NN + x.gn;
             if (is_free(g, x.gn, c)) {
                 const double dx = g.cg_x[d];
@@ -321,8 +339,8 @@ __global__ void __launch_bounds__(kNodeBlock) k_imp_update_b(const FomB g, const
     sx = block_sum1(sx);
     su = block_sum1(su);
     if (threadIdx.x == 0) {
-        g.ipart[blockIdx.x] = sx;
-        g.ipart[g.n_nblk + blockIdx.x] = su;
+        ipart(g, 0, blockIdx.y)[blockIdx.x] = sx;
+        ipart(g, 1, blockIdx.y)[blockIdx.x] = su;
     }
 }
 
@@ -387,28 +405,33 @@ cudaError_t launch_imp_predict_b(const FomB& g, const int* active, int slot1, do
     return cudaGetLastError();
 }
 cudaError_t launch_imp_residual_b(const FomB& g, const int* mask, double c0, cudaStream_t s) {
-    k_imp_residual_b<<<g.n_nblk, kNodeBlock, 0, s>>>(g, mask, c0, 1.0 / c0);   // 1 / c0 once, on the host
+    if (node_split(g)) k_imp_residual_b<1><<<dim3(g.n_nblk, 3), kNodeBlock, 0, s>>>(g, mask, c0, 1.0 / c0);
+    else k_imp_residual_b<3><<<g.n_nblk, kNodeBlock, 0, s>>>(g, mask, c0, 1.0 / c0);   // 1 / c0 once, on the host
     return cudaGetLastError();
 }
 cudaError_t launch_imp_reduce_b(const FomB& g, const int* mask, int mode, int first, double tol2, cudaStream_t s) {
-    k_imp_reduce_b<<<g.n_inst, 128, 0, s>>>(g, mask, mode, first, tol2);
+    k_imp_reduce_b<<<g.n_inst, 128, 0, s>>>(g, mask, mode, first, tol2, node_split(g) ? 3 : 1);
     return cudaGetLastError();
 }
 cudaError_t launch_cg_ap_b(const FomB& g, const int* mask, double c0, cudaStream_t s) {
-    k_cg_ap_b<<<g.n_nblk, kNodeBlock, 0, s>>>(g, mask, c0);
+    if (node_split(g)) k_cg_ap_b<1><<<dim3(g.n_nblk, 3), kNodeBlock, 0, s>>>(g, mask, c0);
+    else k_cg_ap_b<3><<<g.n_nblk, kNodeBlock, 0, s>>>(g, mask, c0);
     return cudaGetLastError();
 }
 cudaError_t launch_cg_step_b(const FomB& g, const int* mask, double c0, double tol2, cudaStream_t s) {
-    k_cg_step_b<<<g.n_nblk, kNodeBlock, 0, s>>>(g, mask, 1.0 / c0, tol2);
+    if (node_split(g)) k_cg_step_b<1><<<dim3(g.n_nblk, 3), kNodeBlock, 0, s>>>(g, mask, 1.0 / c0, tol2);
+    else k_cg_step_b<3><<<g.n_nblk, kNodeBlock, 0, s>>>(g, mask, 1.0 / c0, tol2);
     return cudaGetLastError();
 }
 cudaError_t launch_cg_dir_b(const FomB& g, const int* mask, double c0, cudaStream_t s, cudaGraphConditionalHandle h,
                             int max_it) {
-    k_cg_dir_b<<<g.n_nblk, kNodeBlock, 0, s>>>(g, mask, 1.0 / c0, h, max_it);
+    if (node_split(g)) k_cg_dir_b<1><<<dim3(g.n_nblk, 3), kNodeBlock, 0, s>>>(g, mask, 1.0 / c0, h, max_it);
+    else k_cg_dir_b<3><<<g.n_nblk, kNodeBlock, 0, s>>>(g, mask, 1.0 / c0, h, max_it);
     return cudaGetLastError();
 }
 cudaError_t launch_imp_update_b(const FomB& g, const int* mask, cudaStream_t s) {
-    k_imp_update_b<<<g.n_nblk, kNodeBlock, 0, s>>>(g, mask);
+    if (node_split(g)) k_imp_update_b<1><<<dim3(g.n_nblk, 3), kNodeBlock, 0, s>>>(g, mask);
+    else k_imp_update_b<3><<<g.n_nblk, kNodeBlock, 0, s>>>(g, mask);
     return cudaGetLastError();
 }
 cudaError_t launch_imp_finish_b(const FomB& g, const int* active, int slot1, double dt, double c0, cudaStream_t s) {

@@ -111,7 +111,7 @@ struct FomB {
     double* cg_r;             // CG residual [3][NN]
     double* cg_p;             // CG direction [3][NN]
     double* cg_ap;            // tangent times direction [3][NN]
-    double* ipart;            // partial sums, two per node block
+    double* ipart;            // partial sums [2][3][n_nblk]
     double* rn2;              // per instance: squared Newton residual
     double* r0;               // per instance: squared residual of the predictor
     double* rr;               // per instance: r . z of the current CG iterate (z = M^-1 r / c0)

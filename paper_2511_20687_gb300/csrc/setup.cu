@@ -300,7 +300,7 @@ int setup_fom_group(osam_ctx* ctx, FomGroupH& G, int s, int n, const osam_proble
     B.n_nblk = (int)G.nblk.size();
     B.nblk_off = nbo;
     CKA(B.partial = ctx->alloc<double>(2LL * B.n_nblk));
-    if (B.implicit) CKA(B.ipart = ctx->alloc<double>(2LL * B.n_nblk));
+    if (B.implicit) CKA(B.ipart = ctx->alloc<double>(6LL * B.n_nblk));
     RET(set_eblocks(ctx, G, 128));
     RET(set_tiles(ctx, G));
     std::vector<double> modulus;
