@@ -16,6 +16,7 @@
 
 #include <cstdint>
 
+#include "fixed_math.cuh"
 #include "hex8_math.cuh"
 #include "osam_internal.h"
 #include "trace_item.cuh"
@@ -395,8 +396,13 @@ __global__ void __launch_bounds__(kNodeBlock) k_node_b(const FomB g, const int* 
         }
         if (h2) {
             unext[d] = un;
-            g.us[d] = un * I.invh;
-            if (sizeof(TF) == 4) g.u2[d] = split_f2(un * I.invh);   // FP32 force input
+            if constexpr (sizeof(TF) == 4) {   // FP32 force input, without the FP64 pipe
+                float2 x;
+                fx::split_scaled(un, I.ihm, I.ihe, x.x, x.y);
+                g.u2[d] = x;
+            } else {
+                g.us[d] = un * I.invh;
+            }
         }
     }
 }
