@@ -10,6 +10,7 @@
 
 #include <cstdint>
 
+#include "fixed_math.cuh"
 #include "hex8_math.cuh"
 #include "osam_internal.h"
 
@@ -36,26 +37,10 @@ __device__ __forceinline__ void edge_diffs(const double* x, int sn, long long sc
     }
 }
 
-// Linear elastic, one thread per element.  MODE kAtomic adds ubar into a.f ([3] x strided nodes); kGather writes the
-// element's 24 contributions to the element buffer a.fe [24][ne] (corner-major, component), which a
-// fixed-order gather sums per node (deterministic).  The transposed interpolation is the force's
-// Walsh-basis stage (hex8::walsh_transpose), so the material factors carry its 1/4.
-template <int MODE>
-__global__ void __launch_bounds__(128) k_hex8_vjp_le(const ElemArgs a, const double* ybar, int ysn, long long ysc,
-                                                  double* lam_bar, double* mu_bar, int accumulate) {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= a.ne) return;
-    const int i = e % a.nx;
-    const int t = e / a.nx;
-    const int j = t % a.ny;
-    const int k = t / a.ny;
-    const int sy = a.nx + 1, sz = (a.nx + 1) * (a.ny + 1);
-    const int n0 = i + sy * j + sz * k;
-    int node[8];
-#pragma unroll
-    for (int c8 = 0; c8 < 8; ++c8) node[c8] = n0 + (c8 & 1) + ((c8 >> 1) & 1) * sy + ((c8 >> 2) & 1) * sz;
-    const double lam = a.lam_e ? a.lam_e[e] : a.lam;
-    const double mu = a.mu_e ? a.mu_e[e] : a.mu;
+// Linear elastic vector-Jacobian product of one element in FP64, for operands outside the integer formats.  The
+// transposed interpolation is the force's Walsh-basis stage, so the material factors carry its 1/4.
+__device__ __noinline__ void far_vjp_le(const ElemArgs& a, const double* ybar, int ysn, long long ysc, const int node[8],
+                                        double lam, double mu, double Fe[3][8], double& lb, double& mb) {
     double Dx[3][2][2], Dy[3][2][2], Dz[3][2][2];
     double Ex[3][2][2], Ey[3][2][2], Ez[3][2][2];
     edge_diffs(a.u, a.usn, a.usc, node, a.invh, Dx, Dy, Dz);
@@ -69,7 +54,7 @@ __global__ void __launch_bounds__(128) k_hex8_vjp_le(const ElemArgs a, const dou
     double m1, m2, m3;
     hex8::material_factors<OSAM_LINEAR_ELASTIC, double>(lam, mu, a.wq, a.wq3, m1, m2, m3);
     double Sx[3][2][2], Sy[3][2][2], Sz[3][2][2];
-    double lb = 0.0, mb = 0.0;
+    lb = mb = 0.0;
 #pragma unroll
     for (int p = 0; p < 2; ++p)
 #pragma unroll
@@ -101,25 +86,78 @@ __global__ void __launch_bounds__(128) k_hex8_vjp_le(const ElemArgs a, const dou
                     if (r == 0) Sz[c][p][q] = dP[c][2]; else Sz[c][p][q] += dP[c][2];
                 }
             }
-    double Fe[3][8];
     hex8::walsh_transpose<double>(Sx, Sy, Sz, Fe);
-    if (MODE == kAtomic) {
-        double* ub = static_cast<double*>(a.f);
+}
+
+template <int MODE>
+__device__ __forceinline__ void put(const ElemArgs& a, int e, const int node[8], int c8, int c, double v) {
+    if (MODE == kAtomic)
+        atomicAdd(static_cast<double*>(a.f) + (long long)c * a.fsc + (long long)node[c8] * a.fsn, v);
+    else
+        static_cast<double*>(a.fe)[(long long)(c8 * 3 + c) * a.ne + e] = v;
+}
+
+// Linear elastic, one thread per element, in 64-bit integers: the law is linear, so the cotangent of u is the force
+// of ybar and the parameters' are bilinear in the Walsh coefficients of u and ybar (fixed_math.cuh).  In FP64
+// (396 us on 64x64x64) it was bound by about 1100 FP64 instructions per element.  MODE kAtomic adds ubar into
+// a.f ([3] x strided nodes); kGather writes the element's 24 contributions to the element buffer a.fe [24][ne]
+// (corner-major, component), which a fixed-order gather sums per node (deterministic).
+template <int MODE>
+__global__ void __launch_bounds__(64) k_hex8_vjp_le(const __grid_constant__ ElemArgs a, const double* ybar, int ysn,
+                                                    long long ysc, double* lam_bar, double* mu_bar, int accumulate) {
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= a.ne) return;
+    const int i = e % a.nx;
+    const int t = e / a.nx;
+    const int j = t % a.ny;
+    const int k = t / a.ny;
+    const int sy = a.nx + 1, sz = (a.nx + 1) * (a.ny + 1);
+    const int n0 = i + sy * j + sz * k;
+    const double lam = a.lam_e ? a.lam_e[e] : a.lam;
+    const double mu = a.mu_e ? a.mu_e[e] : a.mu;
+    const double h16 = 2.0 * a.wq * a.invh;    // h / 16
+    int node[8];
+    double U[3][8], Fe[3][8];
 #pragma unroll
-        for (int c = 0; c < 3; ++c)
+    for (int c8 = 0; c8 < 8; ++c8) node[c8] = n0 + (c8 & 1) + ((c8 >> 1) & 1) * sy + (c8 >> 2) * sz;
+    fx::i64 wu[3][8], wy[3][8], dl, dm;
+    int Tu, Ty;
 #pragma unroll
-            for (int c8 = 0; c8 < 8; ++c8) atomicAdd(ub + (long long)c * a.fsc + (long long)node[c8] * a.fsn, Fe[c][c8]);
-    } else {
-        double* fe = static_cast<double*>(a.fe);
+    for (int c = 0; c < 3; ++c)
+#pragma unroll
+        for (int c8 = 0; c8 < 8; ++c8) U[c][c8] = a.u[(long long)c * a.usc + (long long)node[c8] * a.usn];
+    bool ok = fx::block_walsh(U, wu, Tu);
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+#pragma unroll
+        for (int c8 = 0; c8 < 8; ++c8) U[c][c8] = ybar[(long long)c * ysc + (long long)node[c8] * ysn];
+    ok = fx::block_walsh(U, wy, Ty) && ok;
+    ok = ok && fx::force_le_walsh(wy, Ty, lam * h16, mu * h16, Fe);
+    const bool zero = Tu == fx::kNoExponent || Ty == fx::kNoExponent;
+    const int scale = zero ? 0 : 2090 - Tu - Ty;   // 2 (1081 - 6) - 60
+    ok = ok && scale < 1000 && scale > -900;
+    double lb = 0.0, mb = 0.0;
+    if (ok) {
+        fx::contract_le(wu, wy, dl, dm);
+        lb = h16 * fx::f64_scaled(dl, scale);
+        mb = h16 * fx::f64_scaled(dm, scale);
 #pragma unroll
         for (int c8 = 0; c8 < 8; ++c8)
 #pragma unroll
-            for (int c = 0; c < 3; ++c) fe[(long long)(c8 * 3 + c) * a.ne + e] = Fe[c][c8];
+            for (int c = 0; c < 3; ++c) put<MODE>(a, e, node, c8, c, Fe[c][c8]);
+    } else {
+        double Ff[3][8];
+        int far[8];
+        for (int c8 = 0; c8 < 8; ++c8) far[c8] = n0 + (c8 & 1) + ((c8 >> 1) & 1) * sy + (c8 >> 2) * sz;
+        far_vjp_le(a, ybar, ysn, ysc, far, lam, mu, Ff, lb, mb);
+        for (int c8 = 0; c8 < 8; ++c8)
+            for (int c = 0; c < 3; ++c) put<MODE>(a, e, far, c8, c, Ff[c][c8]);
+        const double vol8 = a.w8 / a.invh;     // w detJ = h^3/8 per Gauss point; the gradients are physical
+        lb *= vol8;
+        mb *= vol8;
     }
-    // w detJ = h^3/8 per Gauss point; Gbar above is the physical gradient
-    const double vol8 = a.w8 / a.invh;
-    if (lam_bar) lam_bar[e] = (accumulate ? lam_bar[e] : 0.0) + vol8 * lb;
-    if (mu_bar) mu_bar[e] = (accumulate ? mu_bar[e] : 0.0) + vol8 * mb;
+    if (lam_bar) lam_bar[e] = (accumulate ? lam_bar[e] : 0.0) + lb;
+    if (mu_bar) mu_bar[e] = (accumulate ? mu_bar[e] : 0.0) + mb;
 }
 
 }  // namespace
@@ -128,9 +166,9 @@ cudaError_t launch_hex8_vjp(int material, int scatter, const ElemArgs& a, const 
                             double* lam_bar, double* mu_bar, int acc, cudaStream_t s) {
     if (a.ne <= 0) return cudaSuccess;
     if (material == OSAM_NEO_HOOKEAN) return launch_elem_vjp_nh(scatter, a, ybar, ysn, ysc, lam_bar, mu_bar, acc, s);
-    const int g = grid_for(a.ne, 128);
-    if (scatter == kAtomic) k_hex8_vjp_le<kAtomic><<<g, 128, 0, s>>>(a, ybar, ysn, ysc, lam_bar, mu_bar, acc);
-    else k_hex8_vjp_le<kGather><<<g, 128, 0, s>>>(a, ybar, ysn, ysc, lam_bar, mu_bar, acc);
+    const int g = grid_for(a.ne, 64);
+    if (scatter == kAtomic) k_hex8_vjp_le<kAtomic><<<g, 64, 0, s>>>(a, ybar, ysn, ysc, lam_bar, mu_bar, acc);
+    else k_hex8_vjp_le<kGather><<<g, 64, 0, s>>>(a, ybar, ysn, ysc, lam_bar, mu_bar, acc);
     return cudaGetLastError();
 }
 

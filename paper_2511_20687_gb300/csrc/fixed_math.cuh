@@ -657,17 +657,13 @@ OSAM_HD void le_coefficients(const i64 w[3][8], i64 lam, i64 mu, i64 f[3][8]) {
     }
 }
 
-// The 24 nodal forces of an element from its 24 nodal displacements: exact Walsh sums of the block values,
-// the coefficients above, the inverse sums.  lam, mu: Lame parameters times the factor h / 16 (divided by
-// the factor that the displacements carry).  Returns false for operands outside the formats (not finite,
-// or so small or large that the result's exponent leaves the normal range): the caller then uses FP64.
-OSAM_HD double f64_scaled(i64 x, int scale);
-OSAM_HD bool element_force_le(const double U[3][8], double lam, double mu, double F[3][8]) {
-    const int ek = factor_exponent(lam, mu);
-    if (ek == 2047) return false;
-    i64 w[3][8], f[3][8];
-    int e[3], T = kNoExponent;
+// The Walsh coefficients of an element's 24 nodal values in block format, |w| < 2^58, coefficient =
+// w 2^(T + 6 - 1081) (T = kNoExponent and w = 0 without differences); false for values that are not finite or
+// subnormal
+OSAM_HD bool block_walsh(const double U[3][8], i64 w[3][8], int& T) {
+    int e[3];
     bool bad = false;
+    T = kNoExponent;
 #ifdef __CUDACC__
 #pragma unroll
 #endif
@@ -682,7 +678,7 @@ OSAM_HD bool element_force_le(const double U[3][8], double lam, double mu, doubl
         }
         e[c] = (int)(top >> 20);
         bad |= e[c] == 2047;
-        if (e[c] == 0) {                       // all zero, or subnormal displacements
+        if (e[c] == 0) {                       // all zero, or subnormal
             unsigned long long bits = 0;
             for (int a = 0; a < 8; ++a) {
                 unsigned long long b;
@@ -715,18 +711,31 @@ OSAM_HD bool element_force_le(const double U[3][8], double lam, double mu, doubl
         for (int a = 1; a < 8; ++a) any |= mag(w[c][a]);
         T = imax(T, top_exponent(any, e[c]));
     }
-    // |w| < 2^58 after the shift: 4 w fits beside it, and the 7 terms of a corner below 2^61 each
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+    for (int c = 0; c < 3; ++c) {
+        w[c][0] = 0;
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+        for (int a = 1; a < 8; ++a) w[c][a] = T == kNoExponent ? 0 : shift(w[c][a], e[c] - T - 6);
+    }
+    return !bad;
+}
+
+// The 24 nodal forces of an element from the Walsh coefficients of its displacements (block_walsh): the
+// coefficients above, the inverse sums.  lam, mu: Lame parameters times the factor h / 16 (divided by the factor
+// that the displacements carry).  Returns false for operands outside the formats (or so small or large that the
+// result's exponent leaves the normal range): the caller then uses FP64.
+OSAM_HD double f64_scaled(i64 x, int scale);
+OSAM_HD bool force_le_walsh(const i64 w[3][8], int T, double lam, double mu, double F[3][8]) {
+    const int ek = factor_exponent(lam, mu);
     const bool zero = T == kNoExponent;
     const int scale = 2095 - T - ek;           // 1081 + 1084 - 64 - 6
-    if (bad || (!zero && (scale > 1000 || scale < -900))) return false;
-#ifdef __CUDACC__
-#pragma unroll
-#endif
-    for (int c = 0; c < 3; ++c)
-#ifdef __CUDACC__
-#pragma unroll
-#endif
-        for (int a = 1; a < 8; ++a) w[c][a] = zero ? 0 : shift(w[c][a], e[c] - T - 6);
+    if (ek == 2047 || (!zero && (scale > 1000 || scale < -900))) return false;
+    i64 f[3][8];
+    // |w| < 2^58: 4 w fits beside it, and the 7 terms of a corner below 2^61 each
     le_coefficients(w, factor_value(lam, ek), factor_value(mu, ek), f);
 #ifdef __CUDACC__
 #pragma unroll
@@ -751,6 +760,37 @@ OSAM_HD bool element_force_le(const double U[3][8], double lam, double mu, doubl
         for (int a = 0; a < 8; ++a) F[c][a] = f64_scaled(f[c][a], scale);
     }
     return true;
+}
+OSAM_HD bool element_force_le(const double U[3][8], double lam, double mu, double F[3][8]) {
+    i64 w[3][8];
+    int T;
+    return block_walsh(U, w, T) && force_le_walsh(w, T, lam, mu, F);
+}
+
+// y . dK/dlam u and y . dK/dmu u of an element in units of h / 16, from the Walsh coefficients of u and y: with
+// K's coefficients above, sums of products that are symmetric in u and y,
+//   lam: tr tr' + sum_j S_j S_j' / 3 + sum_c w_xyz^c w_xyz^c' / 9,   S_j = w_ij^i + w_jk^k,
+//   mu:  2 sum w_i^i w_i^i' + sum_(i<c) (w_i^c + w_c^i)(w_i^c + w_c^i)'
+//        + sum [3 w_ij^i w_ij^i' + 3 w_ij^j w_ij^j' + (2 w_ij^k + w_jk^i + w_ik^j) w_ij^k'] / 3 + 4 sum w_xyz^c w_xyz^c' / 9.
+// Operands are raised by 2 bits each (below 2^62), so a product is a b 2^4 / 2^64 and every sum below 2^63.
+OSAM_HD void contract_le(const i64 u[3][8], const i64 y[3][8], i64& dl, i64& dm) {
+    const auto dot = [](i64 a, i64 b) { return mul(split(shl(a, 2)), split(shl(b, 2))); };
+    i64 l1 = dot(u[0][1] + u[1][2] + u[2][4], y[0][1] + y[1][2] + y[2][4]), l2 = 0, l3 = 0, m1 = 0, m2 = 0;
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+    for (int i = 0; i < 3; ++i) {
+        const int j = (i + 1) % 3, k = (i + 2) % 3;
+        const int I = 1 << i, J = 1 << j, K = 1 << k;
+        l2 += dot(u[i][I | J] + u[k][J | K], y[i][I | J] + y[k][J | K]);
+        l3 += dot(u[i][7], y[i][7]);
+        m1 += 2 * dot(u[i][I], y[i][I]) + dot(u[i][J] + u[j][I], y[i][J] + y[j][I]);
+        m2 += dot(3 * u[i][I | J], y[i][I | J]) + dot(3 * u[j][I | J], y[j][I | J]);
+        m2 += dot(2 * u[k][I | J] + u[i][J | K] + u[j][I | K], y[k][I | J]);
+    }
+    const i64 n = mul_third(mul_third(l3));
+    dl = l1 + mul_third(l2) + n;
+    dm = m1 + mul_third(m2) + 4 * n;
 }
 
 // x / 2^scale as an FP64 value, rounded to nearest (integer operations; |x| < 2^63)

@@ -32,16 +32,31 @@ __device__ __forceinline__ double block_sum1(double x) {
     __syncthreads();
     if (l == 0) sx[w] = x;
     __syncthreads();
-    double a = 0.0;
-    if (threadIdx.x == 0)
-        for (int i = 0; i < (int)((blockDim.x + 31) / 32); ++i) a += sx[i];
-    return a;
+    static_assert(kNodeBlock == 128, "four warps");
+    return threadIdx.x == 0 ? (sx[0] + sx[1]) + (sx[2] + sx[3]) : 0.0;
 }
 
 // Partial sums of a node kernel: one per block, in the plane of its component (blockIdx.y, with one component
 // per thread) of [2 quantities][3][n_nblk]; every plane of a launch is summed in a fixed order.
 __device__ __forceinline__ double* ipart(const FomB& g, int quantity, int plane) {
     return g.ipart + (long long)(3 * quantity + plane) * g.n_nblk;
+}
+
+// A thread's share of an instance's block partials of one quantity, in a fixed order with four loads in flight
+// (one after the other they took half of the reduction's time)
+__device__ __forceinline__ double partial_share(const FomB& g, int quantity, int b0, int nb, int planes) {
+    const int total = nb * planes;
+    double s = 0.0;
+    for (int t = (int)threadIdx.x; t < total; t += 4 * kNodeBlock) {
+        double v[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int i = t + q * kNodeBlock;
+            v[q] = i < total ? __ldcg(ipart(g, quantity, i / nb) + b0 + i % nb) : 0.0;
+        }
+        s += (v[0] + v[1]) + (v[2] + v[3]);
+    }
+    return s;
 }
 
 struct NodeCtx {
@@ -132,15 +147,9 @@ __global__ void k_imp_reduce_b(const FomB g, const int* __restrict__ mask, int m
     const int inst = blockIdx.x;
     if (!run(mask, inst)) return;
     if (first < 0) first = g.iloop[0] == 0;  // device-side Newton loop: its counter says which step this is
-    const int b0 = g.nblk_off[inst], b1 = g.nblk_off[inst + 1];
-    double s = 0.0, sz = 0.0;
-    for (int y = 0; y < planes; ++y)
-        for (int b = b0 + (int)threadIdx.x; b < b1; b += blockDim.x) {
-            s += ipart(g, 0, y)[b];
-            sz += ipart(g, 1, y)[b];
-        }
-    s = block_sum1(s);
-    sz = block_sum1(sz);
+    const int b0 = g.nblk_off[inst], nb = g.nblk_off[inst + 1] - b0;
+    const double s = block_sum1(partial_share(g, 0, b0, nb, planes));
+    const double sz = block_sum1(partial_share(g, 1, b0, nb, planes));
     if (threadIdx.x != 0) return;
     if (mode == 0) {
         if (first) g.r0[inst] = s;
@@ -180,11 +189,8 @@ __device__ __forceinline__ bool last_block_sum(const FomB& g, int inst, double& 
     __syncthreads();
     if (!last) return false;
     __threadfence();
-    const int b0 = g.nblk_off[inst], b1 = g.nblk_off[inst + 1];
-    double s = 0.0;
-    for (int y = 0; y < (int)gridDim.y; ++y)
-        for (int b = b0 + (int)threadIdx.x; b < b1; b += blockDim.x) s += __ldcg(ipart(g, 0, y) + b);
-    s = block_sum1(s);
+    const int b0 = g.nblk_off[inst];
+    const double s = block_sum1(partial_share(g, 0, b0, g.nblk_off[inst + 1] - b0, (int)gridDim.y));
     if (threadIdx.x != 0) return false;
     g.iticket[inst] = 0u;
     total = s;
@@ -410,7 +416,7 @@ cudaError_t launch_imp_residual_b(const FomB& g, const int* mask, double c0, cud
     return cudaGetLastError();
 }
 cudaError_t launch_imp_reduce_b(const FomB& g, const int* mask, int mode, int first, double tol2, cudaStream_t s) {
-    k_imp_reduce_b<<<g.n_inst, 128, 0, s>>>(g, mask, mode, first, tol2, node_split(g) ? 3 : 1);
+    k_imp_reduce_b<<<g.n_inst, kNodeBlock, 0, s>>>(g, mask, mode, first, tol2, node_split(g) ? 3 : 1);
     return cudaGetLastError();
 }
 cudaError_t launch_cg_ap_b(const FomB& g, const int* mask, double c0, cudaStream_t s) {

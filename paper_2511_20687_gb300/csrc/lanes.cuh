@@ -96,9 +96,9 @@ __device__ __forceinline__ void deformation(const Lane& L, const i64 U[3], Cols&
     }
 }
 
-// A direction in block format: its scaled gradient columns, gradient = G 2^-base / h; returns the base
-__device__ __forceinline__ int direction(const Lane& L, const double p[3], Cols& G, bool& bad) {
-    i64 w[3];
+// Walsh coefficients of a direction in block format (the lane's pattern, |w| < 2^58); returns the exponent T:
+// coefficient = w 2^(T + 6 - 1081), kNoExponent for a direction without differences (w is then 0)
+__device__ __forceinline__ int block_walsh(const Lane& L, const double p[3], i64 w[3], bool& bad) {
     int e[3], T = kNoExponent;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
@@ -109,10 +109,67 @@ __device__ __forceinline__ int direction(const Lane& L, const double p[3], Cols&
         bad |= e[c] == 2047 || (e[c] == 0 && shl(__double_as_longlong(p[c]), 1) != 0);   // not finite, subnormal
     }
     T = reduce8(T, [](int a, int b) { return max(a, b); });
-    const bool zero = T == kNoExponent;
 #pragma unroll
-    for (int c = 0; c < 3; ++c) gauss_columns(L, pattern_scale(L, zero ? 0 : shift(w[c], e[c] - T - 6)), c, G);
-    return zero ? 0 : 1016 - T;                // 1081 - 59 - 6
+    for (int c = 0; c < 3; ++c) w[c] = T == kNoExponent ? 0 : shift(w[c], e[c] - T - 6);
+    return T;
+}
+
+// A direction in block format: its scaled gradient columns, gradient = G 2^-base / h; returns the base
+__device__ __forceinline__ int direction(const Lane& L, const double p[3], Cols& G, bool& bad) {
+    i64 w[3];
+    const int T = block_walsh(L, p, w, bad);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) gauss_columns(L, pattern_scale(L, w[c]), c, G);
+    return T == kNoExponent ? 0 : 1016 - T;    // 1081 - 59 - 6
+}
+
+// Linear elastic force of the lane's corner from its displacement (element_force_le on 8 lanes): F 2^-scale.  lam, mu times h / 16 as in element_force_le.
+// A pattern's coefficients need those of the two patterns that differ from it in two axes: {j} and {k} for {i},
+// {j, k} and {i, k} for {i, j}.
+__device__ __forceinline__ bool force_le_lanes(const Lane& L, const double p[3], double lam, double mu, i64 F[3], int& scale) {
+    bool bad = false;
+    i64 w[3], A[3], B[3];
+    const int T = block_walsh(L, p, w, bad), ek = factor_exponent(lam, mu);
+    const int order = __popc((unsigned int)L.a), lane = (int)(threadIdx.x & 31u);
+    // order 1: i the pattern's axis; order 2: k the missing axis, i and j the others
+    const int i = order == 1 ? __ffs(L.a) - 1 : (__ffs(~L.a & 7) % 3), j = (i + 1) % 3, k = (i + 2) % 3;
+    const int flip1 = order == 1 ? (1 << i) | (1 << j) : (1 << i) | (1 << k);   // to {j}; to {j, k}
+    const int flip2 = order == 1 ? (1 << i) | (1 << k) : (1 << j) | (1 << k);   // to {k}; to {i, k}
+    i64 u[3], v[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        u[c] = __shfl_sync(0xffffffffu, w[c], lane ^ flip1);
+        v[c] = __shfl_sync(0xffffffffu, w[c], lane ^ flip2);
+    }
+    const auto at = [](const i64 x[3], int c) { return c == 0 ? x[0] : (c == 1 ? x[1] : x[2]); };
+    const i64 wi = at(w, i), wj = at(w, j), wk = at(w, k);
+    i64 ai, aj, ak, bi, bj, bk;
+    if (order == 1) {
+        ai = wi + at(u, j) + at(v, k); aj = ak = 0;
+        bi = 2 * wi; bj = wj + at(u, i); bk = wk + at(v, i);
+    } else if (order == 2) {
+        ai = wi + at(u, k); aj = wj + at(v, k); ak = 0;
+        bi = 3 * wi; bj = 3 * wj; bk = 2 * wk + at(u, i) + at(v, j);
+    } else {
+        ai = wi; aj = wj; ak = wk;
+        bi = 4 * wi; bj = 4 * wj; bk = 4 * wk;
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        A[c] = c == i ? ai : (c == j ? aj : ak);
+        B[c] = c == i ? bi : (c == j ? bj : bk);
+    }
+    const D l = split(factor_value(lam, ek)), m = split(factor_value(mu, ek));
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        i64 f = mul_add(l, split(A[c]), mul(m, split(B[c])));
+        const i64 t = mul_third(f);
+        f = order == 1 ? f : (order == 2 ? t : mul_third(t));
+        F[c] = corner_values(L, L.a ? f : 0);
+    }
+    const bool zero = T == kNoExponent;
+    scale = zero ? 0 : 2095 - T - ek;
+    return !any_lane(bad || ek == 2047 || scale > 1000 || scale < -900);
 }
 
 // Material factors kappa/2 and mu times w as integers: value = X 2^(k - 62), the larger in [2^61, 2^62);

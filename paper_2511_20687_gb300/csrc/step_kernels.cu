@@ -318,8 +318,8 @@ __global__ void __launch_bounds__(kNodeBlock) k_node_b(const FomB g, const int* 
     const double* h2 = slot2 >= 0 ? g.hist + I.hist_off + (long long)slot2 * 9 * I.ns : nullptr;
     const TF* fe = static_cast<const TF*>(g.fe) + I.elem_off;
     TF* fa = static_cast<TF*>(g.f);
-    // all loads of a free node first (state and the element contributions of the three components,
-    // summed per component in the fixed corner order), so that they are in flight together
+    // all loads of a free node first (state and the element contributions, summed in a fixed order), so that
+    // they are in flight together
     double uc[NC], vc[NC], ac[NC], f[NC] = {};
     TF fs[NC] = {};   // the gather sums in the element buffer's precision
 #pragma unroll
@@ -331,25 +331,18 @@ __global__ void __launch_bounds__(kNodeBlock) k_node_b(const FomB g, const int* 
     }
     if (!predict_only && row < 0 && cm != 7) {
         if (MODE == kGather) {
+            TF x[NC][8];
 #pragma unroll
-            for (int az = 0; az < 2; ++az) {
-                const int ke = k - az;
-                if (ke < 0 || ke >= I.nz) continue;
+            for (int corner = 0; corner < 8; ++corner) {
+                const int ie = i - (corner & 1), je = j - ((corner >> 1) & 1), ke = k - (corner >> 2);
+                const bool in = ke >= 0 && ke < I.nz && je >= 0 && je < I.ny && ie >= 0 && ie < I.nx;
+                const long long e = ie + (long long)I.nx * (je + I.ny * ke);
 #pragma unroll
-                for (int ay = 0; ay < 2; ++ay) {
-                    const int je = j - ay;
-                    if (je < 0 || je >= I.ny) continue;
-#pragma unroll
-                    for (int ax = 0; ax < 2; ++ax) {
-                        const int ie = i - ax;
-                        if (ie < 0 || ie >= I.nx) continue;
-                        const long long e = ie + (long long)I.nx * (je + I.ny * ke);
-                        const int corner = ax + 2 * ay + 4 * az;
-#pragma unroll
-                        for (int q = 0; q < NC; ++q) fs[q] += __ldg(fe + (long long)(corner * 3 + c0 + q) * g.NE + e);
-                    }
-                }
+                for (int q = 0; q < NC; ++q) x[q][corner] = in ? __ldg(fe + (long long)(corner * 3 + c0 + q) * g.NE + e) : TF(0);
             }
+#pragma unroll
+            for (int q = 0; q < NC; ++q)   // three additions in a row instead of eight
+                fs[q] = ((x[q][0] + x[q][1]) + (x[q][2] + x[q][3])) + ((x[q][4] + x[q][5]) + (x[q][6] + x[q][7]));
             // FP64: the same sums; FP32 force: summed in FP32 (its own precision) and widened once, by
             // integer operations (f64_of: exact)
 #pragma unroll
