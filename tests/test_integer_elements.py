@@ -126,6 +126,28 @@ def test_element_calls_match_torch(dims, material, shift):
 
 @pytest.mark.gpu
 @pytest.mark.parametrize("material", ["nh", "le"])
+@pytest.mark.parametrize("dims", [(16, 32, 32), (17, 31, 33), (64, 32, 32), (33, 65, 31)])   # sides of the size rules
+def test_large_meshes_match_torch(dims, material):
+    import torch
+
+    from paper_2511_20687_gb300 import osam
+    g = torch.Generator(device="cuda").manual_seed(9)
+    nn = (dims[0] + 1) * (dims[1] + 1) * (dims[2] + 1)
+    ne = dims[0] * dims[1] * dims[2]
+    rand = lambda *s: torch.rand(*s, generator=g, device="cuda", dtype=torch.float64)  # noqa: E731
+    u = H * 0.02 * (rand(nn, 3) - 0.5)
+    u[: nn // 50] += 30 * H          # some elements beyond the fixed-point range, some torn across it
+    lam, mu = 4e8 * (1 + 0.2 * rand(ne)), 4e8 * (1 + 0.2 * rand(ne))
+    f = torch.empty_like(u)
+    osam.hex8_force(dims, H, material, 0.0, 0.0, u, f, lam_e=lam, mu_e=mu)
+    r = reference(torch, dims, H, material, lam, mu, u)
+    near = torch.isfinite(r).all(1)   # the torn layer may be inverted: the law is undefined there
+    near[nn // 50 - 2 * (dims[0] + 1) * (dims[1] + 1): nn // 50 + 2 * (dims[0] + 1) * (dims[1] + 1)] = False
+    assert (f - r)[near].norm() <= 1e-12 * (1 + 100 * 30) * r[near].norm()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("material", ["nh", "le"])
 @pytest.mark.parametrize("bad", [float("nan"), float("inf")])
 def test_non_finite_displacement_spreads_to_its_elements(material, bad):
     import torch
