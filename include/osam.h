@@ -60,7 +60,8 @@ enum { OSAM_MULTIPLICATIVE = 0, OSAM_ADDITIVE = 1 };
  * in native FP64).  OSAM_FP32_FORCE: internal force in FP32 (checked to 1e-5).
  * OSAM_F32X2_FORCE: internal force in double-float arithmetic (pairs of FP32 values, ~48-bit
  * significands) on the FP32 pipes, state and time integration in FP64 (checked to 1e-9 like FP64);
- * uses the deterministic gather scatter.  OSAM_FP64_TANGENT32: OSAM_FP64, except that the Newton
+ * uses the deterministic gather scatter; Neo-Hookean subdomains with OSAM_SCATTER_AUTO take the
+ * fixed-point force of OSAM_FP64, which is more accurate and faster.  OSAM_FP64_TANGENT32: OSAM_FP64, except that the Newton
  * tangent of implicit Neo-Hookean subdomains (its stored Gauss-point linearisation, its action on
  * the conjugate-gradient direction and the element contributions of that action) is in FP32; the
  * Newton residual and its test, the CG vectors and reductions stay FP64, so a converged step meets the
