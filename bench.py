@@ -55,6 +55,13 @@ FP64_NOMINAL_TFLOPS = 1.25
 # x 32 / elements of the phased kernel) and the FP32 issue peak (152 SMs x 128 lanes x 2.07 GHz)
 F32X2_INST_PER_NH_ELEMENT = 12012
 FP32_ISSUE_PEAK_TINST = 152 * 128 * 2.07e9 / 1e12
+# fixed-point force (the FP64 and double-float modes with the scatter left to the library): 32 x 32 + 64-bit integer
+# multiply-add pipe instructions per Neo-Hookean element (ncu, k_force_fx_b) and their issue peak: one per 4 cycles
+# and scheduler (measured), 152 SMs x 4 schedulers x 32 lanes x 2.07 GHz / 4
+INT_MAD_PER_NH_ELEMENT = 1969
+INT_MAD_PEAK_TINST = 152 * 4 * 32 * 2.07e9 / 4 / 1e12
+# bf16 digit products per FP64 product of the fit (split_gemm.cu)
+SPLIT_PRODUCTS = 28
 # DRAM traffic of one force launch of the bench workload (ncu dram__bytes_read.sum + write.sum),
 # valid only for the kernel source and variant (tiled or not) it was captured on.
 FORCE_TRAFFIC = {"source_sha256": "5329782da603ec0d213b49ef60d6836089a9f41f0ba6bc0fa18cff46cede7c3d",
@@ -143,6 +150,15 @@ def measured_hbm_gbs():
             return float(json.load(fh)["hbm_gbs"]), "measured (MEASURED_PEAKS.json hbm_gbs)"
     except (OSError, ValueError, KeyError):
         return 6800.0, "fallback (6.8 TB/s)"
+
+
+def measured_bf16_tflops():
+    """cuBLAS bf16 burst rate in TFLOP/s: the measured figure, else the fallback."""
+    try:
+        with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as fh:
+            return float(json.load(fh)["bf16_tflops"])
+    except (OSError, ValueError, KeyError):
+        return 1900.0
 
 
 def parse():
@@ -247,6 +263,18 @@ class ClockSampler:
             out = {"sm_mhz": statistics.median(sm), "sm_max_mhz": max(mx), "reasons": sorted(reasons),
                    "samples": len(sm)}
         return out
+
+
+def fixed_point_roofline(prof):
+    """Integer multiply-add issue rate of the fixed-point force launches."""
+    achieved = INT_MAD_PER_NH_ELEMENT * prof["force_elements"] / (prof["force_ms"] * 1e-3) / 1e12
+    return {"bound": "alu", "kernel": "k_force_fx_b (Neo-Hookean, 64-bit fixed point)", "achieved": achieved,
+            "peak": INT_MAD_PEAK_TINST, "unit": "Tinst/s (integer multiply-add pipe)",
+            "frac": achieved / INT_MAD_PEAK_TINST,
+            "peak_kind": "152 SMs x 4 schedulers x 32 lanes x 2.07 GHz / 4 cycles (measured issue interval)",
+            "fp64_equivalent_tflops": FLOPS_PER_NH_ELEMENT * prof["force_elements"] / (prof["force_ms"] * 1e-3) / 1e12,
+            "elements_per_launch": prof["force_elements"] // max(1, prof["force_launches"]),
+            "force_ms_per_launch": prof["force_ms"] / max(1, prof["force_launches"])}
 
 
 def source_sha(files=("step_kernels.cu", "hex8_math.cuh", "trace_item.cuh", "fp_bits.cuh")):
@@ -409,7 +437,6 @@ def measure_batched(W, osam, torch, flush, args, device, log, rank=0, world=1):
     bprof = batch.profile_read()
     batch.profile(False)
     batch.close()
-    bach_force = FLOPS_PER_NH_ELEMENT * bprof["force_elements"] / (bprof["force_ms"] * 1e-3) / 1e12
     # the same samples with the tiled force kernel forced (the autotuner's choice is timed against it)
     tb = osam.Batch(specs, rom_ops=ops, device=device, scatter=osam.SCATTER_GATHER_TILED)
     tb.step()
@@ -460,16 +487,10 @@ def measure_batched(W, osam, torch, flush, args, device, log, rank=0, world=1):
            "tuning": tuning, "timing": "host wall clock around each synchronous step call (value) and the "
                                        "library's CUDA events (value_device); L2 flushed between steps; "
                                        "under torchrun a barrier on both sides and the maximum over ranks",
-           "roofline": {"bound": "alu", "kernel": "batched internal force (Neo-Hookean, %s)" %
-                        ("tiled" if tuning.get("tiled") else "%d-thread blocks" % tuning["element_block"]),
-                        "achieved": bach_force, "peak": FP64_PEAK[0], "unit": "TFLOP/s",
-                        "frac": bach_force / FP64_PEAK[0], "flops_per_element": FLOPS_PER_NH_ELEMENT,
-                        "force_ms_per_launch": bprof["force_ms"] / max(1, bprof["force_launches"]),
-                        "elements_per_launch": bprof["force_elements"] // max(1, bprof["force_launches"]),
+           "roofline": {**fixed_point_roofline(bprof),
                         "force_launches_per_step": bprof["force_launches"],
                         "force_time_share": bprof["force_ms"] / prof_tot["elapsed_ms"],
-                        "kernel_launches_per_step": bprof["kernel_launches"],
-                        "peak_kind": FP64_PEAK_KIND[0]},
+                        "kernel_launches_per_step": bprof["kernel_launches"]},
            "tiled_forced": {"value_device": t_upd_all / (t_dev * 1e-3), "steps": 2,
                             "note": "the same samples with the 8x4x4-tile force kernel forced (n x n x 2n "
                                     "meshes, n in 8..32, leave partial tiles on most instances)"}}
@@ -530,9 +551,10 @@ def fit_gemm_roofline(U, A, S, r, rs, log, device=0):
     torch.cuda.empty_cache()
     return {"device_input_seconds": plain_s, "gemm_ms": prof["gemm_ms"], "gemm_flops": prof["gemm_flops"],
             "gemm_launches": prof["gemm_launches"], "gemm_share_of_fit": prof["gemm_ms"] * 1e-3 / plain_s,
-            "roofline": {"bound": "alu", "kernel": "k_gemm_mma (+ k_gemm_reduce), FP64 tensor-core mma.sync m8n8k4", "achieved": achieved,
-                         "peak": FP64_PEAK[0], "unit": "TFLOP/s", "frac": achieved / FP64_PEAK[0],
-                         "peak_kind": FP64_PEAK_KIND[0],
+            "roofline": {"bound": "alu", "kernel": "k_split_gemm (exact splitting, bf16 mma.sync m16n8k16)",
+                         "achieved": SPLIT_PRODUCTS * achieved, "peak": measured_bf16_tflops(), "unit": "TFLOP/s (bf16)",
+                         "frac": SPLIT_PRODUCTS * achieved / measured_bf16_tflops(), "fp64_equivalent_tflops": achieved,
+                         "peak_kind": "measured cuBLAS bf16 burst, or the fallback of one earlier measurement",
                          "timing": "library CUDA events around every GEMM of one device-input fit "
                                    "(osam_fit_profile)"}}
 
@@ -722,12 +744,15 @@ def measure_implicit(W, osam, torch, flush, rom_ops, args, local, log, steps=2, 
             "cg_per_newton": ip["cg_iterations"] / max(1, ip["newton_steps"]),
             "ms_per_step_host_loop": p_ms / steps,
             "tangent_time_share": ip["tangent_ms"] / p_ms if p_ms else None,
-            "roofline": {"bound": "alu", "kernel": "k_tangent_lin_b (Neo-Hookean)", "achieved": achieved,
-                         "peak": FP64_PEAK[0], "unit": "TFLOP/s", "frac": achieved / FP64_PEAK[0],
+            "roofline": {"bound": "hbm", "kernel": "k_fom_lanes<tangent> (Neo-Hookean, 64-bit integers)",
+                         "achieved": ne * TANGENT_BYTES_PER_ELEMENT / 1e6 / max(1e-9, ip["tangent_ms"] / max(1, ip["tangent_launches"])),
+                         "peak": measured_hbm_gbs()[0], "unit": "GB/s",
+                         "frac": (ne * TANGENT_BYTES_PER_ELEMENT / 1e6 / max(1e-9, ip["tangent_ms"] / max(1, ip["tangent_launches"]))
+                                  / measured_hbm_gbs()[0] if measured_hbm_gbs()[0] else None),
                          "traffic": (TANGENT_TRAFFIC["bytes_per_launch"]
                                      if TANGENT_TRAFFIC["source_sha256"] == source_sha(TANGENT_SOURCES) else None),
                          "algorithmic_bytes_per_launch": ne * TANGENT_BYTES_PER_ELEMENT,
-                         "flops_per_element": TANGENT_FLOPS_PER_NH_ELEMENT,
+                         "fp64_equivalent_tflops": achieved,
                          "ms_per_launch": ip["tangent_ms"] / max(1, ip["tangent_launches"]),
                          "peak_kind": FP64_PEAK_KIND[0]},
             "timing": "value: library CUDA events around each controller step, each one graph launch with the "
@@ -941,19 +966,19 @@ def measure_large(W, osam, torch, flush, args, local, log, warmup=3):
             max_its = int(max(its))
         per_launch = prof["force_ms"] / max(1, prof["force_launches"])
         achieved = FLOPS_PER_NH_ELEMENT * prof["force_elements"] / (prof["force_ms"] * 1e-3) / 1e12
-        peak = FP64_PEAK[0] if name == "f64" else FP32_FMA_PEAK_TFLOPS
+        peak = FP32_FMA_PEAK_TFLOPS
         out[name] = {"value": upd / (ms * 1e-3), "ms_per_step": ms / args.large_steps, "steps": args.large_steps,
                      "warmup": warmup, "mean_iterations": float(np.mean(its)), "max_iterations": int(max(its)),
                      "effective_rate": upd / (ms * 1e-3) / float(np.mean(its)),
                      "value_host_loop": p_upd / (p_ms * 1e-3), "tuning": tuning,
-                     "roofline": {"bound": "alu", "kernel": "internal force (Neo-Hookean, %s)" % name,
+                     "roofline": {**fixed_point_roofline(prof), "force_time_share": prof["force_ms"] / p_ms}
+                     if name == "f64" else
+                     {"bound": "alu", "kernel": "internal force (Neo-Hookean, %s)" % name,
                                   "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
                                   "flops_per_element": FLOPS_PER_NH_ELEMENT, "elements_per_launch":
                                   spec.subdomains[0].n_elements, "force_ms_per_launch": per_launch,
                                   "force_time_share": prof["force_ms"] / p_ms,
-                                  "peak_kind": (FP64_PEAK_KIND[0] if name == "f64"
-                                                else "FP32 FMA: 152 SMs x 128 lanes x 2 flops x 2.07 GHz"),
-                                  "frac_of_nominal": (achieved / FP64_NOMINAL_TFLOPS if name == "f64" else None)}}
+                                  "peak_kind": "FP32 FMA: 152 SMs x 128 lanes x 2 flops x 2.07 GHz"}}
         if name == "fp32_force":
             out[name]["iterations"] = f"fixed at {max_its} (the largest FP64 count)"
         log(f"large chain [{name}]: {out[name]['value']:.3e} element-updates/s, {ms / args.large_steps:.1f} ms/step, "
@@ -1325,6 +1350,9 @@ def main():
     def roofline(res, prec_name):
         prof = res["prof"]
         per_launch = prof["force_ms"] / max(1, prof["force_launches"])
+        if args.scatter == "auto":   # both modes' explicit Neo-Hookean force
+            return {**fixed_point_roofline(prof), "traffic": None,
+                    "force_time_share": prof["force_ms"] / res["prof_total_ms"]}
         if prec_name == "f64":
             achieved = FLOPS_PER_NH_ELEMENT * prof["force_elements"] / (prof["force_ms"] * 1e-3) / 1e12
             same = (FORCE_TRAFFIC["source_sha256"] == source_sha()
@@ -1401,7 +1429,7 @@ def main():
             hbm[name] = {"achieved_gbs": gbs, "frac": gbs / hbm_peak if hbm_peak else None}
         hbm = {"algorithmic_bytes_per_element_update": bytes_per_update, "peak_gbs": hbm_peak,
                "peak_kind": hbm_kind, **hbm,
-               "note": "the path is bound by the FP64 (or FP32-issue) pipes, not by HBM"}
+               "note": "the path is bound by the integer multiply-add pipe, not by HBM"}
         mean_it = float(np.mean(head["iters"]))
         line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
                 "warmup": args.warmup, "ms_per_step": head["total_ms"] / args.steps, "higher_is_better": True,

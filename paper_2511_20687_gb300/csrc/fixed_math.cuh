@@ -568,6 +568,56 @@ OSAM_HD bool tangent_point(const Cols& C, const Cols& E, D kap2, D mu, D mu3, i6
     return ok && top < kOne25;
 }
 
+// dP[G] of a Gauss point from its stored linearisation, dalpha = a1 dJ and dbeta = b1 dJ + a1 (F : G): a third of
+// tangent_point's instructions.  q in the units of stress_point (a1, b1 with 60 and 57 fraction bits); G, dP and
+// the checks as in tangent_point.
+OSAM_HD bool tangent_stored(const Linear& q, const Cols& E, i64 dP[3][3]) {
+    D F[3][3], N[3][3], G[3][3], c[3][3];
+    i64 dJ = 0, FG = 0;
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+    for (int k = 0; k < 3; ++k) {
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+        for (int a = 0; a < 3; ++a) {
+            F[k][a] = split(q.F[k][a]);
+            N[k][a] = split(-q.F[k][a]);
+            G[k][a] = split(E.x[k][a]);
+            c[k][a] = split(q.cof[k][a]);
+        }
+        dJ += dot3(c[k][0], G[k][0], c[k][1], G[k][1], c[k][2], G[k][2]);      // 58, below 3.6
+        FG += dot3(F[k][0], G[k][0], F[k][1], G[k][1], F[k][2], G[k][2]);      // 58, below 2.4
+    }
+    bool ok = (hi(dJ) ^ (hi(dJ) >> 31)) < (1 << 26);
+    const D dJd = split(shl(dJ, 4)), a1 = split(shl(q.a1, 1));                 // 62, 61 (below 2)
+    const D dad = split(mul(a1, dJd));                                         // 59
+    // |b1| < 8 with 59 fraction bits; dbeta below 8
+    ok = ok && (hi(q.b1) ^ (hi(q.b1) >> 31)) < (8 << 25);
+    const i64 dbeta = dot2(split(shl(q.b1, 2)), dJd, a1, split(shl(FG, 2)));   // 57
+    ok = ok && (hi(dbeta) ^ (hi(dbeta) >> 31)) < (8 << 25);
+    const D db = split(shl(dbeta, 2)), be = split(shl(q.beta, 2)), ah = split((q.alpha + 1) >> 1);   // 59
+    int top = 0;
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+    for (int x = 0; x < 3; ++x) {
+        const int y = (x + 1) % 3, z = (x + 2) % 3;
+        const i64 d0 = dot4(G[1][y], F[2][z], G[1][z], N[2][y], F[1][y], G[2][z], N[1][z], G[2][y]);   // 58, below 1.7
+        const i64 d1 = dot4(G[2][y], F[0][z], G[2][z], N[0][y], F[2][y], G[0][z], N[2][z], G[0][y]);
+        const i64 d2 = dot4(G[0][y], F[1][z], G[0][z], N[1][y], F[0][y], G[1][z], N[0][z], G[1][y]);
+        dP[0][x] = dot4(db, c[0][x], be, split(shl(d0, 3)), dad, F[0][x], ah, G[0][x]);                // 56
+        dP[1][x] = dot4(db, c[1][x], be, split(shl(d1, 3)), dad, F[1][x], ah, G[1][x]);
+        dP[2][x] = dot4(db, c[2][x], be, split(shl(d2, 3)), dad, F[2][x], ah, G[2][x]);
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+        for (int k = 0; k < 3; ++k) top |= hi(dP[k][x]) ^ (hi(dP[k][x]) >> 31);
+    }
+    return ok && top < kOne25;
+}
+
 // ---- operands with a block exponent --------------------------------------------------------------
 // The 8 nodal values of one component of an element's direction (or linear displacement) share one
 // exponent e: value = V 2^(e - 1081), |V| < 2^59, exact for values within 2^-6 of the largest, else rounded at

@@ -82,7 +82,7 @@ __device__ __noinline__ void far_tangent(const FarIn& x, double F[3][8], double&
     walsh_transpose<double>(Sx, Sy, Sz, F);
 }
 
-// The Newton linearisation of the FP32 tangent (k_tangent_lin32_b): F, cof F, alpha, beta and the coefficients of
+// The Newton linearisation of the tangent: F, cof F, alpha, beta and the coefficients of
 // dalpha = a1 dJ and dbeta = b1 dJ + a1 (F : G), dJ = cof : G, per Gauss point; layout [kLinPerGp][8 Gauss points][NE],
 // Gauss point 4 x + 2 y + z:
 //   a1 = -2/3 alpha / J,  b1 = 2 kappa/2 - (a1 trC / 3 + beta) / J   (from P = alpha F + beta cof,
@@ -260,9 +260,11 @@ __global__ void __launch_bounds__(kLaneBlock, kTangentBlocks) k_elem_vjp(const _
 }
 
 // ---- implicit groups (FomB): element buffer [24][NE] ----------------------------------------------
-// OP kOpTangent: K(u) p of the CG direction; else the internal force of u, with kOpLinearise also the Newton
-// linearisation of the FP32 tangent
-enum { kOpForce, kOpLinearise, kOpTangent };
+// OP kOpTangent: K(u) p of the CG direction from the stored linearisation; else the internal force of u, which
+// also stores it (in FP32 for k_tangent_lin32_b, or as integers).  The u-dependent part of the tangent does not
+// change over the CG iterations of a Newton step (12 of them on average): with it stored a tangent launch issues
+// 1000 instead of 2700 instructions per warp.
+enum { kOpStore32, kOpStore64, kOpTangent };
 template <int OP>
 __global__ void __launch_bounds__(kLaneBlock, OP == kOpTangent ? kTangentBlocks : kForceBlocks) k_fom_lanes(const __grid_constant__ FomB g, const int* __restrict__ mask) {
     constexpr bool TANGENT = OP == kOpTangent;
@@ -274,26 +276,39 @@ __global__ void __launch_bounds__(kLaneBlock, OP == kOpTangent ? kTangentBlocks 
     if (first >= I.ne) return;
     const Elem x = element(first + (int)(threadIdx.x >> 3), I.nx, I.ny, I.ne);
     const Lane L = make_lane();
-    const long long gn = I.node_off + corner_node(x, L.a);
-    i64 U[3], F[3], pk, pm;
-    double p[3];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        U[c] = fixed_u(g.u[0][c * g.NN + gn], I.ihm, I.ihe);
-        if (TANGENT) p[c] = g.cg_p[c * g.NN + gn];
-    }
+    const long long gn = I.node_off + corner_node(x, L.a), st = 8LL * g.NE;
     const double lam = I.lam_e ? I.lam_e[x.e] : I.lam, mu = I.mu_e ? I.mu_e[x.e] : I.mu;
+    // FP32: [22][8 Gauss points][NE] for the one-thread-per-element tangent; integers: [22][NE][8 lanes], 256
+    // consecutive bytes per warp
+    const long long entry = OP == kOpStore32 ? I.elem_off + x.e + (long long)lin_point(L.a) * g.NE : 8 * (I.elem_off + x.e) + L.a;
     Material M;
-    const bool bad = !material(lam, mu, TANGENT ? I.wqi : I.wq, M);
-    int scale = 57 - M.k, base;
+    const bool bad = !material(lam, mu, I.wq, M) || M.k < -900 || M.k > 900;
+    i64 F[3];
     Linear q;
-    Linear* lin = OP == kOpLinearise ? &q : nullptr;
-    const bool ok = TANGENT ? tangent_lanes(L, U, p, M, bad, false, F, scale, pk, pm, base)
-                            : force_lanes(L, U, M.kap2, M.mu, M.mu3, bad || M.k < -900 || M.k > 900, F, lin);
+    int scale;
+    bool ok;
+    if (TANGENT) {
+        const i64* lg = g.lin + entry;
+        double p[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            p[c] = g.cg_p[c * g.NN + gn];
+#pragma unroll
+            for (int d = 0; d < 3; ++d) { q.F[d][c] = __ldg(lg + (3 * c + d) * st); q.cof[d][c] = __ldg(lg + (9 + 3 * c + d) * st); }
+        }
+        q.alpha = __ldg(lg + 18 * st); q.beta = __ldg(lg + 19 * st);
+        q.a1 = __ldg(lg + 20 * st); q.b1 = __ldg(lg + 21 * st);
+        ok = tangent_stored_lanes(L, q, p, M.k + I.ihe + 1, bad || q.alpha == kBadF, F, scale);
+    } else {
+        i64 U[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) U[c] = fixed_u(g.u[0][c * g.NN + gn], I.ihm, I.ihe);
+        ok = force_lanes(L, U, M.kap2, M.mu, M.mu3, bad, F, &q);
+        scale = 57 - M.k;
+    }
     if (!x.live) return;
-    if (OP == kOpLinearise && ok) {
-        float* lg = g.linf + I.elem_off + x.e + (long long)lin_point(L.a) * g.NE;
-        const long long st = 8LL * g.NE;
+    if (OP == kOpStore32 && ok) {
+        float* lg = g.linf + entry;
 #pragma unroll
         for (int d = 0; d < 3; ++d)
 #pragma unroll
@@ -306,6 +321,22 @@ __global__ void __launch_bounds__(kLaneBlock, OP == kOpTangent ? kTangentBlocks 
         lg[20 * st] = f32_scaled(q.a1, 60 - M.k);
         lg[21 * st] = f32_scaled(q.b1, 57 - M.k);
     }
+    if (OP == kOpStore64) {
+        i64* lg = g.lin + entry;
+#pragma unroll
+        for (int d = 0; d < 3; ++d)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                lg[(3 * c + d) * st] = q.F[d][c];
+                lg[(9 + 3 * c + d) * st] = q.cof[d][c];
+            }
+        // the factors times 1/h: ihm 2^-63 of it here, the rest in the tangent's exponent
+        const D r = split(I.ihm);
+        lg[18 * st] = ok ? shl(mul(split(q.alpha), r), 1) : kBadF;
+        lg[19 * st] = shl(mul(split(q.beta), r), 1);
+        lg[20 * st] = shl(mul(split(q.a1), r), 1);
+        lg[21 * st] = shl(mul(split(q.b1), r), 1);
+    }
     double* fe = static_cast<double*>(g.fe) + I.elem_off + x.e;
     if (ok) {
 #pragma unroll
@@ -315,7 +346,7 @@ __global__ void __launch_bounds__(kLaneBlock, OP == kOpTangent ? kTangentBlocks 
                        I.invh, lam, mu, I.wq, I.wq3};
         double Ff[3][8], lb, mb;
         if (TANGENT) far_tangent(in, Ff, lb, mb);
-        else if (OP == kOpLinearise) far_linearise(in, g.linf + I.elem_off + x.e, g.NE, Ff);
+        else if (OP == kOpStore32) far_linearise(in, g.linf + I.elem_off + x.e, g.NE, Ff);
         else far_force(in, Ff);
         for (int c8 = 0; c8 < 8; ++c8)
             for (int c = 0; c < 3; ++c) fe[(long long)(c8 * 3 + c) * g.NE] = Ff[c][c8];
@@ -362,13 +393,14 @@ cudaError_t launch_elem_vjp_nh(int scatter, const ElemArgs& a, const double* yba
 cudaError_t launch_imp_force_nh_b(const FomB& g, const int* mask, cudaStream_t s) {
     if (g.eblock % 32) return cudaErrorInvalidValue;
     const int grid = g.n_eblk * (g.eblock * 8 / kLaneBlock);
-    if (g.linf) k_fom_lanes<kOpLinearise><<<grid, kLaneBlock, 0, s>>>(g, mask);
-    else k_fom_lanes<kOpForce><<<grid, kLaneBlock, 0, s>>>(g, mask);
+    if (g.linf) k_fom_lanes<kOpStore32><<<grid, kLaneBlock, 0, s>>>(g, mask);
+    else if (g.lin) k_fom_lanes<kOpStore64><<<grid, kLaneBlock, 0, s>>>(g, mask);
+    else return cudaErrorInvalidValue;
     return cudaGetLastError();
 }
 
 cudaError_t launch_imp_tangent_nh_b(const FomB& g, const int* mask, cudaStream_t s) {
-    if (g.eblock % 32) return cudaErrorInvalidValue;
+    if (g.eblock % 32 || !g.lin) return cudaErrorInvalidValue;
     k_fom_lanes<kOpTangent><<<g.n_eblk * (g.eblock * 8 / kLaneBlock), kLaneBlock, 0, s>>>(g, mask);
     return cudaGetLastError();
 }

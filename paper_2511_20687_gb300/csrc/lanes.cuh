@@ -207,6 +207,22 @@ __device__ __forceinline__ bool force_lanes(const Lane& L, const i64 U[3], D kap
     return !any_lane(bad);
 }
 
+// tangent action on a direction p (FP64) from the stored linearisation of the lane's Gauss point, whose factors
+// carry 1/h and units 2^k: value of the lane's corner = F 2^-scale
+__device__ __forceinline__ bool tangent_stored_lanes(const Lane& L, const Linear& q, const double p[3], int k, bool bad,
+                                                     i64 F[3], int& scale) {
+    Cols G;
+    i64 dP[3][3];
+    const int base = direction(L, p, G, bad);
+    bad |= !tangent_stored(q, G, dP);
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+        F[c] = corner_values(L, pattern_scale(L, gauss_transpose(L, dP[0][c], dP[1][c], dP[2][c])));
+    scale = 56 + base - k;
+    bad |= scale > 1000 || scale < -900;
+    return !any_lane(bad);
+}
+
 // tangent action on a direction p (FP64): value of the lane's corner = F 2^-scale; the sums over the Gauss points
 // of pk (60 fraction bits) and pm + 2/3 pk (56) with `base` more from the direction's own exponent
 __device__ __forceinline__ bool tangent_lanes(const Lane& L, const i64 U[3], const double p[3], const Material& M,

@@ -23,7 +23,7 @@ namespace osam {
 enum Scatter { kAtomic = 1, kGather = 2 };
 
 constexpr int kMaxSlots = 8;    // subdomains per instance
-constexpr int kLinPerGp = 22;   // floats per Gauss point of the stored Neo-Hookean Newton linearisation
+constexpr int kLinPerGp = 22;   // values per Gauss point of the stored Neo-Hookean Newton linearisation
 constexpr int kNodeBlock = 128; // nodes per block of the node kernels
 
 struct Grid {
@@ -126,7 +126,8 @@ struct FomB {
     int* nact;                // per instance Newton state: 1 iterating, 0 converged, 2 failed
     int* cgact;               // per instance: CG still iterating
     long long* istat;         // per instance: Newton linear solves, CG iterations (since the last reset)
-    float* linf;              // OSAM_FP64_TANGENT32, Neo-Hookean implicit groups: Newton linearisation [kLinPerGp][8][NE]
+    long long* lin;           // Neo-Hookean implicit groups: Newton linearisation [kLinPerGp][NE][8] (fixed_math.cuh)
+    float* linf;              // the same in FP32, [kLinPerGp][8][NE] (OSAM_FP64_TANGENT32; lin is then null)
     float* fe32;              // FP32 element buffer [24][NE] of the FP32 tangent action
     int df32;                 // 1: internal force in double-float arithmetic (element buffer of float2)
     int fixed;                // internal force in 64-bit integers: 1 Neo-Hookean (element buffer of int64; force_fx.cu),

@@ -249,6 +249,8 @@ int setup_fom_group(osam_ctx* ctx, FomGroupH& G, int s, int n, const osam_proble
         if (B.material == OSAM_NEO_HOOKEAN && ctx->precision == OSAM_FP64_TANGENT32) {
             CKA(B.linf = ctx->alloc<float>((long long)kLinPerGp * 8 * NE));
             CKA(B.fe32 = ctx->alloc<float>(24 * NE));
+        } else if (B.material == OSAM_NEO_HOOKEAN) {
+            CKA(B.lin = ctx->alloc<long long>((long long)kLinPerGp * 8 * NE));
         }
         CK(cudaMemsetAsync(B.istat, 0, sizeof(long long) * 2 * n, ctx->stream));
         CKA(B.nact = ctx->alloc<int>(n));

@@ -5,6 +5,7 @@
 // in units of h^2 times the largest difference of the direction.
 #include <cmath>
 #include <cstdio>
+#include <cstdlib>
 
 #include "fixed_math.cuh"
 
@@ -137,7 +138,15 @@ static bool tangent_fixed(const double u[3][8], const double x[3][8], double h, 
         i64 P[3][3], pk, pm;
         columns(wu, g, C);
         columns(wx, g, G);
-        ok = tangent_point(C, G, split(std::llrint(std::ldexp(m1, 62 - k))), split(m), split(mul_third(m)), P, pk, pm) && ok;
+        const D k2 = split(std::llrint(std::ldexp(m1, 62 - k))), m2d = split(m), m3 = split(mul_third(m));
+        ok = tangent_point(C, G, k2, m2d, m3, P, pk, pm) && ok;
+        // from the stored linearisation: dbeta is rounded at 2^-57 in four places, times cof below 2.25, against the
+        // unit 2^-56 of dP, and dP itself once more: 8 units
+        Linear lin;
+        i64 S[3][3], Q[3][3];
+        ok = stress_point(C, k2, m2d, m3, S, &lin) && tangent_stored(lin, G, Q) && ok;
+        for (int d = 0; d < 3; ++d)
+            for (int c = 0; c < 3; ++c) ok = ok && std::llabs(Q[d][c] - P[d][c]) <= 8;
         ks += pk;
         ms += pm;
         for (int b = 1; b < 8; ++b)
