@@ -11,13 +11,16 @@
 // Measured on 40x40x80: 43 us per launch, 186 us for the FP64 kernel; on 96x96x192 480 us, 2360 us.
 // The Gauss points are fully unrolled (43.4 us; with the two planes as a loop 45.3), 255 registers and
 // two warps per scheduler: capping at 168 or 128 registers (480 to 680 bytes of spills read back per thread)
-// measured 45.3 and 47.5 us on 40x40x80, 510 and 523 us on 96x96x192.
+// measured 45.3 and 47.5 us on 40x40x80, 510 and 523 us on 96x96x192; with the Walsh coefficients and one
+// plane's sums in shared memory (168 registers, three blocks per SM, no spills) the 96x96x192 chain step took 58.4
+// instead of 55.5 ms, so more warps do not help: the pipe is the bound.
 #include <cuda_runtime.h>
 
 #include <cstdint>
 
 #include "fixed_math.cuh"
 #include "hex8_math.cuh"
+#include "lanes.cuh"
 #include "osam_internal.h"
 #include "trace_item.cuh"
 
@@ -116,6 +119,51 @@ __global__ void __launch_bounds__(128) k_force_fx_b(const __grid_constant__ FomB
 #pragma unroll
         for (int c = 0; c < 3; ++c) fe[(long long)(c8 * 3 + c) * g.NE] = F[c][c8];
 }
+
+// the same with an element on 8 lanes (lanes.cuh); 8 thread blocks of g.eblock threads per element block
+__global__ void __launch_bounds__(128, 5) k_force_fx_lanes_b(const __grid_constant__ FomB g, const int* __restrict__ active,
+                                                          const __grid_constant__ TraceFuse tr, const double* u) {
+    if ((int)blockIdx.x >= 8 * g.n_eblk) {
+        trace::fused_trace_block(tr, active, g, (int)blockIdx.x - 8 * g.n_eblk);
+        return;
+    }
+    const int2 b = g.eblk[blockIdx.x >> 3];
+    if (active && !active[b.x]) return;
+    const InstFom& I = g.inst[b.x];
+    const int first = b.y + (int)((blockIdx.x & 7u) * (blockDim.x >> 3) + (threadIdx.x >> 3)), e = min(first, I.ne - 1);
+    const int nx = I.nx, ny = I.ny, i = e % nx, t = e / nx, j = t % ny, k = t / ny;
+    const int sy = nx + 1, sz = (nx + 1) * (ny + 1), n0 = i + sy * j + sz * k;
+    const Lane L = make_lane();
+    const long long gn = I.node_off + n0 + (L.a & 1) + ((L.a >> 1) & 1) * sy + (L.a >> 2) * sz;
+    i64 U[3], F[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) U[c] = g.ux[c * g.NN + gn];
+    D kap2 = split(I.fk2), mu = split(I.fmu), mu3 = split(mul_third(I.fmu));
+    bool bad = false;
+    if (I.lam_e || I.mu_e) {   // the element's factors in units of the instance's scale, which is at least theirs
+        Material M;
+        const int top = kFracOut - I.fscale;
+        bad = !material(I.lam_e ? I.lam_e[e] : I.lam, I.mu_e ? I.mu_e[e] : I.mu, I.wq, M) || M.k > top;
+        const i64 m = shift(whole(M.mu), M.k - top);
+        kap2 = split(shift(whole(M.kap2), M.k - top));
+        mu = split(m);
+        mu3 = split(mul_third(m));
+    }
+    const bool ok = force_lanes(L, U, kap2, mu, mu3, bad, F);
+    if (first >= I.ne) return;
+    if (ok) {
+        i64* fe = static_cast<i64*>(g.fe) + I.elem_off + e;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) fe[(long long)(L.a * 3 + c) * g.NE] = (F[c] + 4) >> 3;   // 57 to 54 fraction bits
+    } else if (L.a == 0) {
+        far_element(g, I, u, e, n0);
+    }
+}
+
+// 8 lanes per element up to kLaneElements elements, where the length of one thread's work is the time; they issue
+// two and a half times the instructions.  Time of a substep, 8 lanes against one thread per element: 432 elements
+// 9.6 and 15.8 us, 8192 13.2 and 16.7, 16000 16.2 and 16.9, 27648 21.6 and 19.2, 128000 67 and 52.
+constexpr long long kLaneElements = 16384;
 
 // Corrector of substep j and predictor of substep j + 1 (the arithmetic of k_node_b) on the fixed-point
 // element buffer: the 24 contributions of a node are summed exactly as integers and converted once per
@@ -227,8 +275,9 @@ cudaError_t launch_force_fx_b(const FomB& g, const int* active, const TraceFuse&
     if (!upred || g.eblock > 128) return cudaErrorInvalidValue;
     long long items = 0;
     for (int k = 0; k < tr.n; ++k) items += 3LL * tr.c[k].R;
-    const int grid = g.n_eblk + (int)((items + g.eblock - 1) / g.eblock);
-    k_force_fx_b<<<grid, g.eblock, 0, s>>>(g, active, tr, upred);
+    const int extra = (int)((items + g.eblock - 1) / g.eblock);
+    if (g.NE <= kLaneElements) k_force_fx_lanes_b<<<8 * g.n_eblk + extra, g.eblock, 0, s>>>(g, active, tr, upred);
+    else k_force_fx_b<<<g.n_eblk + extra, g.eblock, 0, s>>>(g, active, tr, upred);
     return cudaGetLastError();
 }
 

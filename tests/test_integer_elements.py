@@ -148,6 +148,31 @@ def test_large_meshes_match_torch(dims, material):
 
 @pytest.mark.gpu
 @pytest.mark.parametrize("material", ["nh", "le"])
+@pytest.mark.parametrize("n,nz", [(16, 64), (17, 57), (24, 30)])   # 16384 elements, the size rule's last, and above it
+@pytest.mark.parametrize("per_element", [False, True])
+def test_step_on_both_sides_of_the_size_rule(material, n, nz, per_element):
+    """Against the FP64 gather kernels (rounding of a step: 1e-12); a tenth of an edge of noise sends many Neo-Hookean
+    elements out of the fixed-point range."""
+    from paper_2511_20687_gb300 import osam
+    p = W.bar_chain("rule", n, [nz, nz], ["fom", "fom"], material, 1e9, 0.25, 1000.0, 1e-3, 1e-6, 4, max_iters=2)
+    rng = np.random.default_rng(5)
+    for sd in p.subdomains:
+        sd.u0 = sd.u0 + W.random_field(sd.n_nodes, 1e-3, 3)
+        sd.u0[sd.dirichlet == 7] = 0.0
+        if per_element:
+            sd.lam_e = sd.lam * (1 + 0.3 * rng.uniform(-1, 1, sd.n_elements))
+            sd.mu_e = sd.mu * (1 + 0.3 * rng.uniform(-1, 1, sd.n_elements))
+    a, b = osam.Problem(p), osam.Problem(p, scatter=osam.SCATTER_GATHER)
+    a.step()
+    b.step()
+    for i in range(2):
+        for f in range(3):
+            x, y = a.state(i)[f], b.state(i)[f]
+            assert np.linalg.norm(x - y) <= 1e-12 * np.linalg.norm(y)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("material", ["nh", "le"])
 @pytest.mark.parametrize("bad", [float("nan"), float("inf")])
 def test_non_finite_displacement_spreads_to_its_elements(material, bad):
     import torch
