@@ -86,7 +86,7 @@ cudaError_t newton_force(const FomB& g, cudaStream_t s) {
 cudaError_t newton_tangent(const FomB& g, cudaStream_t s) {
     if (g.linf) return launch_tangent_lin_b(g, g.cgact, s);
     if (g.material == OSAM_NEO_HOOKEAN) return launch_imp_tangent_nh_b(g, g.cgact, s);
-    if (g.fixed == 2) return launch_tangent_le_b(g, g.cgact, s);
+    if (g.fixed == 2) return launch_force_le_b(g, g.cgact, TraceFuse{}, g.cg_p, s);
     return launch_tangent_b(g, g.cgact, s);
 }
 double cg_floor(const FomB& g) { return g.linf ? kCgTol2F32 : kCgTol2; }

@@ -664,6 +664,70 @@ OSAM_HD i64 shift(i64 x, int n) {
 constexpr int kNoExponent = -100000;
 OSAM_HD int top_exponent(i64 any, int e) { return any == 0 ? kNoExponent : e - lead_zeros(any); }
 
+// Saint Venant-Kirchhoff stress of one Gauss point.  H = G 2^-base (G below 0.32 with 61 fraction bits, base >= -2: gradients of order one):
+//   2 E = H + H^T + H^T H,  S = lam/2 tr(2 E) I + mu (2 E),  P = S + H S,
+// everything in units of 2^-base, so the accuracy is relative to the largest gradient however small it is.  l2, mu: lam/2
+// and mu with 62 fraction bits (any sign); P[column][component] with 56, below 2.
+OSAM_HD bool svk_point(const Cols& C, int base, D l2, D mu, i64 P[3][3]) {
+    D G[3][3];
+    i64 S[3][3], tr = 0;
+    bool wide = false;
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+    for (int k = 0; k < 3; ++k)
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+        for (int c = 0; c < 3; ++c) G[k][c] = split(C.x[k][c]);
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+    for (int i = 0; i < 3; ++i)
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+        for (int j = i; j < 3; ++j) {
+            const i64 q = dot3(G[i][0], G[j][0], G[i][1], G[j][1], G[i][2], G[j][2]);      // 58, below 0.31
+            const i64 e = C.x[j][i] + C.x[i][j] + shift(shl(q, 3), -base);                  // 61, below 2
+            S[i][j] = mul(mu, split(e));                                                    // 59
+            if (i == j) {   // each below 1.3, so that their sum keeps its 61 bits
+                tr += e;
+                wide |= (hi(e) ^ (hi(e) >> 31)) >= (int)(1.3 * (1 << 29));
+            }
+        }
+    const i64 lt = mul(l2, split(tr));                                                      // 59
+    D s[3][3];
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+    for (int i = 0; i < 3; ++i) {
+        S[i][i] += lt;
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+        for (int j = i; j < 3; ++j) {
+            s[i][j] = split(S[i][j]);
+            S[j][i] = S[i][j];
+            s[j][i] = s[i][j];
+        }
+    }
+    int top = 0;
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+    for (int j = 0; j < 3; ++j)
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+        for (int c = 0; c < 3; ++c) {
+            const i64 hs = dot3(G[0][c], s[0][j], G[1][c], s[1][j], G[2][c], s[2][j]);      // 56
+            P[j][c] = ((S[c][j] + 4) >> 3) + shift(hs, -base);
+            top |= hi(P[j][c]) ^ (hi(P[j][c]) >> 31);
+        }
+    return base >= -2 && !wide && top < kOne25;
+}
+
 // Two factors a, b (any finite values) as integers with a common exponent: value = A 2^(e - 1084), |A| < 2^62
 OSAM_HD int factor_exponent(double a, double b) {
     const unsigned int x = hi_word(a) & 0x7fffffffu, y = hi_word(b) & 0x7fffffffu;

@@ -1,4 +1,4 @@
-// FOM set-up and I/O kernels, and the element-level internal-force kernel of the C ABI
+// FOM set-up and I/O kernels, and the dispatch of the element-level internal force of the C ABI
 // (osam_hex8_force / osam_hex8_force_noalloc).  The per-step kernels of the controller, which work
 // on every instance of a batch at once, are in step_kernels.cu; both use hex8_math.cuh.
 #include <cuda_runtime.h>
@@ -13,50 +13,6 @@ namespace osam {
 namespace {
 
 using namespace hex8;
-
-// one thread per element of a single mesh, strided input / output (see ElemArgs)
-template <int MAT, int MODE>
-__global__ void __launch_bounds__(128) k_hex8_force(const ElemArgs a) {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= a.ne) return;
-    const int i = e % a.nx;
-    const int t = e / a.nx;
-    const int j = t % a.ny;
-    const int k = t / a.ny;
-    const int sy = a.nx + 1, sz = (a.nx + 1) * (a.ny + 1);
-    const int n0 = i + sy * j + sz * k;
-    int node[8];
-#pragma unroll
-    for (int c8 = 0; c8 < 8; ++c8) node[c8] = n0 + (c8 & 1) + ((c8 >> 1) & 1) * sy + ((c8 >> 2) & 1) * sz;
-    const double lam = a.lam_e ? a.lam_e[e] : a.lam;
-    const double mu = a.mu_e ? a.mu_e[e] : a.mu;
-    double m1, m2, m3;
-    material_factors<MAT, double>(lam, mu, a.wq, a.wq3, m1, m2, m3);
-    double Dx[3][2][2], Dy[3][2][2], Dz[3][2][2];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        double U[8];
-        const double* uc = a.u + (long long)c * a.usc;
-#pragma unroll
-        for (int c8 = 0; c8 < 8; ++c8) U[c8] = uc[(long long)node[c8] * a.usn];
-        edge_differences<double>(U, a.invh, Dx[c], Dy[c], Dz[c]);
-    }
-    double F[3][8];
-    element_force<MAT, double>(Dx, Dy, Dz, m1, m2, m3, F);
-    if (MODE == kAtomic) {
-        double* f = static_cast<double*>(a.f);
-#pragma unroll
-        for (int c = 0; c < 3; ++c)
-#pragma unroll
-            for (int c8 = 0; c8 < 8; ++c8) atomic_add(f + (long long)c * a.fsc + (long long)node[c8] * a.fsn, F[c][c8]);
-    } else {
-        double* fe = static_cast<double*>(a.fe);
-#pragma unroll
-        for (int c8 = 0; c8 < 8; ++c8)
-#pragma unroll
-            for (int c = 0; c < 3; ++c) fe[(long long)(c8 * 3 + c) * a.ne + e] = F[c][c8];
-    }
-}
 
 // inverse row-sum lumped mass of a uniform cubic mesh: m_n = rho h^3 / 8 x (adjacent elements)
 __global__ void k_lumped_minv(int nx, int ny, int nz, double m_e8, double* minv, double* mass) {
@@ -166,13 +122,10 @@ int grid_for(long long n, int block) { return (int)((n + block - 1) / block); }
 
 cudaError_t launch_hex8_force(int material, int scatter, const ElemArgs& a, cudaStream_t s) {
     if (a.ne <= 0) return cudaSuccess;
-    // Neo-Hookean and linear elastic: in 64-bit integers, no FP64 pipe (lane_kernels.cu, force_le.cu)
+    // in 64-bit integers, no FP64 pipe (lane_kernels.cu, force_le.cu, force_svk.cu)
     if (material == OSAM_NEO_HOOKEAN) return launch_elem_force_nh(scatter, a, s);
     if (material == OSAM_LINEAR_ELASTIC) return launch_elem_force_le(scatter, a, s);
-    const int g = grid_for(a.ne, 128);
-    if (scatter == kAtomic) k_hex8_force<OSAM_SAINT_VENANT_KIRCHHOFF, kAtomic><<<g, 128, 0, s>>>(a);
-    else k_hex8_force<OSAM_SAINT_VENANT_KIRCHHOFF, kGather><<<g, 128, 0, s>>>(a);
-    return cudaGetLastError();
+    return launch_elem_force_svk(scatter, a, s);
 }
 
 cudaError_t launch_lumped_minv(const Grid& g, double rho, double* minv, cudaStream_t s, double* mass) {

@@ -104,10 +104,10 @@ __global__ void __launch_bounds__(128) k_elem_force_le_lanes(const __grid_consta
     }
 }
 
-// FomB groups: x = u / h (g.us) or the CG direction; element buffer [24][NE], trace blocks at the end of the grid
-template <bool TANGENT>
+// FomB groups: u the displacement or the CG direction, read as it is (its rounding through 1/h was the largest
+// error of the FP64 form); element buffer [24][NE], trace blocks at the end of the grid
 __global__ void __launch_bounds__(128) k_fom_force_le(const __grid_constant__ FomB g, const int* __restrict__ active,
-                                                      const __grid_constant__ TraceFuse tr) {
+                                                      const __grid_constant__ TraceFuse tr, const double* u) {
     if ((int)blockIdx.x >= g.n_eblk) {
         trace::fused_trace_block(tr, active, g, (int)blockIdx.x - g.n_eblk);
         return;
@@ -119,16 +119,16 @@ __global__ void __launch_bounds__(128) k_fom_force_le(const __grid_constant__ Fo
     if (e >= I.ne) return;
     const int nx = I.nx, ny = I.ny, i = e % nx, t = e / nx, j = t % ny, k = t / ny;
     const int sy = nx + 1, sz = (nx + 1) * (ny + 1);
-    const double* x = (TANGENT ? g.cg_p : g.us) + I.node_off + (i + sy * j + sz * k);
+    const double* x = u + I.node_off + (i + sy * j + sz * k);
     double U[3][8], F[3][8];
 #pragma unroll
     for (int c = 0; c < 3; ++c)
 #pragma unroll
         for (int c8 = 0; c8 < 8; ++c8)
             U[c][c8] = x[(long long)c * g.NN + (c8 & 1) + ((c8 >> 1) & 1) * sy + (c8 >> 2) * sz];
-    double lam = TANGENT ? I.t1 : I.s1, mu = TANGENT ? I.t2 : I.s2;
+    double lam = I.t1, mu = I.t2;
     if (I.lam_e || I.mu_e) {
-        const double w = 2.0 * (TANGENT ? I.wqi : I.wq);
+        const double w = 2.0 * I.wqi;
         lam = (I.lam_e ? I.lam_e[e] : I.lam) * w;
         mu = (I.mu_e ? I.mu_e[e] : I.mu) * w;
     }
@@ -147,9 +147,8 @@ __global__ void __launch_bounds__(128) k_fom_force_le(const __grid_constant__ Fo
 }
 
 // ... and on 8 lanes: block of g.eblock threads, an element block on 8 of them
-template <bool TANGENT>
 __global__ void __launch_bounds__(128) k_fom_force_le_lanes(const __grid_constant__ FomB g, const int* __restrict__ active,
-                                                            const __grid_constant__ TraceFuse tr) {
+                                                            const __grid_constant__ TraceFuse tr, const double* u) {
     if ((int)blockIdx.x >= 8 * g.n_eblk) {
         trace::fused_trace_block(tr, active, g, (int)blockIdx.x - 8 * g.n_eblk);
         return;
@@ -160,16 +159,16 @@ __global__ void __launch_bounds__(128) k_fom_force_le_lanes(const __grid_constan
     const int first = b.y + (int)((blockIdx.x & 7u) * (blockDim.x >> 3) + (threadIdx.x >> 3)), e = min(first, I.ne - 1);
     const int nx = I.nx, ny = I.ny, i = e % nx, t = e / nx, j = t % ny, k = t / ny;
     const int sy = nx + 1, sz = (nx + 1) * (ny + 1);
-    const double* x = (TANGENT ? g.cg_p : g.us) + I.node_off + (i + sy * j + sz * k);
+    const double* x = u + I.node_off + (i + sy * j + sz * k);
     const Lane L = make_lane();
     double U[3];
     i64 F[3];
     int scale;
 #pragma unroll
     for (int c = 0; c < 3; ++c) U[c] = x[(long long)c * g.NN + (L.a & 1) + ((L.a >> 1) & 1) * sy + (L.a >> 2) * sz];
-    double lam = TANGENT ? I.t1 : I.s1, mu = TANGENT ? I.t2 : I.s2;
+    double lam = I.t1, mu = I.t2;
     if (I.lam_e || I.mu_e) {
-        const double w = 2.0 * (TANGENT ? I.wqi : I.wq);
+        const double w = 2.0 * I.wqi;
         lam = (I.lam_e ? I.lam_e[e] : I.lam) * w;
         mu = (I.mu_e ? I.mu_e[e] : I.mu) * w;
     }
@@ -194,13 +193,13 @@ constexpr long long kLaneElements = 16384;
 
 }  // namespace
 
-cudaError_t launch_elem_force_le(int scatter, const ElemArgs& a, cudaStream_t s) {
+cudaError_t launch_elem_force_le(int scatter, const ElemArgs& a, cudaStream_t s, int lanes) {
     const int grid = grid_for(a.ne, kElemBlock);
     const double w = 2.0 * a.wq * a.invh;   // h / 16
-    if (a.ne <= kLaneElements) {
-        const int lanes = grid_for(a.ne, 16);
-        if (scatter == kAtomic) k_elem_force_le_lanes<kAtomic><<<lanes, 128, 0, s>>>(a, w);
-        else k_elem_force_le_lanes<kGather><<<lanes, 128, 0, s>>>(a, w);
+    if (lanes < 0 ? a.ne <= kLaneElements : lanes) {
+        const int blocks = grid_for(a.ne, 16);
+        if (scatter == kAtomic) k_elem_force_le_lanes<kAtomic><<<blocks, 128, 0, s>>>(a, w);
+        else k_elem_force_le_lanes<kGather><<<blocks, 128, 0, s>>>(a, w);
         return cudaGetLastError();
     }
     if (scatter == kAtomic) k_elem_force_le<kAtomic><<<grid, kElemBlock, 0, s>>>(a, w);
@@ -208,20 +207,13 @@ cudaError_t launch_elem_force_le(int scatter, const ElemArgs& a, cudaStream_t s)
     return cudaGetLastError();
 }
 
-cudaError_t launch_force_le_b(const FomB& g, const int* active, const TraceFuse& tr, cudaStream_t s) {
-    if (g.eblock > 128) return cudaErrorInvalidValue;
+cudaError_t launch_force_le_b(const FomB& g, const int* active, const TraceFuse& tr, const double* u, cudaStream_t s) {
+    if (g.eblock > 128 || !u) return cudaErrorInvalidValue;
     long long items = 0;
     for (int k = 0; k < tr.n; ++k) items += 3LL * tr.c[k].R;
     const int extra = (int)((items + g.eblock - 1) / g.eblock);
-    if (g.NE <= kLaneElements) k_fom_force_le_lanes<false><<<8 * g.n_eblk + extra, g.eblock, 0, s>>>(g, active, tr);
-    else k_fom_force_le<false><<<g.n_eblk + extra, g.eblock, 0, s>>>(g, active, tr);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_tangent_le_b(const FomB& g, const int* mask, cudaStream_t s) {
-    if (g.eblock > 128) return cudaErrorInvalidValue;
-    if (g.NE <= kLaneElements) k_fom_force_le_lanes<true><<<8 * g.n_eblk, g.eblock, 0, s>>>(g, mask, TraceFuse{});
-    else k_fom_force_le<true><<<g.n_eblk, g.eblock, 0, s>>>(g, mask, TraceFuse{});
+    if (g.NE <= kLaneElements) k_fom_force_le_lanes<<<8 * g.n_eblk + extra, g.eblock, 0, s>>>(g, active, tr, u);
+    else k_fom_force_le<<<g.n_eblk + extra, g.eblock, 0, s>>>(g, active, tr, u);
     return cudaGetLastError();
 }
 

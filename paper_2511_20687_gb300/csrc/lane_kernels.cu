@@ -363,11 +363,11 @@ void fixed_point_inverse(double x, long long& m, int& e) {
     e = k - 1;
 }
 
-cudaError_t launch_elem_force_nh(int scatter, const ElemArgs& a, cudaStream_t s) {
+cudaError_t launch_elem_force_nh(int scatter, const ElemArgs& a, cudaStream_t s, int lanes) {
     long long m;
     int e;
     fixed_point_inverse(a.invh, m, e);
-    if (a.ne > kLaneElements) {
+    if (lanes < 0 ? a.ne > kLaneElements : !lanes) {
         if (scatter == kAtomic) k_elem_force_thread<kAtomic><<<grid_for(a.ne, 128), 128, 0, s>>>(a, m, e);
         else k_elem_force_thread<kGather><<<grid_for(a.ne, 128), 128, 0, s>>>(a, m, e);
         return cudaGetLastError();

@@ -172,6 +172,27 @@ __device__ __forceinline__ bool force_le_lanes(const Lane& L, const double p[3],
     return !any_lane(bad || ek == 2047 || scale > 1000 || scale < -900);
 }
 
+// Saint Venant-Kirchhoff force of the lane's corner from its displacement: F 2^-scale; 1/h as ihm 2^(ihe - 62) (the
+// coefficients are multiplied by ihm 2^-63), m1, m2: the material factors lam and mu times h^2 / 32
+__device__ __forceinline__ bool force_svk_lanes(const Lane& L, const double p[3], i64 ihm, int ihe, double m1, double m2,
+                                                i64 F[3], int& scale) {
+    Cols G;
+    i64 P[3][3], w[3];
+    bool bad = false;
+    const int T = block_walsh(L, p, w, bad), e = factor_exponent(m1, m2);
+    const int base = T == kNoExponent ? 0 : 1015 - T - ihe;
+    const D r = split(ihm);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) gauss_columns(L, pattern_scale(L, (mul(split(shl(w[c], 4)), r) + 4) >> 3), c, G);
+    const i64 l = factor_value(m1, e);
+    bad |= !svk_point(G, base, split((l + 1) >> 1), split(factor_value(m2, e)), P);
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+        F[c] = corner_values(L, pattern_scale(L, gauss_transpose(L, P[0][c], P[1][c], P[2][c])));
+    scale = 56 + base - (e - 1022);
+    return !any_lane(bad || e == 2047 || scale > 1000 || scale < -900);
+}
+
 // Material factors kappa/2 and mu times w as integers: value = X 2^(k - 62), the larger in [2^61, 2^62);
 // false unless both are positive and finite
 struct Material {

@@ -84,6 +84,10 @@ int device_setup(cudaStream_t s, double** out) {
         a.fe = base;
         for (int m : {OSAM_LINEAR_ELASTIC, OSAM_NEO_HOOKEAN, OSAM_SAINT_VENANT_KIRCHHOFF})
             if (e == cudaSuccess) e = osam::launch_hex8_force(m, osam::kGather, a, s);
+        for (int lanes = 0; lanes < 2; ++lanes) {   // both kernels of the materials with a size rule
+            if (e == cudaSuccess) e = osam::launch_elem_force_le(osam::kGather, a, s, lanes);
+            if (e == cudaSuccess) e = osam::launch_elem_force_nh(osam::kGather, a, s, lanes);
+        }
         if (e == cudaSuccess) {
             k_gather_aos<<<1, 32, 0, s>>>(1, 1, 1, base, base + 48);
             e = cudaGetLastError();

@@ -67,7 +67,7 @@ struct InstFom {
     long long fk2, fmu, ihm;
     int ihe, fscale;
     double wqi;               // wq / h (weight of the tangent action on a direction that is not divided by h)
-    double s1, s2, t1, t2;    // linear elastic: lam and mu times 2 wq and 2 wqi (element_force_le)
+    double t1, t2;            // linear elastic: lam and mu times 2 wqi (element_force_le)
 };
 
 // kernel view of a FOM slot across instances; nodal arrays are SoA over the concatenated nodes:
@@ -131,7 +131,7 @@ struct FomB {
     float* fe32;              // FP32 element buffer [24][NE] of the FP32 tangent action
     int df32;                 // 1: internal force in double-float arithmetic (element buffer of float2)
     int fixed;                // internal force in 64-bit integers: 1 Neo-Hookean (element buffer of int64; force_fx.cu),
-                              // 2 linear elastic (element buffer of double; force_le.cu)
+                              // 2 linear elastic, 3 Saint Venant-Kirchhoff (element buffer of double; force_le.cu, force_svk.cu)
     long long* ux;            // fixed-point predicted displacement / h [3][NN]
     double* fe2;              // FP64 contributions of the elements outside the fixed-point range [24][NE]
 };
@@ -230,7 +230,7 @@ cudaError_t launch_zero_clamped(int nn, const uint8_t* clamp, double* u, double*
 // batched per-step kernels (step_kernels.cu); `active` masks instances that have converged
 // ------------------------------------------------------------------------------------------------
 // internal force of the predicted displacement held (divided by h) in g.us / g.u2
-// (upred: that displacement itself, required by fixed-point groups)
+// (upred: that displacement itself, required by the integer forces of explicit groups)
 cudaError_t launch_force_b(const FomB& g, const int* active, int scatter, cudaStream_t s,
                            const TraceFuse* tr = nullptr, const double* upred = nullptr);
 cudaError_t launch_force_init_b(const FomB& g, const int* active, cudaStream_t s);  // FP64 gather of f(u[0]) into fe
@@ -248,15 +248,19 @@ cudaError_t launch_node_fx_b(const FomB& g, const int* active, int slot1, int sl
 // Neo-Hookean element level and implicit groups in 64-bit integers, 8 lanes per element (lane_kernels.cu);
 // fixed_point_inverse: x as m 2^(e - 62), m in [2^62, 2^63)
 void fixed_point_inverse(double x, long long& m, int& e);
-cudaError_t launch_elem_force_nh(int scatter, const ElemArgs& a, cudaStream_t s);
+cudaError_t launch_elem_force_nh(int scatter, const ElemArgs& a, cudaStream_t s, int lanes = -1);
 cudaError_t launch_elem_vjp_nh(int scatter, const ElemArgs& a, const double* ybar, int ysn, long long ysc,
                                double* lam_bar, double* mu_bar, int acc, cudaStream_t s);
 cudaError_t launch_imp_force_nh_b(const FomB& g, const int* mask, cudaStream_t s);
 cudaError_t launch_imp_tangent_nh_b(const FomB& g, const int* mask, cudaStream_t s);
 // linear elastic in 64-bit integers (force_le.cu)
-cudaError_t launch_elem_force_le(int scatter, const ElemArgs& a, cudaStream_t s);
-cudaError_t launch_force_le_b(const FomB& g, const int* active, const TraceFuse& tr, cudaStream_t s);
-cudaError_t launch_tangent_le_b(const FomB& g, const int* mask, cudaStream_t s);
+// lanes: 8 lanes per element (1) or one thread (0); -1: by the number of elements
+cudaError_t launch_elem_force_le(int scatter, const ElemArgs& a, cudaStream_t s, int lanes = -1);
+// (u: the displacement, or the direction of the tangent action)
+cudaError_t launch_force_le_b(const FomB& g, const int* active, const TraceFuse& tr, const double* u, cudaStream_t s);
+// Saint Venant-Kirchhoff in 64-bit integers (force_svk.cu)
+cudaError_t launch_elem_force_svk(int scatter, const ElemArgs& a, cudaStream_t s);
+cudaError_t launch_force_svk_b(const FomB& g, const int* active, const TraceFuse& tr, const double* u, cudaStream_t s);
 // double-float mode (force_df.cu)
 cudaError_t launch_split_u2_b(const FomB& g, cudaStream_t s);
 cudaError_t launch_force_df_b(const FomB& g, const int* active, const TraceFuse& tr, cudaStream_t s);

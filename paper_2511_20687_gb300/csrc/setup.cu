@@ -179,7 +179,6 @@ int setup_fom_group(osam_ctx* ctx, FomGroupH& G, int s, int n, const osam_proble
         I.wq3 = g.h * g.h / 96.0;
         I.lam = d.lambda; I.mu = d.mu;
         I.wqi = I.wq * I.invh;
-        I.s1 = 2.0 * I.wq * I.lam; I.s2 = 2.0 * I.wq * I.mu;
         I.t1 = 2.0 * I.wqi * I.lam; I.t2 = 2.0 * I.wqi * I.mu;
         fixed_point_inverse(I.invh, I.ihm, I.ihe);
         if (d.material == OSAM_NEO_HOOKEAN) {
@@ -214,16 +213,16 @@ int setup_fom_group(osam_ctx* ctx, FomGroupH& G, int s, int n, const osam_proble
     CKA(B.hist = ctx->alloc<double>(std::max<long long>(H, 1)));
     CKA(B.us = ctx->alloc<double>(3 * NN));
     B.implicit = descs[0].subdomains[s].integrator == OSAM_IMPLICIT;
-    // Force in 64-bit integers: explicit Neo-Hookean groups and linear elastic groups of the FP64 modes
-    // whose scatter is left to the library (a scatter mode asked for by name runs its own FP64 kernel).
+    // Force in 64-bit integers: explicit Neo-Hookean groups, and linear elastic and Saint Venant-Kirchhoff groups of
+    // the FP64 modes, whose scatter is left to the library (a scatter mode asked for by name runs its own FP64 kernel).
     // The double-float mode's Neo-Hookean force is the fixed-point one too: more accurate than pairs of FP32
     // values, and faster (40x40x80: 40 us per launch against 50).
     const bool integers = descs[0].scatter == OSAM_SCATTER_AUTO || ctx->integer_force;
     const bool fp64 = ctx->precision == OSAM_FP64 || ctx->precision == OSAM_FP64_TANGENT32;
     if (integers && B.material == OSAM_NEO_HOOKEAN && !B.implicit && (fp64 || ctx->precision == OSAM_F32X2_FORCE))
         B.fixed = 1;
-    else if (integers && B.material == OSAM_LINEAR_ELASTIC && fp64)
-        B.fixed = 2;
+    else if (integers && fp64 && B.material != OSAM_NEO_HOOKEAN)
+        B.fixed = B.material == OSAM_LINEAR_ELASTIC ? 2 : 3;
     B.df32 = ctx->precision == OSAM_F32X2_FORCE && !B.fixed;
     if (B.df32 || B.fp32) CKA(B.u2 = ctx->alloc<float2>(3 * NN));   // the FP32 forces' split of u/h
     if (B.fixed == 1) {

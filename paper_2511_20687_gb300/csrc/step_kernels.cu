@@ -341,8 +341,9 @@ __global__ void __launch_bounds__(kNodeBlock) k_node_b(const FomB g, const int* 
                 for (int q = 0; q < NC; ++q) x[q][corner] = in ? __ldg(fe + (long long)(corner * 3 + c0 + q) * g.NE + e) : TF(0);
             }
 #pragma unroll
-            for (int q = 0; q < NC; ++q)   // three additions in a row instead of eight
-                fs[q] = ((x[q][0] + x[q][1]) + (x[q][2] + x[q][3])) + ((x[q][4] + x[q][5]) + (x[q][6] + x[q][7]));
+            for (int corner = 0; corner < 8; ++corner)
+#pragma unroll
+                for (int q = 0; q < NC; ++q) fs[q] += x[q][corner];
             // FP64: the same sums; FP32 force: summed in FP32 (its own precision) and widened once, by
             // integer operations (f64_of: exact)
 #pragma unroll
@@ -393,7 +394,7 @@ __global__ void __launch_bounds__(kNodeBlock) k_node_b(const FomB g, const int* 
                 float2 x;
                 fx::split_scaled(un, I.ihm, I.ihe, x.x, x.y);
                 g.u2[d] = x;
-            } else {
+            } else if (g.fixed == 0) {         // the integer forces read u itself
                 g.us[d] = un * I.invh;
             }
         }
@@ -821,7 +822,8 @@ cudaError_t launch_force_b(const FomB& g, const int* active, int scatter, cudaSt
     const int grid = g.n_eblk + (int)((items + b - 1) / b);
     if (g.df32) return launch_force_df_b(g, active, tr, s);
     if (g.fixed == 1) return launch_force_fx_b(g, active, tr, upred, s);
-    if (g.fixed == 2) return launch_force_le_b(g, active, tr, s);
+    if (g.fixed == 2) return launch_force_le_b(g, active, tr, g.implicit ? g.u[0] : upred, s);
+    if (g.fixed == 3) return launch_force_svk_b(g, active, tr, g.implicit ? g.u[0] : upred, s);
 #define OSAM_LAUNCH(MAT, T, MODE) k_force_b<MAT, T, MODE><<<grid, b, 0, s>>>(g, active, tr)
     const bool fp32 = g.fp32 != 0;
     if (g.tiled && !fp32) {
@@ -889,7 +891,7 @@ cudaError_t launch_node_b(const FomB& g, const int* active, int scatter, int slo
     const bool fp32 = g.fp32 != 0;
     if (g.df32) return launch_node_df_b(g, active, slot1, slot2, predict_only, ucur, unext, dt, s);
     if (g.fixed == 1) return launch_node_fx_b(g, active, slot1, slot2, predict_only, ucur, unext, dt, s);
-    if (g.fixed == 2) scatter = kGather;
+    if (g.fixed >= 2) scatter = kGather;
     const bool split = node_split(g);
     const dim3 grid(g.n_nblk, split ? 3 : 1);
 #define OSAM_NODE(T, M)                                                                                                   \

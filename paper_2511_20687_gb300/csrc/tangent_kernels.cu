@@ -58,12 +58,16 @@ __device__ __forceinline__ void svk_tangent(const double H[3][3], const double G
 
 // element tangent action: the directional derivative of the element forces at u along p, written
 // to the element buffer (same layout and sum factorisation as the force kernels)
+// Blocks of 64 elements whatever the group's element blocks are: bound by the FP64 pipe, the launch lasts as long as
+// the SM with the most elements.
+constexpr int kTangentBlock = 64;
 template <int MAT>
-__global__ void __launch_bounds__(256) k_tangent_b(const FomB g, const int* __restrict__ mask) {
-    const int2 b = g.eblk[blockIdx.x];
+__global__ void __launch_bounds__(kTangentBlock) k_tangent_b(const FomB g, const int* __restrict__ mask) {
+    const int per = g.eblock / kTangentBlock;
+    const int2 b = g.eblk[blockIdx.x / per];
     if (!run_inst(mask, b.x)) return;
     const InstFom I = g.inst[b.x];
-    const int e = b.y + threadIdx.x;
+    const int e = b.y + (int)(blockIdx.x % per) * kTangentBlock + (int)threadIdx.x;
     if (e >= I.ne) return;
     const int i = e % I.nx;
     const int t = e / I.nx;
@@ -280,10 +284,11 @@ cudaError_t launch_tangent_lin_b(const FomB& g, const int* mask, cudaStream_t s)
 
 cudaError_t launch_tangent_b(const FomB& g, const int* mask, cudaStream_t s) {
     if (g.n_eblk == 0) return cudaSuccess;
-    if (g.eblock > 256) return cudaErrorInvalidConfiguration;
+    if (g.eblock % kTangentBlock) return cudaErrorInvalidConfiguration;
+    const int grid = g.n_eblk * (g.eblock / kTangentBlock);
     if (g.material == OSAM_SAINT_VENANT_KIRCHHOFF)
-        k_tangent_b<OSAM_SAINT_VENANT_KIRCHHOFF><<<g.n_eblk, g.eblock, 0, s>>>(g, mask);
-    else k_tangent_b<OSAM_LINEAR_ELASTIC><<<g.n_eblk, g.eblock, 0, s>>>(g, mask);
+        k_tangent_b<OSAM_SAINT_VENANT_KIRCHHOFF><<<grid, kTangentBlock, 0, s>>>(g, mask);
+    else k_tangent_b<OSAM_LINEAR_ELASTIC><<<grid, kTangentBlock, 0, s>>>(g, mask);
     return cudaGetLastError();
 }
 }  // namespace osam

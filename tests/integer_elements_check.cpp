@@ -2,7 +2,8 @@
 // extended precision.  Reads "h lam mu" and 24 displacements and 24 directions [component][corner] per line; writes
 // "ok" of the two and the rms errors (integers, the same formula in double) of the linear elastic force of the
 // direction and of the tangent action, relative to the largest exact entry, and of the two parameter contractions
-// in units of h^2 times the largest difference of the direction.
+// in units of h^2 times the largest difference of the direction; then "ok" and the errors of the Saint
+// Venant-Kirchhoff force of the displacement.
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -167,6 +168,58 @@ static bool tangent_fixed(const double u[3][8], const double x[3][8], double h, 
     return ok;
 }
 
+// Saint Venant-Kirchhoff force from displacements divided by h
+template <class T>
+void svk(const double v[3][8], double h, double lam, double mu, T F[26]) {
+    const Shape<T> S(1.0);
+    for (int p = 0; p < 8; ++p) {
+        T H[3][3], E[3][3], P[3][3], tr = 0;
+        S.grad(v, p, H);
+        for (int i = 0; i < 3; ++i)
+            for (int j = 0; j < 3; ++j) {
+                E[i][j] = H[i][j] + H[j][i];
+                for (int c = 0; c < 3; ++c) E[i][j] += H[c][i] * H[c][j];
+                E[i][j] /= 2;
+                if (i == j) tr += E[i][j];
+            }
+        for (int c = 0; c < 3; ++c)
+            for (int j = 0; j < 3; ++j) {
+                P[c][j] = 0;
+                for (int k = 0; k < 3; ++k)
+                    P[c][j] += (H[c][k] + (c == k)) * (2 * T(mu) * E[k][j] + (k == j ? T(lam) * tr : T(0))) * T(h) * T(h);
+            }
+        S.add(P, p, F);
+    }
+}
+static bool svk_fixed(const double v[3][8], double h, double lam, double mu, double R[26]) {
+    i64 w[3][8], o[3][8] = {};
+    int T;
+    bool ok = block_walsh(v, w, T);
+    const int base = T == kNoExponent ? 0 : 1016 - T;
+    for (int c = 0; c < 3; ++c)
+        for (int a = 1; a < 8; ++a) w[c][a] = scaled(w[c][a], a);
+    const double m1 = lam * h * h / 32, m2 = mu * h * h / 32;
+    const int e = factor_exponent(m1, m2);
+    for (int g = 0; g < 8; ++g) {
+        Cols G;
+        i64 P[3][3];
+        columns(w, g, G);
+        ok = svk_point(G, base, split((factor_value(m1, e) + 1) >> 1), split(factor_value(m2, e)), P) && ok;
+        for (int b = 1; b < 8; ++b)
+            for (int d = 0; d < 3; ++d)
+                if ((b >> d) & 1)
+                    for (int c = 0; c < 3; ++c) o[c][b] += minus(b & ~(1 << d), g) ? -P[d][c] : P[d][c];
+    }
+    for (int c = 0; c < 3; ++c) {
+        for (int b = 1; b < 8; ++b) o[c][b] = scaled(o[c][b], b);
+        for (int b = 1; b < 8; b <<= 1)
+            for (int a = 0; a < 8; ++a)
+                if (!(a & b)) { const i64 l = o[c][a], u = o[c][a | b]; o[c][a] = l - u; o[c][a | b] = l + u; }
+        for (int a = 0; a < 8; ++a) R[8 * c + a] = f64_scaled(o[c][a], 56 + base - (e - 1022));
+    }
+    return ok;
+}
+
 template <class A>
 static double error(const A* x, const Real* y, int n) {
     Real s = 0, t = 0;
@@ -192,7 +245,15 @@ int main() {
             for (int k = 0; k < 8; ++k) top = std::fmax(top, std::fabs((Real)x[c][k] - (Real)x[c][0]));
         top *= (Real)h * h;
         const auto part = [&](const double* f, int k) { return (double)(std::fabs(f[k] - T[k]) / top); };
-        std::printf("%d %d %.3e %.3e %.3e %.3e %.3e %.3e %.3e %.3e\n", a, b, error(&Ef[0][0], E, 24), error(Ed, E, 24),
-                    error(Tf, T, 24), error(Td, T, 24), part(Tf, 24), part(Td, 24), part(Tf, 25), part(Td, 25));
+        Real V[26] = {};
+        double Vd[26] = {}, Vf[26] = {}, y[3][8];   // the displacement divided by h, exact in the reference
+        for (int c = 0; c < 3; ++c)
+            for (int k = 0; k < 8; ++k) y[c][k] = u[c][k] / h;
+        svk<Real>(y, h, lam, mu, V);
+        svk<double>(y, h, lam, mu, Vd);
+        const bool v3 = svk_fixed(y, h, lam, mu, Vf);
+        std::printf("%d %d %.3e %.3e %.3e %.3e %.3e %.3e %.3e %.3e %d %.3e %.3e\n", a, b, error(&Ef[0][0], E, 24), error(Ed, E, 24),
+                    error(Tf, T, 24), error(Td, T, 24), part(Tf, 24), part(Td, 24), part(Tf, 25), part(Td, 25),
+                    v3, error(Vf, V, 24), error(Vd, V, 24));
     }
 }

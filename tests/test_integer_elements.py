@@ -1,4 +1,4 @@
-"""The integer element kernels (linear elastic force, Neo-Hookean force and vector-Jacobian product): their arithmetic on
+"""The integer element kernels (linear elastic, Neo-Hookean and Saint Venant-Kirchhoff force, vector-Jacobian products): their arithmetic on
 the CPU against extended precision, and the element-level calls against plain torch."""
 import math
 import os
@@ -61,6 +61,19 @@ def test_closer_than_fp64(check, nu, amp, kind, size):
         assert np.sqrt(np.mean(r[:, k] ** 2)) <= np.sqrt(np.mean(r[:, k + 1] ** 2))
 
 
+@pytest.mark.parametrize("nu", [0.25, 0.45, -0.1])
+@pytest.mark.parametrize("amp,inside", [(0.0, True), (1e-12, True), (1e-3, True), (0.2, True), (3.0, False)])
+def test_saint_venant_kirchhoff_is_closer_than_fp64(check, nu, amp, inside):
+    """As above, with the error bound of the linear elastic force; strains of order one leave the range."""
+    rng = np.random.default_rng(6)
+    u = H * (0.3 + amp * rng.uniform(-1, 1, (150, 3, 8)))
+    r = check(u, rng.standard_normal((150, 3, 8)), nu)
+    good = r[:, 10] == 1
+    assert good.all() if inside else good.mean() < 0.1
+    assert (r[good, 11] < 1e-15).all()
+    assert not good.any() or np.sqrt(np.mean(r[good, 11] ** 2)) <= np.sqrt(np.mean(r[good, 12] ** 2))
+
+
 @pytest.mark.parametrize("bad", [np.nan, np.inf, 1e-310])
 def test_operands_outside_the_formats_are_reported(check, bad):
     x = np.zeros((1, 3, 8))
@@ -88,6 +101,9 @@ def reference(torch, dims, h, material, lam, mu, u):
     eye = torch.eye(3, device=u.device, dtype=torch.float64)
     if material == "le":
         P = lam * G.diagonal(dim1=-2, dim2=-1).sum(-1)[..., None, None] * eye + mu * (G + G.mT)
+    elif material == "svk":
+        E = 0.5 * (G + G.mT + G.mT @ G)
+        P = (G + eye) @ (lam * E.diagonal(dim1=-2, dim2=-1).sum(-1)[..., None, None] * eye + 2 * mu * E)
     else:
         F = G + eye
         J = torch.det(F)[..., None, None]
@@ -125,7 +141,7 @@ def test_element_calls_match_torch(dims, material, shift):
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("material", ["nh", "le"])
+@pytest.mark.parametrize("material", ["nh", "le", "svk"])
 @pytest.mark.parametrize("dims", [(16, 32, 32), (17, 31, 33), (64, 32, 32), (33, 65, 31)])   # sides of the size rules
 def test_large_meshes_match_torch(dims, material):
     import torch
@@ -147,7 +163,7 @@ def test_large_meshes_match_torch(dims, material):
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("material", ["nh", "le"])
+@pytest.mark.parametrize("material", ["nh", "le", "svk"])
 @pytest.mark.parametrize("n,nz", [(16, 64), (17, 57), (24, 30)])   # 16384 elements, the size rule's last, and above it
 @pytest.mark.parametrize("per_element", [False, True])
 def test_step_on_both_sides_of_the_size_rule(material, n, nz, per_element):
@@ -172,7 +188,7 @@ def test_step_on_both_sides_of_the_size_rule(material, n, nz, per_element):
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("material", ["nh", "le"])
+@pytest.mark.parametrize("material", ["nh", "le", "svk"])
 @pytest.mark.parametrize("bad", [float("nan"), float("inf")])
 def test_non_finite_displacement_spreads_to_its_elements(material, bad):
     import torch
