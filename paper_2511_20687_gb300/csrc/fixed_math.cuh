@@ -948,27 +948,6 @@ OSAM_HD float f32_scaled(i64 x, int scale) {
     return r;
 }
 
-// (hi, lo) FP32 split of u / h by integer operations: hi the product cut to 24 bits, lo the remainder cut to 24 bits
-// (|u / h - (hi + lo)| < 2^-47 |u / h|).  ihm, ihe: 1/h as in fixed_u.
-OSAM_HD void split_scaled(double u, i64 ihm, int ihe, float& hif, float& lof) {
-    unsigned long long b;
-#ifdef __CUDA_ARCH__
-    b = (unsigned long long)__double_as_longlong(u);
-#else
-    __builtin_memcpy(&b, &u, 8);
-#endif
-    const int e = (int)((b >> 52) & 0x7ff);
-    const i64 m = e == 0 ? 0 : (i64)(((b & 0xfffffffffffffULL) | 0x10000000000000ULL) << 10);   // u = m 2^(e - 1085)
-    const i64 p = mul(m, ihm);                                       // below 2^62: u / h = p 2^(e - 1085 + ihe + 2)
-    const int lz = lead_zeros(p);
-    const i64 q = shl(p, lz == 64 ? 0 : lz - 1), top = q & ~(((i64)1 << 39) - 1);   // 24 leading bits of [2^62, 2^63)
-    const int scale = 1083 - e - ihe + (lz == 64 ? 0 : lz - 1);
-    const bool neg = (b >> 63) != 0, odd = e == 2047;
-    const i64 h = odd ? (i64)1 << 62 : top, l = q - top;
-    hif = f32_scaled(neg ? -h : h, odd ? -200 : scale);              // infinite for operands that are not finite
-    lof = odd ? 0.0f : f32_scaled(neg ? -l : l, scale);
-}
-
 // fixed-point u / h of a nodal displacement: mantissa (53 bits) times the 63-bit mantissa of 1/h, shifted
 // to 59 fraction bits; kBadU for |u| / h >= 12 and for non-finite values.  ihm in [2^62, 2^63),
 // 1/h = ihm 2^(ihe - 62).
