@@ -170,7 +170,8 @@ OSAM_HD bool out_of_range(const Range& g) {
 }
 
 // spread check of one component's 8 nodal values (59 fraction bits): no nodal value marked, and the
-// spread below 2.75 edges, so that every Walsh coefficient stays below 11
+// spread below 2.75 edges, so that every Walsh coefficient stays below 11.  Values reach +-12 edges, so their
+// difference (27 fraction bits of the high words) is taken without a sign: it wraps a signed word from 16 edges on.
 OSAM_HD bool spread_bad(const i64 V[8]) {
     int mx = hi(V[0]), mn = hi(V[0]);
 #ifdef __CUDACC__
@@ -180,7 +181,7 @@ OSAM_HD bool spread_bad(const i64 V[8]) {
         mx = imax(mx, hi(V[k]));
         mn = imin(mn, hi(V[k]));
     }
-    return mn < -((kMaxU + 1) << 27) || mx - mn >= 11 * (1 << 25);
+    return mn < -((kMaxU + 1) << 27) || (unsigned int)mx - (unsigned int)mn >= 11u << 25;
 }
 
 // Walsh coefficients of one component of u / h (59 fraction bits) and their multiples that the Gauss

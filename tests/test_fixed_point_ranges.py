@@ -1,0 +1,98 @@
+"""Which elements the integer Neo-Hookean force may evaluate: the range checks at their limits, on the CPU with the
+kernels' own functions and on the GPU against the FP64 kernels."""
+import os
+import shutil
+import subprocess
+
+import numpy as np
+import pytest
+
+from paper_2511_20687_gb300 import workloads as W
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+H = 0.0123
+CORNERS = np.array([[a & 1, (a >> 1) & 1, a >> 2] for a in range(8)], float)
+
+
+def build(tmp_path_factory, source):
+    if shutil.which("g++") is None:
+        pytest.skip("needs g++")
+    exe = str(tmp_path_factory.mktemp("ranges") / "check")
+    subprocess.run(["g++", "-O2", "-std=c++17", "-x", "c++", "-I", os.path.join(ROOT, "paper_2511_20687_gb300/csrc"), "-o",
+                    exe, os.path.join(ROOT, "tests", source)], check=True)
+
+    def run(lines):
+        text = "\n".join(" ".join(repr(float(v)) for v in np.concatenate([np.ravel(a) for a in line])) for line in lines)
+        out = subprocess.run([exe], input=text, capture_output=True, text=True, check=True).stdout
+        return np.array([[float(v) for v in line.split()] for line in out.splitlines()])
+
+    return run
+
+
+@pytest.fixture(scope="module")
+def force(tmp_path_factory):
+    return build(tmp_path_factory, "fixed_point_check.cpp")
+
+
+@pytest.mark.parametrize("stretch", [2.8, 4.0, 8.0, 15.9, 16.1, 16.3, 17.0, 18.0, 20.0, 23.8])
+@pytest.mark.parametrize("component", [0, 1, 2])
+def test_stretch_across_the_format_is_reported(force, stretch, component):
+    """One component of an element spreads over up to 24 edges, half of it on either side of the origin (so that every
+    node is inside the format's 12 edges): out of range for every amount, direction and sign."""
+    lam, mu = W.lame(1e9, 0.25)
+    lines = []
+    for axis in range(3):
+        for sign in (-1.0, 1.0):
+            u = np.zeros((3, 8))
+            u[component] = H * sign * stretch * (CORNERS[:, axis] - 0.5)
+            lines.append(((H, lam, mu), u))
+    assert (force(lines)[:, 0] == 0).all()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("dims", [(6, 5, 4), (41, 41, 41)])   # 8 lanes and one thread per element
+@pytest.mark.parametrize("stretch", [2.9, 16.3, 17.0, 23.0])
+def test_stretched_layer_matches_torch(dims, stretch):
+    """A layer of elements stretched by 2.9 to 23 edges along x (u split evenly about 0); the rest moves rigidly with a
+    hundredth of an edge of noise.  The reference rounds grad u at 2^-53 of u / h (up to 12) on strains of 1e-2, so
+    1e-12 (1 + 100 stretch / 2) relative to the force of the unstretched part."""
+    import torch
+
+    from paper_2511_20687_gb300 import osam
+    from tests.test_integer_elements import reference
+    g = torch.Generator(device="cuda").manual_seed(3)
+    nn = [d + 1 for d in dims]
+    ne = dims[0] * dims[1] * dims[2]
+    u = H * 0.01 * (torch.rand(nn[2], nn[1], nn[0], 3, generator=g, device="cuda", dtype=torch.float64) - 0.5)
+    cut = dims[0] // 2
+    u[:, :, :cut + 1, 0] -= 0.5 * stretch * H
+    u[:, :, cut + 1:, 0] += 0.5 * stretch * H
+    u = u.reshape(-1, 3).contiguous()
+    f = torch.empty_like(u)
+    osam.hex8_force(dims, H, "nh", 4e8, 4e8, u, f)
+    full = lambda v: torch.full((ne,), v, device="cuda", dtype=torch.float64)  # noqa: E731
+    r = reference(torch, dims, H, "nh", full(4e8), full(4e8), u)
+    assert torch.isfinite(r).all()
+    x = torch.arange(nn[0], device="cuda").repeat(nn[1] * nn[2])
+    for part in ((x == cut) | (x == cut + 1), (x < cut) | (x > cut + 1)):
+        assert (f - r)[part].norm() <= 1e-12 * (1 + 50 * stretch) * r[part].norm()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n,nz", [(4, 8), (26, 26)])   # 8 lanes and one thread per element
+def test_step_with_a_stretched_layer(n, nz):
+    """The explicit step across the same kind of layer against the FP64 kernels (rounding of a step: 1e-12; the
+    stretched elements carry almost all of the force, so both paths round the same FP64 formula there)."""
+    from paper_2511_20687_gb300 import osam
+    p = W.single_bar("stretched", n, nz, "nh", 1e9, 0.25, 1000.0, 1e-3, 1e-6, 2)
+    sd = p.subdomains[0]
+    sd.dirichlet = None
+    k = np.arange(nz + 1).repeat((n + 1) ** 2)
+    sd.u0 = W.random_field(sd.n_nodes, 1e-5, 3)
+    sd.u0[:, 2] += np.where(k <= nz // 2, -0.5, 0.5) * 16.3 * sd.h
+    a, b = osam.Problem(p), osam.Problem(p, scatter=osam.SCATTER_GATHER)
+    a.step()
+    b.step()
+    for f in range(3):
+        x, y = a.state(0)[f], b.state(0)[f]
+        assert np.linalg.norm(x - y) <= 1e-12 * np.linalg.norm(y)
