@@ -736,6 +736,33 @@ OSAM_HD int factor_exponent(double a, double b) {
 }
 OSAM_HD i64 factor_value(double x, int e) { return shl(block_value(x, e), 3); }
 
+// Material factors kappa/2 and mu times w as integers: value = X 2^(k - 62), the larger in [2^61, 2^62);
+// false unless both are positive and finite
+struct Material {
+    D kap2, mu, mu3;
+    int k;
+};
+OSAM_HD bool material(double lam, double mu, double w, Material& M) {
+    const int e = factor_exponent(lam, mu), ew = factor_exponent(w, 0.0);
+    const i64 l = factor_value(lam, e), m = factor_value(mu, e);
+    const D wd = split(factor_value(w, ew));
+    const i64 K = mul(split((l >> 1) + mul_third(m)), wd), U = mul(split(m), wd);
+    if (e == 2047 || ew == 2047 || ew == 0 || K <= 0 || U <= 0) return false;
+    const int n = lead_zeros(K | U) - 2;
+    const i64 us = shl(U, n);
+    M.kap2 = split(shl(K, n));
+    M.mu = split(us);
+    M.mu3 = split(mul_third(us));
+    M.k = e + ew - 2042 - n;     // 2 x 1084 - 64 - 62
+    return true;
+}
+
+// An element's forces are computed in its own unit 2^k and kept in the buffer's unit 2^top (one per mesh, so that a
+// node sums integers).  Down to kMaxDown binades below it they are rounded to that unit: 2^-54 of it is then still
+// below the FP64 formula's error (contrast 8 at a strain of 1e-3: 1.7e-13 of the force, FP64 3.9e-13); a softer element
+// keeps its own rounding and is held in FP64.
+constexpr int kMaxDown = 3;
+
 // ---- linear elasticity ---------------------------------------------------------------------------
 // Element force of isotropic linear elasticity in the Walsh basis of the 8 corners.  With raw Walsh
 // coefficients w_S of the nodal values (S a set of axes: signs of those axes), the 2x2x2 Gauss sums of

@@ -4,7 +4,7 @@
 // predicted displacement read as fixed-point u / h (written by the node kernel), the element forces left
 // as 64-bit integers in the element buffer, so the node kernel's sums are exact and cost integer
 // additions.  An element outside the range of the formats is evaluated in FP64 (far_element) into a second
-// buffer and marked in the first.
+// buffer and marked in the first; so is the integer result of an element too soft for the buffer's unit (kMaxDown).
 //
 // k_force_fx_b is bound by the integer multiply-add pipe: ncu counts 1969 instructions on it and 2994 on
 // the integer ALU per warp, against 717 FP64 instructions (67 to 80 cycles each) of the tiled FP64 kernel.
@@ -30,17 +30,14 @@ namespace {
 
 using namespace fx;
 
-// Fixed-point material factor of a positive FP64 value below 2^k (62 fraction bits of value / 2^k)
-__device__ __forceinline__ i64 fixed_factor(double m, int k) {
-    const unsigned long long b = (unsigned long long)__double_as_longlong(m);
-    const int s = (int)(b >> 52) - 1023 - k + 10;    // 62 - 52 bits, scaled by 2^(e - k)
-    const i64 v = (i64)((b & 0xfffffffffffffULL) | 0x10000000000000ULL);
-    if (s >= 0) return shl(v, s);
-    return s < -53 ? 0 : (v + ((i64)1 << (-s - 1))) >> -s;
+// A contribution held in FP64: it goes to fe2, the fixed-point buffer gets the mark
+__device__ __forceinline__ void put_f64(const FomB& g, const InstFom& I, int e, int c8, int c, double v) {
+    const long long d = (long long)(c8 * 3 + c) * g.NE + I.elem_off + e;
+    static_cast<i64*>(g.fe)[d] = kBadF;
+    g.fe2[d] = v;
 }
 
-// Element e in FP64: its 24 contributions go to fe2, the fixed-point buffer gets the mark.  Not inlined,
-// so that its registers and code stay out of the fixed-point path.
+// Element e in FP64.  Not inlined, so that its registers and code stay out of the fixed-point path.
 __device__ __noinline__ void far_element(const FomB& g, const InstFom& I, const double* u, int e, int n0) {
     using namespace hex8;
     const int sy = I.nx + 1, sz = (I.nx + 1) * (I.ny + 1);
@@ -59,15 +56,10 @@ __device__ __noinline__ void far_element(const FomB& g, const InstFom& I, const 
         edge_differences<double>(U, I.invh, Dx[c], Dy[c], Dz[c]);
     }
     element_force<OSAM_NEO_HOOKEAN, double>(Dx, Dy, Dz, m1, m2, m3, F);
-    i64* fe = static_cast<i64*>(g.fe) + I.elem_off + e;
-    double* fe2 = g.fe2 + I.elem_off + e;
 #pragma unroll
     for (int c8 = 0; c8 < 8; ++c8)
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            fe[(long long)(c8 * 3 + c) * g.NE] = kBadF;
-            fe2[(long long)(c8 * 3 + c) * g.NE] = F[c][c8];
-        }
+        for (int c = 0; c < 3; ++c) put_f64(g, I, e, c8, c, F[c][c8]);
 }
 
 __global__ void __launch_bounds__(128) k_force_fx_b(const __grid_constant__ FomB g, const int* __restrict__ active,
@@ -100,18 +92,34 @@ __global__ void __launch_bounds__(128) k_force_fx_b(const __grid_constant__ FomB
         w[c] = walsh_in(V, c);
     }
     i64 kap2 = I.fk2, mu = I.fmu;
+    int down = 0;   // binades of the element's unit below the mesh's
     if (I.lam_e || I.mu_e) {
-        const double le = I.lam_e ? I.lam_e[e] : I.lam, me = I.mu_e ? I.mu_e[e] : I.mu;
-        double m1, m2, m3;
-        hex8::material_factors<OSAM_NEO_HOOKEAN, double>(le, me, I.wq, I.wq3, m1, m2, m3);
-        kap2 = fixed_factor(m1, kFracOut - I.fscale);
-        mu = fixed_factor(m2, kFracOut - I.fscale);
+        Material M;
+        bad |= !material(I.lam_e ? I.lam_e[e] : I.lam, I.mu_e ? I.mu_e[e] : I.mu, I.wq, M);
+        kap2 = whole(M.kap2);
+        mu = whole(M.mu);
+        down = kFracOut - I.fscale - M.k;
+        bad |= down < 0 || M.k < -900;
     }
     i64 F[3][8];
     bad |= !element_force_nh(w, kap2, mu, mul_third(mu), F);
     if (bad) {
         far_element(g, I, u, e, n0);
         return;
+    }
+    if (down > kMaxDown) {
+#pragma unroll
+        for (int c8 = 0; c8 < 8; ++c8)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) put_f64(g, I, e, c8, c, f64_scaled(F[c][c8], I.fscale + down));
+        return;
+    }
+    if (down) {
+        const i64 half = (i64)1 << (down - 1);
+#pragma unroll
+        for (int c8 = 0; c8 < 8; ++c8)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) F[c][c8] = (F[c][c8] + half) >> down;
     }
     i64* fe = static_cast<i64*>(g.fe) + I.elem_off + e;
 #pragma unroll
@@ -140,21 +148,26 @@ __global__ void __launch_bounds__(128, 5) k_force_fx_lanes_b(const __grid_consta
     for (int c = 0; c < 3; ++c) U[c] = g.ux[c * g.NN + gn];
     D kap2 = split(I.fk2), mu = split(I.fmu), mu3 = split(mul_third(I.fmu));
     bool bad = false;
-    if (I.lam_e || I.mu_e) {   // the element's factors in units of the instance's scale, which is at least theirs
+    int down = 0;
+    if (I.lam_e || I.mu_e) {
         Material M;
-        const int top = kFracOut - I.fscale;
-        bad = !material(I.lam_e ? I.lam_e[e] : I.lam, I.mu_e ? I.mu_e[e] : I.mu, I.wq, M) || M.k > top;
-        const i64 m = shift(whole(M.mu), M.k - top);
-        kap2 = split(shift(whole(M.kap2), M.k - top));
-        mu = split(m);
-        mu3 = split(mul_third(m));
+        bad = !material(I.lam_e ? I.lam_e[e] : I.lam, I.mu_e ? I.mu_e[e] : I.mu, I.wq, M);
+        kap2 = M.kap2;
+        mu = M.mu;
+        mu3 = M.mu3;
+        down = kFracOut - I.fscale - M.k;
+        bad |= down < 0 || M.k < -900;
     }
     const bool ok = force_lanes(L, U, kap2, mu, mu3, bad, F);
     if (first >= I.ne) return;
-    if (ok) {
-        i64* fe = static_cast<i64*>(g.fe) + I.elem_off + e;
+    if (ok && down > kMaxDown) {
 #pragma unroll
-        for (int c = 0; c < 3; ++c) fe[(long long)(L.a * 3 + c) * g.NE] = (F[c] + 4) >> 3;   // 57 to 54 fraction bits
+        for (int c = 0; c < 3; ++c) put_f64(g, I, e, L.a, c, f64_scaled(F[c], I.fscale + down + 3));   // 57 fraction bits
+    } else if (ok) {
+        i64* fe = static_cast<i64*>(g.fe) + I.elem_off + e;
+        const int n = 3 + down;   // 57 to 54 fraction bits
+#pragma unroll
+        for (int c = 0; c < 3; ++c) fe[(long long)(L.a * 3 + c) * g.NE] = (F[c] + ((i64)1 << (n - 1))) >> n;
     } else if (L.a == 0) {
         far_element(g, I, u, e, n0);
     }

@@ -193,27 +193,6 @@ __device__ __forceinline__ bool force_svk_lanes(const Lane& L, const double p[3]
     return !any_lane(bad || e == 2047 || scale > 1000 || scale < -900);
 }
 
-// Material factors kappa/2 and mu times w as integers: value = X 2^(k - 62), the larger in [2^61, 2^62);
-// false unless both are positive and finite
-struct Material {
-    D kap2, mu, mu3;
-    int k;
-};
-__device__ __forceinline__ bool material(double lam, double mu, double w, Material& M) {
-    const int e = factor_exponent(lam, mu), ew = factor_exponent(w, 0.0);
-    const i64 l = factor_value(lam, e), m = factor_value(mu, e);
-    const D wd = split(factor_value(w, ew));
-    const i64 K = mul(split((l >> 1) + mul_third(m)), wd), U = mul(split(m), wd);
-    if (e == 2047 || ew == 2047 || ew == 0 || K <= 0 || U <= 0) return false;
-    const int n = lead_zeros(K | U) - 2;
-    const i64 us = shl(U, n);
-    M.kap2 = split(shl(K, n));
-    M.mu = split(us);
-    M.mu3 = split(mul_third(us));
-    M.k = e + ew - 2042 - n;     // 2 x 1084 - 64 - 62
-    return true;
-}
-
 // corner forces of the lane's corner (57 fraction bits, units 2^k); false if the element is out of range
 // (lin: also the linearisation of the lane's Gauss point)
 __device__ __forceinline__ bool force_lanes(const Lane& L, const i64 U[3], D kap2, D mu, D mu3, bool bad, i64 F[3],

@@ -108,23 +108,24 @@ int set_eblocks(osam_ctx* ctx, FomGroupH& G, int block) {
 // Neo-Hookean law linearises to the same lambda, mu).  A relative allowance of 1e-9 keeps a step that
 // sits exactly on the limit.
 int check_stability(osam_ctx* ctx, FomGroupH& G, int s, int n, const osam_problem_desc* descs,
-                    std::vector<double>& modulus) {
-    unsigned long long* mod = ctx->alloc<unsigned long long>(n);
+                    std::vector<double>& factor) {
+    unsigned long long* mod = ctx->alloc<unsigned long long>(2 * n);   // also max(kappa / 2, mu), into factor
     int* bad = ctx->alloc<int>(1);
     CKA(mod); CKA(bad);
-    CK(cudaMemsetAsync(mod, 0, sizeof(unsigned long long) * n, ctx->stream));
+    CK(cudaMemsetAsync(mod, 0, sizeof(unsigned long long) * 2 * n, ctx->stream));
     CK(cudaMemsetAsync(bad, 0, sizeof(int), ctx->stream));
     CK(launch_cfl_modulus(G.d, mod, bad, ctx->stream));
     std::vector<unsigned long long> mh;
     std::vector<int> bh;
-    RET(to_host(ctx, mh, mod, n));
+    RET(to_host(ctx, mh, mod, 2 * n));
     RET(to_host(ctx, bh, bad, 1));
     if (bh[0]) return ctx->fail(OSAM_EINVAL, "subdomain %d: material not positive definite (mu > 0 and "
                                              "3 lambda + 2 mu > 0 required)", s);
+    factor.resize(n);
+    std::memcpy(factor.data(), mh.data() + n, sizeof(double) * n);
     for (int i = 0; i < n; ++i) {
         double m;
         std::memcpy(&m, &mh[i], sizeof(double));
-        modulus.push_back(m);
         const double lim = G.grid[i].h * std::sqrt(descs[i].subdomains[s].rho / m);
         const double dt = ctx->slots[s].dt;
         if (!G.d.implicit && dt > lim * (1.0 + 1e-9))
@@ -151,11 +152,11 @@ int set_tiles(osam_ctx* ctx, FomGroupH& G) {
     return OSAM_OK;
 }
 
-// Scales of the fixed-point force of one Neo-Hookean instance.  The unit of its element forces is the
-// power of two at or above the largest material factor: of the uniform kappa/2 and mu, or, with
-// per-element parameters, of mu <= modulus / 2 (modulus = max(3 lambda + 2 mu, 2 mu) >= 6 kappa/2).
-void fixed_point_scales(InstFom& I, double modulus) {
-    const double top = I.lam_e || I.mu_e ? 0.5 * modulus * I.wq : std::max(I.m1, I.m2);
+// Scales of the fixed-point force of one Neo-Hookean instance.  The unit of its element buffer is the power of two
+// above the largest material factor: of the uniform kappa/2 and mu, or, with per-element parameters, of factor =
+// max_e max(kappa_e / 2, mu_e), raised by a few roundings so that no element's own unit lies above it.
+void fixed_point_scales(InstFom& I, double factor) {
+    const double top = I.lam_e || I.mu_e ? factor * I.wq * (1.0 + 0x1p-48) : std::max(I.m1, I.m2);
     int k;
     std::frexp(top, &k);
     I.fscale = 54 - k;
@@ -309,10 +310,10 @@ int setup_fom_group(osam_ctx* ctx, FomGroupH& G, int s, int n, const osam_proble
     if (B.implicit) CKA(B.ipart = ctx->alloc<double>(6LL * B.n_nblk));
     RET(set_eblocks(ctx, G, 128));
     RET(set_tiles(ctx, G));
-    std::vector<double> modulus;
-    RET(check_stability(ctx, G, s, n, descs, modulus));
+    std::vector<double> factor;
+    RET(check_stability(ctx, G, s, n, descs, factor));
     if (B.fixed == 1) {
-        for (int i = 0; i < n; ++i) fixed_point_scales(G.inst[i], modulus[i]);
+        for (int i = 0; i < n; ++i) fixed_point_scales(G.inst[i], factor[i]);
         RET(upload(ctx, G.inst_d, G.inst.data(), sizeof(InstFom) * n));
     }
     if (B.df32 || B.fp32) CK(launch_split_u2_b(B, ctx->stream));
