@@ -41,7 +41,7 @@ constexpr int kFracM = 62;    // material factors in units of the instance's sca
 constexpr int kFracOut = 54;  // element forces in units of the instance's scale
 constexpr int kMaxU = 12;     // largest |u| / h of the fixed format
 constexpr i64 kBadU = (i64)1 << 63;    // stored for a node outside it (-16)
-constexpr i64 kBadF = (i64)1 << 63;    // stored for an element force that is held in FP64 instead
+constexpr i64 kBadF = (i64)1 << 63;    // stored linearisation of a Gauss point outside the range
 
 struct D {
     int h, l;
@@ -974,6 +974,35 @@ OSAM_HD float f32_scaled(i64 x, int scale) {
     __builtin_memcpy(&r, &b, 4);
 #endif
     return r;
+}
+
+// An element buffer entry is an integer force (below 2^60: four equal leading bits) or, for an element outside the
+// integer path, the FP64 force itself: its leading bits differ for every value in -2^769 .. 2^-767 and 2^-767 .. inf
+// and for NaN.  The others have codes: zero (and what rounds to it, below 2^-767) is stored as -0, -inf (and what
+// lies below -2^769) as a NaN of its own.  A group whose unit is outside 2^+-kMaxUnit does not take this buffer.
+constexpr int kMaxUnit = 500;
+constexpr i64 kMinusInf = 0x7ff8000000000002LL;
+OSAM_HD bool held_f64(i64 x) { return (unsigned int)((hi(x) >> 28) + 1) > 1u; }
+OSAM_HD i64 hold_f64(double v) {
+    i64 b;
+#ifdef __CUDA_ARCH__
+    b = __double_as_longlong(v);
+#else
+    __builtin_memcpy(&b, &v, 8);
+#endif
+    if (held_f64(b)) return b;
+    if (b >= 0) return (i64)1 << 63;
+    return shl(b, 1) > shl(0x7ff0000000000000LL, 1) ? 0x7ff8000000000000LL : kMinusInf;   // NaN, or -2^769 and below
+}
+OSAM_HD double f64_held(i64 b) {
+    if (b == kMinusInf) b = (i64)0xfff0000000000000ULL;
+    double v;
+#ifdef __CUDA_ARCH__
+    v = __longlong_as_double(b);
+#else
+    __builtin_memcpy(&v, &b, 8);
+#endif
+    return v;
 }
 
 // fixed-point u / h of a nodal displacement: mantissa (53 bits) times the 63-bit mantissa of 1/h, shifted

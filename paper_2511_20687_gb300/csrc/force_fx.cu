@@ -3,8 +3,8 @@
 // The force of the FP64 explicit path when the launch is left to the library: one thread per element, the
 // predicted displacement read as fixed-point u / h (written by the node kernel), the element forces left
 // as 64-bit integers in the element buffer, so the node kernel's sums are exact and cost integer
-// additions.  An element outside the range of the formats is evaluated in FP64 (far_element) into a second
-// buffer and marked in the first; so is the integer result of an element too soft for the buffer's unit (kMaxDown).
+// additions.  An element outside the range of the formats is evaluated in FP64 (far_element), and its entries hold
+// the FP64 values (hold_f64); so do those of an element too soft for the buffer's unit (kMaxDown).
 //
 // k_force_fx_b is bound by the integer multiply-add pipe: ncu counts 1969 instructions on it and 2994 on
 // the integer ALU per warp, against 717 FP64 instructions (67 to 80 cycles each) of the tiled FP64 kernel.
@@ -30,11 +30,9 @@ namespace {
 
 using namespace fx;
 
-// A contribution held in FP64: it goes to fe2, the fixed-point buffer gets the mark
+// A contribution held in FP64 in its entry of the buffer
 __device__ __forceinline__ void put_f64(const FomB& g, const InstFom& I, int e, int c8, int c, double v) {
-    const long long d = (long long)(c8 * 3 + c) * g.NE + I.elem_off + e;
-    static_cast<i64*>(g.fe)[d] = kBadF;
-    g.fe2[d] = v;
+    static_cast<i64*>(g.fe)[(long long)(c8 * 3 + c) * g.NE + I.elem_off + e] = hold_f64(v);
 }
 
 // Element e in FP64.  Not inlined, so that its registers and code stay out of the fixed-point path.
@@ -231,7 +229,7 @@ __global__ void __launch_bounds__(kNodeBlock) k_node_fx_b(const __grid_constant_
                     i64 x[NC];
 #pragma unroll
                     for (int q = 0; q < NC; ++q) x[q] = __ldg(fe + (long long)(corner * 3 + c0 + q) * g.NE + e);
-                    if (x[0] == kBadF) { far |= 1u << corner; continue; }
+                    if (held_f64(x[0])) { far |= 1u << corner; continue; }
 #pragma unroll
                     for (int q = 0; q < NC; ++q) s[q] += x[q];
                 }
@@ -245,7 +243,7 @@ __global__ void __launch_bounds__(kNodeBlock) k_node_fx_b(const __grid_constant_
             const long long e = (i - (corner & 1)) +
                                 (long long)nx * ((j - ((corner >> 1) & 1)) + ny * (k - (corner >> 2)));
 #pragma unroll
-            for (int q = 0; q < NC; ++q) f[q] += g.fe2[(long long)(corner * 3 + c0 + q) * g.NE + I.elem_off + e];
+            for (int q = 0; q < NC; ++q) f[q] += f64_held(fe[(long long)(corner * 3 + c0 + q) * g.NE + e]);
         }
     }
 #pragma unroll

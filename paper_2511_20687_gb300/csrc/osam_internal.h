@@ -132,8 +132,7 @@ struct FomB {
     int df32;                 // 1: internal force in double-float arithmetic (element buffer of float2)
     int fixed;                // internal force in 64-bit integers: 1 Neo-Hookean (element buffer of int64; force_fx.cu),
                               // 2 linear elastic, 3 Saint Venant-Kirchhoff (element buffer of double; force_le.cu, force_svk.cu)
-    long long* ux;            // fixed-point predicted displacement / h [3][NN]
-    double* fe2;              // FP64 contributions of the elements outside the fixed-point range [24][NE]
+    long long* ux;            // fixed-point predicted displacement / h [3][NN], in the memory of us
 };
 
 // A node kernel takes one thread per node and component instead of one per node while that leaves it

@@ -10,6 +10,7 @@
 #include <vector>
 
 #include "ctx.h"
+#include "fixed_math.cuh"
 
 namespace osam {
 namespace host {
@@ -155,13 +156,15 @@ int set_tiles(osam_ctx* ctx, FomGroupH& G) {
 // Scales of the fixed-point force of one Neo-Hookean instance.  The unit of its element buffer is the power of two
 // above the largest material factor: of the uniform kappa/2 and mu, or, with per-element parameters, of factor =
 // max_e max(kappa_e / 2, mu_e), raised by a few roundings so that no element's own unit lies above it.
-void fixed_point_scales(InstFom& I, double factor) {
+// False for a unit so small or large that the buffer's FP64 entries would leave their range.
+bool fixed_point_scales(InstFom& I, double factor) {
     const double top = I.lam_e || I.mu_e ? factor * I.wq * (1.0 + 0x1p-48) : std::max(I.m1, I.m2);
     int k;
     std::frexp(top, &k);
     I.fscale = 54 - k;
     I.fk2 = std::llrint(std::ldexp(I.m1, 62 - k));
     I.fmu = std::llrint(std::ldexp(I.m2, 62 - k));
+    return std::abs(k) <= fx::kMaxUnit;
 }
 
 int setup_fom_group(osam_ctx* ctx, FomGroupH& G, int s, int n, const osam_problem_desc* descs) {
@@ -224,12 +227,6 @@ int setup_fom_group(osam_ctx* ctx, FomGroupH& G, int s, int n, const osam_proble
         B.fixed = 1;
     else if (integers && fp64 && B.material != OSAM_NEO_HOOKEAN)
         B.fixed = B.material == OSAM_LINEAR_ELASTIC ? 2 : 3;
-    B.df32 = ctx->precision == OSAM_F32X2_FORCE && !B.fixed;
-    if (B.df32 || B.fp32) CKA(B.u2 = ctx->alloc<float2>(3 * NN));   // the FP32 forces' split of u/h
-    if (B.fixed == 1) {
-        CKA(B.ux = ctx->alloc<long long>(3 * NN));
-        CKA(B.fe2 = ctx->alloc<double>(24 * NE));
-    }
     if (B.implicit) {
         ctx->any_implicit = true;
         CKA(B.ut = ctx->alloc<double>(3 * NN));
@@ -313,9 +310,15 @@ int setup_fom_group(osam_ctx* ctx, FomGroupH& G, int s, int n, const osam_proble
     std::vector<double> factor;
     RET(check_stability(ctx, G, s, n, descs, factor));
     if (B.fixed == 1) {
-        for (int i = 0; i < n; ++i) fixed_point_scales(G.inst[i], factor[i]);
+        // us holds u / h in FP64 for the initial force and after a change of state, and the fixed-point predictor,
+        // which the node kernel writes before every force of a step
+        B.ux = reinterpret_cast<long long*>(B.us);
+        for (int i = 0; i < n; ++i)
+            if (!fixed_point_scales(G.inst[i], factor[i])) B.fixed = 0;
         RET(upload(ctx, G.inst_d, G.inst.data(), sizeof(InstFom) * n));
     }
+    B.df32 = ctx->precision == OSAM_F32X2_FORCE && !B.fixed;
+    if (B.df32 || B.fp32) CKA(B.u2 = ctx->alloc<float2>(3 * NN));   // the FP32 forces' split of u/h
     if (B.df32 || B.fp32) CK(launch_split_u2_b(B, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
     return OSAM_OK;

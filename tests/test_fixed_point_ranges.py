@@ -141,3 +141,78 @@ def test_step_of_a_soft_and_a_stiff_half(n, nz, contrast, precision):
     kn = np.arange(nz + 1).repeat((n + 1) ** 2)
     for half in (kn < nz // 2, kn > nz // 2):
         assert np.linalg.norm((x - y)[half]) <= 2e-12 * np.linalg.norm(y[half])
+
+
+def test_buffer_entry_holds_either_kind(tmp_path):
+    """Integers below 2^60 and FP64 values share an entry: every value comes back, zero and -inf through their codes."""
+    if shutil.which("g++") is None:
+        pytest.skip("needs g++")
+    (tmp_path / "held.cpp").write_text("""
+#include <cmath>
+#include <cstdio>
+#include <initializer_list>
+#include <limits>
+#include "fixed_math.cuh"
+using namespace osam::fx;
+int main() {
+    const double inf = std::numeric_limits<double>::infinity(), nan = std::numeric_limits<double>::quiet_NaN();
+    int bad = 0;
+    for (int e = -766; e < 769; ++e)
+        for (double m : {1.0, 1.25, 2.0 - 0x1p-52})
+            for (double s : {-1.0, 1.0}) {
+                const double v = std::ldexp(s * m, e);
+                bad += !held_f64(hold_f64(v)) || f64_held(hold_f64(v)) != v;
+            }
+    for (double v : {0.0, -0.0, inf, -inf, -0x1p-900, 0x1p1000, -0x1p768})
+        bad += !held_f64(hold_f64(v)) || f64_held(hold_f64(v)) != v;
+    for (double v : {nan, -nan}) bad += !held_f64(hold_f64(v)) || !std::isnan(f64_held(hold_f64(v)));
+    bad += f64_held(hold_f64(0x1p-800)) != 0.0 || f64_held(hold_f64(-0x1p900)) != -inf;
+    for (int n = 0; n < 60; ++n)
+        for (i64 x : {(i64)1 << n, ((i64)1 << n) - 1, ((i64)2 << n) - 1, (i64)0x123456789abcdefLL >> n})
+            bad += held_f64(x) || held_f64(-x) || held_f64(~x);
+    std::printf("%d\\n", bad);
+}
+""")
+    exe = str(tmp_path / "held")
+    subprocess.run(["g++", "-O2", "-std=c++17", "-x", "c++", "-I", os.path.join(ROOT, "paper_2511_20687_gb300/csrc"), "-o",
+                    exe, str(tmp_path / "held.cpp")], check=True)
+    assert subprocess.run([exe], capture_output=True, text=True, check=True).stdout.strip() == "0"
+
+
+@pytest.mark.gpu
+def test_fixed_point_group_takes_no_more_memory():
+    """The default explicit group holds its element forces and predictor in the FP64 group's buffers."""
+    import torch
+
+    from paper_2511_20687_gb300 import osam
+    p = W.single_bar("memory", 40, 80, "nh", 1e9, 0.25, 1000.0, 1e-3, 1e-7, 2)
+
+    def taken(**kw):
+        torch.cuda.synchronize()
+        before = torch.cuda.mem_get_info()[0]
+        q = osam.Problem(p, **kw)
+        torch.cuda.synchronize()
+        used = before - torch.cuda.mem_get_info()[0]
+        q.close()
+        return used
+
+    taken()                                       # one-time allocations of the library
+    gather = taken(scatter=osam.SCATTER_GATHER)
+    assert taken() <= gather + (4 << 20)          # the tuner's block lists; a second buffer would be 24 MB
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("scale", [1e-170, 1.0, 1e160])
+def test_units_outside_the_buffers_range(scale):
+    """Moduli and density scaled together leave the motion as it is; 1e-170 and 1e160 take the FP64 kernels."""
+    from paper_2511_20687_gb300 import osam
+    out = []
+    for s, mode in ((scale, osam.SCATTER_AUTO), (1.0, osam.SCATTER_GATHER)):
+        p = W.single_bar("units", 4, 8, "nh", 1e9, 0.25, 1000.0, 1e-3, 1e-6, 4)
+        sd = p.subdomains[0]
+        sd.lam, sd.mu, sd.rho = sd.lam * s, sd.mu * s, sd.rho * s
+        q = osam.Problem(p, scatter=mode)
+        q.step()
+        out.append(q.state(0))
+    for x, y in zip(*out):
+        assert np.linalg.norm(x - y) <= 1e-12 * np.linalg.norm(y)
