@@ -16,7 +16,8 @@
 // intermediate sums may wrap as long as the result fits).
 //
 // Range (checked per element; an element outside is evaluated in FP64 by the caller): |u| / h below
-// kMaxU at every node, the spread of each displacement component over the element below 2.75 edges, column
+// kMaxU at every node, the spread of each displacement component over the element (the kernels with a corner per lane:
+// along each of its edges) below 2.75 edges, column
 // norms of F at the Gauss points below 1.5 (any rotation, 50% stretch), J in (0.53, 1.98), |beta| < 4
 // and pair sums of P below 2 in units of the instance's material scale.  Every intermediate then fits
 // its format; the bounds are at each step.
@@ -182,6 +183,15 @@ OSAM_HD bool spread_bad(const i64 V[8]) {
         mn = imin(mn, hi(V[k]));
     }
     return mn < -((kMaxU + 1) << 27) || (unsigned int)mx - (unsigned int)mn >= 11u << 25;
+}
+
+// The same for the kernels with a corner per lane, from the high words of two corners joined by an edge: further apart
+// than 2.75 edges.  With all 12 edges below it a Walsh coefficient (a signed sum of four edge differences) is below 11,
+// and an entry of F at a Gauss point (1 or 0 plus a mean of four) below 3.75.  The difference is taken modulo 32 edges:
+// values within +-12 that are further apart than 2.75 are also seen apart.
+OSAM_HD bool edge_bad(int a, int b) {
+    const int d = (int)((unsigned int)a - (unsigned int)b);
+    return (d ^ (d >> 31)) >= 11 << 25;
 }
 
 // Walsh coefficients of one component of u / h (59 fraction bits) and their multiples that the Gauss

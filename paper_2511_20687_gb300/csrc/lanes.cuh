@@ -77,19 +77,15 @@ __device__ __forceinline__ T reduce8(T x, Op op) {
     return x;
 }
 
-// Columns of F from this lane's fixed-point u / h (59 fraction bits); bad: a node outside the format, or a Walsh
-// coefficient at or above 11 (found from the values cut to 23 fraction bits, which cannot wrap)
+// Columns of F from this lane's fixed-point u / h (59 fraction bits); bad: a node outside the format, or an edge of the
+// element out of range (edge_bad)
 __device__ __forceinline__ void deformation(const Lane& L, const i64 U[3], Cols& C, bool& bad) {
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-        bad |= hi(U[c]) < -((kMaxU + 1) << 27);
-        int v = hi(U[c]) >> 4;
+        const int v = hi(U[c]);
+        bad |= v < -((kMaxU + 1) << 27);
 #pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            const int o = __shfl_xor_sync(0xffffffffu, v, 1 << d), n = (int)L.n[d];
-            v += (o ^ n) - n;
-        }
-        bad |= L.a != 0 && (v >= (11 << 23) || v <= -(11 << 23));
+        for (int d = 0; d < 3; ++d) bad |= edge_bad(v, __shfl_xor_sync(0xffffffffu, v, 1 << d));
         i64 w = walsh_sums(L, U[c]);
         if (L.a == 1 << c) w += (i64)1 << kFracF;
         gauss_columns(L, pattern_scale(L, L.a ? w : 0), c, C);

@@ -216,3 +216,34 @@ def test_units_outside_the_buffers_range(scale):
         out.append(q.state(0))
     for x, y in zip(*out):
         assert np.linalg.norm(x - y) <= 1e-12 * np.linalg.norm(y)
+
+
+@pytest.fixture(scope="module")
+def lanes(tmp_path_factory):
+    return build(tmp_path_factory, "lane_range_check.cpp")
+
+
+def test_lane_range_check_bounds_every_intermediate(lanes):
+    """Whatever passes the lane kernels' check keeps its Walsh coefficients below 11 and its gradients below 3.75, so no
+    64-bit value wraps; elements that wrap are refused, among them one corner pulled out by 10.9 edges (coefficients
+    of 10.9, a gradient of 7.8 in a format that ends at 4) and components spread over up to 24 edges."""
+    rng = np.random.default_rng(12)
+    lines = []
+    for _ in range(4000):   # corners reached by steps of up to 2.8 edges along random paths: many at the limit
+        size = rng.choice([0.5, 2.0, 2.74, 2.8, 6.0, 12.0])
+        v = np.zeros(8)
+        for a in range(1, 8):
+            near = [v[a ^ d] for d in (1, 2, 4) if a & d]
+            v[a] = np.mean([max(near), min(near)]) + size * rng.choice([-1, 1]) * rng.choice([1.0, rng.uniform()])
+        lines.append((np.clip(v - 0.5 * (v.max() + v.min()), -11.99, 11.99),))
+    for corner in range(8):
+        for x in (-10.9, 10.9):
+            lines.append((np.eye(8)[corner] * x,))
+    for axis in range(3):
+        for x in (2.8, 8.0, 16.0, 20.0, 23.9):
+            lines.append((x * (CORNERS[:, axis] - 0.5),))
+    r = lanes(lines)
+    ok = r[:, 0] == 1
+    assert 500 < ok.sum() < 3900
+    assert (r[ok, 1] < 11.001).all() and (r[ok, 2] < 3.751).all() and not r[ok, 3].any()
+    assert r[~ok, 3].any() and not ok[4000:].any()
