@@ -16,7 +16,7 @@
 // intermediate sums may wrap as long as the result fits).
 //
 // Range (checked per element; an element outside is evaluated in FP64 by the caller): |u| / h below
-// kMaxU at every node, the spread of each displacement component over the element (the kernels with a corner per lane:
+// 2^22 at every node (from kMaxU on its nodal values are taken modulo 32 edges: refit), the spread of each displacement component over the element (the kernels with a corner per lane:
 // along each of its edges) below 2.75 edges, column
 // norms of F at the Gauss points below 1.5 (any rotation, 50% stretch), J in (0.53, 1.98), |beta| < 4
 // and pair sums of P below 2 in units of the instance's material scale.  Every intermediate then fits
@@ -41,7 +41,7 @@ constexpr int kFracF = 61;    // F at the Gauss points, range +-4
 constexpr int kFracM = 62;    // material factors in units of the instance's scale, at most 1
 constexpr int kFracOut = 54;  // element forces in units of the instance's scale
 constexpr int kMaxU = 12;     // largest |u| / h of the fixed format
-constexpr i64 kBadU = (i64)1 << 63;    // stored for a node outside it (-16)
+constexpr i64 kBadU = (i64)1 << 63;    // fixed_u of a node outside it (-16)
 constexpr i64 kBadF = (i64)1 << 63;    // stored linearisation of a Gauss point outside the range
 
 struct D {
@@ -190,8 +190,8 @@ OSAM_HD bool spread_bad(const i64 V[8]) {
 // and an entry of F at a Gauss point (1 or 0 plus a mean of four) below 3.75.  The difference is taken modulo 32 edges:
 // values within +-12 that are further apart than 2.75 are also seen apart.
 OSAM_HD bool edge_bad(int a, int b) {
-    const int d = (int)((unsigned int)a - (unsigned int)b);
-    return (d ^ (d >> 31)) >= 11 << 25;
+    constexpr unsigned int kEdge = 11u << 25;
+    return (unsigned int)a - (unsigned int)b + kEdge >= 2 * kEdge;
 }
 
 // Walsh coefficients of one component of u / h (59 fraction bits) and their multiples that the Gauss
@@ -1036,6 +1036,49 @@ OSAM_HD i64 fixed_u(double u, i64 ihm, int ihe) {
     else v = s > 62 ? 0 : (p + ((i64)1 << (s - 1))) >> s;
     if (v >= (i64)kMaxU << kFracU || v < 0) return kBadU;
     return (i64)b < 0 ? -v : v;
+}
+
+// The same for an element with a node beyond the format: u / h modulo 32 edges, so that differences inside the element
+// are exact while they stay below 16 edges, and with 8 fraction bits in `coarse`, which tells whether they do.  False
+// for |u| / h >= 2^22 and for non-finite values.
+constexpr int kCoarseSpread = 702;   // 2.75 edges, less the cut of two values
+OSAM_HD bool wrapped_u(double u, i64 ihm, int ihe, i64& v, int& coarse) {
+    unsigned long long b;
+#ifdef __CUDA_ARCH__
+    b = (unsigned long long)__double_as_longlong(u);
+#else
+    __builtin_memcpy(&b, &u, 8);
+#endif
+    v = coarse = 0;
+    const int e = (int)((b >> 52) & 0x7ff);
+    if (e == 0) return true;
+    const i64 p = mul((i64)(((b & 0xfffffffffffffULL) | 0x10000000000000ULL) << 10), ihm);
+    const int s = 1 - (e - 1023 + ihe);                       // u / h in [2^(1 - s), 2^(3 - s))
+    if (s < -19) return false;
+    if (s <= 0) v = shl(p, -s);
+    else v = s > 62 ? 0 : (p + ((i64)1 << (s - 1))) >> s;
+    coarse = s + 51 > 62 ? 0 : (int)(p >> (s + 51));
+    if ((i64)b < 0) {
+        v = (i64)(0ULL - (unsigned long long)v);
+        coarse = -coarse;
+    }
+    return true;
+}
+
+// one component of such an element: its 8 nodal values again; true if it is out of range all the same
+OSAM_HD bool refit(const double U[8], i64 ihm, int ihe, i64 V[8]) {
+    int mx = -0x7fffffff, mn = 0x7fffffff;
+    bool bad = false;
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+    for (int a = 0; a < 8; ++a) {
+        int x;
+        bad |= !wrapped_u(U[a], ihm, ihe, V[a], x);
+        mx = imax(mx, x);
+        mn = imin(mn, x);
+    }
+    return bad || mx - mn >= kCoarseSpread;                   // |x| < 2^30
 }
 
 }  // namespace fx

@@ -60,6 +60,22 @@ __device__ __noinline__ void far_element(const FomB& g, const InstFom& I, const 
         for (int c = 0; c < 3; ++c) put_f64(g, I, e, c8, c, F[c][c8]);
 }
 
+// In an instance with displacements beyond the format (g.wide) the nodal values are modulo 32 edges, and u itself tells
+// whether the element's differences are in range; its own function, away from the registers of the force
+__device__ __noinline__ bool torn_element(const FomB& g, const InstFom& I, const double* u, int n0) {
+    const int sy = I.nx + 1, sz = (I.nx + 1) * (I.ny + 1);
+    bool bad = false;
+    for (int c = 0; c < 3; ++c) {
+        const double* x = u + (long long)c * g.NN + I.node_off + n0;
+        double U[8];
+        i64 V[8];
+#pragma unroll
+        for (int c8 = 0; c8 < 8; ++c8) U[c8] = x[(c8 & 1) + ((c8 >> 1) & 1) * sy + (c8 >> 2) * sz];
+        bad |= refit(U, I.ihm, I.ihe, V);
+    }
+    return bad;
+}
+
 __global__ void __launch_bounds__(128) k_force_fx_b(const __grid_constant__ FomB g, const int* __restrict__ active,
                                                     const __grid_constant__ TraceFuse tr, const double* u) {
     if ((int)blockIdx.x >= g.n_eblk) {
@@ -78,15 +94,17 @@ __global__ void __launch_bounds__(128) k_force_fx_b(const __grid_constant__ FomB
     const int k = t / ny;
     const int sy = nx + 1, sz = (nx + 1) * (ny + 1);
     const int n0 = i + sy * j + sz * k;
-    WalshIn w[3];
+    const bool wide = g.wide[b.x] != 0;
     bool bad = false;
+    if (wide) bad = torn_element(g, I, u, n0);
+    WalshIn w[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
         const i64* x = g.ux + (long long)c * g.NN + I.node_off + n0;
         i64 V[8];
 #pragma unroll
         for (int c8 = 0; c8 < 8; ++c8) V[c8] = x[(c8 & 1) + ((c8 >> 1) & 1) * sy + ((c8 >> 2) & 1) * sz];
-        bad |= spread_bad(V);
+        bad |= spread_bad(V) && !wide;
         w[c] = walsh_in(V, c);
     }
     i64 kap2 = I.fk2, mu = I.fmu;
@@ -146,10 +164,19 @@ __global__ void __launch_bounds__(128, 5) k_force_fx_lanes_b(const __grid_consta
     for (int c = 0; c < 3; ++c) U[c] = g.ux[c * g.NN + gn];
     D kap2 = split(I.fk2), mu = split(I.fmu), mu3 = split(mul_third(I.fmu));
     bool bad = false;
+    if (g.wide[b.x]) {   // values modulo 32 edges: the edges from u itself
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            i64 v;
+            int x;
+            bad |= !wrapped_u(u[c * g.NN + gn], I.ihm, I.ihe, v, x);
+            bad |= coarse_edge_bad(x);
+        }
+    }
     int down = 0;
     if (I.lam_e || I.mu_e) {
         Material M;
-        bad = !material(I.lam_e ? I.lam_e[e] : I.lam, I.mu_e ? I.mu_e[e] : I.mu, I.wq, M);
+        bad |= !material(I.lam_e ? I.lam_e[e] : I.lam, I.mu_e ? I.mu_e[e] : I.mu, I.wq, M);
         kap2 = M.kap2;
         mu = M.mu;
         mu3 = M.mu3;
@@ -274,7 +301,13 @@ __global__ void __launch_bounds__(kNodeBlock) k_node_fx_b(const __grid_constant_
         }
         if (h2) {
             unext[d] = un;
-            g.ux[d] = fixed_u(un, I.ihm, I.ihe);
+            i64 x = fixed_u(un, I.ihm, I.ihe);
+            if (x == kBadU) {   // beyond the format: modulo 32 edges, and the force looks at u from now on
+                int coarse;
+                wrapped_u(un, I.ihm, I.ihe, x, coarse);
+                g.wide[b.x] = 1;
+            }
+            g.ux[d] = x;
         }
     }
 }

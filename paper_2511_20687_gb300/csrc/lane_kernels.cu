@@ -167,6 +167,7 @@ __global__ void __launch_bounds__(kLaneBlock, kForceBlocks) k_elem_force(const _
     const double lam = a.lam_e ? a.lam_e[x.e] : a.lam, mu = a.mu_e ? a.mu_e[x.e] : a.mu;
     Material M;
     bool bad = !material(lam, mu, a.wq, M);
+    refit_lanes([&](int c) { return a.u[(long long)c * a.usc + (long long)node * a.usn]; }, ihm, ihe, U, bad);
     const bool ok = force_lanes(L, U, M.kap2, M.mu, M.mu3, bad || M.k < -900 || M.k > 900, F);
     if (!x.live) return;
     if (ok) {
@@ -181,6 +182,42 @@ __global__ void __launch_bounds__(kLaneBlock, kForceBlocks) k_elem_force(const _
 }
 
 // the same with one thread per element (the arithmetic of force_fx.cu)
+template <int MODE>
+__device__ __forceinline__ bool thread_force(const ElemArgs& a, const Elem& x, const WalshIn w[3], bool bad) {
+    const double lam = a.lam_e ? a.lam_e[x.e] : a.lam, mu = a.mu_e ? a.mu_e[x.e] : a.mu;
+    Material M;
+    bad |= !material(lam, mu, a.wq, M) || M.k < -900 || M.k > 900;
+    i64 F[3][8];
+    bad |= !element_force_nh(w, whole(M.kap2), whole(M.mu), whole(M.mu3), F);
+    if (bad) return false;
+#pragma unroll
+    for (int c8 = 0; c8 < 8; ++c8)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) put<MODE>(a, x, c8, c, f64_scaled(F[c][c8], kFracOut - M.k));
+    return true;
+}
+
+// ... with a node beyond the format: the element's values modulo 32 edges
+template <int MODE>
+__device__ __noinline__ void moved_force(const ElemArgs& a, const Elem& x, i64 ihm, int ihe) {
+    WalshIn w[3];
+    bool bad = false;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        double X[8];
+        i64 V[8];
+#pragma unroll
+        for (int c8 = 0; c8 < 8; ++c8) X[c8] = a.u[(long long)c * a.usc + (long long)corner_node(x, c8) * a.usn];
+        bad |= refit(X, ihm, ihe, V);
+        w[c] = walsh_in(V, c);
+    }
+    if (thread_force<MODE>(a, x, w, bad)) return;
+    double Ff[3][8];
+    far_force(far_in(a, x, nullptr, 0, 0, a.lam_e ? a.lam_e[x.e] : a.lam, a.mu_e ? a.mu_e[x.e] : a.mu), Ff);
+    for (int c8 = 0; c8 < 8; ++c8)
+        for (int c = 0; c < 3; ++c) put<MODE>(a, x, c8, c, Ff[c][c8]);
+}
+
 template <int MODE>
 __global__ void __launch_bounds__(128) k_elem_force_thread(const __grid_constant__ ElemArgs a, i64 ihm, int ihe) {
     const int first = blockIdx.x * 128 + (int)threadIdx.x;
@@ -197,22 +234,7 @@ __global__ void __launch_bounds__(128) k_elem_force_thread(const __grid_constant
         bad |= spread_bad(V);
         w[c] = walsh_in(V, c);
     }
-    const double lam = a.lam_e ? a.lam_e[x.e] : a.lam, mu = a.mu_e ? a.mu_e[x.e] : a.mu;
-    Material M;
-    bad |= !material(lam, mu, a.wq, M) || M.k < -900 || M.k > 900;
-    i64 F[3][8];
-    bad |= !element_force_nh(w, whole(M.kap2), whole(M.mu), whole(M.mu3), F);
-    if (bad) {
-        double Ff[3][8];
-        far_force(far_in(a, x, nullptr, 0, 0, lam, mu), Ff);
-        for (int c8 = 0; c8 < 8; ++c8)
-            for (int c = 0; c < 3; ++c) put<MODE>(a, x, c8, c, Ff[c][c8]);
-        return;
-    }
-#pragma unroll
-    for (int c8 = 0; c8 < 8; ++c8)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) put<MODE>(a, x, c8, c, f64_scaled(F[c][c8], kFracOut - M.k));
+    if (!thread_force<MODE>(a, x, w, bad)) moved_force<MODE>(a, x, ihm, ihe);
 }
 
 // Element-level force: 8 lanes per element up to this many elements, above it one thread per element, which
@@ -236,7 +258,8 @@ __global__ void __launch_bounds__(kLaneBlock, kTangentBlocks) k_elem_vjp(const _
     }
     const double lam = a.lam_e ? a.lam_e[x.e] : a.lam, mu = a.mu_e ? a.mu_e[x.e] : a.mu;
     Material M;
-    const bool bad = !material(lam, mu, wqi, M);
+    bool bad = !material(lam, mu, wqi, M);
+    refit_lanes([&](int c) { return a.u[(long long)c * a.usc + (long long)node * a.usn]; }, ihm, ihe, U, bad);
     int scale, base;
     const bool ok = tangent_lanes(L, U, p, M, bad, lam_bar || mu_bar, F, scale, pk, pm, base);
     if (!x.live) return;
@@ -282,7 +305,7 @@ __global__ void __launch_bounds__(kLaneBlock, OP == kOpTangent ? kTangentBlocks 
     // consecutive bytes per warp
     const long long entry = OP == kOpStore32 ? I.elem_off + x.e + (long long)lin_point(L.a) * g.NE : 8 * (I.elem_off + x.e) + L.a;
     Material M;
-    const bool bad = !material(lam, mu, I.wq, M) || M.k < -900 || M.k > 900;
+    bool bad = !material(lam, mu, I.wq, M) || M.k < -900 || M.k > 900;
     i64 F[3];
     Linear q;
     int scale;
@@ -303,6 +326,7 @@ __global__ void __launch_bounds__(kLaneBlock, OP == kOpTangent ? kTangentBlocks 
         i64 U[3];
 #pragma unroll
         for (int c = 0; c < 3; ++c) U[c] = fixed_u(g.u[0][c * g.NN + gn], I.ihm, I.ihe);
+        refit_lanes([&](int c) { return g.u[0][c * g.NN + gn]; }, I.ihm, I.ihe, U, bad);
         ok = force_lanes(L, U, M.kap2, M.mu, M.mu3, bad, F, &q);
         scale = 57 - M.k;
     }

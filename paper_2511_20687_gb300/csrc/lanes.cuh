@@ -77,13 +77,33 @@ __device__ __forceinline__ T reduce8(T x, Op op) {
     return x;
 }
 
-// Columns of F from this lane's fixed-point u / h (59 fraction bits); bad: a node outside the format, or an edge of the
-// element out of range (edge_bad)
+// an edge of the element beyond range, from the lanes' coarse nodal values; every lane of the warp takes part
+__device__ __forceinline__ bool coarse_edge_bad(int v) {
+    bool bad = false;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) bad |= abs(v - __shfl_xor_sync(0xffffffffu, v, 1 << d)) >= kCoarseSpread;
+    return bad;
+}
+
+// Nodal values of a warp in which a node is beyond the format (kMaxU edges), again from u(c) in FP64 and modulo 32 edges;
+// bad: an element that is out of range all the same
+template <typename Load>
+__device__ __forceinline__ void refit_lanes(Load u, i64 ihm, int ihe, i64 U[3], bool& bad) {
+    if (!__any_sync(0xffffffffu, U[0] == kBadU || U[1] == kBadU || U[2] == kBadU)) return;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        int v;
+        bad |= !wrapped_u(u(c), ihm, ihe, U[c], v);
+        bad |= coarse_edge_bad(v);
+    }
+}
+
+// Columns of F from this lane's fixed-point u / h (59 fraction bits; no node marked); bad: an edge of the element out
+// of range (edge_bad)
 __device__ __forceinline__ void deformation(const Lane& L, const i64 U[3], Cols& C, bool& bad) {
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
         const int v = hi(U[c]);
-        bad |= v < -((kMaxU + 1) << 27);
 #pragma unroll
         for (int d = 0; d < 3; ++d) bad |= edge_bad(v, __shfl_xor_sync(0xffffffffu, v, 1 << d));
         i64 w = walsh_sums(L, U[c]);

@@ -133,6 +133,7 @@ struct FomB {
     int fixed;                // internal force in 64-bit integers: 1 Neo-Hookean (element buffer of int64; force_fx.cu),
                               // 2 linear elastic, 3 Saint Venant-Kirchhoff (element buffer of double; force_le.cu, force_svk.cu)
     long long* ux;            // fixed-point predicted displacement / h [3][NN], in the memory of us
+    int* wide;                // fixed-point groups, per instance: a predictor has been beyond the format's 12 edges
 };
 
 // A node kernel takes one thread per node and component instead of one per node while that leaves it

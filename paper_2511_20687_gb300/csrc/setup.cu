@@ -313,6 +313,8 @@ int setup_fom_group(osam_ctx* ctx, FomGroupH& G, int s, int n, const osam_proble
         // us holds u / h in FP64 for the initial force and after a change of state, and the fixed-point predictor,
         // which the node kernel writes before every force of a step
         B.ux = reinterpret_cast<long long*>(B.us);
+        CKA(B.wide = ctx->alloc<int>(n));
+        CK(cudaMemsetAsync(B.wide, 0, sizeof(int) * n, ctx->stream));
         for (int i = 0; i < n; ++i)
             if (!fixed_point_scales(G.inst[i], factor[i])) B.fixed = 0;
         RET(upload(ctx, G.inst_d, G.inst.data(), sizeof(InstFom) * n));
@@ -724,6 +726,8 @@ int autotune(osam_ctx* ctx, bool fixed) {
         }
     }
     CK(cudaMemsetAsync(G.d.f, 0, sizeof(double) * 3 * NN, ctx->stream));
+    // the trial steps took boundary values from history slots that nothing had filled
+    if (G.d.wide) CK(cudaMemsetAsync(G.d.wide, 0, sizeof(int) * G.d.n_inst, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
     if (!fixed) ctx->scatter = best_scatter;
     for (Slot& S : ctx->slots)

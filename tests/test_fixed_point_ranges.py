@@ -247,3 +247,102 @@ def test_lane_range_check_bounds_every_intermediate(lanes):
     assert 500 < ok.sum() < 3900
     assert (r[ok, 1] < 11.001).all() and (r[ok, 2] < 3.751).all() and not r[ok, 3].any()
     assert r[~ok, 3].any() and not ok[4000:].any()
+
+
+@pytest.fixture(scope="module")
+def refit(tmp_path_factory):
+    return build(tmp_path_factory, "fixed_point_refit_check.cpp")
+
+
+@pytest.mark.parametrize("amp", [1e-3, 0.25])
+@pytest.mark.parametrize("shift", [0.0, 11.0, 13.0, 15.9, 16.1, 31.0, 33.0, 500.0, 1e5])
+def test_translated_element_stays_in_range(refit, shift, amp):
+    """An element anywhere within 2^22 edges keeps the format's accuracy (1.6e-15, see test_fixed_point.py) up to the
+    rounding of u / h at 2^-62 of it, times the ten units that a corner force amplifies it by; and stays closer than
+    the same formula in double."""
+    lam, mu = W.lame(1e9, 0.25)
+    rng = np.random.default_rng(13)
+    lines = [((H, lam, mu), H * (0.5 * amp * rng.uniform(-1, 1, (3, 8)) + shift * rng.choice([-1, 1], (3, 1))))
+             for _ in range(200)]
+    r = refit(lines)
+    assert r[:, 0].all() and r[:, 3].all()
+    assert r[:, 1].max() < 1.6e-15 + 10 * shift * 2.0 ** -62
+    assert np.sqrt(np.mean(r[:, 1] ** 2)) <= np.sqrt(np.mean(r[:, 2] ** 2))
+
+
+@pytest.mark.parametrize("stretch", [2.8, 16.3, 29.5, 31.0, 32.0, 33.0, 64.0, 1024.0, 1e6, 5e6, np.inf, np.nan])
+def test_torn_element_is_reported_however_far(refit, stretch):
+    """Among them spreads that vanish modulo 32 edges."""
+    lam, mu = W.lame(1e9, 0.25)
+    lines = []
+    for axis in range(3):
+        for component in range(3):
+            u = np.zeros((3, 8))
+            u[component] = H * np.where(CORNERS[:, axis] > 0, stretch, 0.0)
+            lines.append(((H, lam, mu), u))
+    assert (refit(lines)[:, 0] == 0).all()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("dims", [(6, 5, 4), (41, 41, 41)])   # 8 lanes and one thread per element
+@pytest.mark.parametrize("edges", [13, 64, 4096])
+def test_translated_mesh_gets_the_same_force(dims, edges):
+    """u and h on a binary grid, so that a translation changes no digit of the differences: every element's force and
+    gradient stay the same bit for bit, and a node's differ by the order of eight FP64 additions (a few 2^-53; the FP64
+    kernels' own rounding at strains of 1e-2 is 1e-14)."""
+    import torch
+
+    from paper_2511_20687_gb300 import osam
+    h = 2.0 ** -6
+    g = torch.Generator(device="cuda").manual_seed(17)
+    nn = (dims[0] + 1) * (dims[1] + 1) * (dims[2] + 1)
+    u = torch.randint(-2 ** 20, 2 ** 20, (nn, 3), generator=g, device="cuda").double() * 2.0 ** -32
+    y = torch.rand(nn, 3, generator=g, device="cuda", dtype=torch.float64)
+    out = []
+    for x in (u, u + edges * h):
+        f, ub = torch.empty_like(u), torch.empty_like(u)
+        osam.hex8_force(dims, h, "nh", 4e8, 4e8, x, f)
+        osam.hex8_force_vjp(dims, h, "nh", 4e8, 4e8, x, y, ub)
+        out.append((f, ub))
+    for a, b in zip(*out):
+        assert (a - b).norm() <= 1e-15 * a.norm()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n,nz,integrator", [(4, 8, "explicit"), (26, 26, "explicit"), (4, 8, "implicit")])
+@pytest.mark.parametrize("shift", [14.0, 40.0])
+def test_step_of_a_translated_bar(n, nz, integrator, shift):
+    """Against the oracle: u / h is rounded at 2^-53 of the shift on strains of 1e-2."""
+    from oracle import oracle as O
+    from paper_2511_20687_gb300 import osam
+    p = W.single_bar("moved", n, nz, "nh", 1e9, 0.25, 1000.0, 1e-3, 1e-6, 2)
+    sd = p.subdomains[0]
+    sd.dirichlet = np.zeros(sd.n_nodes, np.uint8)
+    sd.integrator = integrator
+    sd.u0 = sd.u0 + shift * sd.h
+    a, b = osam.Problem(p), O.Problem(p)
+    a.step()
+    b.step()
+    for f in range(3):
+        x, y = a.state(0)[f], b.state(0)[f]
+        assert np.linalg.norm(x - y) <= 1e-12 * (1 + 100 * shift) * np.linalg.norm(y)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n,nz", [(4, 8), (26, 26)])   # 8 lanes and one thread per element
+def test_step_with_a_layer_torn_by_the_modulus(n, nz):
+    """A layer stretched by 32 edges, which vanishes modulo 32, against the FP64 kernels as in
+    test_step_with_a_stretched_layer."""
+    from paper_2511_20687_gb300 import osam
+    p = W.single_bar("torn", n, nz, "nh", 1e9, 0.25, 1000.0, 1e-3, 1e-6, 2)
+    sd = p.subdomains[0]
+    sd.dirichlet = None
+    k = np.arange(nz + 1).repeat((n + 1) ** 2)
+    sd.u0 = W.random_field(sd.n_nodes, 1e-5, 3)
+    sd.u0[:, 2] += np.where(k <= nz // 2, -0.5, 0.5) * 32.0 * sd.h
+    a, b = osam.Problem(p), osam.Problem(p, scatter=osam.SCATTER_GATHER)
+    a.step()
+    b.step()
+    for f in range(3):
+        x, y = a.state(0)[f], b.state(0)[f]
+        assert np.linalg.norm(x - y) <= 1e-12 * np.linalg.norm(y)
