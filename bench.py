@@ -61,7 +61,7 @@ FP32_ISSUE_PEAK_TINST = 152 * 128 * 2.07e9 / 1e12
 INT_MAD_PER_NH_ELEMENT = 1969
 INT_MAD_PEAK_TINST = 152 * 4 * 32 * 2.07e9 / 4 / 1e12
 # bf16 digit products per FP64 product of the fit (split_gemm.cu)
-SPLIT_PRODUCTS = 28
+SPLIT_PRODUCTS = 34
 # DRAM traffic of one force launch of the bench workload (ncu dram__bytes_read.sum + write.sum),
 # valid only for the kernel source and variant (tiled or not) it was captured on.
 FORCE_TRAFFIC = {"source_sha256": "5329782da603ec0d213b49ef60d6836089a9f41f0ba6bc0fa18cff46cede7c3d",

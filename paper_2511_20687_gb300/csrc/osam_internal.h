@@ -325,7 +325,21 @@ cudaError_t launch_gemm_nn(int m, int n, int k, const double* A, int lda, const 
                            int ldc, double alpha, double beta, cudaStream_t s);
 cudaError_t launch_gemm_nt(int m, int n, int k, const double* A, int lda, const double* B, int ldb, double* C,
                            int ldc, double alpha, double beta, cudaStream_t s);
-// the same on the bf16 tensor cores by exact splitting (split_gemm.cu); element strides (ai, ak), (bk, bj)
+// The FP64 kernel on element strides (ai, ak), (bk, bj): k in p.nsplit parts with their partial results in ws
+// [nsplit][m][n] (none for one part).  flag: only the 64 x 64 tiles of C marked in it, numbered by gemm_tile.
+constexpr int kGemmTile = 64;
+struct GemmSplit { int nsplit, kchunk; };
+GemmSplit gemm_split(int m, int n, int k, int sms);
+cudaError_t launch_gemm_f64(int m, int n, int k, const double* A, long long ai, long long ak, const double* B,
+                            long long bk, long long bj, double* C, long long ldc, double alpha, double beta,
+                            const GemmSplit& p, double* ws, const int* flag, int sym, cudaStream_t s);
+// tile of entry (i, j) of an m x n result; sym: a tile below the diagonal is its mirror image's
+__host__ __device__ inline long long gemm_tile(long long i, long long j, int n, int sym) {
+    const long long ti = i / kGemmTile, tj = j / kGemmTile, ntn = (n + kGemmTile - 1) / kGemmTile;
+    return sym && ti > tj ? tj * ntn + ti : ti * ntn + tj;
+}
+// the same on the bf16 tensor cores by splitting, where its error is certified to be below the FP64 kernel's
+// (split_gemm.cu), else by that kernel
 constexpr int kSplitChunk = 1024;
 cudaError_t launch_split_gemm(int m, int n, int k, const double* A, long long ai, long long ak, const double* B,
                               long long bk, long long bj, double* C, long long ldc, double alpha, double beta,

@@ -84,8 +84,9 @@ __global__ void k_build_Rt(int nrow, int r, const int* dnode, const double* dw, 
 // ws[z][m][n]; k_gemm_reduce then adds the partials in ascending z (deterministic) and applies
 // alpha and beta.  The output tiles are numbered along grid.x, column tile fastest (blocks that
 // share a row tile of A run together and find it in L2), so m is bounded only by 32-bit indices.
-constexpr int TM = 64, TN = 64, TK = 16;
+constexpr int TM = kGemmTile, TN = kGemmTile, TK = 16;
 constexpr double kSplitMin = 4.2e6;
+constexpr int kSplitMinK = 128;
 
 // The GEMM runs on the FP64 tensor cores: 128 threads per 64x64 output tile, each warp a 32x32 quarter
 // as 4 x 4 accumulators of mma.sync m8n8k4 (FP64 in and out, each MMA 8x8x4 fused multiply-adds).
@@ -101,7 +102,8 @@ __device__ __forceinline__ void dmma_8x8x4(double& d0, double& d1, double a, dou
 
 __global__ void __launch_bounds__(128) k_gemm_mma(int m, int n, int kdim, int kchunk, const double* A, long long ai,
                                                   long long ak, const double* B, long long bk, long long bj,
-                                                  double* C, long long ldc, double alpha, double beta, double* ws) {
+                                                  double* C, long long ldc, double alpha, double beta, double* ws,
+                                                  const int* __restrict__ flag, int sym) {
     __shared__ double As[TK][TM + TPAD];
     __shared__ double Bs[TK][TN + TPAD];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -109,6 +111,7 @@ __global__ void __launch_bounds__(128) k_gemm_mma(int m, int n, int kdim, int kc
     const int g = lane >> 2, t4 = lane & 3;
     const int ntn = (n + TN - 1) / TN;
     const int i0 = (int)(blockIdx.x / ntn) * TM, j0 = (int)(blockIdx.x % ntn) * TN;
+    if (flag && !flag[gemm_tile(i0, j0, n, sym)]) return;   // only the flagged tiles
     const int kbeg = blockIdx.z * kchunk;
     const int kend = min(kdim, kbeg + kchunk);
     const bool a_along_i = ai == 1 && ak != 1;   // A stored [k][m]
@@ -164,10 +167,10 @@ __global__ void __launch_bounds__(128) k_gemm_mma(int m, int n, int kdim, int kc
 }
 
 __global__ void k_gemm_reduce(int m, int n, int nsplit, const double* __restrict__ ws, double* C, long long ldc,
-                              double alpha, double beta) {
+                              double alpha, double beta, const int* __restrict__ flag, int sym) {
     const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const long long mn = (long long)m * n;
-    if (idx >= mn) return;
+    if (idx >= mn || (flag && !flag[gemm_tile(idx / n, idx % n, n, sym)])) return;
     double s = 0.0;
     for (int z = 0; z < nsplit; ++z) s += ws[z * mn + idx];
     double* cp = C + (idx / n) * ldc + idx % n;
@@ -208,49 +211,23 @@ cudaError_t launch_gemm(int m, int n, int k, const double* A, long long ai, long
     return e;
 }
 
-// Split the reduction when the output tiles alone cannot fill the GPU (four 4-warp blocks per SM
-// wanted) and the reduction is long: chunks of at least 512 k, a multiple of the k tile.
 cudaError_t launch_gemm_impl(int m, int n, int k, const double* A, long long ai, long long ak, const double* B,
                              long long bk, long long bj, double* C, long long ldc, double alpha, double beta,
                              cudaStream_t s) {
     if (m <= 0 || n <= 0) return cudaSuccess;
     // From a few million products on, on the bf16 tensor cores (split_gemm.cu); below, the splitting's extra
-    // launches cost more than the FP64 tensor pipe takes.
-    if (k >= 16 && (double)m * n * k >= kSplitMin)
+    // launches cost more than the FP64 tensor pipe takes.  Rows shorter than 128 are left to FP64: in so few elements
+    // the certificate that the splitting needs is close to failing on ordinary operands (it fails at 16, passes at 64).
+    if (k >= kSplitMinK && (double)m * n * k >= kSplitMin)
         return launch_split_gemm(m, n, k, A, ai, ak, B, bk, bj, C, ldc, alpha, beta, s);
-    const long long tiles = (long long)grid_for(n, TN) * grid_for(m, TM);
     int dev = 0, sms = 152;
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const long long want = 4LL * sms;
-    int nsplit = 1;
-    if (tiles < want && k >= 2 * 512)
-        nsplit = (int)std::min<long long>((want + tiles - 1) / tiles, k / 512);
-    // prefer a block count that is a multiple of the SM count: every SM then runs the same number of
-    // equal blocks (a 64-tile Gram split 10 ways leaves some SMs three blocks and others two)
-    if (nsplit > 1)
-        for (long long ns = nsplit; ns <= std::min<long long>(k / 512, 4LL * nsplit); ++ns)
-            if ((tiles * ns) % sms == 0) { nsplit = (int)ns; break; }
-    int kchunk = k;
-    if (nsplit > 1) {
-        kchunk = (k + nsplit - 1) / nsplit;
-        kchunk = (kchunk + TK - 1) / TK * TK;
-        nsplit = (k + kchunk - 1) / kchunk;
-    }
-    if (tiles > 0x7fffffffLL) return cudaErrorInvalidValue;
-    dim3 g((unsigned)tiles, 1, nsplit);
-    if (nsplit == 1) {
-        k_gemm_mma<<<g, 128, 0, s>>>(m, n, k, k, A, ai, ak, B, bk, bj, C, ldc, alpha, beta, nullptr);
-        return cudaGetLastError();
-    }
+    const GemmSplit p = gemm_split(m, n, k, sms);
+    if (p.nsplit == 1) return launch_gemm_f64(m, n, k, A, ai, ak, B, bk, bj, C, ldc, alpha, beta, p, nullptr, nullptr, 0, s);
     double* ws = nullptr;
-    cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&ws), sizeof(double) * (size_t)nsplit * m * n, s);
+    cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&ws), sizeof(double) * (size_t)p.nsplit * m * n, s);
     if (e != cudaSuccess) return e;
-    k_gemm_mma<<<g, 128, 0, s>>>(m, n, k, kchunk, A, ai, ak, B, bk, bj, C, ldc, alpha, beta, ws);
-    e = cudaGetLastError();
-    if (e == cudaSuccess) {
-        k_gemm_reduce<<<grid_for((long long)m * n, 256), 256, 0, s>>>(m, n, nsplit, ws, C, ldc, alpha, beta);
-        e = cudaGetLastError();
-    }
+    e = launch_gemm_f64(m, n, k, A, ai, ak, B, bk, bj, C, ldc, alpha, beta, p, ws, nullptr, 0, s);
     cudaError_t f = cudaFreeAsync(ws, s);
     return e != cudaSuccess ? e : f;
 }
@@ -418,6 +395,44 @@ int gemm_profile(int enable, double* ms, double* flops, long long* launches) {
     if (flops) *flops = P.flops;
     if (launches) *launches = P.launches;
     return OSAM_OK;
+}
+
+// Split the reduction when the output tiles alone cannot fill the GPU (four 4-warp blocks per SM
+// wanted) and the reduction is long: chunks of at least 512 k, a multiple of the k tile.
+GemmSplit gemm_split(int m, int n, int k, int sms) {
+    const long long tiles = (long long)grid_for(n, TN) * grid_for(m, TM);
+    const long long want = 4LL * sms;
+    int nsplit = 1;
+    if (tiles < want && k >= 2 * 512)
+        nsplit = (int)std::min<long long>((want + tiles - 1) / tiles, k / 512);
+    // prefer a block count that is a multiple of the SM count: every SM then runs the same number of
+    // equal blocks (a 64-tile Gram split 10 ways leaves some SMs three blocks and others two)
+    if (nsplit > 1)
+        for (long long ns = nsplit; ns <= std::min<long long>(k / 512, 4LL * nsplit); ++ns)
+            if ((tiles * ns) % sms == 0) { nsplit = (int)ns; break; }
+    int kchunk = k;
+    if (nsplit > 1) {
+        kchunk = (k + nsplit - 1) / nsplit;
+        kchunk = (kchunk + TK - 1) / TK * TK;
+        nsplit = (k + kchunk - 1) / kchunk;
+    }
+    return GemmSplit{nsplit, kchunk};
+}
+
+cudaError_t launch_gemm_f64(int m, int n, int k, const double* A, long long ai, long long ak, const double* B,
+                            long long bk, long long bj, double* C, long long ldc, double alpha, double beta,
+                            const GemmSplit& p, double* ws, const int* flag, int sym, cudaStream_t s) {
+    const long long tiles = (long long)grid_for(n, TN) * grid_for(m, TM);
+    if (tiles > 0x7fffffffLL) return cudaErrorInvalidValue;
+    const dim3 g((unsigned)tiles, 1, p.nsplit);
+    const bool direct = p.nsplit == 1;
+    k_gemm_mma<<<g, 128, 0, s>>>(m, n, k, p.kchunk, A, ai, ak, B, bk, bj, C, ldc, alpha, beta, direct ? nullptr : ws, flag, sym);
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess && !direct) {
+        k_gemm_reduce<<<grid_for((long long)m * n, 256), 256, 0, s>>>(m, n, p.nsplit, ws, C, ldc, alpha, beta, flag, sym);
+        e = cudaGetLastError();
+    }
+    return e;
 }
 
 // row-major helpers: C[m][n] (ldc) = alpha * A^T B, A is [k][m] (lda), B is [k][n] (ldb)
