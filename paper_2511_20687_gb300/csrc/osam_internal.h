@@ -330,6 +330,7 @@ cudaError_t launch_gemm_nt(int m, int n, int k, const double* A, int lda, const 
 constexpr int kGemmTile = 64;
 struct GemmSplit { int nsplit, kchunk; };
 GemmSplit gemm_split(int m, int n, int k, int sms);
+GemmSplit gemm_split_tiles(long long tiles, long long most, int k, int sms);   // for that many tiles; at most `most` parts
 cudaError_t launch_gemm_f64(int m, int n, int k, const double* A, long long ai, long long ak, const double* B,
                             long long bk, long long bj, double* C, long long ldc, double alpha, double beta,
                             const GemmSplit& p, double* ws, const int* flag, int sym, cudaStream_t s);

@@ -400,7 +400,9 @@ int gemm_profile(int enable, double* ms, double* flops, long long* launches) {
 // Split the reduction when the output tiles alone cannot fill the GPU (four 4-warp blocks per SM
 // wanted) and the reduction is long: chunks of at least 512 k, a multiple of the k tile.
 GemmSplit gemm_split(int m, int n, int k, int sms) {
-    const long long tiles = (long long)grid_for(n, TN) * grid_for(m, TM);
+    return gemm_split_tiles((long long)grid_for(n, TN) * grid_for(m, TM), 0x7fffffff, k, sms);
+}
+GemmSplit gemm_split_tiles(long long tiles, long long most, int k, int sms) {
     const long long want = 4LL * sms;
     int nsplit = 1;
     if (tiles < want && k >= 2 * 512)
@@ -410,6 +412,7 @@ GemmSplit gemm_split(int m, int n, int k, int sms) {
     if (nsplit > 1)
         for (long long ns = nsplit; ns <= std::min<long long>(k / 512, 4LL * nsplit); ++ns)
             if ((tiles * ns) % sms == 0) { nsplit = (int)ns; break; }
+    nsplit = (int)std::max(1LL, std::min<long long>(nsplit, most));
     int kchunk = k;
     if (nsplit > 1) {
         kchunk = (k + nsplit - 1) / nsplit;

@@ -517,7 +517,10 @@ cudaError_t launch_split_gemm(int m, int n, int k, const double* A, long long ai
     nsplit = (chunks + per - 1) / per;
     if (nsplit > 65535) return cudaErrorInvalidValue;
     const bool direct = nsplit == 1 && !sym && alpha == 1.0 && beta == 0.0;   // straight into C
-    const GemmSplit f64 = gemm_split(m, n, k, sms);
+    // The FP64 kernel meets few tiles as a rule: k in as many parts as one tile needs to fill the GPU (one failing tile
+    // of 500 x 64 x 403440: 76 parts 24.4 ms, 601 parts 3.9 ms), within the products' workspace or 256 MB
+    const long long most = std::max<long long>(nsplit, (1LL << 25) / ((long long)m * n));
+    const GemmSplit f64 = gemm_split_tiles(1, most, k, sms);
     const size_t nex = (size_t)m * chunks + (sym ? 0 : (size_t)n * chunks);
     // the partial results: first the certificate's, then the products', then the FP64 kernel's for the flagged tiles
     const size_t nws = std::max<size_t>(direct ? 0 : (size_t)nsplit * m * n, f64.nsplit > 1 ? (size_t)f64.nsplit * m * n : 0);
