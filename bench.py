@@ -60,19 +60,16 @@ FP32_ISSUE_PEAK_TINST = 152 * 128 * 2.07e9 / 1e12
 # and scheduler (measured), 152 SMs x 4 schedulers x 32 lanes x 2.07 GHz / 4
 INT_MAD_PER_NH_ELEMENT = 1969
 INT_MAD_PEAK_TINST = 152 * 4 * 32 * 2.07e9 / 4 / 1e12
+LANE_ELEMENTS = 16384   # the explicit force's size rule (force_fx.cu)
 # bf16 digit products per FP64 product of the fit (split_gemm.cu)
 SPLIT_PRODUCTS = 34
 # DRAM traffic of one force launch of the bench workload (ncu dram__bytes_read.sum + write.sum),
 # valid only for the kernel source and variant (tiled or not) it was captured on.
 FORCE_TRAFFIC = {"source_sha256": "5329782da603ec0d213b49ef60d6836089a9f41f0ba6bc0fa18cff46cede7c3d",
                  "bytes_per_launch": 3.567616e6, "tiled": True, "register_cap": 0}
-# the same for the Neo-Hookean tangent-action kernel of the implicit block (sources TANGENT_SOURCES)
-# bytes one tangent launch must move per element: the stored linearisation (22 doubles x 8 Gauss
-# points) + p at 8 nodes / 8 elements per node (24 B); the element buffer stays in L2
+# bytes one tangent launch of the implicit block must move per element: the stored linearisation (22 64-bit integers x 8
+# Gauss points) + p at 8 nodes / 8 elements per node (24 B); the element buffer stays in L2
 TANGENT_BYTES_PER_ELEMENT = 22 * 8 * 8 + 24
-TANGENT_TRAFFIC = {"source_sha256": "cd475f28af922fbeaa85abd62d838d03451fea6f47a72d3046ce0d821fae63fc",
-                   "bytes_per_launch": 1.947856e8}
-
 
 STATE_BYTES_PER_NODE_UPDATE = 152
 # FP64 flops of one Neo-Hookean element tangent action K(u) p of the implicit Newton-CG (FMA = 2
@@ -84,9 +81,6 @@ TANGENT_FLOPS_PER_NH_ELEMENT = 1832
 # bytes the FP32 tangent kernel must move per element: the FP32 linearisation (22 floats x 8 Gauss
 # points) from HBM, p at 8 nodes / 8 elements per node (24 B), the FP32 element buffer out (24 floats)
 TANGENT32_BYTES_PER_ELEMENT = 22 * 8 * 4 + 24 + 24 * 4
-# DRAM traffic of one FP32-tangent launch (ncu, same sources as TANGENT_TRAFFIC)
-TANGENT32_TRAFFIC = {"source_sha256": "cd475f28af922fbeaa85abd62d838d03451fea6f47a72d3046ce0d821fae63fc",
-                     "bytes_per_launch": 9.375027e7}
 # FP64 flops of one Saint Venant-Kirchhoff element force: the 504 flops of the sum factorisation
 # around the constitutive law (as for Neo-Hookean) + 8 x 115 (Green-Lagrange strain 48, S 13, P = F S 54)
 FLOPS_PER_SVK_ELEMENT = 1424
@@ -266,15 +260,18 @@ class ClockSampler:
 
 
 def fixed_point_roofline(prof):
-    """Integer multiply-add issue rate of the fixed-point force launches."""
+    """Integer multiply-add issue rate of the fixed-point force launches (the kernel with one thread per element; up to
+    LANE_ELEMENTS elements per launch the one with 8 lanes per element runs, whose instructions are not counted here)."""
+    per_launch = prof["force_elements"] // max(1, prof["force_launches"])
+    common = {"bound": "alu", "peak": INT_MAD_PEAK_TINST, "unit": "Tinst/s (integer multiply-add pipe)",
+              "peak_kind": "152 SMs x 4 schedulers x 32 lanes x 2.07 GHz / 4 cycles (measured issue interval)",
+              "fp64_equivalent_tflops": FLOPS_PER_NH_ELEMENT * prof["force_elements"] / (prof["force_ms"] * 1e-3) / 1e12,
+              "elements_per_launch": per_launch, "force_ms_per_launch": prof["force_ms"] / max(1, prof["force_launches"])}
+    if per_launch <= LANE_ELEMENTS:
+        return {**common, "kernel": "k_force_fx_lanes_b (Neo-Hookean, 64-bit fixed point)", "achieved": None, "frac": None}
     achieved = INT_MAD_PER_NH_ELEMENT * prof["force_elements"] / (prof["force_ms"] * 1e-3) / 1e12
-    return {"bound": "alu", "kernel": "k_force_fx_b (Neo-Hookean, 64-bit fixed point)", "achieved": achieved,
-            "peak": INT_MAD_PEAK_TINST, "unit": "Tinst/s (integer multiply-add pipe)",
-            "frac": achieved / INT_MAD_PEAK_TINST,
-            "peak_kind": "152 SMs x 4 schedulers x 32 lanes x 2.07 GHz / 4 cycles (measured issue interval)",
-            "fp64_equivalent_tflops": FLOPS_PER_NH_ELEMENT * prof["force_elements"] / (prof["force_ms"] * 1e-3) / 1e12,
-            "elements_per_launch": prof["force_elements"] // max(1, prof["force_launches"]),
-            "force_ms_per_launch": prof["force_ms"] / max(1, prof["force_launches"])}
+    return {**common, "kernel": "k_force_fx_b (Neo-Hookean, 64-bit fixed point)", "achieved": achieved,
+            "frac": achieved / INT_MAD_PEAK_TINST}
 
 
 def source_sha(files=("step_kernels.cu", "hex8_math.cuh", "trace_item.cuh", "fp_bits.cuh")):
@@ -283,9 +280,6 @@ def source_sha(files=("step_kernels.cu", "hex8_math.cuh", "trace_item.cuh", "fp_
     for f in files:
         h.update(open(os.path.join(ROOT, "paper_2511_20687_gb300", "csrc", f), "rb").read())
     return h.hexdigest()
-
-
-TANGENT_SOURCES = ("tangent_kernels.cu", "hex8_math.cuh", "nh_tangent.cuh", "fp_bits.cuh")
 
 
 # ---------------------------------------------------------------------------------------------
@@ -715,9 +709,7 @@ def measure_implicit(W, osam, torch, flush, rom_ops, args, local, log, steps=2, 
         "roofline": {"bound": "hbm", "kernel": "k_tangent_lin32_b (Neo-Hookean, FP32)",
                      "achieved": t_gbs, "peak": hbm_peak, "unit": "GB/s",
                      "frac": t_gbs / hbm_peak if (t_gbs and hbm_peak) else None, "peak_kind": hbm_kind,
-                     "algorithmic_bytes_per_launch": t_bytes, "ms_per_launch": t_launch_ms,
-                     "traffic": (TANGENT32_TRAFFIC["bytes_per_launch"]
-                                 if TANGENT32_TRAFFIC["source_sha256"] == source_sha(TANGENT_SOURCES) else None)},
+                     "algorithmic_bytes_per_launch": t_bytes, "ms_per_launch": t_launch_ms, "traffic": None},
         "speedup_vs_fp64_tangent": (t_upd / t_ms) / (upd / total_ms),
         "parity": "1e-9 relative L2 vs the oracle, 1e-10 vs the FP64 tangent (tests/test_gpu_implicit.py)"}
     log(f"implicit, FP32 tangent: {t_ms / steps:.1f} ms/step, {fp32_tangent['newton_per_substep']:.2f} "
@@ -746,15 +738,14 @@ def measure_implicit(W, osam, torch, flush, rom_ops, args, local, log, steps=2, 
             "tangent_time_share": ip["tangent_ms"] / p_ms if p_ms else None,
             "roofline": {"bound": "hbm", "kernel": "k_fom_lanes<tangent> (Neo-Hookean, 64-bit integers)",
                          "achieved": ne * TANGENT_BYTES_PER_ELEMENT / 1e6 / max(1e-9, ip["tangent_ms"] / max(1, ip["tangent_launches"])),
-                         "peak": measured_hbm_gbs()[0], "unit": "GB/s",
+                         "peak": hbm_peak, "unit": "GB/s",
                          "frac": (ne * TANGENT_BYTES_PER_ELEMENT / 1e6 / max(1e-9, ip["tangent_ms"] / max(1, ip["tangent_launches"]))
-                                  / measured_hbm_gbs()[0] if measured_hbm_gbs()[0] else None),
-                         "traffic": (TANGENT_TRAFFIC["bytes_per_launch"]
-                                     if TANGENT_TRAFFIC["source_sha256"] == source_sha(TANGENT_SOURCES) else None),
+                                  / hbm_peak if hbm_peak else None),
+                         "traffic": None,
                          "algorithmic_bytes_per_launch": ne * TANGENT_BYTES_PER_ELEMENT,
                          "fp64_equivalent_tflops": achieved,
                          "ms_per_launch": ip["tangent_ms"] / max(1, ip["tangent_launches"]),
-                         "peak_kind": FP64_PEAK_KIND[0]},
+                         "peak_kind": hbm_kind},
             "timing": "value: library CUDA events around each controller step, each one graph launch with the "
                       "Newton and CG loops as device-side WHILE nodes (L2 flushed between steps); roofline and "
                       "counts: a second pass of the same steps driven from the host with CUDA events around "
@@ -865,9 +856,9 @@ def measure_next_rows(W, osam, torch, flush, rom_ops, args, local, log, steps=5,
         "workload": f"{args.n}x{args.n}x{args.nz} Saint Venant-Kirchhoff FOM + cubic OpInf ROM r=20 "
                     f"(r_s={svk_fit['r_s']}, fitted on {svk_fit['n_snap']} snapshots of an SVK FOM-FOM run)",
         "fit_seconds": svk_fit["gpu_seconds"],
-        "roofline": {"bound": "alu", "kernel": "k_force_*<SaintVenantKirchhoff>", "achieved": achieved,
-                     "peak": FP64_PEAK[0], "unit": "TFLOP/s", "frac": achieved / FP64_PEAK[0],
-                     "flops_per_element": FLOPS_PER_SVK_ELEMENT,
+        "roofline": {"bound": "alu", "kernel": "k_fom_force_svk (Saint Venant-Kirchhoff, 64-bit integers)", "achieved": None,
+                     "peak": INT_MAD_PEAK_TINST, "unit": "Tinst/s (integer multiply-add pipe)", "frac": None,
+                     "fp64_equivalent_tflops": achieved, "flops_per_element": FLOPS_PER_SVK_ELEMENT,
                      "force_ms_per_launch": prof["force_ms"] / max(1, prof["force_launches"])}}
     # oracle beside each variant, on a small bar of the same kind (3x3x[8,8] FOMs, 20 substeps)
     small = W.bar_chain("s_add", 3, [8, 8], ["fom", "fom"], "nh", 1e9, 0.25, 1000.0, 1e-3, 1e-6, 20, max_iters=64)
@@ -1429,7 +1420,8 @@ def main():
             hbm[name] = {"achieved_gbs": gbs, "frac": gbs / hbm_peak if hbm_peak else None}
         hbm = {"algorithmic_bytes_per_element_update": bytes_per_update, "peak_gbs": hbm_peak,
                "peak_kind": hbm_kind, **hbm,
-               "note": "the path is bound by the integer multiply-add pipe, not by HBM"}
+               "note": "the path is bound by the integer force kernel (its multiply-add pipe on large launches, its own "
+                       "latencies on one mesh), not by HBM"}
         mean_it = float(np.mean(head["iters"]))
         line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
                 "warmup": args.warmup, "ms_per_step": head["total_ms"] / args.steps, "higher_is_better": True,

@@ -54,10 +54,19 @@ enum { OSAM_LINEAR_ELASTIC = 0, OSAM_NEO_HOOKEAN = 1, OSAM_SAINT_VENANT_KIRCHHOF
  * Newmark (beta = 1/4, gamma = 1/2, average acceleration) */
 enum { OSAM_EXPLICIT = 0, OSAM_IMPLICIT = 1 };
 enum { OSAM_MULTIPLICATIVE = 0, OSAM_ADDITIVE = 1 };
-/* OSAM_FP64: FP64 state and arithmetic; the internal force of explicit Neo-Hookean subdomains whose scatter
- * is OSAM_SCATTER_AUTO is evaluated in 64-bit fixed point with an error below native FP64's (elements
- * outside its range -- displacement gradients of order one half, displacements beyond 12 element edges --
- * in native FP64).  OSAM_FP32_FORCE: internal force in FP32 (checked to 1e-5).
+/* OSAM_FP64: FP64 state and arithmetic.  Element operators run in 64-bit integers (Neo-Hookean in fixed
+ * point in each element's own material unit, linear elastic and Saint Venant-Kirchhoff with a common
+ * exponent per element), with an error against exact arithmetic that is not above native FP64's:
+ *  - the internal force of explicit subdomains whose scatter is OSAM_SCATTER_AUTO (OSAM_FP64 and
+ *    OSAM_FP64_TANGENT32: every material; OSAM_F32X2_FORCE: Neo-Hookean), and with it the residual and the
+ *    linear elastic tangent of implicit linear elastic and Saint Venant-Kirchhoff subdomains;
+ *  - the Newton residual of implicit Neo-Hookean subdomains and, in OSAM_FP64, their tangent, whatever the
+ *    scatter;
+ *  - osam_hex8_force, osam_hex8_force_noalloc, osam_hex8_force_vjp and osam_adjoint.
+ * A scatter asked for by name selects the FP64 (or double-float) kernels for the first group.  Elements
+ * outside the integers' range -- Neo-Hookean and Saint Venant-Kirchhoff displacement gradients of order
+ * one half, displacements beyond 2^22 element edges, operands that are not finite -- are evaluated in FP64.
+ * OSAM_FP32_FORCE: internal force in FP32 (checked to 1e-5).
  * OSAM_F32X2_FORCE: internal force in double-float arithmetic (pairs of FP32 values, ~48-bit
  * significands) on the FP32 pipes, state and time integration in FP64 (checked to 1e-9 like FP64);
  * uses the deterministic gather scatter; Neo-Hookean subdomains with OSAM_SCATTER_AUTO take the
@@ -74,8 +83,8 @@ enum { OSAM_FP64 = 0, OSAM_FP32_FORCE = 1, OSAM_F32X2_FORCE = 2, OSAM_FP64_TANGE
  * GATHER_TILED the gather scheme with the FP64 force evaluated by 8x4x4 element tiles that share
  * their edge interpolation (same results bit for bit), GATHER_TILED_LOWREG the tiled kernel capped at
  * 128 registers (4 instead of 3 resident tiles per SM); the FP32 variants ignore these.  AUTO times
- * the candidates at initialisation and keeps the fastest (explicit Neo-Hookean FP64 subdomains: element
- * blocks of the fixed-point force, gather scheme) */
+ * the candidates at initialisation and keeps the fastest (subdomains with an integer force: its element
+ * blocks, gather scheme) */
 enum {
     OSAM_SCATTER_AUTO = 0,
     OSAM_SCATTER_ATOMIC = 1,
@@ -375,7 +384,11 @@ typedef struct {
     double* C;                /* [r][r(r+1)(r+2)/6] cubic operator (cubic fits), or NULL */
 } osam_fit_output;
 
-/* The regularisation lambda is a field of osam_fit_input (next to the other fit settings it goes with,
+/* The fit's products round like FP64 ones: those with at least 128 terms and 4.2e6 multiplications run on the bf16
+ * tensor cores as digit products where their error is certified to be no larger (per 64 x 64 tile of the result),
+ * else in FP64.
+ *
+ * The regularisation lambda is a field of osam_fit_input (next to the other fit settings it goes with,
  * e.g. the same input serves opinf_select, which ignores it and scans its candidates) rather than a
  * separate argument. */
 OSAM_API int opinf_fit(const osam_fit_input* in, osam_fit_output* out);

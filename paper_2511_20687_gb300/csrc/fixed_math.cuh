@@ -6,7 +6,8 @@
 // order one: its FP64 error is set by F's own rounding (2^-53 of 1), however small grad u is, so 64-bit
 // integers with a fixed binary point carry it more accurately at a fifth of the time.  Measured against
 // a 113-bit reference over displacement gradients from 1e-12 to 0.3, any rotation, nu 0.25 and 0.45: error of an
-// element force 1.1e-17 to 3.5e-16 mu h^2 (rms) here, 4.2e-17 to 4.0e-16 in FP64, smaller in every case.
+// element force 1.1e-17 to 3.5e-16 mu h^2 (rms) here, 4.2e-17 to 4.0e-16 in FP64, smaller in every case.  That is for an
+// element in its own material's unit; kept in a buffer with the unit of a mesh it loses up to kMaxDown bits.
 //
 // Values are int64 with a stated number of fraction bits.  A product takes its operands as balanced
 // digits x = h 2^32 + l (l signed) and returns the rounded high word,
@@ -19,7 +20,7 @@
 // 2^22 at every node (from kMaxU on its nodal values are taken modulo 32 edges: refit), the spread of each displacement component over the element (the kernels with a corner per lane:
 // along each of its edges) below 2.75 edges, column
 // norms of F at the Gauss points below 1.5 (any rotation, 50% stretch), J in (0.53, 1.98), |beta| < 4
-// and pair sums of P below 2 in units of the instance's material scale.  Every intermediate then fits
+// and pair sums of P below 2 in units of the element's material scale.  Every intermediate then fits
 // its format; the bounds are at each step.
 #pragma once
 
@@ -38,8 +39,8 @@ typedef long long i64;
 
 constexpr int kFracU = 59;    // u / h, range +-16
 constexpr int kFracF = 61;    // F at the Gauss points, range +-4
-constexpr int kFracM = 62;    // material factors in units of the instance's scale, at most 1
-constexpr int kFracOut = 54;  // element forces in units of the instance's scale
+constexpr int kFracM = 62;    // material factors in units of the element's scale, at most 1
+constexpr int kFracOut = 54;  // element forces in units of the element's scale, or of the mesh's in the buffer
 constexpr int kMaxU = 12;     // largest |u| / h of the fixed format
 constexpr i64 kBadU = (i64)1 << 63;    // fixed_u of a node outside it (-16)
 constexpr i64 kBadF = (i64)1 << 63;    // stored linearisation of a Gauss point outside the range

@@ -6,14 +6,18 @@
 // additions.  An element outside the range of the formats is evaluated in FP64 (far_element), and its entries hold
 // the FP64 values (hold_f64); so do those of an element too soft for the buffer's unit (kMaxDown).
 //
-// k_force_fx_b is bound by the integer multiply-add pipe: ncu counts 1969 instructions on it and 2994 on
-// the integer ALU per warp, against 717 FP64 instructions (67 to 80 cycles each) of the tiled FP64 kernel.
-// Measured on 40x40x80: 43 us per launch, 186 us for the FP64 kernel; on 96x96x192 480 us, 2360 us.
+// ncu counts 1969 instructions of k_force_fx_b on the integer multiply-add pipe (4 cycles each) and 2994 on the integer
+// ALU per warp, against 717 FP64 instructions (67 to 80 cycles each) of the tiled FP64 kernel.  On large launches the
+// pipe is the bound (0.82 of its issue rate at 5.6 M elements, 0.72 at 1.8 M); on one 40x40x80 mesh (3.3 waves of
+// blocks) it issues 0.63 of that rate warm, and at 1.9 warps per scheduler the warps wait for their own results and for
+// instructions (ncu, cold: per issued instruction 1.5 warps in fixed latencies, 1.0 without an instruction, 0.6 in
+// dispatch, 0.6 for memory, 0.3 for the pipe): the unrolled code is 80 KB, and moving it changes the time by 1 to 2%.
+// Measured on 40x40x80: 40 us per launch, 186 us for the FP64 kernel; on 96x96x192 478 us, 2360 us.
 // The Gauss points are fully unrolled (43.4 us; with the two planes as a loop 45.3), 255 registers and
 // two warps per scheduler: capping at 168 or 128 registers (480 to 680 bytes of spills read back per thread)
 // measured 45.3 and 47.5 us on 40x40x80, 510 and 523 us on 96x96x192; with the Walsh coefficients and one
 // plane's sums in shared memory (168 registers, three blocks per SM, no spills) the 96x96x192 chain step took 58.4
-// instead of 55.5 ms, so more warps do not help: the pipe is the bound.
+// instead of 55.5 ms: more warps did not help.
 #include <cuda_runtime.h>
 
 #include <cstdint>

@@ -138,7 +138,7 @@ struct FomB {
 
 // A node kernel takes one thread per node and component instead of one per node while that leaves it
 // below eight warps per scheduler: its time is then the length of one thread's chain of FP64 instructions
-// and loads, a third with one component.
+// and loads, a third with one component.  (GB300's 152 SMs: the library is built for no other chip.)
 constexpr int kNodeSplitBlocks = 152 * 8 / 3;
 inline bool node_split(const FomB& g) { return g.n_nblk <= kNodeSplitBlocks; }
 

@@ -218,7 +218,8 @@ int setup_fom_group(osam_ctx* ctx, FomGroupH& G, int s, int n, const osam_proble
     CKA(B.us = ctx->alloc<double>(3 * NN));
     B.implicit = descs[0].subdomains[s].integrator == OSAM_IMPLICIT;
     // Force in 64-bit integers: explicit Neo-Hookean groups, and linear elastic and Saint Venant-Kirchhoff groups of
-    // the FP64 modes, whose scatter is left to the library (a scatter mode asked for by name runs its own FP64 kernel).
+    // the FP64 modes (explicit or implicit), whose scatter is left to the library: a scatter mode asked for by name runs
+    // its own FP64 kernel.  Implicit Neo-Hookean groups take the integer kernels of lane_kernels.cu whatever the scatter.
     // The double-float mode's Neo-Hookean force is the fixed-point one too: more accurate than pairs of FP32
     // values, and faster (40x40x80: 40 us per launch against 50).
     const bool integers = descs[0].scatter == OSAM_SCATTER_AUTO || ctx->integer_force;
