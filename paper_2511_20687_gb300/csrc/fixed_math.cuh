@@ -24,11 +24,11 @@
 // its format; the bounds are at each step.
 #pragma once
 
+#include <cmath>
 #ifdef __CUDACC__
 #include <cuda_runtime.h>
 #define OSAM_HD __host__ __device__ __forceinline__
 #else
-#include <cmath>
 #define OSAM_HD inline
 #endif
 
@@ -49,6 +49,7 @@ struct D {
     int h, l;
 };
 
+// |x| below 2^63 - 2^31: the high digit of a larger value would not fit its word
 OSAM_HD D split(i64 x) {
     D d;
     d.l = (int)(unsigned int)x;
@@ -553,7 +554,7 @@ OSAM_HD bool tangent_point(const Cols& C, const Cols& E, D kap2, D mu, D mu3, i6
     const i64 cf = shl(mul(kap2, split(shl(s.J, 3))), 1) - shl(s.beta, 2);      // 59, below 8
     const i64 T = mul(split(shl(da, 2)), nd) + mul(al, FGd);                    // 57
     const i64 Q = mul(split(cf), dJd) - mul_third(T);                           // 57, below 14
-    ok = ok && (hi(Q) ^ (hi(Q) >> 31)) < (4 << 25);
+    ok = ok && (hi(Q) ^ (hi(Q) >> 31)) < (4 << 25) - 1;
     const D db = split(mul(s.inv, split(shl(Q, 4))));                  // 59
     const D be = split(shl(s.beta, 2)), dad = split(da), ah = split((s.alpha + 1) >> 1);   // 59
     int top = 0;
@@ -1016,9 +1017,20 @@ OSAM_HD double f64_held(i64 b) {
     return v;
 }
 
-// fixed-point u / h of a nodal displacement: mantissa (53 bits) times the 63-bit mantissa of 1/h, shifted
-// to 59 fraction bits; kBadU for |u| / h >= 12 and for non-finite values.  ihm in [2^62, 2^63),
-// 1/h = ihm 2^(ihe - 62).
+// x (positive, normal) as m 2^(e - 62), m in [2^62, 2^63 - 2^31) (or half of that, where x's mantissa is within 2^-32 of 2):
+// a value that split() takes
+inline void mantissa63(double x, long long& m, int& e) {
+    int k;
+    m = (long long)std::ldexp(std::frexp(x, &k), 63);
+    e = k - 1;
+    if (m >= 0x7fffffff80000000LL) {
+        m >>= 1;       // exact: a double's mantissa leaves the low 10 bits zero
+        ++e;
+    }
+}
+
+// fixed-point u / h of a nodal displacement: the mantissa as 62 bits (63 would not split near 2) times the mantissa of 1/h
+// (mantissa63: 1/h = ihm 2^(ihe - 62)), shifted to 59 fraction bits; kBadU for |u| / h >= 12 and for non-finite values.
 OSAM_HD i64 fixed_u(double u, i64 ihm, int ihe) {
     unsigned long long b;
 #ifdef __CUDA_ARCH__
@@ -1028,10 +1040,10 @@ OSAM_HD i64 fixed_u(double u, i64 ihm, int ihe) {
 #endif
     const int e = (int)((b >> 52) & 0x7ff);
     if (e == 0) return 0;                                     // zero and subnormals
-    const i64 m = (i64)(((b & 0xfffffffffffffULL) | 0x10000000000000ULL) << 10);   // [2^62, 2^63)
-    const i64 p = mul(m, ihm);                                // [2^60, 2^62): u/h = p 2^(e - 1023 + ihe - 60)
-    const int s = 1 - (e - 1023 + ihe);                       // right shift to 59 fraction bits
-    if (s < -2) return kBadU;                                 // |u| / h >= 8 2^.. (p 2^3 would leave 63 bits)
+    const i64 m = (i64)(((b & 0xfffffffffffffULL) | 0x10000000000000ULL) << 9);    // [2^61, 2^62)
+    const i64 p = mul(m, ihm);                                // [2^58, 2^61): u/h = p 2^(e - 1023 + ihe - 59)
+    const int s = 1023 - e - ihe;                             // right shift to 59 fraction bits
+    if (s < -3) return kBadU;                                 // (p 2^4 could leave 64 bits)
     i64 v;
     if (s <= 0) v = shl(p, -s);
     else v = s > 62 ? 0 : (p + ((i64)1 << (s - 1))) >> s;
@@ -1053,9 +1065,9 @@ OSAM_HD bool wrapped_u(double u, i64 ihm, int ihe, i64& v, int& coarse) {
     v = coarse = 0;
     const int e = (int)((b >> 52) & 0x7ff);
     if (e == 0) return true;
-    const i64 p = mul((i64)(((b & 0xfffffffffffffULL) | 0x10000000000000ULL) << 10), ihm);
-    const int s = 1 - (e - 1023 + ihe);                       // u / h in [2^(1 - s), 2^(3 - s))
-    if (s < -19) return false;
+    const i64 p = mul((i64)(((b & 0xfffffffffffffULL) | 0x10000000000000ULL) << 9), ihm);
+    const int s = 1023 - e - ihe;                             // u / h in [2^(-1 - s), 2^(2 - s))
+    if (s < -20) return false;
     if (s <= 0) v = shl(p, -s);
     else v = s > 62 ? 0 : (p + ((i64)1 << (s - 1))) >> s;
     coarse = s + 51 > 62 ? 0 : (int)(p >> (s + 51));

@@ -382,9 +382,7 @@ int elem_grid(int ne) { return grid_for(8LL * ne, kLaneBlock); }
 }  // namespace
 
 void fixed_point_inverse(double x, long long& m, int& e) {
-    int k;
-    m = (long long)std::ldexp(std::frexp(x, &k), 63);
-    e = k - 1;
+    mantissa63(x, m, e);
 }
 
 cudaError_t launch_elem_force_nh(int scatter, const ElemArgs& a, cudaStream_t s, int lanes) {

@@ -246,7 +246,7 @@ cudaError_t launch_force_fx_b(const FomB& g, const int* active, const TraceFuse&
 cudaError_t launch_node_fx_b(const FomB& g, const int* active, int slot1, int slot2, int predict_only,
                              const double* ucur, double* unext, double dt, cudaStream_t s);
 // Neo-Hookean element level and implicit groups in 64-bit integers, 8 lanes per element (lane_kernels.cu);
-// fixed_point_inverse: x as m 2^(e - 62), m in [2^62, 2^63)
+// fixed_point_inverse: x as m 2^(e - 62) for the kernels' 1/h (mantissa63, fixed_math.cuh)
 void fixed_point_inverse(double x, long long& m, int& e);
 cudaError_t launch_elem_force_nh(int scatter, const ElemArgs& a, cudaStream_t s, int lanes = -1);
 cudaError_t launch_elem_vjp_nh(int scatter, const ElemArgs& a, const double* ybar, int ysn, long long ysc,

@@ -346,3 +346,74 @@ def test_step_with_a_layer_torn_by_the_modulus(n, nz):
     for f in range(3):
         x, y = a.state(0)[f], b.state(0)[f]
         assert np.linalg.norm(x - y) <= 1e-12 * np.linalg.norm(y)
+
+
+@pytest.fixture(scope="module")
+def fixed_u(tmp_path_factory):
+    return build(tmp_path_factory, "fixed_u_check.cpp")
+
+
+NEAR_TWO = [np.nextafter(0.5, 1), 0.5 * (1 + 1e-11), np.nextafter(0.0078125, 1), 2.0 ** -7 * (1 + 2.0 ** -33)]
+
+
+@pytest.mark.parametrize("h", [H, 0.0125, 1.0, 0.5, np.nextafter(0.5, 0)] + NEAR_TWO)
+def test_displacements_of_every_mantissa(fixed_u, h):
+    """Mantissas of u and of 1/h up to the largest: half a unit of rounding and 0.75 2^-58 of the value, in units of
+    2^-59; only |u| / h >= 12 is marked."""
+    rng = np.random.default_rng(31)
+    m = np.concatenate([1 + rng.uniform(0, 1, 200), 2 - 2.0 ** -np.arange(1, 53), 1 + 2.0 ** -np.arange(1, 53)])
+    u = np.concatenate([s * m * 2.0 ** e for s in (-1, 1) for e in range(-60, 12)])
+    r = fixed_u([(h, v) for v in u])
+    x = np.abs(r[:, 2])
+    bound = 0.51 + 1.5 * x
+    assert (np.isnan(r[:, 0]) == (x >= 12)).mean() > 0.999 and not np.isnan(r[x < 11.99, 0]).any()
+    assert np.isnan(r[x > 12.01, 0]).all()
+    near = ~np.isnan(r[:, 0])
+    assert (np.abs(r[near, 0]) <= bound[near]).all()
+    assert (np.abs(r[:, 1]) <= bound).all()
+    assert (np.abs(r[:, 3] - 256 * r[:, 2]) <= 1.001).all()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("material", ["nh", "le", "svk"])
+@pytest.mark.parametrize("h", NEAR_TWO)
+@pytest.mark.parametrize("dims", [(5, 4, 3), (41, 41, 41)])   # 8 lanes and one thread per element
+def test_edges_just_above_a_power_of_two(material, h, dims):
+    """1/h with a mantissa just below 2, against plain torch as in test_integer_elements.py (strains of 1e-2: 1e-12)."""
+    import torch
+
+    from paper_2511_20687_gb300 import osam
+    from tests.test_integer_elements import reference
+    g = torch.Generator(device="cuda").manual_seed(19)
+    nn = (dims[0] + 1) * (dims[1] + 1) * (dims[2] + 1)
+    ne = dims[0] * dims[1] * dims[2]
+    u = h * 0.02 * (torch.rand(nn, 3, generator=g, device="cuda", dtype=torch.float64) - 0.5)
+    f = torch.empty_like(u)
+    osam.hex8_force(dims, h, material, 4e8, 4e8, u, f)
+    full = torch.full((ne,), 4e8, device="cuda", dtype=torch.float64)
+    r = reference(torch, dims, h, material, full, full, u.clone().requires_grad_(material != "svk"))
+    assert (f - r).norm() <= 1e-12 * r.norm()
+    if material != "svk":
+        y = torch.rand(nn, 3, generator=g, device="cuda", dtype=torch.float64)
+        ub = torch.empty_like(u)
+        osam.hex8_force_vjp(dims, h, material, 4e8, 4e8, u, y, ub)
+        v = u.clone().requires_grad_(True)
+        w, = torch.autograd.grad(reference(torch, dims, h, material, full, full, v), v, y)
+        assert (ub - w).norm() <= 1e-12 * w.norm()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("material", ["nh", "le", "svk"])
+@pytest.mark.parametrize("integrator", ["explicit", "implicit"])
+def test_step_with_edges_just_above_a_power_of_two(material, integrator):
+    """The step against the oracle (1e-9 as everywhere)."""
+    from oracle import oracle as O
+    from paper_2511_20687_gb300 import osam
+    p = W.single_bar("near", 4, 8, material, 1e9, 0.25, 1000.0, 1e-3, 1e-6, 2, h=float(np.nextafter(0.0078125, 1)))
+    p.subdomains[0].integrator = integrator
+    a, b = osam.Problem(p), O.Problem(p)
+    a.step()
+    b.step()
+    for f in range(3):
+        x, y = a.state(0)[f], b.state(0)[f]
+        assert np.linalg.norm(x - y) <= 1e-9 * np.linalg.norm(y)
